@@ -63,6 +63,8 @@ Layout make_layout(const mc_desc& d) {
   o += round_up((3 * (size_t)d.L + 4 + 3 * kScaleBlocks) * sizeof(double), 256);
   y.off_fver = o;
   o += round_up(sizeof(unsigned long long) + (size_t)d.L * sizeof(int), 256);
+  y.off_bexp = o;
+  o += round_up((size_t)(7 + y.nfar) * (size_t)d.L * sizeof(int), 256);   // either apply mode
   y.lp = d.dtype == MC_F32 ? 1 : d.dtype == MC_BF16 ? 2 : 0;
   if (y.lp) {
     const size_t es = y.lp == 1 ? 4 : 2;
@@ -168,6 +170,12 @@ static bool fused_ok(const mc_chain* c) {
 // chains use the direct residual.
 static bool split_resid_ok(const mc_chain* c) { return c->d.stair <= 2 && c->lay.nfar == 0; }
 
+// block_exp of a plane's blocks (written by the factorisation).
+static int* plane_exp(const mc_chain* c, int plane) {
+  return (int*)(c->ws + c->lay.off_bexp) + (size_t)plane * (size_t)c->lay.L;
+}
+const int* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); }
+
 // n stair sweeps src -> dst (in place allowed) as fused launches of at most
 // kMaxFusedSweeps sweeps, each followed by the normalisation (with the step
 // error after the last).  With resid (block-tridiagonal chains only) the last
@@ -198,6 +206,9 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
     a.A = c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe;
     a.B = c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe;
     a.C = c->planes + kPlaneNINV * pe;
+    a.eA = plane_exp(c, coupled ? kPlaneWLO : kPlaneTLO);
+    a.eB = plane_exp(c, coupled ? kPlaneWUP : kPlaneTUP);
+    a.eC = plane_exp(c, kPlaneNINV);
     a.x_in = in;
     a.W = c->xb;
     a.Z = c->z;
@@ -224,17 +235,8 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
       a.prev = K == 1 ? in : c->xb;
       a.rsum = rsum;
     }
-    // block Gauss-Seidel runs at most min(K, L/2) units at once (one per sweep
-    // in flight), one block per unit; the launcher caps the grid at the blocks
-    // resident at once
-    int nb = c->nb_fused;
-    if (a.bgs) {
-      const int64_t par = K < (L + 1) / 2 ? K : (L + 1) / 2;
-      nb = par < (1 << 30) ? (int)par : (1 << 30);
-    }
-    if (c->tune_bps > 0 && c->tune_bps * c->num_sms < nb) nb = c->tune_bps * c->num_sms;
     CK(cudaMemsetAsync(c->fclaim, 0, cnt_bytes, s));
-    CK(launch_sweeps_fused(a, coupled, nb, s));
+    CK(launch_sweeps_fused(a, coupled, c->tune_bps, c->num_sms, s));
     if (ev && final) CK(cudaEventRecord(ev[1], s));
     CK(launch_fused_scale(c->flsum, L, K, with_resid ? rsum : nullptr, a.P0, scale, scale + 4,
                           &c->hdr->ticket[4], s));
@@ -409,11 +411,6 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   if (lay.L < sms) wr = lay.L;
   if (wr > kMaxWarps) wr = kMaxWarps;
   c->nb_resid = (int)((wr + kWarpsPerBlock - 1) / kWarpsPerBlock);
-  // fused launches claim units dynamically: the full resident grid, but no
-  // more warps than levels
-  int64_t wf = wps * sms;
-  if (wf > lay.L) wf = lay.L;
-  c->nb_fused = (int)((wf + kWarpsPerBlock - 1) / kWarpsPerBlock);
   c->tune_bps = 0;
   c->tune_lpu = 1;
   int64_t nbn = (lay.N + 4 * kNormThreads - 1) / (4 * kNormThreads);
@@ -491,6 +488,7 @@ int mc_create_banded(const mc_desc* desc, const double* const* diags, void* work
     double* plane = c->planes + (size_t)(y.far_base + j) * pe;
     fd.off[j] = d;
     fd.plane[j] = plane;
+    fd.bexp[j] = plane_exp(c, y.far_base + j);
     if (launch_layout_diag(diags[-d + lo], d, plane, y, c->user) != cudaSuccess) rc = MC_ERR_CUDA;
   }
   if (rc == MC_OK && cudaMemcpyAsync((char*)c->hdr + kFarDescOffset, &fd, sizeof(fd),
@@ -526,10 +524,21 @@ int mc::chain_factor_async(mc_chain* c) {
   }
   CK(launch_factor(c->planes, c->lay, c->hdr, c->d.apply == MC_APPLY_COUPLED, c->num_sms,
                    c->user));
+  const size_t pe = c->lay.plane_bytes / sizeof(double);
+  const bool coupled = c->d.apply == MC_APPLY_COUPLED;
+  if (c->lay.lp == 0) {   // the planes that FP64 sweeps stream
+    static const int kOps[2][3] = {{kPlaneTLO, kPlaneTUP, kPlaneNINV}, {kPlaneWLO, kPlaneWUP, -1}};
+    for (int i = 0; i < 3; ++i) {
+      const int p = kOps[coupled][i];
+      if (p >= 0) CK(launch_block_exp(c->planes + p * pe, plane_exp(c, p), c->lay, c->user));
+    }
+    for (int j = 0; j < c->lay.nfar; ++j) {
+      const int p = c->lay.far_base + j;
+      CK(launch_block_exp(c->planes + p * pe, plane_exp(c, p), c->lay, c->user));
+    }
+  }
   if (c->lay.lp) {
-    const size_t pe = c->lay.plane_bytes / sizeof(double);
     const int bf16 = c->lay.lp == 2;
-    const bool coupled = c->d.apply == MC_APPLY_COUPLED;
     CK(launch_lp_convert(c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe, c->ws + c->lay.off_lpA,
                          bf16, lpSc(c), 2, c->lay, c->lay.lp_bs, c->user));
     CK(launch_lp_convert(c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe, c->ws + c->lay.off_lpB,

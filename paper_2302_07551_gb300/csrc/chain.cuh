@@ -19,7 +19,6 @@ struct mc_chain {
   double* flsum;             // fused launches: [2][L] level sums, 2 scales, block partials
   int* fver;                 // [L] completion counters, after the queue counter
   unsigned long long* fclaim;
-  int nb_fused;              // grid of the fused multi-sweep kernel
   int tune_bps;              // blocks per SM of the fused launches (0: default)
   int tune_lpu;              // levels per unit of the low-precision fused launches
   cudaGraphExec_t gexec;     // cached chunk graph of mc_solve
@@ -36,6 +35,8 @@ int chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaStream
 int chain_factor_async(mc_chain* c);
 // Enqueue the direct residual of x (and q = (-T_dd)^{-1} r when q != NULL).
 int chain_residual_async(mc_chain* c, const double* x, cudaStream_t s, float* q);
+// block_exp per level of one plane (mc_internal.cuh).
+const int* chain_bexp(const mc_chain* c, int plane);
 const void* chain_lpA(mc_chain* c);
 const void* chain_lpB(mc_chain* c);
 const float* chain_lpC(mc_chain* c);

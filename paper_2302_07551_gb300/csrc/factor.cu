@@ -2,6 +2,7 @@
 // the operators that apply Q_{l,l}^{-1} in Algorithm 2 (steps 2 and 3).
 #include <math.h>
 
+#include "fixed_dev.cuh"
 #include "mc_internal.cuh"
 
 namespace mc {
@@ -301,7 +302,28 @@ __global__ void k_layout_diag(const double* __restrict__ diag, int d, double* __
   }
 }
 
+// block_exp (mc_internal.cuh): one warp per block, read once.
+__global__ void __launch_bounds__(256) k_block_exp(const double* __restrict__ plane, int* bexp,
+                                                   int64_t L, int m, int ms) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t l = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; l < L; l += nw) {
+    const double* p = plane + (size_t)l * ms;
+    unsigned e = 0u;   // a negative entry reads as >= 2048
+    for (int i = lane; i < m * m; i += 32) e = max(e, (unsigned)__double2hiint(__ldcs(p + i)) >> 20);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) bexp[l] = (e >= (unsigned)dev::kMinFixedExp && e < 2047u) ? (int)e : kNoFixed;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_block_exp(const double* plane, int* bexp, const Layout& lay, cudaStream_t s) {
+  int64_t nb = (lay.L + 7) / 8;
+  if (nb > 2048) nb = 2048;
+  k_block_exp<<<(int)nb, 256, 0, s>>>(plane, bexp, lay.L, lay.m, lay.ms);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_layout_diag(const double* diag, int d, double* plane, const Layout& lay,
                                cudaStream_t s) {

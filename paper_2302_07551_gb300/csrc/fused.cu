@@ -1,7 +1,7 @@
 // Several staircase sweeps (Algorithm 2, repeated) in one persistent launch.
 //
 // Work units are (sweep k, half-sweep h, level l), claimed in that order from
-// one queue counter.  Half-sweep 1 of sweep k (the diagonal-only stair rows)
+// one queue counter by teams of warps (team_dev.cuh).  Half-sweep 1 of sweep k (the diagonal-only stair rows)
 // reads its neighbours as left by half-sweep 2 of sweep k-1; half-sweep 2
 // reads its neighbours as left by half-sweep 1 of sweep k.  So each unit
 // depends on exactly two earlier units, the neighbour levels l-1 and l+1, and
@@ -14,9 +14,9 @@
 // updates) have completed, which is exactly the condition it waits for.  The
 // last sweep writes Z instead, so that W keeps z_{K-1} for the step error.
 //
-// Progress: a warp handles its claimed units in increasing queue order and
+// Progress: a team handles its claimed units in increasing queue order and
 // every unit depends only on units earlier in the queue, all claimed by
-// running warps, so the earliest unfinished unit can always proceed.  Each
+// running teams, so the earliest unfinished unit can always proceed.  Each
 // wait is still bounded (FusedArgs::wait_ns of the GPU's global timer); on
 // expiry the warp latches MC_ERR_TIMEOUT and carries on, so the launch
 // always ends.
@@ -30,13 +30,14 @@
 // streams the off-diagonal blocks of half the levels once, a third of one
 // sweep's bytes in inverse mode, instead of all three blocks of every level.
 //
-// Values and level sums do not depend on which warp handles which unit, and
+// Values and level sums do not depend on which team handles which unit, and
 // the sums are reduced per level in a fixed order: results are bitwise
 // reproducible for any grid.
 #include <math.h>
 
 #include "mc_internal.cuh"
 #include "sweep_dev.cuh"
+#include "team_dev.cuh"
 #include "wave_dev.cuh"
 
 namespace mc {
@@ -45,85 +46,251 @@ namespace {
 
 using namespace dev;
 
-template <int R, bool COUPLED, bool PAIRED>
-__global__ void __launch_bounds__(256, Tune<R>::MINB) k_sweeps(FusedArgs a) {
-  extern __shared__ double vsh[];
-  const int lane = threadIdx.x & 31;
-  double* slice = vsh + (threadIdx.x >> 5) * 3 * 32 * R;
-  const unsigned long long sweeps = (unsigned long long)a.K * (unsigned long long)a.L;
-  const unsigned long long total = sweeps + (a.with_resid ? (unsigned long long)a.P0 : 0ull);
-  unsigned long long q0 = claim_unit(a.claim, lane);
-  unsigned long long q = __shfl_sync(kFull, q0, 0);
-  while (q < total) {
-    // claim the next unit now; its index is needed only after this one
-    q0 = claim_unit(a.claim, lane);
-    if (q >= sweeps) {
-      // residual unit of diagonal-only level l: neighbours must hold z_K
-      const int64_t u = (int64_t)(q - sweeps);
-      const int64_t l = 2 * u + a.par0;
-      wait_neighbours(a.ver, l, a.L, (int)a.K, &a.hdr->status, lane, a.wait_ns);
-      const double t = level_resid_split<R, PAIRED>(a.RA, a.RB, a.Z, a.prev, l, a.L, a.m, a.ms,
-                                                    slice, lane);
-      if (lane == 0) a.rsum[u] = t;
-      q = __shfl_sync(kFull, q0, 0);
-      continue;
-    }
-    const int64_t k = (int64_t)(q / (unsigned long long)a.L);
-    const int64_t r = (int64_t)q - k * a.L;
-    const bool h2 = r >= a.P0;
-    const int64_t l = h2 ? 2 * (r - a.P0) + (1 - a.par0) : 2 * r + a.par0;
-    const bool last = k == a.K - 1;
-    double* dst = last ? a.Z : a.W;
-    // half-sweep 1 reads z_k (x_in for k = 0); half-sweep 2 reads z_{k+1}
-    const double* src = h2 ? dst : (k == 0 ? a.x_in : a.W);
-    const int need = (int)(h2 ? k + 1 : k);
-    if (need > 0) wait_neighbours(a.ver, l, a.L, need, &a.hdr->status, lane, a.wait_ns);
-    // e^T z is needed of the last two sweeps only
-    const bool want = k >= a.K - 2;
-    const double t = level_sweep2<R, COUPLED, PAIRED, true, true>(
-        a.A, a.B, a.C, src, src, dst, l, a.L, a.m, a.ms, slice, lane, 1.0, nullptr, nullptr,
-        nullptr, want);
-    if (want && lane == 0) a.lsum[(k & 1) * a.L + l] = t;
-    publish(a.ver + l, (int)(k + 1), lane);
-    q = __shfl_sync(kFull, q0, 0);
-  }
+// Threads per block and blocks per SM of a team kernel: 24 warps an SM.
+template <int TW>
+struct TeamBlock {
+  static constexpr int T = (TW == 3 || TW == 6) ? 192 : 256;
+  static constexpr int B = 768 / T;
+};
+
+// Largest exponent over the team's warps.
+template <int TW>
+__device__ __forceinline__ int team_max(const int* e) {
+  int v = e[0];
+#pragma unroll
+  for (int i = 1; i < TW; ++i) v = max(v, e[i]);
+  return v;
 }
 
-// Block-banded chains (Algorithm 2 with off-staircase terms, inverse mode):
-// every row also adds sum_d T_{l,l+d} x_{l+d} over the far diagonals |d| >= 2
-// from the sweep's input, at levels of both parities, so the sweeps cannot
-// update in place.  Y_0 = x_in; sweep k reads Y_k and writes Y_{k+1} into W
-// (k even) or Z (k odd), over Y_{k-1}.  A unit of sweep k at level l waits
-// until every level within the band l - bw .. l + bw has finished sweep k - 1
-// (its inputs are ready and every reader of the Y_{k-1} it overwrites is
-// done); a coupled-row unit also waits for half-sweep 1 of sweep k at l - 1
-// and l + 1.
-template <int R>
-__global__ void __launch_bounds__(256, Tune<R>::MINB) k_sweeps_banded(FusedArgs a) {
-  extern __shared__ double vsh[];
-  const int lane = threadIdx.x & 31;
-  double* slice = vsh + (threadIdx.x >> 5) * 3 * 32 * R;
-  const unsigned long long total = (unsigned long long)a.K * (unsigned long long)a.L;
-  unsigned long long q0 = claim_unit(a.claim, lane);
-  unsigned long long q = __shfl_sync(kFull, q0, 0);
-  while (q < total) {
-    q0 = claim_unit(a.claim, lane);
-    const int64_t k = (int64_t)(q / (unsigned long long)a.L);
-    const int64_t r = (int64_t)q - k * a.L;
-    const bool h2 = r >= a.P0;
-    const int64_t l = h2 ? 2 * (r - a.P0) + (1 - a.par0) : 2 * r + a.par0;
-    const double* y = k == 0 ? a.x_in : ((k & 1) ? a.W : a.Z);   // Y_k
-    double* dst = (k & 1) ? a.Z : a.W;                             // Y_{k+1}
-    if (k > 0 || h2)
-      wait_band(a.ver, l, a.L, a.bw, (int)k, (int)(h2 ? k + 1 : k), &a.hdr->status, lane,
-                a.wait_ns);
-    const double* near = h2 ? dst : y;
-    const bool want = k >= a.K - 2;
-    const double t = level_sweep2<R, false, false, true, true>(
-        a.A, a.B, a.C, near, near, dst, l, a.L, a.m, a.ms, slice, lane, 1.0, a.far, y, y, want);
-    if (want && lane == 0) a.lsum[(k & 1) * a.L + l] = t;
-    publish(a.ver + l, (int)(k + 1), lane);
+// Rows first, first + stride, ... of one vector into a staged slot.
+template <int TW, int RW>
+__device__ __forceinline__ void stage_rows(double* v, uint64_t* x, int* emax,
+                                           const double (&y)[RW], int first, int stride, int w,
+                                           int lane) {
+  unsigned e = 0u;
+#pragma unroll
+  for (int i = 0; i < RW; ++i) {
+    v[first + stride * i] = y[i];
+    x[first + stride * i] = fixed_entry(y[i]);
+    e = max(e, (unsigned)__double2hiint(y[i]) >> 20);
+  }
+  e = __reduce_max_sync(kFull, e);
+  if (lane == 0) emax[w] = (int)e;
+}
+
+// Sum of the warps' values in warp order (valid on the team's first warp).
+template <int TW>
+__device__ __forceinline__ double team_total(double t, double* part, int w, int lane, int bar) {
+  if constexpr (TW == 1) return t;
+  if (lane == 0) part[w] = t;
+  team_sync<TW>(bar);
+  double v = part[0];
+#pragma unroll
+  for (int i = 1; i < TW; ++i) v += part[i];
+  return v;
+}
+
+// Shared memory of one team: a ring of two staged products (a warp that writes
+// slot i + 1 has passed the barrier of slot i, so every warp of the team has
+// finished reading slot i - 1), the largest exponents found by each warp, the
+// units to come, and partial level sums.
+// The staged vectors are read in 16-byte pairs, so every team's slots start on a
+// 16-byte boundary.
+template <int TW, int RW>
+struct alignas(16) TeamShared {
+  TeamSlot<32 * RW * TW> slot[2];
+  int emax[2][2][TW];
+  unsigned long long next[2];
+  double part[TW];
+};
+
+// MC: the block size if it equals 32 RW TW, else 0.  BANDED: block-banded
+// chains (Algorithm 2 with off-staircase terms, inverse mode): every row also
+// adds sum_d T_{l,l+d} x_{l+d} over the far diagonals |d| >= 2 from the sweep's
+// input, at levels of both parities, so the sweeps cannot update in place.
+// Y_0 = x_in; sweep k reads Y_k and writes Y_{k+1} into W (k even) or Z (k
+// odd), over Y_{k-1}.  A unit of sweep k at level l waits until every level
+// within the band l - bw .. l + bw has finished sweep k - 1 (its inputs are
+// ready and every reader of the Y_{k-1} it overwrites is done); a coupled-row
+// unit also waits for half-sweep 1 of sweep k at l - 1 and l + 1.
+//
+// A level's completion counter grows by TW per write (each warp of the team
+// releases its own rows).
+template <int TW, int RW, int MC, bool COUPLED, bool PAIRED, bool BANDED>
+__global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(FusedArgs a) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  using Sh = TeamShared<TW, RW>;
+  static_assert(sizeof(Sh) % 16 == 0 && sizeof(TeamSlot<32 * RW * TW>) % 16 == 0, "pair loads");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / TW, w = warp % TW, tt = threadIdx.x - team * TW * 32;
+  Sh& sh = reinterpret_cast<Sh*>(team_smem)[team];
+  const int bar = 1 + team;
+  const int m = MC ? MC : a.m;
+  const int row0 = 32 * RW * w;
+  const unsigned long long sweeps = (unsigned long long)a.K * (unsigned long long)a.L;
+  const unsigned long long total = sweeps + (a.with_resid ? (unsigned long long)a.P0 : 0ull);
+  // paired chains: T_lo is zero in rows m/2.. of columns ..m/2, T_up in rows
+  // ..m/2 of columns m/2.. (RW = 1: a warp's rows lie on one side)
+  const int lo0 = PAIRED && 2 * row0 >= m ? m / 2 : 0;
+  const int up1 = PAIRED && 2 * row0 < m ? m / 2 : m;
+  int s = 0;   // ring position
+  // one warp claims for the team; with one warp a unit ahead of use, with more
+  // two ahead (the unit travels through shared memory with a barrier)
+  unsigned long long q0 = w == 0 ? claim_unit(a.claim, lane) : 0ull, q;
+  if constexpr (TW == 1) {
     q = __shfl_sync(kFull, q0, 0);
+  } else {
+    if (w == 0 && lane == 0) sh.next[1] = q0;
+    if (w == 0) q0 = claim_unit(a.claim, lane);
+    team_sync<TW>(bar);
+    q = sh.next[1];
+  }
+  int turn = 0;
+  while (q < total) {
+    unsigned long long qn = 0ull;
+    if constexpr (TW == 1) {
+      q0 = claim_unit(a.claim, lane);   // its index is needed only after this unit
+    } else if (w == 0 && lane == 0) {
+      sh.next[turn] = q0;
+    }
+    const bool resid = !BANDED && q >= sweeps;
+    const int64_t k = resid ? a.K : (int64_t)(q / (unsigned long long)a.L);
+    const int64_t r = (int64_t)q - k * a.L;
+    const bool h2 = !resid && r >= a.P0;
+    const int64_t l = h2 ? 2 * (r - a.P0) + (1 - a.par0) : 2 * r + a.par0;
+    const bool has_lo = l > 0, has_up = l < a.L - 1;
+    const bool last = k == a.K - 1;
+    double* dst = BANDED ? ((k & 1) ? a.Z : a.W) : (last ? a.Z : a.W);
+    // half-sweep 1 reads z_k (x_in for k = 0); half-sweep 2 reads z_{k+1}; a
+    // residual unit z_K and z_{K-1}
+    const double* y = k == 0 ? a.x_in : (BANDED && !(k & 1)) ? a.Z : a.W;
+    const double* src = resid ? a.Z : h2 ? dst : y;
+    const int need = (int)(h2 ? k + 1 : k);
+    if constexpr (BANDED) {
+      if (need > 0)
+        wait_band(a.ver, l, a.L, a.bw, (int)k * TW, need * TW, &a.hdr->status, lane, a.wait_ns);
+    } else {
+      if (need > 0) wait_neighbours(a.ver, l, a.L, need * TW, &a.hdr->status, lane, a.wait_ns);
+    }
+    // stage both neighbours: thread tt of the team loads rows tt, tt + 32 TW
+    {
+      unsigned e0 = 0u, e1 = 0u;
+      double x0[RW], x1[RW];
+#pragma unroll
+      for (int i = 0; i < RW; ++i) {
+        const int row = tt + 32 * TW * i;
+        x0[i] = has_lo && row < m ? __ldcg(src + (l - 1) * m + row) : 0.0;
+        x1[i] = has_up && row < m ? __ldcg(src + (l + 1) * m + row) : 0.0;
+      }
+      if (resid) {
+#pragma unroll
+        for (int i = 0; i < RW; ++i) {
+          const int row = tt + 32 * TW * i;
+          if (has_lo && row < m) x0[i] -= __ldcg(a.prev + (l - 1) * m + row);
+          if (has_up && row < m) x1[i] -= __ldcg(a.prev + (l + 1) * m + row);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < RW; ++i) {
+        const int row = tt + 32 * TW * i;
+        sh.slot[s].v[0][row] = x0[i];
+        sh.slot[s].v[1][row] = x1[i];
+        sh.slot[s].x[0][row] = fixed_entry(x0[i]);
+        sh.slot[s].x[1][row] = fixed_entry(x1[i]);
+        e0 = max(e0, (unsigned)__double2hiint(x0[i]) >> 20);
+        e1 = max(e1, (unsigned)__double2hiint(x1[i]) >> 20);
+      }
+      e0 = __reduce_max_sync(kFull, e0);
+      e1 = __reduce_max_sync(kFull, e1);
+      if (lane == 0) {
+        sh.emax[s][0][w] = (int)e0;
+        sh.emax[s][1][w] = (int)e1;
+      }
+    }
+    team_sync<TW>(bar);
+    if constexpr (TW > 1) {
+      qn = sh.next[turn];
+      turn ^= 1;
+      if (w == 0) q0 = claim_unit(a.claim, lane);
+    }
+    double acc[RW];
+#pragma unroll
+    for (int i = 0; i < RW; ++i) acc[i] = 0.0;
+    if (resid) {
+      // ||T_lo d_{l-1} + T_up d_{l+1}||_1, d = z_K - z_{K-1} (signed: FP64 pipe)
+      if (has_lo)
+        rows_f64<RW, MC>(acc, a.RA + (size_t)l * a.ms, sh.slot[s].v[0], lo0, m, m, row0, lane);
+      if (has_up)
+        rows_f64<RW, MC>(acc, a.RB + (size_t)l * a.ms, sh.slot[s].v[1], 0, up1, m, row0, lane);
+      double t = 0.0;
+#pragma unroll
+      for (int i = 0; i < RW; ++i) t += fabs(acc[i]);
+      t = team_total<TW>(warp_sum(t), sh.part, w, lane, bar);
+      if (w == 0 && lane == 0) a.rsum[r] = t;
+      s ^= 1;
+      q = TW == 1 ? __shfl_sync(kFull, q0, 0) : qn;
+      continue;
+    }
+    if (has_lo)
+      rows_product<RW, MC>(acc, a.A + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], a.eA[l],
+                           team_max<TW>(sh.emax[s][0]), lo0, m, m, row0, lane);
+    if (has_up)
+      rows_product<RW, MC>(acc, a.B + (size_t)l * a.ms, sh.slot[s].v[1], sh.slot[s].x[1], a.eB[l],
+                           team_max<TW>(sh.emax[s][1]), 0, up1, m, row0, lane);
+    if constexpr (BANDED) {
+      const int n = a.far->n;
+      for (int j = 0; j < n; ++j) {
+        const int64_t kk = l + a.far->off[j];
+        if (kk < 0 || kk >= a.L) continue;
+        s ^= 1;
+        double x0[RW];
+#pragma unroll
+        for (int i = 0; i < RW; ++i) {
+          const int row = tt + 32 * TW * i;
+          x0[i] = row < m ? __ldcg(y + kk * m + row) : 0.0;
+        }
+        stage_rows<TW, RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], x0, tt, 32 * TW, w,
+                           lane);
+        team_sync<TW>(bar);
+        rows_product<RW, MC>(acc, a.far->plane[j] + (size_t)l * a.ms, sh.slot[s].v[0],
+                             sh.slot[s].x[0], a.far->bexp[j][l], team_max<TW>(sh.emax[s][0]), 0,
+                             m, m, row0, lane);
+      }
+    }
+    if constexpr (!COUPLED) {
+      s ^= 1;
+      stage_rows<TW, RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], acc, row0 + lane, 32, w,
+                         lane);
+      team_sync<TW>(bar);
+#pragma unroll
+      for (int i = 0; i < RW; ++i) acc[i] = 0.0;
+      rows_product<RW, MC>(acc, a.C + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], a.eC[l],
+                           team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
+    }
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < RW; ++i) {
+      const int row = row0 + lane + 32 * i;
+      if (row < m) {
+        dst[l * m + row] = acc[i];
+        t += acc[i];
+      }
+    }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) {
+      if constexpr (TW == 1)
+        st_release(a.ver + l, (int)(k + 1));
+      else
+        red_release(a.ver + l, 1);
+    }
+    // e^T z is needed of the last two sweeps only (FP64 adds cost issue slots)
+    if (k >= a.K - 2) {
+      t = team_total<TW>(warp_sum(t), sh.part, w, lane, bar);
+      if (w == 0 && lane == 0) a.lsum[(k & 1) * a.L + l] = t;
+    }
+    s ^= 1;
+    q = TW == 1 ? __shfl_sync(kFull, q0, 0) : qn;
   }
 }
 
@@ -302,19 +469,66 @@ __global__ void __launch_bounds__(256) k_fused_scale(const double* lsum, int64_t
   }
 }
 
-template <int R, bool C, bool P = false>
-cudaError_t sweeps_r(const FusedArgs& a, int nb, cudaStream_t s) {
-  static bool done = false;
-  const size_t smem = (size_t)kWarpsPerBlock * 3 * 32 * R * sizeof(double);
-  if (!done && smem > 40 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_sweeps<R, C, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+// bps: resident blocks per SM (0: all the kernel's occupancy allows); no more
+// teams than levels.
+template <int TW, int RW, int MC, bool C, bool P, bool BANDED>
+cudaError_t sweeps_k(const FusedArgs& a, int bps, int sms, cudaStream_t s) {
+  constexpr int T = TeamBlock<TW>::T, teams = T / 32 / TW;
+  static int occ = 0;
+  const size_t smem = teams * sizeof(TeamShared<TW, RW>);
+  if (occ == 0) {
+    cudaError_t e = cudaFuncSetAttribute(k_sweeps<TW, RW, MC, C, P, BANDED>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int o = 0;
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_sweeps<TW, RW, MC, C, P, BANDED>, T,
+                                                        smem);
     if (e != cudaSuccess) return e;
-    done = true;
+    occ = o < 1 ? 1 : o;
   }
-  k_sweeps<R, C, P><<<nb, 256, smem, s>>>(a);
+  int64_t nb = (int64_t)(bps > 0 && bps < occ ? bps : occ) * sms;
+  const int64_t need = (a.L + teams - 1) / teams;
+  if (nb > need) nb = need;
+  k_sweeps<TW, RW, MC, C, P, BANDED><<<(int)nb, T, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int TW, int RW, bool C, bool P, bool BANDED>
+cudaError_t sweeps_m(const FusedArgs& a, int bps, int sms, cudaStream_t s) {
+  if constexpr (P)
+    return sweeps_k<TW, RW, 32 * RW * TW, C, P, BANDED>(a, bps, sms, s);
+  else
+    return a.m == 32 * RW * TW ? sweeps_k<TW, RW, 32 * RW * TW, C, P, BANDED>(a, bps, sms, s)
+                               : sweeps_k<TW, RW, 0, C, P, BANDED>(a, bps, sms, s);
+}
+
+// Team of a block size: two rows per lane (half the warps per level, so half
+// the staging and waiting per streamed byte) while a half-sweep has more units
+// than teams in flight; one row per lane (twice the warps per level) when it
+// has fewer, so that units neither wait for their neighbours' previous sweep
+// nor leave warps without work.
+template <bool C, bool BANDED>
+cudaError_t sweeps_team(const FusedArgs& a, int bps, int sms, cudaStream_t s) {
+  const int r = (a.m + 31) / 32;
+  const int64_t teams2 = 24ll * sms / ((r + 1) / 2);
+  const bool narrow = r == 1 || a.L / 2 < teams2 + teams2 / 2;
+  if (narrow) {
+    switch (r) {
+      case 1: return sweeps_m<1, 1, C, false, BANDED>(a, bps, sms, s);
+      case 2: return sweeps_m<2, 1, C, false, BANDED>(a, bps, sms, s);
+      case 3:
+      case 4: return sweeps_m<4, 1, C, false, BANDED>(a, bps, sms, s);
+      case 5:
+      case 6: return sweeps_m<6, 1, C, false, BANDED>(a, bps, sms, s);
+      default: return sweeps_m<8, 1, C, false, BANDED>(a, bps, sms, s);
+    }
+  }
+  switch ((r + 1) / 2) {
+    case 1: return sweeps_m<1, 2, C, false, BANDED>(a, bps, sms, s);
+    case 2: return sweeps_m<2, 2, C, false, BANDED>(a, bps, sms, s);
+    case 3: return sweeps_m<3, 2, C, false, BANDED>(a, bps, sms, s);
+    default: return sweeps_m<4, 2, C, false, BANDED>(a, bps, sms, s);
+  }
 }
 
 // nb: units that can run at once (capped here at the blocks resident at once,
@@ -339,25 +553,16 @@ cudaError_t bgs_fused_r(const FusedArgs& a, int nb, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int R>
-cudaError_t banded_r(const FusedArgs& a, int nb, cudaStream_t s) {
-  static bool done = false;
-  const size_t smem = (size_t)kWarpsPerBlock * 3 * 32 * R * sizeof(double);
-  if (!done && smem > 40 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_sweeps_banded<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    done = true;
-  }
-  k_sweeps_banded<R><<<nb, 256, smem, s>>>(a);
-  return cudaGetLastError();
-}
-
 template <bool C>
-cudaError_t sweeps_dispatch(const FusedArgs& a, int nb, cudaStream_t s) {
+cudaError_t sweeps_dispatch(const FusedArgs& a, int bps, int sms, cudaStream_t s) {
+  if (a.m < 1 || a.m > kMaxM) return cudaErrorInvalidValue;
   if (a.bgs) {
     if (a.far || a.paired) return cudaErrorInvalidValue;
+    // at most min(K, L/2) units run at once (one per sweep in flight), one
+    // block per unit; the launcher caps the grid at the blocks resident at once
+    const int64_t par = a.K < (a.L + 1) / 2 ? a.K : (a.L + 1) / 2;
+    int nb = par < (1 << 30) ? (int)par : (1 << 30);
+    if (bps > 0 && bps * sms < nb) nb = bps * sms;
     switch ((a.m + 31) / 32) {
       case 1: return bgs_fused_r<1, C>(a, nb, s);
       case 2: return bgs_fused_r<2, C>(a, nb, s);
@@ -366,50 +571,32 @@ cudaError_t sweeps_dispatch(const FusedArgs& a, int nb, cudaStream_t s) {
       case 5: return bgs_fused_r<5, C>(a, nb, s);
       case 6: return bgs_fused_r<6, C>(a, nb, s);
       case 7: return bgs_fused_r<7, C>(a, nb, s);
-      case 8: return bgs_fused_r<8, C>(a, nb, s);
-      default: return cudaErrorInvalidValue;
+      default: return bgs_fused_r<8, C>(a, nb, s);
     }
   }
   if (a.far) {
-    if (C) return cudaErrorInvalidValue;   // block-banded chains: inverse mode only
-    switch ((a.m + 31) / 32) {
-      case 1: return banded_r<1>(a, nb, s);
-      case 2: return banded_r<2>(a, nb, s);
-      case 3: return banded_r<3>(a, nb, s);
-      case 4: return banded_r<4>(a, nb, s);
-      case 5: return banded_r<5>(a, nb, s);
-      case 6: return banded_r<6>(a, nb, s);
-      case 7: return banded_r<7>(a, nb, s);
-      case 8: return banded_r<8>(a, nb, s);
-      default: return cudaErrorInvalidValue;
-    }
+    if constexpr (C)
+      return cudaErrorInvalidValue;   // block-banded chains: inverse mode only
+    else
+      return sweeps_team<false, true>(a, bps, sms, s);
   }
   if (a.paired && !C) {
     switch (a.m / 32) {
-      case 2: return sweeps_r<2, false, true>(a, nb, s);
-      case 4: return sweeps_r<4, false, true>(a, nb, s);
-      case 6: return sweeps_r<6, false, true>(a, nb, s);
-      case 8: return sweeps_r<8, false, true>(a, nb, s);
+      case 2: return sweeps_m<2, 1, false, true, false>(a, bps, sms, s);
+      case 4: return sweeps_m<4, 1, false, true, false>(a, bps, sms, s);
+      case 6: return sweeps_m<6, 1, false, true, false>(a, bps, sms, s);
+      case 8: return sweeps_m<8, 1, false, true, false>(a, bps, sms, s);
       default: return cudaErrorInvalidValue;
     }
   }
-  switch ((a.m + 31) / 32) {
-    case 1: return sweeps_r<1, C>(a, nb, s);
-    case 2: return sweeps_r<2, C>(a, nb, s);
-    case 3: return sweeps_r<3, C>(a, nb, s);
-    case 4: return sweeps_r<4, C>(a, nb, s);
-    case 5: return sweeps_r<5, C>(a, nb, s);
-    case 6: return sweeps_r<6, C>(a, nb, s);
-    case 7: return sweeps_r<7, C>(a, nb, s);
-    case 8: return sweeps_r<8, C>(a, nb, s);
-    default: return cudaErrorInvalidValue;
-  }
+  return sweeps_team<C, false>(a, bps, sms, s);
 }
 
 }  // namespace
 
-cudaError_t launch_sweeps_fused(const FusedArgs& a, int coupled, int n_blocks, cudaStream_t s) {
-  return coupled ? sweeps_dispatch<true>(a, n_blocks, s) : sweeps_dispatch<false>(a, n_blocks, s);
+cudaError_t launch_sweeps_fused(const FusedArgs& a, int coupled, int bps, int sms,
+                                cudaStream_t s) {
+  return coupled ? sweeps_dispatch<true>(a, bps, sms, s) : sweeps_dispatch<false>(a, bps, sms, s);
 }
 
 cudaError_t launch_wait_selftest(int preset, unsigned long long wait_ns, Header* hdr, int* ver,

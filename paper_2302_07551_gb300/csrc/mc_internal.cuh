@@ -42,6 +42,7 @@ struct FarDesc {
   int32_t n;
   int32_t off[kMaxFar];           // d: the Q^T block (l, l + d)
   const double* plane[kMaxFar];   // L blocks, column-major, stride ms
+  const int* bexp[kMaxFar];       // per block: largest exponent (block_exp)
 };
 constexpr size_t kFarDescOffset = 512;   // byte offset inside the 4 KB header
 
@@ -62,6 +63,7 @@ struct Layout {
   // per-level residual sums, the scales, queue counter + per-level completion
   // counters
   size_t off_fsum, off_fver;
+  size_t off_bexp;       // per plane and level: largest exponent of the block (block_exp)
   // low-precision storage (dtype MC_F32 / MC_BF16)
   int lp;                // 0: none, 1: FP32, 2: BF16
   int64_t lp_bs;         // elements per stored block of the A/B planes
@@ -70,6 +72,10 @@ struct Layout {
 };
 
 Layout make_layout(const mc_desc& d);
+
+// block_exp of a block whose products run on the FP64 pipe alone (negative,
+// non-finite or only tiny entries).
+constexpr int kNoFixed = 0;
 
 // Arguments of one half-sweep (Algorithm 2, step 1+2 or step 3).
 struct PhaseArgs {
@@ -102,6 +108,9 @@ struct FusedArgs {
   const double* A;       // TLO / WLO plane
   const double* B;       // TUP / WUP plane
   const double* C;       // NINV plane (inverse mode)
+  const int* eA;         // block_exp of A, B, C per level
+  const int* eB;
+  const int* eC;
   const double* x_in;    // z_0 (read by the first half-sweep only)
   double* W;             // z_1 .. z_{K-1}, in place
   double* Z;             // z_K
@@ -174,13 +183,19 @@ cudaError_t launch_layout_diag(const double* diag, int d, double* plane, const L
                                cudaStream_t s);
 cudaError_t launch_factor(double* planes, const Layout& lay, Header* hdr, int coupled,
                           int num_sms, cudaStream_t s);
+// block_exp of the blocks of one plane: the largest biased exponent of the
+// block's entries if all are >= 0, finite and the largest is not tiny, else
+// kNoFixed.
+cudaError_t launch_block_exp(const double* plane, int* bexp, const Layout& lay, cudaStream_t s);
 cudaError_t launch_phase(const PhaseArgs& a, int coupled, int n_blocks, cudaStream_t s);
 // Block Gauss-Seidel step: one warp walks the levels in order (z_{l-1} fresh,
 // x_{l+1} old); e^T z into hdr->stats[0].
 cudaError_t launch_bgs(const PhaseArgs& a, int coupled, cudaStream_t s);
 int phase_blocks_per_sm(int m);   // resident 256-thread blocks of k_phase per SM
 cudaError_t launch_normalise(const NormArgs& a, int n_blocks, cudaStream_t s);
-cudaError_t launch_sweeps_fused(const FusedArgs& a, int coupled, int n_blocks, cudaStream_t s);
+// bps: resident blocks per SM (0: the kernel's occupancy); sms: SMs of the GPU.
+cudaError_t launch_sweeps_fused(const FusedArgs& a, int coupled, int bps, int sms,
+                                cudaStream_t s);
 // One warp waits (at most wait_ns) for counters preset to `preset` to reach 1;
 // MC_ERR_TIMEOUT is latched in hdr when they never do.
 cudaError_t launch_wait_selftest(int preset, unsigned long long wait_ns, Header* hdr, int* ver,

@@ -1,0 +1,162 @@
+// Level products of the fused FP64 sweeps by teams of warps.
+//
+// A team of TW warps owns one unit (one level of one half-sweep).  Warp w owns
+// the rows 32 RW w .. 32 RW (w + 1) - 1, RW = 1 or 2 per lane, of every block, so
+// each block column is one coalesced 256-byte load per 32 rows, every
+// multiply-add lands in the lane's own accumulators and no partial sums cross
+// the warps; the neighbour vectors are staged once per team in shared memory.
+// Splitting the rows of large blocks keeps 16 loads per lane in flight with
+// 80 registers at any m, and shortens a unit's time, which is what a chain
+// with few levels waits for.
+//
+// The multiply-adds are shared between the FP64 pipe and the integer pipes
+// (fixed_dev.cuh), which moves the bound from the FP64 pipe (98 % busy, 74 % of
+// the HBM copy rate) to HBM.  64 sweeps with residual units: L = 32768, m = 64
+// 41.8 -> 29.4 ms (4.98 -> 7.1 TB/s streamed, FP64 pipe 87 %, ALU 40 %); 32
+// coupled sweeps, L = 5001, m = 100, 7.32 -> 5.63 ms; 16 sweeps of 4096 paired
+// levels of 256, 19.2 -> 12.7 ms (one warp per level with 8 rows a lane: 21.2);
+// block Hessenberg, L = 4096, 64 sweeps, 11.9 -> 8.0 ms (with four of eight
+// entries on the integer pipes 8.3, L = 32768 unchanged).
+#pragma once
+#include "fixed_dev.cuh"
+#include "sweep_dev.cuh"
+#include "wave_dev.cuh"
+
+namespace mc {
+namespace dev {
+
+// Which entries of a batch of `total` per lane go to the fixed-point
+// accumulators: n8 of every 8, spread evenly.  Three of eight where every lane
+// owns rows: the FP64 pipe then needs 10 clocks an entry and SM where
+// streaming it at the read rate of HBM takes 10.7.  Four of eight where some
+// lanes of the last 32-row group own none (their FP64 slots are lost).
+__host__ __device__ constexpr bool fixed_slot(int idx, int total, int n8) {
+  const int n = (n8 * total + 4) / 8;
+  return ((idx + 1) * n) / total != (idx * n) / total;
+}
+
+template <int RW>
+struct TeamTune {
+  static constexpr int U = RW == 1 ? 16 : 8;   // columns per batch
+};
+
+// Vectors staged for one product: FP64 and integer forms, zero beyond m.
+template <int W>
+struct TeamSlot {
+  double v[2][W];
+  uint64_t x[2][W];
+};
+
+template <int TW>
+__device__ __forceinline__ void team_sync(int bar) {
+  if constexpr (TW == 1)
+    __syncwarp();
+  else
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(TW * 32) : "memory");
+}
+
+// acc[r] += sum over columns [j0b, j1) of M(row0 + lane + 32 r, j) v_j.  MC:
+// the block size when it fills the team's rows (no bounds checks), else 0.
+// b0 = etot = largest exponent of the block + of the vector.
+template <int RW, int MC>
+__device__ __forceinline__ void rows_mix(double (&acc)[RW], const double* __restrict__ M,
+                                         const double* v, const uint64_t* xv, int etot, int j0b,
+                                         int j1, int m_, int row0, int lane, bool& bad) {
+  constexpr int U = TeamTune<RW>::U, T = U * RW, N8 = MC ? 3 : 4;
+  const int m = MC ? MC : m_;
+  uint32_t fa[RW][4], seen[RW];
+#pragma unroll
+  for (int r = 0; r < RW; ++r) {
+    fa[r][0] = fa[r][1] = fa[r][2] = fa[r][3] = 0u;
+    seen[r] = 0u;
+  }
+  const double* p = M + (size_t)j0b * m + row0 + lane;
+#pragma unroll 1
+  for (int j0 = j0b; j0 < j1; j0 += U, p += (size_t)U * m) {
+    double t[U][RW];
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+#pragma unroll
+      for (int r = 0; r < RW; ++r)
+        t[q][r] = (MC || (j0 + q < j1 && row0 + lane + 32 * r < m))
+                      ? ld_stream(p + (size_t)q * m + 32 * r)
+                      : 0.0;
+#pragma unroll
+    for (int q = 0; q < U; q += 2) {
+      const double2 vv = *reinterpret_cast<const double2*>(v + j0 + q);
+      const ulonglong2 xx = *reinterpret_cast<const ulonglong2*>(xv + j0 + q);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const double vj = h ? vv.y : vv.x;
+        const uint64_t xj = h ? xx.y : xx.x;
+        const uint32_t xl = (uint32_t)xj & 0xfffff800u, xh = (uint32_t)(xj >> 32);
+        const int b = etot - (int)((uint32_t)xj & 0x7ffu);
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+          if (fixed_slot((q + h) * RW + r, T, N8))
+            fixed_fma(fa[r], seen[r], t[q + h][r], xl, xh, b);
+          else
+            acc[r] = fma(t[q + h][r], vj, acc[r]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < RW; ++r) acc[r] += fixed_value(fa[r], seen[r], etot, bad);
+}
+
+// As rows_mix on the FP64 pipe alone.
+template <int RW, int MC>
+__device__ __forceinline__ void rows_f64(double (&acc)[RW], const double* __restrict__ M,
+                                         const double* v, int j0b, int j1, int m_, int row0,
+                                         int lane) {
+  constexpr int U = TeamTune<RW>::U;
+  const int m = MC ? MC : m_;
+  const double* p = M + (size_t)j0b * m + row0 + lane;
+#pragma unroll 1
+  for (int j0 = j0b; j0 < j1; j0 += U, p += (size_t)U * m) {
+    double t[U][RW];
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+#pragma unroll
+      for (int r = 0; r < RW; ++r)
+        t[q][r] = (MC || (j0 + q < j1 && row0 + lane + 32 * r < m))
+                      ? ld_stream(p + (size_t)q * m + 32 * r)
+                      : 0.0;
+#pragma unroll
+    for (int q = 0; q < U; q += 2) {
+      const double2 vv = *reinterpret_cast<const double2*>(v + j0 + q);
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        acc[r] = fma(t[q][r], vv.x, acc[r]);
+        acc[r] = fma(t[q + 1][r], vv.y, acc[r]);
+      }
+    }
+  }
+}
+
+// acc += M v on both pipes where the block's and the vector's exponents allow
+// it, on the FP64 pipe alone otherwise or when a row's sum left the window
+// (decided per warp from the data alone).
+template <int RW, int MC>
+__device__ __forceinline__ void rows_product(double (&acc)[RW], const double* M, const double* v,
+                                             const uint64_t* xv, int eb, int ev, int j0, int j1,
+                                             int m, int row0, int lane) {
+  bool plain = eb == kNoFixed || !fixed_vec_ok(ev);
+  if (!plain) {
+    double old[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) old[r] = acc[r];
+    bool bad = false;
+    rows_mix<RW, MC>(acc, M, v, xv, eb + ev, j0, j1, m, row0, lane, bad);
+    plain = __any_sync(kFull, bad);
+    if (plain) {
+#pragma unroll
+      for (int r = 0; r < RW; ++r) acc[r] = old[r];
+    }
+  }
+  if (plain) rows_f64<RW, MC>(acc, M, v, j0, j1, m, row0, lane);
+}
+
+}  // namespace dev
+}  // namespace mc
