@@ -202,6 +202,33 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
   for (int64_t done = 0; done < n;) {
     const int64_t K = n - done < kMaxFusedSweeps ? n - done : kMaxFusedSweeps;
     const bool final = done + K == n;
+    if (c->cluster) {
+      ResidentArgs a{};
+      a.A = c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe;
+      a.B = c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe;
+      a.C = c->planes + kPlaneNINV * pe;
+      a.TLO = c->planes + kPlaneTLO * pe;
+      a.TUP = c->planes + kPlaneTUP * pe;
+      a.x_in = in;
+      a.x_out = dst;
+      a.hdr = c->hdr;
+      a.stats_out = final ? stats_out : nullptr;
+      a.L = L;
+      a.K = K;
+      a.m = c->lay.m;
+      a.ms = c->lay.ms;
+      a.par0 = c->d.stair == 1 ? 0 : 1;
+      a.with_step = final && step;
+      a.with_resid = final && resid;
+      CK(launch_resident(a, coupled, c->cluster, s));
+      if (ev && final) {
+        CK(cudaEventRecord(ev[1], s));
+        CK(cudaEventRecord(ev[2], s));
+      }
+      in = dst;
+      done += K;
+      continue;
+    }
     FusedArgs a{};
     a.A = c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe;
     a.B = c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe;
@@ -411,6 +438,9 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   if (lay.L < sms) wr = lay.L;
   if (wr > kMaxWarps) wr = kMaxWarps;
   c->nb_resid = (int)((wr + kWarpsPerBlock - 1) / kWarpsPerBlock);
+  c->cluster = (desc->stair <= 2 && lay.nfar == 0 && !desc->paired && !lay.lp)
+                   ? resident_cluster(lay, desc->apply == MC_APPLY_COUPLED)
+                   : 0;
   c->tune_bps = 0;
   c->tune_lpu = 1;
   int64_t nbn = (lay.N + 4 * kNormThreads - 1) / (4 * kNormThreads);
@@ -616,7 +646,8 @@ int mc_profile(mc_chain* c, const double* x_in, double* x_out, int64_t nsweeps, 
   if (c->lay.lp)
     ms_host[3] = 2.0;   // residual (r, q) + the fused correction sweeps
   else if (fused)
-    ms_host[3] = 3.0 * (double)((nsweeps + kMaxFusedSweeps - 1) / kMaxFusedSweeps);
+    ms_host[3] = (c->cluster ? 1.0 : 3.0) *
+                 (double)((nsweeps + kMaxFusedSweeps - 1) / kMaxFusedSweeps);
   else
     ms_host[3] = 2.0 * (double)nsweeps;   // comparison splitting sweep + normalisation
   ms_host[4] = fused ? 1.0 : 0.0;

@@ -145,6 +145,23 @@ struct FusedArgs {
   double* rsum;
 };
 
+// K sweeps of a chain that fits one cluster's shared memory, with the sums and
+// the normalisation (resident.cu).
+struct ResidentArgs {
+  const double* A;       // TLO / WLO, TUP / WUP, NINV planes
+  const double* B;
+  const double* C;
+  const double* TLO;     // residual (coupled mode)
+  const double* TUP;
+  const double* x_in;
+  double* x_out;         // may equal x_in
+  Header* hdr;
+  double* stats_out;     // optional extra copy of [s, step, resid]
+  int64_t L, K;
+  int m, ms, par0;
+  int with_step, with_resid;
+};
+
 struct NormArgs {
   const double* r;       // NULL, or ||Q^T z||_1 (stats[2] = *r / e^T z)
   const double* z;
@@ -196,6 +213,9 @@ cudaError_t launch_normalise(const NormArgs& a, int n_blocks, cudaStream_t s);
 // bps: resident blocks per SM (0: the kernel's occupancy); sms: SMs of the GPU.
 cudaError_t launch_sweeps_fused(const FusedArgs& a, int coupled, int bps, int sms,
                                 cudaStream_t s);
+// CTAs of the cluster that holds a chain of this layout, 0 if none does.
+int resident_cluster(const Layout& lay, int coupled);
+cudaError_t launch_resident(const ResidentArgs& a, int coupled, int cluster, cudaStream_t s);
 // One warp waits (at most wait_ns) for counters preset to `preset` to reach 1;
 // MC_ERR_TIMEOUT is latched in hdr when they never do.
 cudaError_t launch_wait_selftest(int preset, unsigned long long wait_ns, Header* hdr, int* ver,

@@ -1,0 +1,68 @@
+"""Chains kept resident in one thread-block cluster: sizes at the edges of the cluster sizes, of the
+lanes per level, of the register-held operators and of the shared memory, against the oracle, and the
+neighbouring sizes that run through global memory."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+mc = pytest.importorskip("paper_2302_07551_gb300")
+
+
+# 2 x cluster sizes 1..16, level counts that do not divide, m through every lane group, threads' worth of
+# rows (256 per half-sweep and CTA), more, and the largest blocks that still fit
+@pytest.mark.parametrize("apply,stair", [("inverse", 1), ("inverse", 2), ("coupled", 1)])
+@pytest.mark.parametrize("L,m", [(2, 3), (3, 2), (4, 5), (5, 1), (8, 16), (15, 4), (16, 9), (17, 8), (31, 7),
+                                 (32, 1), (33, 16), (63, 15), (100, 8), (257, 16), (300, 12), (513, 4), (1030, 8),
+                                 (1100, 3), (700, 2), (90, 33), (35, 47), (34, 60), (150, 32), (2, 90), (2, 160)])
+def test_sweeps_match_the_oracle(L, m, apply, stair):
+    """Iterates after K sweeps: 1e-12 relative L1, the suite's bound; e^T z and the residual of the
+    last sweep as in the other sweep tests."""
+    blocks = synth.qbd(L, m, 0.8, seed=7 * L + m)
+    ch = mc.Chain(*(torch.from_numpy(b).cuda() for b in blocks), apply=apply, stair=stair)
+    oc = oracle.Chain(*blocks)
+    x0 = np.full(L * m, 1.0 / (L * m))
+    method = oracle.STAIR1 if stair == 1 else oracle.STAIR2
+    for K in (1, 2, 33):
+        st = torch.zeros(3, dtype=torch.float64, device="cuda")
+        x = ch.sweep(torch.from_numpy(x0).cuda(), nsweeps=K, stats=st).cpu().numpy()
+        ref = oc.sweeps(x0, K, method)
+        assert np.abs(x - ref).sum() <= 1e-12 * np.abs(ref).sum(), K
+        assert abs(float(st[2]) - oc.residual(x)) <= 1e-12 * oc.residual(x) + 8 * m * 2.0 ** -53 * np.abs(blocks[1]).max()
+    ch.sync()
+
+
+def test_in_place_and_repeated_calls_are_bitwise_equal():
+    L, m = 200, 8
+    blocks = synth.qbd(L, m, 0.8, seed=1)
+    ch = mc.Chain(*(torch.from_numpy(b).cuda() for b in blocks))
+    x = torch.rand(L * m, dtype=torch.float64, device="cuda")
+    x /= x.sum()
+    a = ch.sweep(x, nsweeps=5)
+    b = ch.sweep(x, nsweeps=5)
+    y = x.clone()
+    ch.sweep(y, y, nsweeps=5)
+    assert torch.equal(a, b) and torch.equal(a, y)
+
+
+def test_chains_on_several_streams_at_once():
+    """Clusters of independent chains overlap on the device; every result equals the one alone."""
+    L, m, K = 64, 8, 400
+    chains, alone = [], []
+    x = torch.full((L * m,), 1.0 / (L * m), dtype=torch.float64, device="cuda")
+    for i in range(24):
+        b = [torch.from_numpy(t).cuda() for t in synth.qbd(L, m, 0.8, seed=i)]
+        torch.cuda.synchronize()
+        chains.append(mc.Chain(*b, stream=torch.cuda.Stream()))
+        alone.append(chains[-1].sweep(x, nsweeps=K))
+        torch.cuda.synchronize()
+    outs = [torch.empty_like(x) for _ in chains]
+    torch.cuda.synchronize()
+    for ch, o in zip(chains, outs):
+        ch.sweep(x, o, nsweeps=K)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, o) for a, o in zip(alone, outs))
