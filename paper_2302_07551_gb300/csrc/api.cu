@@ -176,6 +176,17 @@ static int* plane_exp(const mc_chain* c, int plane) {
 }
 const int* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); }
 
+// Versioned words of a resident cooperative launch.  FP64: two words a value in
+// z and xb (such chains use neither otherwise); low precision: one, both rows in
+// z (xb holds the refinement update).
+static ResidentWords resident_words(const mc_chain* c) {
+  ResidentWords w{};
+  w.first = (unsigned long long*)c->z;
+  w.last = c->lay.lp ? w.first + (size_t)c->res_ctas * c->lay.m : (unsigned long long*)c->xb;
+  w.state = (char*)c->hdr + kGridStateOffset;
+  return w;
+}
+
 // n stair sweeps src -> dst (in place allowed) as fused launches of at most
 // kMaxFusedSweeps sweeps, each followed by the normalisation (with the step
 // error after the last).  With resid (block-tridiagonal chains only) the last
@@ -202,7 +213,7 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
   for (int64_t done = 0; done < n;) {
     const int64_t K = n - done < kMaxFusedSweeps ? n - done : kMaxFusedSweeps;
     const bool final = done + K == n;
-    if (c->cluster) {
+    if (c->res_ctas) {
       ResidentArgs a{};
       a.A = c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe;
       a.B = c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe;
@@ -220,7 +231,9 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
       a.par0 = c->d.stair == 1 ? 0 : 1;
       a.with_step = final && step;
       a.with_resid = final && resid;
-      CK(launch_resident(a, coupled, c->cluster, s));
+      a.part = c->rpart;
+      a.words = resident_words(c);
+      CK(launch_resident(a, c->lay, coupled, c->res_ctas, c->res_grid, s));
       if (ev && final) {
         CK(cudaEventRecord(ev[1], s));
         CK(cudaEventRecord(ev[2], s));
@@ -327,7 +340,7 @@ static int enqueue_residual(mc_chain* c, const double* x, cudaStream_t s, float*
   r.ms = c->lay.ms;
   r.paired = c->d.paired;
   r.far = c->lay.nfar ? (const FarDesc*)((const char*)c->hdr + kFarDescOffset) : nullptr;
-  CK(launch_residual(r, c->nb_resid, s));
+  CK(launch_residual(r, c->nb_resid, c->num_sms, s));
   return MC_OK;
 }
 
@@ -344,17 +357,36 @@ static float* lpD(mc_chain* c) { return (float*)(c->ws + c->lay.off_d); }
 // must hold (-T_dd)^{-1} r for the current xa), pi <- (pi + d)/e^T(pi + d)
 // with the step error, then r and q of the new iterate.
 static int enqueue_lp_sweeps_fused(mc_chain* c, int64_t K, cudaStream_t s) {
+  if (c->res_ctas) {
+    ResidentLpArgs a{};
+    a.A = lpA(c);
+    a.B = lpB(c);
+    a.C = lpC(c);
+    a.sc = lpSc(c);
+    a.q = lpQ(c);
+    a.d = lpD(c);
+    a.hdr = c->hdr;
+    a.words = resident_words(c);
+    a.L = c->lay.L;
+    a.K = K;
+    a.abs_ = c->lay.lp_bs;
+    a.cbs = c->lay.lp_cbs;
+    a.m = c->lay.m;
+    a.par0 = c->d.stair == 1 ? 0 : 1;
+    CK(launch_resident_lp(a, c->lay, c->d.apply == MC_APPLY_COUPLED, c->res_ctas, c->res_grid, s));
+    return MC_OK;
+  }
   const size_t cnt_bytes = sizeof(unsigned long long) + (size_t)c->lay.L * sizeof(int);
   CK(cudaMemsetAsync(c->fclaim, 0, cnt_bytes, s));
   CK(launch_sweeps_lp(lpA(c), lpB(c), lpC(c), lpSc(c), lpD(c), lpQ(c), c->lay.L, c->lay.m,
                       c->d.stair == 1 ? 0 : 1, c->lay.lp_bs, c->lay.lp_cbs, c->lay.lp == 2,
                       c->d.apply == MC_APPLY_COUPLED, K, c->fver, c->fclaim, c->hdr, kFusedWaitNs,
-                      c->num_sms, c->tune_lpu, c->tune_bps, s));
+                      c->num_sms, c->tune_lpu, c->tune_bps, (unsigned long long*)c->z, s));
   return MC_OK;
 }
 
 static int enqueue_refine_step(mc_chain* c, int inner, cudaStream_t s) {
-  CK(cudaMemsetAsync(lpD(c), 0, (size_t)c->lay.N * sizeof(float), s));
+  if (!c->res_ctas) CK(cudaMemsetAsync(lpD(c), 0, (size_t)c->lay.N * sizeof(float), s));
   const int rc = enqueue_lp_sweeps_fused(c, inner, s);
   if (rc != MC_OK) return rc;
   double* bpart = (double*)(c->ws + c->lay.off_bpart);
@@ -383,16 +415,35 @@ const float* mc::chain_lpSc(mc_chain* c) { return lpSc(c); }
 float* mc::chain_lpQ(mc_chain* c) { return lpQ(c); }
 float* mc::chain_lpD(mc_chain* c) { return lpD(c); }
 
+// Words of a resident cooperative launch to version 0.
+static cudaError_t reset_words(mc_chain* c) {
+  if (!c->res_ctas || !c->res_grid) return cudaSuccess;
+  const size_t row = (size_t)c->res_ctas * c->lay.m * sizeof(unsigned long long);
+  const ResidentWords w = resident_words(c);
+  const size_t bytes = c->lay.lp ? row : 2 * row;
+  cudaError_t e = cudaMemsetAsync(w.state, 0, 16, c->user);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.first, 0, bytes, c->user);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.last, 0, bytes, c->user);
+  return e;
+}
+
+// Clear the status latched in the fetched header and return it (a wait that
+// gave up leaves a resident launch's counters anywhere: they start again).
+static int clear_status(mc_chain* c) {
+  const int st = c->hh->status;
+  if (st != 0) {
+    CK(cudaMemsetAsync(&c->hdr->status, 0, sizeof(int32_t), c->user));
+    if (st == MC_ERR_TIMEOUT) CK(reset_words(c));
+    CK(cudaStreamSynchronize(c->user));
+  }
+  return st;
+}
+
 // Wait for the stream, fetch the header, clear a latched status.
 static int sync_header(mc_chain* c) {
   CK(cudaMemcpyAsync(c->hh, c->hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->user));
   CK(cudaStreamSynchronize(c->user));
-  const int st = c->hh->status;
-  if (st != 0) {
-    CK(cudaMemsetAsync(&c->hdr->status, 0, sizeof(int32_t), c->user));
-    CK(cudaStreamSynchronize(c->user));
-  }
-  return st;
+  return clear_status(c);
 }
 
 int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaStream_t stream,
@@ -438,9 +489,8 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   if (lay.L < sms) wr = lay.L;
   if (wr > kMaxWarps) wr = kMaxWarps;
   c->nb_resid = (int)((wr + kWarpsPerBlock - 1) / kWarpsPerBlock);
-  c->cluster = (desc->stair <= 2 && lay.nfar == 0 && !desc->paired && !lay.lp)
-                   ? resident_cluster(lay, desc->apply == MC_APPLY_COUPLED)
-                   : 0;
+  if (desc->stair <= 2 && lay.nfar == 0 && !desc->paired)
+    c->res_ctas = resident_ctas(lay, desc->apply == MC_APPLY_COUPLED, &c->res_grid);
   c->tune_bps = 0;
   c->tune_lpu = 1;
   int64_t nbn = (lay.N + 4 * kNormThreads - 1) / (4 * kNormThreads);
@@ -458,7 +508,9 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   }
   memset(c->hh, 0, sizeof(Header));
   int rc = MC_OK;
-  if (cudaMemsetAsync(c->ws + lay.off_hdr, 0, 4096, c->user) != cudaSuccess) rc = MC_ERR_CUDA;
+  if (cudaMemsetAsync(c->ws + lay.off_hdr, 0, 4096, c->user) != cudaSuccess ||
+      reset_words(c) != cudaSuccess)
+    rc = MC_ERR_CUDA;
   if (rc != MC_OK) {
     mc_destroy(c);
     return rc;
@@ -646,7 +698,7 @@ int mc_profile(mc_chain* c, const double* x_in, double* x_out, int64_t nsweeps, 
   if (c->lay.lp)
     ms_host[3] = 2.0;   // residual (r, q) + the fused correction sweeps
   else if (fused)
-    ms_host[3] = (c->cluster ? 1.0 : 3.0) *
+    ms_host[3] = (c->res_ctas ? 1.0 : 3.0) *
                  (double)((nsweeps + kMaxFusedSweeps - 1) / kMaxFusedSweeps);
   else
     ms_host[3] = 2.0 * (double)nsweeps;   // comparison splitting sweep + normalisation
@@ -786,12 +838,8 @@ static int solve_refine(mc_chain* c, double* pi, double tol, double eps, int64_t
       CK(cudaStreamSynchronize(c->user));
     }
     k += chunk;
-    st = c->hh->status;
-    if (st != 0) {
-      CK(cudaMemsetAsync(&c->hdr->status, 0, sizeof(int32_t), c->user));
-      CK(cudaStreamSynchronize(c->user));
-      return st;
-    }
+    st = clear_status(c);
+    if (st != 0) return st;
     d = c->hh->stats[1];
     r = c->hh->stats[2];
     if (d_prev > 0.0 && d > 0.0) kappa = pow(d / d_prev, 1.0 / (double)chunk);
@@ -850,12 +898,8 @@ int mc_solve(mc_chain* c, const double* x0, double* pi, double tol, double eps, 
       CK(cudaStreamSynchronize(c->user));
     }
     k += chunk;
-    st = c->hh->status;
-    if (st != 0) {
-      CK(cudaMemsetAsync(&c->hdr->status, 0, sizeof(int32_t), c->user));
-      CK(cudaStreamSynchronize(c->user));
-      return st;
-    }
+    st = clear_status(c);
+    if (st != 0) return st;
     d = c->hh->stats[1];
     if (mode != kResidNone) r = c->hh->stats[2];
     if (d_prev > 0.0 && d > 0.0) kappa = pow(d / d_prev, 1.0 / (double)chunk);

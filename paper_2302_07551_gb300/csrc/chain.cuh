@@ -19,7 +19,7 @@ struct mc_chain {
   double* flsum;             // fused launches: [2][L] level sums, 2 scales, block partials
   int* fver;                 // [L] completion counters, after the queue counter
   unsigned long long* fclaim;
-  int cluster;               // CTAs of the cluster that keeps the chain resident (0: none)
+  int res_ctas, res_grid;    // CTAs that keep the chain on chip (0: none); 1: cooperative launch
   int tune_bps;              // blocks per SM of the fused launches (0: default)
   int tune_lpu;              // levels per unit of the low-precision fused launches
   cudaGraphExec_t gexec;     // cached chunk graph of mc_solve

@@ -46,13 +46,6 @@ namespace {
 
 using namespace dev;
 
-// Threads per block and blocks per SM of a team kernel: 24 warps an SM.
-template <int TW>
-struct TeamBlock {
-  static constexpr int T = (TW == 3 || TW == 6) ? 192 : 256;
-  static constexpr int B = 768 / T;
-};
-
 // Largest exponent over the team's warps.
 template <int TW>
 __device__ __forceinline__ int team_max(const int* e) {
@@ -166,6 +159,9 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
     const double* y = k == 0 ? a.x_in : (BANDED && !(k & 1)) ? a.Z : a.W;
     const double* src = resid ? a.Z : h2 ? dst : y;
     const int need = (int)(h2 ? k + 1 : k);
+    // the blocks' exponents: loaded while this team waits
+    const int ea = resid ? 0 : a.eA[l], eb = resid ? 0 : a.eB[l];
+    const int ec = COUPLED || resid ? 0 : a.eC[l];
     if constexpr (BANDED) {
       if (need > 0)
         wait_band(a.ver, l, a.L, a.bw, (int)k * TW, need * TW, &a.hdr->status, lane, a.wait_ns);
@@ -232,10 +228,10 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
       continue;
     }
     if (has_lo)
-      rows_product<RW, MC>(acc, a.A + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], a.eA[l],
+      rows_product<RW, MC>(acc, a.A + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], ea,
                            team_max<TW>(sh.emax[s][0]), lo0, m, m, row0, lane);
     if (has_up)
-      rows_product<RW, MC>(acc, a.B + (size_t)l * a.ms, sh.slot[s].v[1], sh.slot[s].x[1], a.eB[l],
+      rows_product<RW, MC>(acc, a.B + (size_t)l * a.ms, sh.slot[s].v[1], sh.slot[s].x[1], eb,
                            team_max<TW>(sh.emax[s][1]), 0, up1, m, row0, lane);
     if constexpr (BANDED) {
       const int n = a.far->n;
@@ -243,6 +239,7 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
         const int64_t kk = l + a.far->off[j];
         if (kk < 0 || kk >= a.L) continue;
         s ^= 1;
+        const int ef = a.far->bexp[j][l];
         double x0[RW];
 #pragma unroll
         for (int i = 0; i < RW; ++i) {
@@ -253,7 +250,7 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
                            lane);
         team_sync<TW>(bar);
         rows_product<RW, MC>(acc, a.far->plane[j] + (size_t)l * a.ms, sh.slot[s].v[0],
-                             sh.slot[s].x[0], a.far->bexp[j][l], team_max<TW>(sh.emax[s][0]), 0,
+                             sh.slot[s].x[0], ef, team_max<TW>(sh.emax[s][0]), 0,
                              m, m, row0, lane);
       }
     }
@@ -264,7 +261,7 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
       team_sync<TW>(bar);
 #pragma unroll
       for (int i = 0; i < RW; ++i) acc[i] = 0.0;
-      rows_product<RW, MC>(acc, a.C + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], a.eC[l],
+      rows_product<RW, MC>(acc, a.C + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], ec,
                            team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
     }
     double t = 0.0;

@@ -20,6 +20,7 @@
 
 #include "mc_internal.cuh"
 #include "lowprec_dev.cuh"
+#include "lpteam_dev.cuh"
 #include "wave_dev.cuh"
 
 namespace mc {
@@ -105,6 +106,57 @@ __global__ void __launch_bounds__(256) k_sweeps_lp(LpArgs a, int64_t K, int lpu,
     }
     publish_levels(ver, l0, 2, n, (int)(k + 1), lane);
     q = __shfl_sync(0xffffffffu, q0, 0);
+  }
+}
+
+// The correction sweeps of a short chain (lpteam_dev.cuh): units are single
+// levels, claimed in order by teams of TW warps, two teams' worth ahead.  16
+// warps per SM: the prefetched operators take 64 to 96 registers a thread.
+template <typename S, int ROWS, int TW, bool COUPLED>
+__global__ void __launch_bounds__(256, 2) k_lp_team(LpLevels a, int64_t K, int parity,
+                                                    unsigned long long* claim, Header* hdr,
+                                                    unsigned long long wait_ns) {
+  extern __shared__ __align__(16) unsigned char lp_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / TW, w = warp % TW, tt = threadIdx.x - team * TW * 32, bar = 1 + team;
+  auto& sh = reinterpret_cast<LpTeamShared<ROWS, TW>*>(lp_smem)[team];
+  const int64_t P0 = (a.L - parity + 1) / 2;
+  const unsigned long long total = (unsigned long long)K * (unsigned long long)a.L;
+  unsigned long long q0 = w == 0 ? claim_unit(claim, lane) : 0ull, q;
+  if constexpr (TW == 1) {
+    q = __shfl_sync(0xffffffffu, q0, 0);
+  } else {
+    if (w == 0 && lane == 0) sh.next[1] = q0;
+    if (w == 0) q0 = claim_unit(claim, lane);
+    lp_sync<TW>(bar);
+    q = sh.next[1];
+  }
+  auto unit = [&](unsigned long long i) {
+    const int64_t k = (int64_t)(i / (unsigned long long)a.L);
+    const int64_t r = (int64_t)i - k * a.L;
+    const bool h2 = r >= P0;
+    return LpUnit{h2 ? 2 * (r - P0) + (1 - parity) : 2 * r + parity, (int)(h2 ? k + 1 : k),
+                  (int)(k + 1), k == 0 && !h2, k == K - 1};
+  };
+  int turn = 0;
+  while (q < total) {
+    unsigned long long qn = 0ull;
+    if constexpr (TW == 1)
+      q0 = claim_unit(claim, lane);
+    else if (w == 0 && lane == 0)
+      sh.next[turn] = q0;
+    const LpUnit u = unit(q);
+    LpAhead<S, ROWS, TW, COUPLED> p;
+    p.load(a, u, w, tt, lane);
+    lp_team_unit<S, ROWS, TW, COUPLED>(a, sh, u, p, w, tt, lane, bar, &hdr->status, wait_ns,
+                                       [&]() {
+                                         if constexpr (TW > 1) {
+                                           qn = sh.next[turn];
+                                           turn ^= 1;
+                                           if (w == 0) q0 = claim_unit(claim, lane);
+                                         }
+                                       });
+    q = TW == 1 ? __shfl_sync(0xffffffffu, q0, 0) : qn;
   }
 }
 
@@ -214,6 +266,30 @@ cudaError_t lp_fused_launch(const LpArgs& a, const LpFused& f, int num_sms, cuda
   return cudaGetLastError();
 }
 
+template <typename S, int ROWS, int TW, bool C>
+cudaError_t lp_team_launch(const LpLevels& a, const LpFused& f, int parity, int num_sms,
+                           cudaStream_t s) {
+  constexpr int teams = kWarpsPerBlock / TW;
+  const size_t smem = teams * sizeof(LpTeamShared<ROWS, TW>);
+  static_assert(teams * sizeof(LpTeamShared<ROWS, TW>) <= 48 * 1024, "no opt-in needed");
+  int64_t nb = 2ll * num_sms;
+  const int64_t need = (a.L + teams - 1) / teams;
+  if (nb > need) nb = need;
+  k_lp_team<S, ROWS, TW, C><<<(int)nb, 256, smem, s>>>(a, f.K, parity, f.claim, f.hdr, f.wait_ns);
+  return cudaGetLastError();
+}
+
+// Warps per level of the team kernel: a warp holds one or two batches of columns.
+int lp_team_warps(int m) { return m <= 64 ? 4 : 8; }
+
+template <typename S, bool C>
+cudaError_t lp_team_dispatch(const LpLevels& a, const LpFused& f, int parity, int num_sms,
+                             cudaStream_t s) {
+  if (a.m <= 64) return lp_team_launch<S, 64, 4, C>(a, f, parity, num_sms, s);
+  if (a.m <= 128) return lp_team_launch<S, 128, 8, C>(a, f, parity, num_sms, s);
+  return lp_team_launch<S, 256, 8, C>(a, f, parity, num_sms, s);
+}
+
 template <typename T, bool C>
 cudaError_t lp_dispatch(const LpArgs& a, const LpFused& f, int nb, cudaStream_t s) {
   // nb: the number of SMs
@@ -255,9 +331,24 @@ cudaError_t launch_sweeps_lp(const void* A, const void* B, const float* C, const
                              float* d, const float* q, int64_t L, int m, int parity, int64_t abs_,
                              int64_t cbs, int bf16, int coupled, int64_t K, int* ver,
                              unsigned long long* claim, Header* hdr, unsigned long long wait_ns,
-                             int num_sms, int lpu, int bps, cudaStream_t s) {
+                             int num_sms, int lpu, int bps, unsigned long long* dv,
+                             cudaStream_t s) {
   if (lpu != 1 && lpu != 2 && lpu != 4) return cudaErrorInvalidValue;
   const int nb = num_sms;
+  // Short chains, whose half-sweep's units all run at once as teams (BF16: with
+  // 16-byte columns); otherwise enough units are in flight to stream from HBM,
+  // and one warp per level with more resident warps is faster.
+  if (m > 32 && (!bf16 || m % 8 == 0) && L / 2 * lp_team_warps(m) <= 16ll * num_sms) {
+    const cudaError_t e = cudaMemsetAsync(dv, 0, (size_t)L * m * sizeof(*dv), s);
+    if (e != cudaSuccess) return e;
+    const LpLevels v{A, B, C, sc, q, dv, d, L, abs_, cbs, m};
+    const LpFused f{K, ver, claim, hdr, wait_ns, lpu, bps};
+    if (bf16)
+      return coupled ? lp_team_dispatch<unsigned short, true>(v, f, parity, num_sms, s)
+                     : lp_team_dispatch<unsigned short, false>(v, f, parity, num_sms, s);
+    return coupled ? lp_team_dispatch<float, true>(v, f, parity, num_sms, s)
+                   : lp_team_dispatch<float, false>(v, f, parity, num_sms, s);
+  }
   LpArgs a{};
   a.A = A;
   a.B = B;

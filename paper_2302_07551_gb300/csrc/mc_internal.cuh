@@ -145,21 +145,42 @@ struct FusedArgs {
   double* rsum;
 };
 
-// K sweeps of a chain that fits one cluster's shared memory, with the sums and
-// the normalisation (resident.cu).
+// Chains that stay on chip (resident.cu).  Versioned words of a chain spread
+// over a cooperative launch: two rows of CTAs x m values, and the launch's
+// counters (16 bytes).
+constexpr size_t kGridStateOffset = 1024;   // byte offset inside the 4 KB header
+struct ResidentWords {
+  unsigned long long* first;
+  unsigned long long* last;
+  void* state;
+};
 struct ResidentArgs {
   const double* A;       // TLO / WLO, TUP / WUP, NINV planes
   const double* B;
   const double* C;
-  const double* TLO;     // residual (coupled mode)
+  const double* TLO;     // residual
   const double* TUP;
   const double* x_in;
   double* x_out;         // may equal x_in
+  double* part;          // 6 doubles per CTA
   Header* hdr;
   double* stats_out;     // optional extra copy of [s, step, resid]
+  ResidentWords words;
   int64_t L, K;
   int m, ms, par0;
   int with_step, with_resid;
+};
+struct ResidentLpArgs {
+  const void* A;
+  const void* B;
+  const float* C;
+  const float* sc;
+  const float* q;
+  float* d;
+  Header* hdr;
+  ResidentWords words;
+  int64_t L, K, abs_, cbs;
+  int m, par0;
 };
 
 struct NormArgs {
@@ -213,9 +234,13 @@ cudaError_t launch_normalise(const NormArgs& a, int n_blocks, cudaStream_t s);
 // bps: resident blocks per SM (0: the kernel's occupancy); sms: SMs of the GPU.
 cudaError_t launch_sweeps_fused(const FusedArgs& a, int coupled, int bps, int sms,
                                 cudaStream_t s);
-// CTAs of the cluster that holds a chain of this layout, 0 if none does.
-int resident_cluster(const Layout& lay, int coupled);
-cudaError_t launch_resident(const ResidentArgs& a, int coupled, int cluster, cudaStream_t s);
+// CTAs that keep a chain of this layout on chip, as one cluster (*grid = 0) or
+// as a cooperative launch (*grid = 1); 0 if it does not fit.
+int resident_ctas(const Layout& lay, int coupled, int* grid);
+cudaError_t launch_resident(const ResidentArgs& a, const Layout& lay, int coupled, int ctas,
+                            int grid, cudaStream_t s);
+cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& lay, int coupled, int ctas,
+                               int grid, cudaStream_t s);
 // One warp waits (at most wait_ns) for counters preset to `preset` to reach 1;
 // MC_ERR_TIMEOUT is latched in hdr when they never do.
 cudaError_t launch_wait_selftest(int preset, unsigned long long wait_ns, Header* hdr, int* ver,
@@ -227,7 +252,8 @@ constexpr int kScaleBlocks = 64;
 cudaError_t launch_fused_scale(const double* lsum, int64_t L, int64_t K, const double* rsum,
                                int64_t P, double* out, double* part, unsigned* ticket,
                                cudaStream_t s);
-cudaError_t launch_residual(const ResidArgs& a, int n_blocks, cudaStream_t s);
+// n_blocks: grid for m <= 32; sms: SMs of the GPU.
+cudaError_t launch_residual(const ResidArgs& a, int n_blocks, int sms, cudaStream_t s);
 cudaError_t launch_fill(double* x, int64_t n, double v, cudaStream_t s);
 // Latch MC_ERR_ARG unless the paired zero quadrants of TLO / TUP are zero.
 cudaError_t launch_check_paired(const double* tlo, const double* tup, const Layout& lay,
@@ -240,12 +266,13 @@ cudaError_t launch_lp_convert(const double* src, void* dst, int bf16, float* sc,
 // All K correction sweeps of a refinement step in one launch (ver, claim:
 // zeroed counters as for launch_sweeps_fused; parity of half-sweep 1); lpu:
 // levels per claimed unit (1, 2 or 4); bps: resident blocks per SM (0: the
-// kernel's occupancy).
+// kernel's occupancy); dv: N words of scratch.
 cudaError_t launch_sweeps_lp(const void* A, const void* B, const float* C, const float* sc,
                              float* d, const float* q, int64_t L, int m, int parity, int64_t abs_,
                              int64_t cbs, int bf16, int coupled, int64_t K, int* ver,
                              unsigned long long* claim, Header* hdr, unsigned long long wait_ns,
-                             int num_sms, int lpu, int bps, cudaStream_t s);
+                             int num_sms, int lpu, int bps, unsigned long long* dv,
+                             cudaStream_t s);
 cudaError_t launch_update(const double* pi, const float* d, double* out, int64_t N, double* bpart,
                           int nb, Header* hdr, double* s_out, cudaStream_t s);
 

@@ -1,6 +1,6 @@
-// Small chains: all sweeps of a call, the sums, the residual and the
-// normalisation in one launch of one thread-block cluster
-// (resident_dev.cuh).
+// Chains that stay on chip (resident_dev.cuh).  FP64: all sweeps of a call, the
+// sums, the residual and the normalisation in one launch.  Low precision: the
+// correction sweeps of a refinement step.
 #include <math.h>
 
 #include <mutex>
@@ -13,17 +13,41 @@ namespace {
 
 using namespace res;
 
+template <typename V>
+__device__ __forceinline__ void attach(ClusterLink<V>& ln, const ResidentWords&, int* status) {
+  ln.status = status;
+}
+template <typename V>
+__device__ __forceinline__ void attach(GridLink<V>& ln, const ResidentWords& w, int* status) {
+  ln.first = w.first;
+  ln.last = w.last;
+  ln.g = reinterpret_cast<GridState*>(w.state);
+  ln.status = status;
+}
+
+// The end of a launch: every CTA of a cluster stays until the others have read
+// its shared memory; one CTA of a grid counts the versions up.
+template <typename V>
+__device__ __forceinline__ void finish(const ClusterLink<V>&) {
+  cg::this_cluster().sync();
+}
+template <typename V>
+__device__ __forceinline__ void finish(const GridLink<V>& ln) {
+  ln.done();
+}
+
 // K FP64 sweeps from x_in, then x_out = z_K / e^T z_K with the step error
 // (with_step) and ||Q^T x_out||_1 from the splitting (with_resid, see
 // fused.cu) into the header and stats_out.
-template <bool COUPLED>
+template <bool COUPLED, typename Link>
 __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double sh[2][kThreads / 32 + 1][3];
   __shared__ double rcp[2];
-  __shared__ unsigned long long bars[2];
-  cg::cluster_group cl = cg::this_cluster();
-  const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
+  __shared__ unsigned long long two[2];
+  Link ln;
+  attach(ln, a.words, &a.hdr->status);
+  const int C = ln.ctas(), r = ln.rank();
   Chain<double, double, double> h{};
   h.A = a.A;
   h.B = a.B;
@@ -33,7 +57,7 @@ __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
   h.L = (int)a.L;
   h.m = a.m;
   h.par0 = a.par0;
-  sweeps<double, double, double, COUPLED>(h, (int)a.K, smem, bars, &a.hdr->status);
+  sweeps<double, double, double, COUPLED>(h, (int)a.K, smem, two, ln);
   const int L = h.L, m = h.m;
   const int l0 = range_begin(L, C, r), n = range_begin(L, C, r + 1) - l0;
   const Carve k = carve<double, double, double, COUPLED>((L + C - 1) / C, m);
@@ -53,7 +77,7 @@ __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
     const Cover c = cover(m, (n + 1) / 2);
     double* rs = reinterpret_cast<double*>(smem + k.g);   // |r| per row
     for_rows<double>(
-        c, m, nh,
+        c, m, nh, reinterpret_cast<double*>(smem + k.p),
         [&](int u, int i, int j0, int S) {
           const int t = t0 + 2 * u;
           const int64_t l = l0 + t;
@@ -73,7 +97,7 @@ __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
     for (int e = threadIdx.x; e < nh * m && threadIdx.x < 32 * warps; e += 32 * warps)
       v[2] += rs[e];
   }
-  cluster_sum3(v, warps, sh[0]);
+  all_sum3(v, warps, sh[0], ln, a.part);
   const double s = v[0], so = a.K > 1 ? v[1] : 1.0, res = v[2];
   if (threadIdx.x == 0) {   // divisions are many FP64 instructions: one thread
     rcp[0] = 1.0 / s;
@@ -87,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
     if (a.with_step) w[0] += fabs(p - x[m + e] * pinv);
     a.x_out[(int64_t)l0 * m + e] = p;
   }
-  cluster_sum3(w, warps, sh[1]);   // after its barrier no CTA reads sh[0] of another
+  all_sum3(w, warps, sh[1], ln, a.part + 3 * C);   // after its barrier no CTA reads sh[0] of another
   if (r == 0 && threadIdx.x == 0) {
     if (!((s > 0.0) && isfinite(s))) latch(a.hdr, MC_ERR_BREAKDOWN);
     const double st[3] = {a.K > 1 ? s / so : s, w[0], a.with_resid ? res * inv : nan("")};
@@ -96,92 +120,186 @@ __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
       if (a.stats_out) a.stats_out[i] = st[i];
     }
   }
-  cl.sync();   // every CTA stays until the others have read its sums
+  finish(ln);
+}
+
+// The K correction sweeps of a refinement step from the zero vector.
+template <typename S, bool COUPLED, template <typename> class LinkT>
+__global__ void __launch_bounds__(kThreads) k_resident_lp(ResidentLpArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned long long two[2];
+  LinkT<float> ln;
+  attach(ln, a.words, &a.hdr->status);
+  Chain<S, float, float> h{};
+  h.A = reinterpret_cast<const S*>(a.A);
+  h.B = reinterpret_cast<const S*>(a.B);
+  h.C = a.C;
+  h.as = a.abs_;
+  h.cs = a.cbs;
+  h.sc = a.sc;
+  h.q = a.q;
+  h.L = (int)a.L;
+  h.m = a.m;
+  h.par0 = a.par0;
+  sweeps<S, float, float, COUPLED>(h, (int)a.K, smem, two, ln);
+  const int l0 = ln.s.l0, n = ln.s.n;
+  for (int e = threadIdx.x; e < n * h.m; e += kThreads)
+    a.d[(int64_t)l0 * h.m + e] = ln.s.x[h.m + e];
+  finish(ln);
 }
 
 constexpr size_t kMaxDyn = 227 * 1024 - 1024;   // opt-in limit less the static arrays
 
-// Whether a cluster of C CTAs with all of an SM's shared memory can run.
-template <typename K>
-bool cluster_runs(K kernel, int C) {
-  cudaLaunchConfig_t cfg{};
+// Kernels by storage type (FP64, FP32, BF16), apply mode and link.
+using Kernel64 = void (*)(ResidentArgs);
+using KernelLp = void (*)(ResidentLpArgs);
+Kernel64 kernel64(int coupled, bool grid) {
+  if (grid)
+    return coupled ? k_resident<true, GridLink<double>> : k_resident<false, GridLink<double>>;
+  return coupled ? k_resident<true, ClusterLink<double>> : k_resident<false, ClusterLink<double>>;
+}
+template <typename S>
+KernelLp kernel_lp_of(int coupled, bool grid) {
+  if (grid) return coupled ? k_resident_lp<S, true, GridLink> : k_resident_lp<S, false, GridLink>;
+  return coupled ? k_resident_lp<S, true, ClusterLink> : k_resident_lp<S, false, ClusterLink>;
+}
+KernelLp kernel_lp(int lp, int coupled, bool grid) {
+  return lp == 1 ? kernel_lp_of<float>(coupled, grid) : kernel_lp_of<unsigned short>(coupled, grid);
+}
+
+size_t smem_bytes(const Layout& y, int coupled, int C) {
+  const int n = (int)((y.L + C - 1) / C), m = y.m;
+  if (y.lp == 0)
+    return coupled ? carve<double, double, double, true>(n, m).total
+                   : carve<double, double, double, false>(n, m).total;
+  if (y.lp == 1)
+    return coupled ? carve<float, float, float, true>(n, m).total
+                   : carve<float, float, float, false>(n, m).total;
+  return coupled ? carve<unsigned short, float, float, true>(n, m).total
+                 : carve<unsigned short, float, float, false>(n, m).total;
+}
+
+void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, bool grid, int C, size_t smem,
+            cudaStream_t s) {
   cfg.gridDim = dim3(C);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kMaxDyn;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = C;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  if (grid) {
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+  } else {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  }
   cfg.attrs = &at;
   cfg.numAttrs = 1;
+}
+
+// Whether a cluster of C CTAs with all of an SM's shared memory can run.
+bool cluster_runs(const void* kernel, int C) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  config(cfg, at, false, C, kMaxDyn, 0);
   int n = 0;
   return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
 }
 
-template <typename K>
-bool opt_in(K kernel) {
+bool opt_in(const void* kernel, bool cluster) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)kMaxDyn) == cudaSuccess &&
-         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-             cudaSuccess;
+         (!cluster || cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                           1) == cudaSuccess);
 }
 
-// Largest cluster of the current device: 16 (the non-portable opt-in), 8 or
-// none; found once per device.
-int cluster_limit() {
+// What the current device allows, found once per device: the largest cluster
+// (16, the non-portable opt-in, 8 or 0) and the SMs of a cooperative launch with
+// one CTA each (0: none).
+struct Limits {
+  bool known;
+  int cluster, grid;
+};
+Limits limits() {
   constexpr int kDevices = 64;
   static std::mutex mu;
-  static int limit[kDevices];   // 0: not asked yet, -1: none
+  static Limits all[kDevices];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return Limits{};
   std::lock_guard<std::mutex> lk(mu);
-  if (limit[dev] == 0) {
-    limit[dev] = -1;
-    if (opt_in(k_resident<true>) && opt_in(k_resident<false>))
-      for (int C = 16; C >= 8; C /= 2)
-        if (cluster_runs(k_resident<true>, C) && cluster_runs(k_resident<false>, C)) {
-          limit[dev] = C;
-          break;
+  Limits& l = all[dev];
+  if (!l.known) {
+    bool ok = true;
+    for (int c = 0; c < 2; ++c) {
+      ok = ok && opt_in((const void*)kernel64(c, false), true) &&
+           opt_in((const void*)kernel64(c, true), false);
+      for (int lp = 1; lp <= 2; ++lp)
+        ok = ok && opt_in((const void*)kernel_lp(lp, c, false), true) &&
+             opt_in((const void*)kernel_lp(lp, c, true), false);
+    }
+    if (ok) {
+      for (int C = 16; C >= 8 && !l.cluster; C /= 2) {
+        bool runs = true;
+        for (int c = 0; c < 2; ++c) {
+          runs = runs && cluster_runs((const void*)kernel64(c, false), C);
+          for (int lp = 1; lp <= 2; ++lp)
+            runs = runs && cluster_runs((const void*)kernel_lp(lp, c, false), C);
         }
+        if (runs) l.cluster = C;
+      }
+      int sms = 0, coop = 0;
+      if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+          cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop)
+        l.grid = sms;
+    }
     cudaGetLastError();
+    l.known = true;
   }
-  return limit[dev] > 0 ? limit[dev] : 0;
-}
-
-template <bool C>
-cudaError_t launch(const ResidentArgs& a, int cluster, cudaStream_t s) {
-  const int n = (int)((a.L + cluster - 1) / cluster);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(cluster);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = carve<double, double, double, C>(n, a.m).total;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cluster;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_resident<C>, a);
+  return l;
 }
 
 }  // namespace
 
-// The largest cluster that leaves every CTA two levels (one of each parity), if
-// the chain fits its shared memory.
-int resident_cluster(const Layout& y, int coupled) {
+// Every CTA owns at least two levels (one of each parity).  A cluster (short
+// hops) while its 16 SMs keep up: FP64 up to 96 K multiply-adds a sweep (3000
+// clocks of the 32 FP64 lanes a clock), low precision up to 64 KB of shared
+// memory a CTA (500 clocks of its bandwidth); else all SMs.
+int resident_ctas(const Layout& y, int coupled, int* grid) {
+  *grid = 0;
   if (y.L > (1 << 20)) return 0;
-  int C = cluster_limit();
+  const Limits lim = limits();
+  int C = lim.cluster;
   while (C > 1 && y.L < 2 * C) C /= 2;
-  if (C < 1) return 0;
-  const int n = (int)((y.L + C - 1) / C);
-  const size_t bytes = coupled ? carve<double, double, double, true>(n, y.m).total
-                               : carve<double, double, double, false>(n, y.m).total;
-  return bytes <= kMaxDyn ? C : 0;
+  const double entries = (double)y.L * y.m * y.m * (coupled ? 2 : 3);
+  const size_t most = y.lp ? 64 * 1024 : kMaxDyn;
+  // low precision, m > 32: the team kernel (lpteam_dev.cuh) keeps more warps on a
+  // level and is faster where it applies (500 levels of 64, FP32 inverse, 3.4 us a
+  // sweep against 4.6)
+  if (y.lp && y.m > 32 && (y.lp == 1 || y.m % 8 == 0)) return 0;
+  if (C > 0 && smem_bytes(y, coupled, C) <= most && (y.lp || entries <= 96e3)) return C;
+  int G = lim.grid;
+  if (G > y.L / 2) G = (int)(y.L / 2);
+  if (G > 0 && smem_bytes(y, coupled, G) <= kMaxDyn) {
+    *grid = 1;
+    return G;
+  }
+  return 0;
 }
 
-cudaError_t launch_resident(const ResidentArgs& a, int coupled, int cluster, cudaStream_t s) {
-  return coupled ? launch<true>(a, cluster, s) : launch<false>(a, cluster, s);
+cudaError_t launch_resident(const ResidentArgs& a, const Layout& y, int coupled, int ctas,
+                            int grid, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  config(cfg, at, grid != 0, ctas, smem_bytes(y, coupled, ctas), s);
+  return cudaLaunchKernelEx(&cfg, kernel64(coupled, grid != 0), a);
+}
+
+cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& y, int coupled, int ctas,
+                               int grid, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  config(cfg, at, grid != 0, ctas, smem_bytes(y, coupled, ctas), s);
+  return cudaLaunchKernelEx(&cfg, kernel_lp(y.lp, coupled, grid != 0), a);
 }
 
 }  // namespace mc

@@ -27,6 +27,7 @@
 
 #include "mc_internal.cuh"
 #include "sweep_dev.cuh"
+#include "team_dev.cuh"
 
 namespace mc {
 
@@ -241,6 +242,84 @@ __global__ void __launch_bounds__(256, Tune<R>::MINB) k_residual(ResidArgs a) {
   }
 }
 
+// k_residual for blocks of more than 32 rows: a team of TW warps per level, one
+// row per lane (team_dev.cuh).  One warp per level with up to 8 rows a lane kept
+// few loads in flight and left most of the GPU idle on short chains (512 levels
+// of 256 with q: the refinement's outer step 563 -> 320 us, of which the FP64
+// pipe needs 213).
+template <int TW>
+struct ResidShared {
+  double v[3][32 * TW];
+  double r[32 * TW];
+};
+
+template <int TW, int MC, bool WITH_Q, bool PAIRED>
+__global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_resid_team(ResidArgs a) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  __shared__ double red[32];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / TW, w = warp % TW, bar = 1 + team, row = 32 * w + lane;
+  constexpr int teams = TeamBlock<TW>::T / 32 / TW;
+  ResidShared<TW>& sh = reinterpret_cast<ResidShared<TW>*>(team_smem)[team];
+  const int m = MC ? MC : a.m, row0 = 32 * w;
+  const int lo0 = PAIRED && 2 * row0 >= m ? m / 2 : 0;
+  const int up1 = PAIRED && 2 * row0 < m ? m / 2 : m;
+  const bool in = row < m;
+  double wsum = 0.0;
+  for (int64_t l = (int64_t)blockIdx.x * teams + team; l < a.L; l += (int64_t)gridDim.x * teams) {
+    const bool has_lo = l > 0, has_up = l < a.L - 1;
+    sh.v[0][row] = has_lo && in ? a.x[(l - 1) * m + row] : 0.0;
+    sh.v[1][row] = in ? a.x[l * m + row] : 0.0;
+    sh.v[2][row] = has_up && in ? a.x[(l + 1) * m + row] : 0.0;
+    team_sync<TW>(bar);
+    double acc[1] = {0.0};
+    if (has_lo)
+      rows_f64<1, MC>(acc, a.TLO + (size_t)l * a.ms, sh.v[0], lo0, m, m, row0, lane);
+    rows_f64<1, MC>(acc, a.TDD + (size_t)l * a.ms, sh.v[1], 0, m, m, row0, lane);
+    if (has_up)
+      rows_f64<1, MC>(acc, a.TUP + (size_t)l * a.ms, sh.v[2], 0, up1, m, row0, lane);
+    if (a.far) {
+      for (int j = 0; j < a.far->n; ++j) {
+        const int64_t k = l + a.far->off[j];
+        if (k < 0 || k >= a.L) continue;
+        sh.r[row] = in ? a.x[k * m + row] : 0.0;
+        team_sync<TW>(bar);
+        rows_f64<1, MC>(acc, a.far->plane[j] + (size_t)l * a.ms, sh.r, 0, m, m, row0, lane);
+        team_sync<TW>(bar);
+      }
+    }
+    wsum += fabs(acc[0]);
+    if constexpr (WITH_Q) {
+      sh.r[row] = acc[0];
+      team_sync<TW>(bar);
+      acc[0] = 0.0;
+      rows_f64<1, MC>(acc, a.NINV + (size_t)l * a.ms, sh.r, 0, m, m, row0, lane);
+      if (in) a.q[l * m + row] = (float)acc[0];
+    }
+    team_sync<TW>(bar);   // the vectors are rewritten for the next level
+  }
+  wsum = warp_sum(wsum);
+  constexpr int nwb = TeamBlock<TW>::T / 32;
+  if (lane == 0) {
+    a.rpart[blockIdx.x * nwb + warp] = wsum;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&a.hdr->ticket[1], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double e = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x * nwb; i += blockDim.x) e += __ldcg(a.rpart + i);
+  e = block_sum(e, red);
+  if (threadIdx.x == 0) {
+    a.hdr->stats[2] = e;
+    if (a.out) a.out[0] = e;
+    a.hdr->ticket[1] = 0u;
+  }
+}
+
 __global__ void k_fill(double* x, int64_t n, double v) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -307,19 +386,29 @@ cudaError_t phase_dispatch(const PhaseArgs& a, int nb, cudaStream_t s) {
   }
 }
 
-template <int R, bool P = false>
-cudaError_t resid_r(const ResidArgs& a, int nb, cudaStream_t s) {
-  static bool done = false, done_q = false;
-  if (a.q) {
-    const cudaError_t e = allow_smem(k_residual<R, true, P>, vec_smem<R>(), done_q);
-    if (e != cudaSuccess) return e;
-    k_residual<R, true, P><<<nb, 256, vec_smem<R>(), s>>>(a);
-    return cudaGetLastError();
-  }
-  const cudaError_t e = allow_smem(k_residual<R, false, P>, vec_smem<R>(), done);
-  if (e != cudaSuccess) return e;
-  k_residual<R, false, P><<<nb, 256, vec_smem<R>(), s>>>(a);
+template <int TW, int MC, bool Q, bool P>
+cudaError_t resid_team(const ResidArgs& a, int sms, cudaStream_t s) {
+  constexpr int T = TeamBlock<TW>::T, teams = T / 32 / TW;
+  int64_t nb = (int64_t)TeamBlock<TW>::B * sms;
+  const int64_t need = (a.L + teams - 1) / teams;
+  if (nb > need) nb = need;
+  if (nb * (T / 32) > kMaxWarps) nb = kMaxWarps / (T / 32);
+  k_resid_team<TW, MC, Q, P><<<(int)nb, T, teams * sizeof(ResidShared<TW>), s>>>(a);
   return cudaGetLastError();
+}
+
+template <int TW, bool P = false>
+cudaError_t resid_m(const ResidArgs& a, int sms, cudaStream_t s) {
+  static_assert(TeamBlock<TW>::T / 32 / TW * sizeof(ResidShared<TW>) <= 40 * 1024, "no opt-in");
+  if constexpr (P)
+    return a.q ? resid_team<TW, 32 * TW, true, true>(a, sms, s)
+               : resid_team<TW, 32 * TW, false, true>(a, sms, s);
+  else if (a.m == 32 * TW)
+    return a.q ? resid_team<TW, 32 * TW, true, false>(a, sms, s)
+               : resid_team<TW, 32 * TW, false, false>(a, sms, s);
+  else
+    return a.q ? resid_team<TW, 0, true, false>(a, sms, s)
+               : resid_team<TW, 0, false, false>(a, sms, s);
 }
 
 }  // namespace
@@ -360,25 +449,31 @@ cudaError_t launch_normalise(const NormArgs& a, int n_blocks, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_residual(const ResidArgs& a, int nb, cudaStream_t s) {
+cudaError_t launch_residual(const ResidArgs& a, int nb, int sms, cudaStream_t s) {
+  const int r = (a.m + 31) / 32;
   if (a.paired) {
-    switch (a.m / 32) {
-      case 2: return resid_r<2, true>(a, nb, s);
-      case 4: return resid_r<4, true>(a, nb, s);
-      case 6: return resid_r<6, true>(a, nb, s);
-      case 8: return resid_r<8, true>(a, nb, s);
+    switch (r) {
+      case 2: return resid_m<2, true>(a, sms, s);
+      case 4: return resid_m<4, true>(a, sms, s);
+      case 6: return resid_m<6, true>(a, sms, s);
+      case 8: return resid_m<8, true>(a, sms, s);
       default: return cudaErrorInvalidValue;
     }
   }
-  switch ((a.m + 31) / 32) {
-    case 1: return resid_r<1>(a, nb, s);
-    case 2: return resid_r<2>(a, nb, s);
-    case 3: return resid_r<3>(a, nb, s);
-    case 4: return resid_r<4>(a, nb, s);
-    case 5: return resid_r<5>(a, nb, s);
-    case 6: return resid_r<6>(a, nb, s);
-    case 7: return resid_r<7>(a, nb, s);
-    case 8: return resid_r<8>(a, nb, s);
+  switch (r) {
+    case 1:
+      if (a.q)
+        k_residual<1, true, false><<<nb, 256, vec_smem<1>(), s>>>(a);
+      else
+        k_residual<1, false, false><<<nb, 256, vec_smem<1>(), s>>>(a);
+      return cudaGetLastError();
+    case 2: return resid_m<2>(a, sms, s);
+    case 3:
+    case 4: return resid_m<4>(a, sms, s);
+    case 5:
+    case 6: return resid_m<6>(a, sms, s);
+    case 7:
+    case 8: return resid_m<8>(a, sms, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -40,6 +40,13 @@ struct TeamTune {
   static constexpr int U = RW == 1 ? 16 : 8;   // columns per batch
 };
 
+// Threads per block and blocks per SM of a team kernel: 24 warps an SM.
+template <int TW>
+struct TeamBlock {
+  static constexpr int T = (TW == 3 || TW == 6) ? 192 : 256;
+  static constexpr int B = 768 / T;
+};
+
 // Vectors staged for one product: FP64 and integer forms, zero beyond m.
 template <int W>
 struct TeamSlot {

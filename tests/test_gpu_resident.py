@@ -1,6 +1,6 @@
-"""Chains kept resident in one thread-block cluster: sizes at the edges of the cluster sizes, of the
-lanes per level, of the register-held operators and of the shared memory, against the oracle, and the
-neighbouring sizes that run through global memory."""
+"""Chains kept on chip, in one thread-block cluster or over all SMs: sizes at the edges of the cluster
+sizes, of the lanes per level, of the register-held operators and of the shared memory, against the
+oracle, and the neighbouring sizes that run through global memory."""
 import numpy as np
 import pytest
 import torch
@@ -18,7 +18,8 @@ mc = pytest.importorskip("paper_2302_07551_gb300")
 @pytest.mark.parametrize("apply,stair", [("inverse", 1), ("inverse", 2), ("coupled", 1)])
 @pytest.mark.parametrize("L,m", [(2, 3), (3, 2), (4, 5), (5, 1), (8, 16), (15, 4), (16, 9), (17, 8), (31, 7),
                                  (32, 1), (33, 16), (63, 15), (100, 8), (257, 16), (300, 12), (513, 4), (1030, 8),
-                                 (1100, 3), (700, 2), (90, 33), (35, 47), (34, 60), (150, 32), (2, 90), (2, 160)])
+                                 (1100, 3), (700, 2), (90, 33), (35, 47), (34, 60), (150, 32), (2, 90), (2, 160),
+                                 (303, 33), (304, 17), (305, 60), (640, 40), (2500, 20), (1250, 32), (5000, 8)])
 def test_sweeps_match_the_oracle(L, m, apply, stair):
     """Iterates after K sweeps: 1e-12 relative L1, the suite's bound; e^T z and the residual of the
     last sweep as in the other sweep tests."""
@@ -49,12 +50,14 @@ def test_in_place_and_repeated_calls_are_bitwise_equal():
     assert torch.equal(a, b) and torch.equal(a, y)
 
 
-def test_chains_on_several_streams_at_once():
-    """Clusters of independent chains overlap on the device; every result equals the one alone."""
-    L, m, K = 64, 8, 400
+@pytest.mark.parametrize("L,m,n", [(64, 8, 24), (320, 32, 6)])
+def test_chains_on_several_streams_at_once(L, m, n):
+    """Independent chains, as clusters or as launches over all SMs, in flight on several streams:
+    every result equals the one alone."""
+    K = 400
     chains, alone = [], []
     x = torch.full((L * m,), 1.0 / (L * m), dtype=torch.float64, device="cuda")
-    for i in range(24):
+    for i in range(n):
         b = [torch.from_numpy(t).cuda() for t in synth.qbd(L, m, 0.8, seed=i)]
         torch.cuda.synchronize()
         chains.append(mc.Chain(*b, stream=torch.cuda.Stream()))
@@ -66,3 +69,21 @@ def test_chains_on_several_streams_at_once():
         ch.sweep(x, o, nsweeps=K)
     torch.cuda.synchronize()
     assert all(torch.equal(a, o) for a, o in zip(alone, outs))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("apply", ["inverse", "coupled"])
+@pytest.mark.parametrize("L,m", [(2, 4), (33, 8), (64, 12), (305, 32), (600, 24), (400, 64), (40, 100), (900, 96), (306, 256)])
+def test_refinement_solutions(L, m, apply, dtype):
+    """Solutions from low-precision correction sweeps on chip and by teams of warps, against the
+    oracle's FP64 solution: the suite's 1e-10 relative L1."""
+    blocks = synth.qbd(L, m, 0.5, seed=L + m)
+    ch = mc.Chain(*(torch.from_numpy(b).cuda() for b in blocks), apply=apply, dtype=dtype)
+    pi, res = ch.solve(tol=1e-12, check_every=24, maxit=40000)
+    assert res["residual"] <= 1e-12
+    if L * m * m > 3e6:       # the oracle would take too long: the residual decides
+        return
+    ref = oracle.Chain(*blocks).solve(tol=1e-13, maxit=40000, check_every=24)["x"]
+    assert np.abs(pi.cpu().numpy() - ref).sum() <= 1e-10
+    again, _ = ch.solve(tol=1e-12, check_every=24, maxit=40000)
+    assert torch.equal(pi, again)
