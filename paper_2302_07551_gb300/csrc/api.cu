@@ -174,7 +174,7 @@ static bool split_resid_ok(const mc_chain* c) { return c->d.stair <= 2 && c->lay
 static int* plane_exp(const mc_chain* c, int plane) {
   return (int*)(c->ws + c->lay.off_bexp) + (size_t)plane * (size_t)c->lay.L;
 }
-const int* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); }
+int* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); }
 
 // Versioned words of a resident cooperative launch.  FP64: two words a value in
 // z and xb (such chains use neither otherwise); low precision: one, both rows in
@@ -509,6 +509,8 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   memset(c->hh, 0, sizeof(Header));
   int rc = MC_OK;
   if (cudaMemsetAsync(c->ws + lay.off_hdr, 0, 4096, c->user) != cudaSuccess ||
+      cudaMemsetAsync(c->ws + lay.off_bexp, 0, (size_t)(7 + lay.nfar) * lay.L * sizeof(int),
+                      c->user) != cudaSuccess ||
       reset_words(c) != cudaSuccess)
     rc = MC_ERR_CUDA;
   if (rc != MC_OK) {
@@ -537,7 +539,7 @@ int mc_create(const mc_desc* desc, const double* dn, const double* loc, const do
   mc_chain* c = nullptr;
   const int rc = chain_init(desc, workspace, ws_bytes, (cudaStream_t)cuda_stream, &c);
   if (rc != MC_OK) return rc;
-  if (launch_layout(dn, loc, up, c->planes, c->lay, c->hdr, c->user) != cudaSuccess) {
+  if (launch_layout(dn, loc, up, c->planes, plane_exp(c, 0), c->lay, c->user) != cudaSuccess) {
     mc_destroy(c);
     return MC_ERR_CUDA;
   }
@@ -560,7 +562,7 @@ int mc_create_banded(const mc_desc* desc, const double* const* diags, void* work
   const size_t pe = y.plane_bytes / sizeof(double);
   // near diagonals as in mc_create: Q^T (l, l-1) <- Q_{l-1,l} (e = +1),
   // (l, l+1) <- Q_{l+1,l} (e = -1), (l, l) <- Q_{l,l}
-  if (launch_layout(diags[lo - 1], diags[lo], diags[lo + 1], c->planes, y, c->hdr, c->user) !=
+  if (launch_layout(diags[lo - 1], diags[lo], diags[lo + 1], c->planes, plane_exp(c, 0), y, c->user) !=
       cudaSuccess)
     rc = MC_ERR_CUDA;
   FarDesc fd{};
@@ -571,7 +573,9 @@ int mc_create_banded(const mc_desc* desc, const double* const* diags, void* work
     fd.off[j] = d;
     fd.plane[j] = plane;
     fd.bexp[j] = plane_exp(c, y.far_base + j);
-    if (launch_layout_diag(diags[-d + lo], d, plane, y, c->user) != cudaSuccess) rc = MC_ERR_CUDA;
+    if (launch_layout_diag(diags[-d + lo], d, plane, plane_exp(c, y.far_base + j), y, c->user) !=
+        cudaSuccess)
+      rc = MC_ERR_CUDA;
   }
   if (rc == MC_OK && cudaMemcpyAsync((char*)c->hdr + kFarDescOffset, &fd, sizeof(fd),
                                      cudaMemcpyHostToDevice, c->user) != cudaSuccess)
@@ -604,21 +608,9 @@ int mc::chain_factor_async(mc_chain* c) {
     CK(launch_check_paired(c->planes + kPlaneTLO * pe, c->planes + kPlaneTUP * pe, c->lay, c->hdr,
                            c->user));
   }
-  CK(launch_factor(c->planes, c->lay, c->hdr, c->d.apply == MC_APPLY_COUPLED, c->num_sms,
-                   c->user));
   const size_t pe = c->lay.plane_bytes / sizeof(double);
   const bool coupled = c->d.apply == MC_APPLY_COUPLED;
-  if (c->lay.lp == 0) {   // the planes that FP64 sweeps stream
-    static const int kOps[2][3] = {{kPlaneTLO, kPlaneTUP, kPlaneNINV}, {kPlaneWLO, kPlaneWUP, -1}};
-    for (int i = 0; i < 3; ++i) {
-      const int p = kOps[coupled][i];
-      if (p >= 0) CK(launch_block_exp(c->planes + p * pe, plane_exp(c, p), c->lay, c->user));
-    }
-    for (int j = 0; j < c->lay.nfar; ++j) {
-      const int p = c->lay.far_base + j;
-      CK(launch_block_exp(c->planes + p * pe, plane_exp(c, p), c->lay, c->user));
-    }
-  }
+  CK(launch_factor(c->planes, plane_exp(c, 0), c->lay, c->hdr, coupled, c->num_sms, c->user));
   if (c->lay.lp) {
     const int bf16 = c->lay.lp == 2;
     CK(launch_lp_convert(c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe, c->ws + c->lay.off_lpA,

@@ -1,5 +1,6 @@
 // Set-up kernels: block layout of Q^T, batched LU of the diagonal blocks and
 // the operators that apply Q_{l,l}^{-1} in Algorithm 2 (steps 2 and 3).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "fixed_dev.cuh"
@@ -9,267 +10,473 @@ namespace mc {
 
 namespace {
 
+// Copy of one block (or of a 2048-entry chunk of it) by a warp, zero where the
+// block is missing and beyond m * m; returns the largest exponent field of its
+// entries on every lane (block_exp).
+constexpr int kChunk = 2048;
+__device__ __forceinline__ unsigned copy_chunk(const double* src, double* dst, int e0, int mm,
+                                               int ms, int lane) {
+  unsigned big = 0u;
+  const int e1 = min(e0 + kChunk, ms);
+  for (int e = e0 + lane; e < e1; e += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = src && e + 32 * q < mm ? __ldcs(src + e + 32 * q) : 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (e + 32 * q < e1) dst[e + 32 * q] = v[q];
+      big = max(big, (unsigned)__double2hiint(v[q]) >> 20);
+    }
+  }
+  return __reduce_max_sync(0xffffffffu, big);
+}
+
 // Planes TLO, TUP, TDD from the generator blocks (Sect. 2 block partition of
 // Q^T).  A row-major Q block is the column-major storage of its transpose, so
 // T_{l,l-1} = (Q_{l-1,l})^T is up[l-1] copied verbatim, T_{l,l+1} =
 // (Q_{l+1,l})^T is dn[l+1], T_{l,l} = loc[l].  Missing boundary blocks and
-// the padding beyond m*m are zero.
-__global__ void k_layout(const double* __restrict__ dn, const double* __restrict__ loc,
-                         const double* __restrict__ up, double* __restrict__ tlo,
-                         double* __restrict__ tup, double* __restrict__ tdd, int64_t L, int m,
-                         int ms) {
+// the padding beyond m*m are zero.  The exponents of TLO and TUP come with the
+// copy, without another pass.
+__global__ void __launch_bounds__(256) k_layout(const double* dn, const double* loc,
+                                                const double* up, double* tlo, double* tup,
+                                                double* tdd, int* elo, int* eup, int64_t L, int m,
+                                                int ms) {
   const int64_t mm = (int64_t)m * m;
-  const int64_t total = L * ms;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t l = t / ms, e = t % ms;
-    double a = 0.0, b = 0.0, c = 0.0;
-    if (e < mm) {
-      if (l > 0) a = up[(l - 1) * mm + e];
-      if (l < L - 1) b = dn[(l + 1) * mm + e];
-      c = loc[l * mm + e];
-    }
-    tlo[t] = a;
-    tup[t] = b;
-    tdd[t] = c;
+  const int chunks = (ms + kChunk - 1) / kChunk, lane = threadIdx.x & 31;
+  const int64_t total = 3 * L * chunks, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total; t += nw) {
+    const int64_t b = t / chunks, l = b / 3;
+    const int p = (int)(b - 3 * l), e0 = (int)(t - b * chunks) * kChunk;
+    const double* src = p == 0   ? (l > 0 ? up + (l - 1) * mm : nullptr)
+                        : p == 1 ? (l < L - 1 ? dn + (l + 1) * mm : nullptr)
+                                 : loc + l * mm;
+    double* dst = (p == 0 ? tlo : p == 1 ? tup : tdd) + (size_t)l * ms;
+    const unsigned e = copy_chunk(src, dst, e0, (int)mm, ms, lane);
+    if (p < 2 && lane == 0) atomicMax((p == 0 ? elo : eup) + l, (int)e);
   }
 }
 
-// LU without pivoting of T_dd (column-major, in A), then X = T_dd^{-1} by
-// forward and backward substitution on the identity, stored as -X = (-T_dd)^{-1}.
-// One CTA per level; A and X live in shared memory (m <= 112).  Every step
-// ends with a CTA barrier; all loops are bounded.
-template <bool SMEM>
-__global__ void __launch_bounds__(256) k_lu_inv(const double* tdd, double* lu,
-                                                double* ninv, int64_t L, int m, int ms,
-                                                Header* hdr) {
-  extern __shared__ double sm[];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int mm = m * m;
-  for (int64_t l = blockIdx.x; l < L; l += gridDim.x) {
-    double* A = SMEM ? sm : lu + (size_t)l * ms;
-    double* X = SMEM ? sm + mm : ninv + (size_t)l * ms;
-    const double* src = tdd + (size_t)l * ms;
-    for (int e = tid; e < mm; e += nt) {
-      A[e] = src[e];
-      X[e] = (e % m == e / m) ? 1.0 : 0.0;
+// ---- LU and inverse by Gauss-Jordan elimination ------------------------------
+//
+// Step k of an in-place Gauss-Jordan inversion without pivoting updates the
+// whole matrix by a rank-1 product of column k over the pivot and row k.  Row k
+// from the diagonal on is U's row k at that moment and the scaled column below
+// it is L's column k, so the factors come on the way.  Per block m^3
+// multiply-adds, what LU and two triangular solves take, but in m equal steps
+// of a full m x m update in which no thread idles and no triangle is walked.
+//
+// The matrix stays in registers: thread (ti, tj) of a G x G grid owns the
+// entries (ti + G a, tj + G b), a, b < R.  A step: the owners of row and column k
+// have put them into shared memory; one warp forms 1 / pivot and the scaled
+// column (a division is a dozen FP64 instructions, 16 clocks each); everybody
+// does R^2 multiply-adds; the owners put row and column k + 1 there.  Row k, column k
+// and the pivot take their new values from the same update, with the
+// multipliers -1/pivot for row k and 1 for column k and the old entries zero.
+// A diagonal entry is kept in two parts, its value at the start (or the inverse
+// pivot) and the sum of its updates, added where it is used: m updates rounded
+// at the size of the dominant diagonal would be most of the inverse's error
+// (m = 256: 6.9e-16 against 0.9e-16 relative, 3.3e-16 for blocked LU and solves).
+// Bound: the FP64 pipe (89 % busy at m = 64; a tenth of its instructions are the
+// pivot's).  8192 blocks of 64: 7.7 -> 4.65 ms (3.4 at the pipe's rate).
+template <int G, int R>
+__device__ __forceinline__ void gj_update(double (&A)[R][R], const double* row, const double* cs,
+                                          int ti, int tj, int kb, bool own_row, bool own_col) {
+  double c[R], r[R];
+#pragma unroll
+  for (int a = 0; a < R; ++a) {
+    c[a] = cs[ti + G * a];
+    r[a] = row[tj + G * a];
+  }
+#pragma unroll
+  for (int b = 0; b < R; ++b)
+    if (b == kb && own_col) {
+      r[b] = 1.0;
+#pragma unroll
+      for (int a = 0; a < R; ++a) A[a][b] = 0.0;
     }
-    __syncthreads();
-    bool bad = false;
-    for (int k = 0; k < m; ++k) {
-      const double piv = A[k * m + k];
-      if (!(piv != 0.0) || !isfinite(piv)) { bad = true; break; }
-      for (int i = k + 1 + tid; i < m; i += nt) A[k * m + i] = A[k * m + i] / piv;
+#pragma unroll
+  for (int a = 0; a < R; ++a)
+    if (a == kb && own_row) {
+#pragma unroll
+      for (int b = 0; b < R; ++b) A[a][b] = 0.0;
+    }
+#pragma unroll
+  for (int a = 0; a < R; ++a)
+#pragma unroll
+    for (int b = 0; b < R; ++b) A[a][b] = fma(-c[a], r[b], A[a][b]);
+#pragma unroll
+  for (int a = 0; a < R; ++a)
+    if (a == kb && own_row && own_col) A[a][a] = 0.0;   // 1/pivot is kept apart
+}
+
+// Blocks of up to 128 rows: G = 16 (one block per CTA) or G = 4 (m <= 16: 16 blocks
+// per CTA, half a warp each).
+template <int G, int R>
+struct GjBlock {
+  static constexpr int N = 256 / (G * G), MP = G * R;
+  static constexpr int B = R <= 4 ? 3 : R <= 6 ? 2 : 1;   // CTAs per SM
+  static size_t doubles(int m) { return ((size_t)6 * MP + (size_t)m * (m + 1) + 1) / 2 * 2; }
+};
+
+template <int G, int R>
+__global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __restrict__ tdd,
+                                                             double* lu, double* ninv, int* eninv,
+                                                             int64_t L, int m, int ms, int per,
+                                                             Header* hdr) {
+  extern __shared__ double sm[];
+  __shared__ int s_bad[256 / (G * G)];
+  constexpr int N = GjBlock<G, R>::N, MP = G * R;
+  const int grp = threadIdx.x / (G * G), t = threadIdx.x % (G * G), ti = t % G, tj = t / G;
+  double* row = sm + (size_t)grp * per;   // [2][MP]
+  double* col = row + 2 * MP;             // [2][MP]
+  double* cs = col + 2 * MP;              // [MP]
+  double* base = cs + MP;                 // [MP] first part of the diagonal
+  double* LU = base + MP;                 // column j at j (m + 1)
+  auto sync = []() {
+    if constexpr (G == 16)
       __syncthreads();
-      const int nr = m - k - 1;
-      for (int idx = tid; idx < nr * nr; idx += nt) {
-        const int i = k + 1 + idx % nr, j = k + 1 + idx / nr;
-        A[j * m + i] = fma(-A[k * m + i], A[j * m + k], A[j * m + i]);
+    else
+      __syncwarp();
+  };
+  for (int64_t l0 = (int64_t)blockIdx.x * N; l0 < L; l0 += (int64_t)gridDim.x * N) {
+    const int64_t l = l0 + grp;
+    const bool live = l < L;
+    double A[R][R];
+#pragma unroll
+    for (int a = 0; a < R; ++a)
+#pragma unroll
+      for (int b = 0; b < R; ++b) {
+        const int i = ti + G * a, j = tj + G * b;
+        A[a][b] = live && i < m && j < m ? tdd[(size_t)l * ms + (size_t)j * m + i]
+                                         : (i == j ? 1.0 : 0.0);
+        if (a == b && ti == tj) {
+          base[i] = A[a][b];
+          A[a][b] = 0.0;
+        }
       }
-      __syncthreads();
+    if (ti == 0)
+#pragma unroll
+      for (int b = 0; b < R; ++b) row[tj + G * b] = A[0][b];
+    if (tj == 0)
+#pragma unroll
+      for (int a = 0; a < R; ++a) col[ti + G * a] = A[a][0];
+    if (t == 0) s_bad[grp] = 0;
+    sync();
+    bool bad = false;
+#pragma unroll
+    for (int kb = 0; kb < R; ++kb) {
+#pragma unroll 1
+      for (int kk = 0; kk < G; ++kk) {
+        const int k = kb * G + kk;
+        if (k >= m || (G == 16 && bad)) break;
+        const double* rw = row + (k & 1) * MP;
+        const double* cl = col + (k & 1) * MP;
+        if (G != 16 || (threadIdx.x >> 5) == (k & 7)) {
+          const double piv = base[k] + rw[k];
+          if (!(piv != 0.0) || !isfinite(piv)) s_bad[grp] = 1;
+          const double p = 1.0 / piv;
+          for (int i = G == 16 ? (int)(threadIdx.x & 31) : t; i < m; i += G == 16 ? 32 : G * G) {
+            const double c = cl[i] * p;
+            cs[i] = i == k ? -p : c;
+            if (i > k) LU[k * (m + 1) + i] = c;
+            if (i >= k) LU[i * (m + 1) + k] = i == k ? piv : rw[i];
+          }
+        }
+        sync();
+        bad = s_bad[grp] != 0;
+        if (ti == kk && tj == kk) base[k] = -cs[k];
+        gj_update<G, R>(A, rw, cs, ti, tj, kb, ti == kk, tj == kk);
+        double* rn = row + ((k + 1) & 1) * MP;
+        double* cn = col + ((k + 1) & 1) * MP;
+        const bool step = kk == G - 1;   // row k + 1 lies in the next register block
+        constexpr int R1 = R - 1;
+        const int nk = step ? 0 : kk + 1;
+        if (ti == nk)
+#pragma unroll
+          for (int b = 0; b < R; ++b)
+            rn[tj + G * b] = step ? A[kb < R1 ? kb + 1 : kb][b] : A[kb][b];
+        if (tj == nk)
+#pragma unroll
+          for (int a = 0; a < R; ++a)
+            cn[ti + G * a] = step ? A[a][kb < R1 ? kb + 1 : kb] : A[a][kb];
+        sync();
+      }
     }
     if (bad) {
-      if (tid == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
-      __syncthreads();
-      continue;
+      if (live && t == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
+    } else if (live) {
+      unsigned e = 0u;
+#pragma unroll
+      for (int a = 0; a < R; ++a)
+#pragma unroll
+        for (int b = 0; b < R; ++b) {
+          const int i = ti + G * a, j = tj + G * b;
+          if (i < m && j < m) {
+            // 0 - x: no -0, whose sign bit would read as negative
+            const double v = (i == j ? -base[i] : 0.0) - A[a][b];
+            ninv[(size_t)l * ms + (size_t)j * m + i] = v;
+            e = max(e, (unsigned)__double2hiint(v) >> 20);
+          }
+        }
+      const unsigned mask = G == 16 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
+      e = __reduce_max_sync(mask, e);
+      if ((threadIdx.x & (G == 16 ? 31 : 15)) == 0) atomicMax(eninv + l, (int)e);
+      for (int j = tj; j < m; j += G)
+        for (int i = ti; i < m; i += G)
+          lu[(size_t)l * ms + (size_t)j * m + i] = LU[j * (m + 1) + i];
     }
-    // X <- L^{-1} X (unit lower triangular, column oriented)
-    for (int k = 0; k < m - 1; ++k) {
-      const int nr = m - k - 1;
-      for (int idx = tid; idx < nr * m; idx += nt) {
-        const int i = k + 1 + idx % nr, c = idx / nr;
-        X[c * m + i] = fma(-A[k * m + i], X[c * m + k], X[c * m + i]);
-      }
-      __syncthreads();
-    }
-    // X <- U^{-1} X
-    for (int k = m - 1; k >= 0; --k) {
-      const double ukk = A[k * m + k];
-      for (int c = tid; c < m; c += nt) X[c * m + k] = X[c * m + k] / ukk;
-      __syncthreads();
-      for (int idx = tid; idx < k * m; idx += nt) {
-        const int i = idx % k, c = idx / k;
-        X[c * m + i] = fma(-A[k * m + i], X[c * m + k], X[c * m + i]);
-      }
-      __syncthreads();
-    }
-    double* dlu = lu + (size_t)l * ms;
-    double* dni = ninv + (size_t)l * ms;
-    for (int e = tid; e < mm; e += nt) {
-      if (SMEM) dlu[e] = A[e];
-      dni[e] = -X[e];
-    }
-    __syncthreads();
+    sync();   // the buffers are rewritten for the next block
   }
 }
 
-// Blocked LU and inverse for blocks too large for shared memory (m > 112):
-// one 512-thread CTA per level, column panels of kB = 32.
-//   LU (right-looking): factor the panel (rows p0..m-1) in shared memory,
-//   solve U12 = L11^{-1} A12 in shared memory, update the trailing block
-//   A22 -= L21 U12 in place.
-//   Inverse: X = U^{-1} L^{-1} one identity column panel at a time, kept in
-//   shared memory: forward substitution by row panels (triangle by a warp per
-//   right-hand side, rows below by a panel product), then backward
-//   substitution the same way; the panel is stored as -X = (-T_dd)^{-1}.
-constexpr int kB = 32, kLd = 256, kLdU = kB + 1, kBigThreads = 512;
+// Blocks of 129 to 256 rows: a cluster of 2 x 2 CTAs, a 32 x 32 grid of threads
+// with R x R entries each (512 KB of the four SMs' registers at m = 256).  Row k
+// and column k go into the shared memory of the CTAs that need them; one cluster
+// barrier a step.  512 blocks of 256: 33.7 -> 21 ms (13.7 at the pipe's rate; a
+// step waits for the pivot and the barrier, and 36 clusters run at once).
+template <int R>
+struct GjBig {
+  static constexpr int H = 16 * R;   // a CTA's rows and columns
+  static constexpr size_t doubles = 6 * H + 2 + (size_t)H * (H + 1);
+};
 
-__global__ void __launch_bounds__(kBigThreads, 1) k_factor_big(const double* __restrict__ tdd,
-                                                               double* lu, double* ninv,
-                                                               int64_t L, int m, int ms,
-                                                               Header* hdr) {
+template <int R>
+__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
+    k_gj_cluster(const double* __restrict__ tdd, double* lu, double* ninv, int* eninv, int64_t L,
+                 int m, int ms, Header* hdr) {
   extern __shared__ double sm[];
-  double* Pan = sm;                  // panel / right-hand sides: [kB][kLd]
-  double* U12 = sm + kB * kLd;       // U12 block: [column][kLdU]
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
-  const int nwarp = nt >> 5;
-  const int np = (m + kB - 1) / kB;
-  for (int64_t l = blockIdx.x; l < L; l += gridDim.x) {
-    double* A = lu + (size_t)l * ms;
-    double* X = ninv + (size_t)l * ms;
+  constexpr int H = GjBig<R>::H;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), cr = rank & 1, cc = rank >> 1;
+  const int ti = threadIdx.x % 16, tj = threadIdx.x / 16;
+  double* row = sm;              // [2][H]: row k at this CTA's columns
+  double* col = row + 2 * H;     // [2][H]: column k at this CTA's rows
+  double* cs = col + 2 * H;      // [H]
+  double* base = cs + H;         // [H] first part of the diagonal (cr == cc)
+  double* piv = base + H;        // [2]
+  double* LU = piv + 2;          // local column lj at lj (H + 1)
+  double* row_peer = cl.map_shared_rank(row, rank ^ 1);   // the other rows, same columns
+  double* col_peer = cl.map_shared_rank(col, rank ^ 2);   // the other columns, same rows
+  const int i0 = ti + 16 * cr, j0 = tj + 16 * cc;   // entries (i0 + 32 a, j0 + 32 b)
+  for (int64_t l = blockIdx.x / 4; l < L; l += gridDim.x / 4) {
     const double* T = tdd + (size_t)l * ms;
-    for (int e = tid; e < m * m; e += nt) A[e] = T[e];
-    __syncthreads();
-    bool ok = true;
-    for (int p = 0; p < np && ok; ++p) {
-      const int p0 = p * kB, w = min(kB, m - p0), nr = m - p0;
-      for (int e = tid; e < w * nr; e += nt) {
-        const int k = e / nr, i = e % nr;
-        Pan[k * kLd + i] = A[(size_t)(p0 + k) * m + p0 + i];
-      }
-      __syncthreads();
-      for (int k = 0; k < w; ++k) {
-        const double piv = Pan[k * kLd + k];
-        if (!(piv != 0.0) || !isfinite(piv)) { ok = false; break; }
-        for (int i = k + 1 + tid; i < nr; i += nt) Pan[k * kLd + i] = Pan[k * kLd + i] / piv;
-        __syncthreads();
-        const int nc = w - k - 1, nrr = nr - k - 1;
-        for (int e = tid; e < nc * nrr; e += nt) {
-          const int j = k + 1 + e / nrr, i = k + 1 + e % nrr;
-          Pan[j * kLd + i] = fma(-Pan[k * kLd + i], Pan[j * kLd + k], Pan[j * kLd + i]);
+    double A[R][R];
+#pragma unroll
+    for (int a = 0; a < R; ++a)
+#pragma unroll
+      for (int b = 0; b < R; ++b) {
+        const int i = i0 + 32 * a, j = j0 + 32 * b;
+        A[a][b] = i < m && j < m ? T[(size_t)j * m + i] : (i == j ? 1.0 : 0.0);
+        if (a == b && i0 == j0) {
+          base[ti + 16 * a] = A[a][b];
+          A[a][b] = 0.0;
         }
-        __syncthreads();
       }
-      if (!ok) break;
-      for (int e = tid; e < w * nr; e += nt) {
-        const int k = e / nr, i = e % nr;
-        A[(size_t)(p0 + k) * m + p0 + i] = Pan[k * kLd + i];
+    // put row and column k = 32 q + s (s < 32) into buffer f, q a register block
+    auto publish = [&](int q, int s, int f) {
+      if (cr == (s >> 4) && ti == (s & 15)) {
+#pragma unroll
+        for (int a = 0; a < R; ++a)
+          if (a == q) {
+#pragma unroll
+            for (int b = 0; b < R; ++b) {
+              row[f * H + tj + 16 * b] = A[a][b];
+              row_peer[f * H + tj + 16 * b] = A[a][b];
+            }
+          }
       }
-      const int nc2 = m - p0 - w;
-      if (nc2 > 0) {
-        for (int e = tid; e < w * nc2; e += nt) {
-          const int c = e / w, k = e % w;
-          U12[c * kLdU + k] = A[(size_t)(p0 + w + c) * m + p0 + k];
-        }
-        __syncthreads();
-        for (int c = tid; c < nc2; c += nt) {
-          double* u = U12 + c * kLdU;
-          for (int k = 0; k < w; ++k) {
-            const double uk = u[k];
-            for (int i = k + 1; i < w; ++i) u[i] = fma(-Pan[k * kLd + i], uk, u[i]);
+      if (cc == (s >> 4) && tj == (s & 15)) {
+#pragma unroll
+        for (int b = 0; b < R; ++b)
+          if (b == q) {
+#pragma unroll
+            for (int a = 0; a < R; ++a) {
+              col[f * H + ti + 16 * a] = A[a][b];
+              col_peer[f * H + ti + 16 * a] = A[a][b];
+              if (a == q && cr == (s >> 4) && ti == (s & 15))
+                for (int p = 0; p < 4; ++p)
+                  cl.map_shared_rank(piv, p)[f] = base[ti + 16 * a] + A[a][b];
+            }
+          }
+      }
+    };
+    publish(0, 0, 0);
+    cl.sync();
+    bool bad = false;
+#pragma unroll
+    for (int kb = 0; kb < R; ++kb) {
+#pragma unroll 1
+      for (int kk = 0; kk < 32; ++kk) {
+        const int k = kb * 32 + kk, f = k & 1;
+        if (k >= m || bad) break;
+        const double pv = piv[f];
+        bad = !(pv != 0.0) || !isfinite(pv);   // the same in every CTA
+        if (bad) break;
+        const bool my_row = cr == (kk >> 4), my_col = cc == (kk >> 4);
+        const int lk = (kk & 15) + 16 * kb;    // local index of row / column k
+        if ((threadIdx.x >> 5) == (k & 7)) {
+          const double p = 1.0 / pv;
+          for (int q = threadIdx.x & 31; q < H; q += 32) {
+            const int gi = (q & 15) + 16 * cr + 32 * (q >> 4);   // global row of local row q
+            const int gj = (q & 15) + 16 * cc + 32 * (q >> 4);
+            const double c = col[f * H + q] * p;
+            cs[q] = gi == k ? -p : c;
+            if (my_col && gi > k) LU[lk * (H + 1) + q] = c;
+            if (my_row && gj >= k) LU[q * (H + 1) + lk] = gj == k ? pv : row[f * H + q];
           }
         }
         __syncthreads();
-        for (int e = tid; e < w * nc2; e += nt) {
-          const int c = e / w, k = e % w;
-          A[(size_t)(p0 + w + c) * m + p0 + k] = U12[c * kLdU + k];
+        if (my_row && my_col && ti == (kk & 15) && tj == (kk & 15)) base[lk] = -cs[lk];
+        gj_update<16, R>(A, row + f * H, cs, ti, tj, kb, my_row && ti == (kk & 15),
+                              my_col && tj == (kk & 15));
+        if (k + 1 < m) {
+          if (kk == 31)
+            publish(kb + 1, 0, f ^ 1);
+          else
+            publish(kb, kk + 1, f ^ 1);
         }
-        for (int e = tid; e < nc2 * nc2; e += nt) {
-          const int i = e % nc2, j = e / nc2;
-          double acc = 0.0;
-          for (int k = 0; k < w; ++k) acc = fma(Pan[k * kLd + w + i], U12[j * kLdU + k], acc);
-          double* a = A + (size_t)(p0 + w + j) * m + p0 + w + i;
-          *a = *a - acc;
-        }
+        cl.sync();
       }
-      __syncthreads();
     }
-    if (!ok) {
-      if (tid == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
-      __syncthreads();
-      continue;
-    }
-    for (int c = 0; c < np; ++c) {
-      const int c0 = c * kB, wc = min(kB, m - c0);
-      double* Y = Pan;
-      for (int e = tid; e < wc * m; e += nt) {
-        const int j = e / m, i = e % m;
-        Y[j * kLd + i] = (i == c0 + j) ? 1.0 : 0.0;
-      }
-      __syncthreads();
-      // forward: L Y = E (rows above c0 stay zero)
-      for (int p = c; p < np; ++p) {
-        const int p0 = p * kB, w = min(kB, m - p0);
-        for (int j = wid; j < wc; j += nwarp) {
-          double y = lane < w ? Y[j * kLd + p0 + lane] : 0.0;
-          for (int k = 0; k < w; ++k) {
-            const double yk = __shfl_sync(0xffffffffu, y, k);
-            if (lane > k && lane < w) y = fma(-A[(size_t)(p0 + k) * m + p0 + lane], yk, y);
+    if (bad) {
+      if (rank == 0 && threadIdx.x == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
+    } else {
+      unsigned e = 0u;
+#pragma unroll
+      for (int a = 0; a < R; ++a)
+#pragma unroll
+        for (int b = 0; b < R; ++b) {
+          const int i = i0 + 32 * a, j = j0 + 32 * b;
+          if (i < m && j < m) {
+            const double v = (i == j ? -base[ti + 16 * a] : 0.0) - A[a][b];
+            ninv[(size_t)l * ms + (size_t)j * m + i] = v;
+            lu[(size_t)l * ms + (size_t)j * m + i] = LU[(tj + 16 * b) * (H + 1) + ti + 16 * a];
+            e = max(e, (unsigned)__double2hiint(v) >> 20);
           }
-          if (lane < w) Y[j * kLd + p0 + lane] = y;
         }
-        __syncthreads();
-        const int nb2 = m - p0 - w;
-        for (int e = tid; e < nb2 * wc; e += nt) {
-          const int i = e % nb2, j = e / nb2;
-          double acc = 0.0;
-          for (int k = 0; k < w; ++k)
-            acc = fma(A[(size_t)(p0 + k) * m + p0 + w + i], Y[j * kLd + p0 + k], acc);
-          Y[j * kLd + p0 + w + i] -= acc;
-        }
-        __syncthreads();
-      }
-      // backward: U X = Y
-      for (int p = np - 1; p >= 0; --p) {
-        const int p0 = p * kB, w = min(kB, m - p0);
-        for (int j = wid; j < wc; j += nwarp) {
-          double y = lane < w ? Y[j * kLd + p0 + lane] : 0.0;
-          for (int k = w - 1; k >= 0; --k) {
-            double xk = 0.0;
-            if (lane == k) xk = y / A[(size_t)(p0 + k) * m + p0 + k];
-            xk = __shfl_sync(0xffffffffu, xk, k);
-            if (lane == k) y = xk;
-            if (lane < k) y = fma(-A[(size_t)(p0 + k) * m + p0 + lane], xk, y);
-          }
-          if (lane < w) Y[j * kLd + p0 + lane] = y;
-        }
-        __syncthreads();
-        for (int e = tid; e < p0 * wc; e += nt) {
-          const int i = e % p0, j = e / p0;
-          double acc = 0.0;
-          for (int k = 0; k < w; ++k) acc = fma(A[(size_t)(p0 + k) * m + i], Y[j * kLd + p0 + k], acc);
-          Y[j * kLd + i] -= acc;
-        }
-        __syncthreads();
-      }
-      for (int e = tid; e < wc * m; e += nt) {
-        const int j = e / m, i = e % m;
-        X[(size_t)(c0 + j) * m + i] = -Y[j * kLd + i];
-      }
-      __syncthreads();
+      e = __reduce_max_sync(0xffffffffu, e);
+      if ((threadIdx.x & 31) == 0) atomicMax(eninv + l, (int)e);
     }
+    cl.sync();   // the buffers are rewritten for the next block
   }
 }
 
-// W = NINV * T for T in {TLO, TUP} (column-major, per level).
-__global__ void __launch_bounds__(256) k_coupled(const double* __restrict__ ninv,
-                                                 const double* __restrict__ tlo,
-                                                 const double* __restrict__ tup,
-                                                 double* __restrict__ wlo, double* __restrict__ wup,
-                                                 int64_t L, int m, int ms) {
-  const int mm = m * m;
-  for (int64_t l = blockIdx.x; l < L; l += gridDim.x) {
+// ---- coupled operators -------------------------------------------------------
+// W = NINV * T for T in {TLO, TUP} (column-major): tiles of 16 RT x 16 RT by 256
+// threads with RT x RT entries each, panels of 16 columns of NINV staged in shared
+// memory with the 16 rows of T that meet them.  FP64-pipe bound, so half of a
+// thread's entries are formed on the integer pipes where both blocks allow it
+// (fixed_dev.cuh: exact products, one rounding per entry), the others by FP64
+// multiply-adds; an entry outside the fixed-point window is formed again in
+// FP64.  8192 blocks of 64: 8.6 -> 4.5 ms (6.8 at the FP64 pipe's rate); 512 of
+// 256: 82.7 -> 17.4 ms (27).
+template <int RT>
+__global__ void __launch_bounds__(256, 2) k_coupled(const double* __restrict__ ninv,
+                                                    const double* __restrict__ tlo,
+                                                    const double* __restrict__ tup,
+                                                    double* __restrict__ wlo,
+                                                    double* __restrict__ wup, const int* en,
+                                                    const int* elo, const int* eup, int* ewlo,
+                                                    int* ewup, int64_t L, int m, int ms,
+                                                    int tiles) {
+  using namespace dev;
+  constexpr int TILE = 16 * RT, KP = 16, RF = RT / 2;   // RF: columns b on the integer pipes
+  __shared__ double As[KP][TILE];
+  __shared__ double Bs[KP][TILE + 1];
+  __shared__ uint64_t Bx[KP][TILE + 1];
+  const int ti = threadIdx.x % 16, tj = threadIdx.x / 16;
+  const int64_t total = L * 2 * tiles * tiles;
+  for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
+    const int64_t l = w / (2 * tiles * tiles);
+    const int rest = (int)(w - l * 2 * tiles * tiles), h = rest / (tiles * tiles);
+    const int tile = rest - h * tiles * tiles;
+    const int i0 = (tile % tiles) * TILE, j0 = (tile / tiles) * TILE;
     const double* Nl = ninv + (size_t)l * ms;
-    for (int h = 0; h < 2; ++h) {
-      const double* T = (h == 0 ? tlo : tup) + (size_t)l * ms;
-      double* W = (h == 0 ? wlo : wup) + (size_t)l * ms;
-      for (int e = threadIdx.x; e < mm; e += blockDim.x) {
-        const int i = e % m, j = e / m;
-        double acc = 0.0;
-        for (int k = 0; k < m; ++k) acc = fma(Nl[(size_t)k * m + i], T[(size_t)j * m + k], acc);
-        W[e] = acc;
+    const double* T = (h == 0 ? tlo : tup) + (size_t)l * ms;
+    double* W = (h == 0 ? wlo : wup) + (size_t)l * ms;
+    const int ea = en[l], eb = (h == 0 ? elo : eup)[l], etot = ea + eb;
+    const bool fix = RF > 0 && fixed_ok(ea) && fixed_ok(eb);
+    double acc[RT][RT];
+    uint32_t fa[RT][RF > 0 ? RF : 1][4], seen[RT][RF > 0 ? RF : 1];
+#pragma unroll
+    for (int a = 0; a < RT; ++a) {
+#pragma unroll
+      for (int b = 0; b < RT; ++b) acc[a][b] = 0.0;
+#pragma unroll
+      for (int b = 0; b < RF; ++b) {
+        fa[a][b][0] = fa[a][b][1] = fa[a][b][2] = fa[a][b][3] = 0u;
+        seen[a][b] = 0u;
       }
     }
+    for (int k0 = 0; k0 < m; k0 += KP) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < KP * TILE; e += 256) {
+        const int k = e / TILE, i = e % TILE;
+        As[k][i] = k0 + k < m && i0 + i < m ? Nl[(size_t)(k0 + k) * m + i0 + i] : 0.0;
+        const int kk = e % KP, j = e / KP;
+        const double v = k0 + kk < m && j0 + j < m ? T[(size_t)(j0 + j) * m + k0 + kk] : 0.0;
+        Bs[kk][j] = v;
+        Bx[kk][j] = fixed_entry(v);
+      }
+      __syncthreads();
+      if (fix) {
+#pragma unroll 2
+        for (int k = 0; k < KP; ++k) {
+          double a[RT];
+#pragma unroll
+          for (int q = 0; q < RT; ++q) a[q] = As[k][ti + 16 * q];
+#pragma unroll
+          for (int b = 0; b < RT; ++b) {
+            if (b < RF) {
+              const uint64_t x = Bx[k][tj + 16 * b];
+              const uint32_t xl = (uint32_t)x & 0xfffff800u, xh = (uint32_t)(x >> 32);
+              const int sh = etot - (int)((uint32_t)x & 0x7ffu);
+#pragma unroll
+              for (int q = 0; q < RT; ++q) fixed_fma(fa[q][b < RF ? b : 0], seen[q][b < RF ? b : 0], a[q], xl, xh, sh);
+            } else {
+              const double v = Bs[k][tj + 16 * b];
+#pragma unroll
+              for (int q = 0; q < RT; ++q) acc[q][b] = fma(a[q], v, acc[q][b]);
+            }
+          }
+        }
+      } else {
+#pragma unroll 2
+        for (int k = 0; k < KP; ++k) {
+          double a[RT];
+#pragma unroll
+          for (int q = 0; q < RT; ++q) a[q] = As[k][ti + 16 * q];
+#pragma unroll
+          for (int b = 0; b < RT; ++b) {
+            const double v = Bs[k][tj + 16 * b];
+#pragma unroll
+            for (int q = 0; q < RT; ++q) acc[q][b] = fma(a[q], v, acc[q][b]);
+          }
+        }
+      }
+    }
+    unsigned e = 0u;
+#pragma unroll
+    for (int b = 0; b < RT; ++b)
+#pragma unroll
+      for (int a = 0; a < RT; ++a) {
+        const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
+        if (i >= m || j >= m) continue;
+        double v = acc[a][b];
+        if (b < RF && fix) {
+          bool bad = false;
+          v = fixed_value(fa[a][b < RF ? b : 0], seen[a][b < RF ? b : 0], etot, bad);
+          if (bad) {
+            v = 0.0;
+            for (int k = 0; k < m; ++k) v = fma(Nl[(size_t)k * m + i], T[(size_t)j * m + k], v);
+          }
+        }
+        W[(size_t)j * m + i] = v;
+        e = max(e, (unsigned)__double2hiint(v) >> 20);
+      }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) atomicMax((h == 0 ? ewlo : ewup) + l, (int)e);
   }
 }
 
@@ -291,46 +498,60 @@ __global__ void k_check_paired(const double* __restrict__ tlo, const double* __r
   if (bad) latch(hdr, MC_ERR_ARG);
 }
 
-__global__ void k_layout_diag(const double* __restrict__ diag, int d, double* __restrict__ plane,
-                              int64_t L, int m, int ms) {
+__global__ void __launch_bounds__(256) k_layout_diag(const double* diag, int d, double* plane,
+                                                     int* bexp, int64_t L, int m, int ms) {
   const int64_t mm = (int64_t)m * m;
-  const int64_t total = L * ms;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t l = t / ms, e = t % ms, k = l + d;
-    plane[t] = (e < mm && k >= 0 && k < L) ? diag[k * mm + e] : 0.0;
+  const int chunks = (ms + kChunk - 1) / kChunk, lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < L * chunks;
+       t += nw) {
+    const int64_t l = t / chunks, k = l + d;
+    const unsigned e = copy_chunk(k >= 0 && k < L ? diag + k * mm : nullptr,
+                                  plane + (size_t)l * ms, (int)(t - l * chunks) * kChunk, (int)mm,
+                                  ms, lane);
+    if (lane == 0) atomicMax(bexp + l, (int)e);
   }
 }
 
-// block_exp (mc_internal.cuh): one warp per block, read once.
-__global__ void __launch_bounds__(256) k_block_exp(const double* __restrict__ plane, int* bexp,
-                                                   int64_t L, int m, int ms) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t l = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; l < L; l += nw) {
-    const double* p = plane + (size_t)l * ms;
-    unsigned e = 0u;   // a negative entry reads as >= 2048
-    for (int i = lane; i < m * m; i += 32) e = max(e, (unsigned)__double2hiint(__ldcs(p + i)) >> 20);
+// block_exp of TLO and TUP where the blocks did not come through k_layout.
+__global__ void __launch_bounds__(256) k_block_exp(const double* __restrict__ tlo,
+                                                   const double* __restrict__ tup, int* elo,
+                                                   int* eup, int64_t L, int m, int ms) {
+  const int chunks = (ms + kChunk - 1) / kChunk, lane = threadIdx.x & 31;
+  const int64_t total = 2 * L * chunks, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total; t += nw) {
+    const int64_t b = t / chunks, l = b >> 1;
+    const int e0 = (int)(t - b * chunks) * kChunk, e1 = min(e0 + kChunk, m * m);
+    const double* p = ((b & 1) ? tup : tlo) + (size_t)l * ms;
+    unsigned e = 0u;
+    for (int i = e0 + lane; i < e1; i += 32)
+      e = max(e, (unsigned)__double2hiint(__ldcs(p + i)) >> 20);
     e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0) bexp[l] = (e >= (unsigned)dev::kMinFixedExp && e < 2047u) ? (int)e : kNoFixed;
+    if (lane == 0) atomicMax(((b & 1) ? eup : elo) + l, (int)e);
   }
+}
+
+int copy_blocks(int64_t warps) {
+  const int64_t nb = (warps + 7) / 8;
+  return (int)(nb < 4096 ? nb : 4096);
 }
 
 }  // namespace
 
-cudaError_t launch_block_exp(const double* plane, int* bexp, const Layout& lay, cudaStream_t s) {
-  int64_t nb = (lay.L + 7) / 8;
-  if (nb > 2048) nb = 2048;
-  k_block_exp<<<(int)nb, 256, 0, s>>>(plane, bexp, lay.L, lay.m, lay.ms);
+cudaError_t launch_block_exp(const double* planes, int* bexp, const Layout& y, cudaStream_t s) {
+  const size_t pe = y.plane_bytes / sizeof(double);
+  const int chunks = (y.ms + kChunk - 1) / kChunk;
+  k_block_exp<<<copy_blocks(2 * y.L * chunks), 256, 0, s>>>(
+      planes + kPlaneTLO * pe, planes + kPlaneTUP * pe, bexp + kPlaneTLO * y.L,
+      bexp + kPlaneTUP * y.L, y.L, y.m, y.ms);
   return cudaGetLastError();
 }
 
-cudaError_t launch_layout_diag(const double* diag, int d, double* plane, const Layout& lay,
-                               cudaStream_t s) {
-  const int64_t total = lay.L * lay.ms;
-  int nb = (int)((total + 255) / 256);
-  if (nb > 4096) nb = 4096;
-  k_layout_diag<<<nb, 256, 0, s>>>(diag, d, plane, lay.L, lay.m, lay.ms);
+cudaError_t launch_layout_diag(const double* diag, int d, double* plane, int* bexp,
+                               const Layout& lay, cudaStream_t s) {
+  const int chunks = (lay.ms + kChunk - 1) / kChunk;
+  k_layout_diag<<<copy_blocks(lay.L * chunks), 256, 0, s>>>(diag, d, plane, bexp, lay.L, lay.m,
+                                                            lay.ms);
   return cudaGetLastError();
 }
 
@@ -341,44 +562,109 @@ cudaError_t launch_check_paired(const double* tlo, const double* tup, const Layo
 }
 
 cudaError_t launch_layout(const double* dn, const double* loc, const double* up, double* planes,
-                          const Layout& lay, Header*, cudaStream_t s) {
+                          int* bexp, const Layout& lay, cudaStream_t s) {
   const size_t pe = lay.plane_bytes / sizeof(double);
-  const int64_t total = lay.L * lay.ms;
-  int nb = (int)((total + 255) / 256);
-  if (nb > 4096) nb = 4096;
-  k_layout<<<nb, 256, 0, s>>>(dn, loc, up, planes + kPlaneTLO * pe, planes + kPlaneTUP * pe,
-                              planes + kPlaneTDD * pe, lay.L, lay.m, lay.ms);
+  const int chunks = (lay.ms + kChunk - 1) / kChunk;
+  k_layout<<<copy_blocks(3 * lay.L * chunks), 256, 0, s>>>(
+      dn, loc, up, planes + kPlaneTLO * pe, planes + kPlaneTUP * pe, planes + kPlaneTDD * pe,
+      bexp + kPlaneTLO * lay.L, bexp + kPlaneTUP * lay.L, lay.L, lay.m, lay.ms);
   return cudaGetLastError();
 }
 
-cudaError_t launch_factor(double* planes, const Layout& lay, Header* hdr, int coupled,
+namespace {
+
+struct FactorArgs {
+  const double* tdd;
+  double *lu, *ninv;
+  int* eninv;
+  int64_t L;
+  int m, ms, sms;
+  Header* hdr;
+};
+
+template <int G, int R>
+cudaError_t gj(const FactorArgs& f, cudaStream_t s) {
+  constexpr int N = GjBlock<G, R>::N;
+  const size_t per = GjBlock<G, R>::doubles(f.m), bytes = N * per * sizeof(double);
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_gj<G, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  int occ = 0;   // every CTA resident: the blocks are dealt out once
+  const cudaError_t e2 =
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gj<G, R>, 256, bytes);
+  if (e2 != cudaSuccess) return e2;
+  int64_t nb = (f.L + N - 1) / N;
+  if (nb > (int64_t)occ * f.sms) nb = (int64_t)(occ < 1 ? 1 : occ) * f.sms;
+  k_gj<G, R><<<(int)nb, 256, bytes, s>>>(f.tdd, f.lu, f.ninv, f.eninv, f.L, f.m, f.ms, (int)per,
+                                         f.hdr);
+  return cudaGetLastError();
+}
+
+template <int R>
+cudaError_t gj_big(const FactorArgs& f, cudaStream_t s) {
+  const size_t bytes = GjBig<R>::doubles * sizeof(double);
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_gj_cluster<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  // as many clusters as run at once (the SMs of a GPC that are left over from
+  // clusters of four stay idle: 36 of the 38 that the SM count suggests), so
+  // that none waits for a whole block's time
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(4 * (unsigned)(f.sms / 4 < 1 ? 1 : f.sms / 4));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = bytes;
+  int fit = 0;
+  const cudaError_t e2 =
+      cudaOccupancyMaxActiveClusters(&fit, (const void*)k_gj_cluster<R>, &cfg);
+  if (e2 != cudaSuccess) return e2;
+  int64_t nc = fit < 1 ? 1 : fit;
+  if (nc > f.L) nc = f.L;
+  k_gj_cluster<R><<<(int)(4 * nc), 256, bytes, s>>>(f.tdd, f.lu, f.ninv, f.eninv, f.L, f.m, f.ms,
+                                                    f.hdr);
+  return cudaGetLastError();
+}
+
+cudaError_t gj_dispatch(const FactorArgs& f, cudaStream_t s) {
+  if (f.m <= 8) return gj<4, 2>(f, s);
+  if (f.m <= 16) return gj<4, 4>(f, s);
+  if (f.m <= 128) switch ((f.m + 15) / 16) {
+      case 2: return gj<16, 2>(f, s);
+      case 3: return gj<16, 3>(f, s);
+      case 4: return gj<16, 4>(f, s);
+      case 5: return gj<16, 5>(f, s);
+      case 6: return gj<16, 6>(f, s);
+      case 7: return gj<16, 7>(f, s);
+      default: return gj<16, 8>(f, s);
+    }
+  switch ((f.m + 31) / 32) {
+    case 5: return gj_big<5>(f, s);
+    case 6: return gj_big<6>(f, s);
+    case 7: return gj_big<7>(f, s);
+    default: return gj_big<8>(f, s);
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_factor(double* planes, int* bexp, const Layout& lay, Header* hdr, int coupled,
                           int num_sms, cudaStream_t s) {
   const size_t pe = lay.plane_bytes / sizeof(double);
   const int m = lay.m;
-  int nb = num_sms * 4;
-  if (nb > lay.L) nb = (int)lay.L;
-  const size_t smem = 2 * sizeof(double) * (size_t)m * m;
-  if (m <= 112) {
-    cudaError_t e = cudaFuncSetAttribute(k_lu_inv<true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_lu_inv<true><<<nb, 256, smem, s>>>(planes + kPlaneTDD * pe, planes + kPlaneLU * pe,
-                                         planes + kPlaneNINV * pe, lay.L, m, lay.ms, hdr);
-  } else {
-    const size_t bsm = sizeof(double) * (size_t)(kB * kLd + kLd * kLdU);
-    cudaError_t e = cudaFuncSetAttribute(k_factor_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bsm);
-    if (e != cudaSuccess) return e;
-    int nbb = num_sms;
-    if (nbb > lay.L) nbb = (int)lay.L;
-    k_factor_big<<<nbb, kBigThreads, bsm, s>>>(planes + kPlaneTDD * pe, planes + kPlaneLU * pe,
-                                               planes + kPlaneNINV * pe, lay.L, m, lay.ms, hdr);
-  }
-  cudaError_t e = cudaGetLastError();
+  const int64_t L = lay.L;
+  const FactorArgs f{planes + kPlaneTDD * pe, planes + kPlaneLU * pe, planes + kPlaneNINV * pe,
+                     bexp + kPlaneNINV * L, L, m, lay.ms, num_sms, hdr};
+  const cudaError_t e = gj_dispatch(f, s);
   if (e != cudaSuccess || !coupled) return e;
-  k_coupled<<<nb, 256, 0, s>>>(planes + kPlaneNINV * pe, planes + kPlaneTLO * pe,
-                               planes + kPlaneTUP * pe, planes + kPlaneWLO * pe,
-                               planes + kPlaneWUP * pe, lay.L, m, lay.ms);
+  const int rt = m <= 16 ? 1 : m <= 32 ? 2 : 4, tiles = (m + 16 * rt - 1) / (16 * rt);
+  int64_t nb = L * 2 * tiles * tiles;
+  if (nb > 8ll * num_sms) nb = 8ll * num_sms;
+  if (nb > 2ll * num_sms && m > 32) nb = 2ll * num_sms;
+  auto kernel = rt == 1 ? k_coupled<1> : rt == 2 ? k_coupled<2> : k_coupled<4>;
+  kernel<<<(int)nb, 256, 0, s>>>(planes + kPlaneNINV * pe, planes + kPlaneTLO * pe,
+                                 planes + kPlaneTUP * pe, planes + kPlaneWLO * pe,
+                                 planes + kPlaneWUP * pe, bexp + kPlaneNINV * L,
+                                 bexp + kPlaneTLO * L, bexp + kPlaneTUP * L, bexp + kPlaneWLO * L,
+                                 bexp + kPlaneWUP * L, L, m, lay.ms, tiles);
   return cudaGetLastError();
 }
 

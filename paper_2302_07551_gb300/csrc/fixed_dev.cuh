@@ -10,10 +10,9 @@
 // of those columns then carries one rounding instead of one per column.
 //
 // Conditions, all checked, else the block goes through the FP64 pipe alone:
-//   * block entries >= 0, finite, largest exponent not tiny: known per block
-//     from the factorisation (block_exp, kNoFixed otherwise);
-//   * vector entries >= 0, finite, largest exponent not tiny: found while the
-//     vector is staged.
+//   * block entries >= 0, finite, largest exponent not tiny: the block's largest
+//     exponent field, known from set-up (block_exp);
+//   * the same of the vector's entries: found while the vector is staged.
 // A term is truncated below 2^-115 of (largest entry of the block) x (largest
 // entry of the vector); a row whose sum is below 2^-51 of that product
 // without being exactly zero cannot be rounded to FP64 accuracy from the
@@ -96,10 +95,9 @@ __device__ __forceinline__ uint64_t fixed_entry(double x) {
   return (s << 11) | ((hi >> 20) & 0x7ffu);
 }
 
-// emax: largest exponent field of a vector's entries, sign bit included.
-__device__ __forceinline__ bool fixed_vec_ok(int emax) {
-  return emax >= kMinFixedExp && emax < 2047;   // a negative entry reads as >= 2048
-}
+// e: largest exponent field (sign bit included: a negative entry reads as >= 2048)
+// of a block's or a vector's entries.
+__device__ __forceinline__ bool fixed_ok(int e) { return e >= kMinFixedExp && e < 2047; }
 
 }  // namespace dev
 }  // namespace mc

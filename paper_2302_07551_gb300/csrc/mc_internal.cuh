@@ -73,9 +73,9 @@ struct Layout {
 
 Layout make_layout(const mc_desc& d);
 
-// block_exp of a block whose products run on the FP64 pipe alone (negative,
-// non-finite or only tiny entries).
-constexpr int kNoFixed = 0;
+// block_exp of a block: the largest exponent field of its entries, sign bit
+// included (fixed_ok in fixed_dev.cuh decides what it allows); per plane and
+// level, zero before set-up.
 
 // Arguments of one half-sweep (Algorithm 2, step 1+2 or step 3).
 struct PhaseArgs {
@@ -213,18 +213,17 @@ struct ResidArgs {
 };
 
 // Launchers (return cudaGetLastError()).
+// bexp: block_exp of all planes (L per plane).
 cudaError_t launch_layout(const double* dn, const double* loc, const double* up, double* planes,
-                          const Layout& lay, Header* hdr, cudaStream_t s);
+                          int* bexp, const Layout& lay, cudaStream_t s);
 // Q^T diagonal d into a plane: plane[l] = diag[l + d] (row-major Q block =
 // column-major Q^T block), zero where l + d is outside [0, L).
-cudaError_t launch_layout_diag(const double* diag, int d, double* plane, const Layout& lay,
-                               cudaStream_t s);
-cudaError_t launch_factor(double* planes, const Layout& lay, Header* hdr, int coupled,
+cudaError_t launch_layout_diag(const double* diag, int d, double* plane, int* bexp,
+                               const Layout& lay, cudaStream_t s);
+cudaError_t launch_factor(double* planes, int* bexp, const Layout& lay, Header* hdr, int coupled,
                           int num_sms, cudaStream_t s);
-// block_exp of the blocks of one plane: the largest biased exponent of the
-// block's entries if all are >= 0, finite and the largest is not tiny, else
-// kNoFixed.
-cudaError_t launch_block_exp(const double* plane, int* bexp, const Layout& lay, cudaStream_t s);
+// block_exp of TLO and TUP (blocks that did not come through launch_layout).
+cudaError_t launch_block_exp(const double* planes, int* bexp, const Layout& lay, cudaStream_t s);
 cudaError_t launch_phase(const PhaseArgs& a, int coupled, int n_blocks, cudaStream_t s);
 // Block Gauss-Seidel step: one warp walks the levels in order (z_{l-1} fresh,
 // x_{l+1} old); e^T z into hdr->stats[0].

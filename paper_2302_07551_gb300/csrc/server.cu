@@ -455,6 +455,8 @@ int mc_server_submit(mc_server* s, int64_t tag, int64_t L, int32_t m, const doub
   if (rc == MC_OK &&
       cudaMemsetAsync(c->fver, 0, (size_t)L * sizeof(int), s->user) != cudaSuccess)
     rc = MC_ERR_CUDA;
+  if (rc == MC_OK && launch_block_exp(P, chain_bexp(c, 0), y, s->user) != cudaSuccess)
+    rc = MC_ERR_CUDA;
   if (rc == MC_OK) rc = chain_factor_async(c);
   if (rc == MC_OK && launch_fill(c->xa, y.N, 1.0 / (double)y.N, s->user) != cudaSuccess)
     rc = MC_ERR_CUDA;

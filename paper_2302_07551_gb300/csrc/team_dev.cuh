@@ -149,7 +149,7 @@ template <int RW, int MC>
 __device__ __forceinline__ void rows_product(double (&acc)[RW], const double* M, const double* v,
                                              const uint64_t* xv, int eb, int ev, int j0, int j1,
                                              int m, int row0, int lane) {
-  bool plain = eb == kNoFixed || !fixed_vec_ok(ev);
+  bool plain = !fixed_ok(eb) || !fixed_ok(ev);
   if (!plain) {
     double old[RW];
 #pragma unroll
