@@ -3,6 +3,8 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "fixed_dev.cuh"
 #include "mc_internal.cuh"
 
@@ -364,13 +366,105 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
 
 // ---- coupled operators -------------------------------------------------------
 // W = NINV * T for T in {TLO, TUP} (column-major): tiles of 16 RT x 16 RT by 256
-// threads with RT x RT entries each, panels of 16 columns of NINV staged in shared
-// memory with the 16 rows of T that meet them.  FP64-pipe bound, so half of a
+// threads with up to RT x RT entries each (fewer in the last tiles of a block),
+// panels of 16 columns of NINV staged in shared memory with the 16 rows of T that
+// meet them.  FP64-pipe bound, so half of a
 // thread's entries are formed on the integer pipes where both blocks allow it
 // (fixed_dev.cuh: exact products, one rounding per entry), the others by FP64
 // multiply-adds; an entry outside the fixed-point window is formed again in
 // FP64.  8192 blocks of 64: 8.6 -> 4.5 ms (6.8 at the FP64 pipe's rate); 512 of
 // 256: 82.7 -> 17.4 ms (27).
+constexpr int kPanel = 16;   // columns of NINV per panel
+template <int TILE>
+struct CoupledShared {
+  double A[kPanel][TILE];
+  double B[kPanel][TILE + 1];
+  uint64_t X[kPanel][TILE + 1];   // integer form of B
+};
+
+// One tile: rows i0 + ti + 16 a (a < RA), columns j0 + tj + 16 b (b < RB) of W.
+template <int TILE, int RA, int RB, bool FIX>
+__device__ __forceinline__ unsigned coupled_tile(CoupledShared<TILE>& sh, const double* Nl,
+                                                 const double* T, double* W, int etot, int i0,
+                                                 int j0, int m) {
+  using namespace dev;
+  constexpr int RF = FIX ? RB / 2 : 0, RX = RF > 0 ? RF : 1;   // columns on the integer pipes
+  const int ti = threadIdx.x % 16, tj = threadIdx.x / 16;
+  double acc[RA][RB];
+  uint32_t fa[RA][RX][4], seen[RA][RX];
+#pragma unroll
+  for (int a = 0; a < RA; ++a) {
+#pragma unroll
+    for (int b = 0; b < RB; ++b) acc[a][b] = 0.0;
+#pragma unroll
+    for (int b = 0; b < RX; ++b) {
+      fa[a][b][0] = fa[a][b][1] = fa[a][b][2] = fa[a][b][3] = 0u;
+      seen[a][b] = 0u;
+    }
+  }
+  for (int k0 = 0; k0 < m; k0 += kPanel) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < kPanel * 16 * RA; e += 256) {
+      const int k = e / (16 * RA), i = e % (16 * RA);
+      sh.A[k][i] = k0 + k < m && i0 + i < m ? Nl[(size_t)(k0 + k) * m + i0 + i] : 0.0;
+    }
+    for (int e = threadIdx.x; e < kPanel * 16 * RB; e += 256) {
+      const int k = e % kPanel, j = e / kPanel;
+      const double v = k0 + k < m && j0 + j < m ? T[(size_t)(j0 + j) * m + k0 + k] : 0.0;
+      sh.B[k][j] = v;
+      if (RF > 0) sh.X[k][j] = fixed_entry(v);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int k = 0; k < kPanel; ++k) {
+      double a[RA];
+#pragma unroll
+      for (int q = 0; q < RA; ++q) a[q] = sh.A[k][ti + 16 * q];
+#pragma unroll
+      for (int b = 0; b < RB; ++b) {
+        if (b < RF) {
+          const uint64_t x = sh.X[k][tj + 16 * b];
+          const uint32_t xl = (uint32_t)x & 0xfffff800u, xh = (uint32_t)(x >> 32);
+          const int s = etot - (int)((uint32_t)x & 0x7ffu);
+#pragma unroll
+          for (int q = 0; q < RA; ++q)
+            fixed_fma(fa[q][b < RF ? b : 0], seen[q][b < RF ? b : 0], a[q], xl, xh, s);
+        } else {
+          const double v = sh.B[k][tj + 16 * b];
+#pragma unroll
+          for (int q = 0; q < RA; ++q) acc[q][b] = fma(a[q], v, acc[q][b]);
+        }
+      }
+    }
+  }
+  unsigned e = 0u;
+#pragma unroll
+  for (int b = 0; b < RB; ++b)
+#pragma unroll
+    for (int a = 0; a < RA; ++a) {
+      const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
+      if (i >= m || j >= m) continue;
+      double v = acc[a][b];
+      if (b < RF) {
+        bool bad = false;
+        v = fixed_value(fa[a][b < RF ? b : 0], seen[a][b < RF ? b : 0], etot, bad);
+        if (bad) {
+          v = 0.0;
+          for (int k = 0; k < m; ++k) v = fma(Nl[(size_t)k * m + i], T[(size_t)j * m + k], v);
+        }
+      }
+      W[(size_t)j * m + i] = v;
+      e = max(e, (unsigned)__double2hiint(v) >> 20);
+    }
+  return e;
+}
+
+// 16-row groups of a tile that starts at x, rounded up to a size that has code.
+__device__ __forceinline__ int tile_groups(int x, int m) {
+  const int g = (m - x + 15) / 16;
+  return g >= 3 ? 4 : g;
+}
+
 template <int RT>
 __global__ void __launch_bounds__(256, 2) k_coupled(const double* __restrict__ ninv,
                                                     const double* __restrict__ tlo,
@@ -380,103 +474,66 @@ __global__ void __launch_bounds__(256, 2) k_coupled(const double* __restrict__ n
                                                     const int* elo, const int* eup, int* ewlo,
                                                     int* ewup, int64_t L, int m, int ms,
                                                     int tiles) {
-  using namespace dev;
-  constexpr int TILE = 16 * RT, KP = 16, RF = RT / 2;   // RF: columns b on the integer pipes
-  __shared__ double As[KP][TILE];
-  __shared__ double Bs[KP][TILE + 1];
-  __shared__ uint64_t Bx[KP][TILE + 1];
-  const int ti = threadIdx.x % 16, tj = threadIdx.x / 16;
+  constexpr int TILE = 16 * RT;
+  __shared__ CoupledShared<TILE> sh;
   const int64_t total = L * 2 * tiles * tiles;
   for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
-    const int64_t l = w / (2 * tiles * tiles);
-    const int rest = (int)(w - l * 2 * tiles * tiles), h = rest / (tiles * tiles);
-    const int tile = rest - h * tiles * tiles;
+    // tile by tile over all levels: every CTA gets its share of full and partial tiles
+    const int tile = (int)(w / (2 * L));
+    const int64_t rest = w - tile * 2 * L, l = rest >> 1;
+    const int h = (int)(rest & 1);
     const int i0 = (tile % tiles) * TILE, j0 = (tile / tiles) * TILE;
     const double* Nl = ninv + (size_t)l * ms;
     const double* T = (h == 0 ? tlo : tup) + (size_t)l * ms;
     double* W = (h == 0 ? wlo : wup) + (size_t)l * ms;
     const int ea = en[l], eb = (h == 0 ? elo : eup)[l], etot = ea + eb;
-    const bool fix = RF > 0 && fixed_ok(ea) && fixed_ok(eb);
-    double acc[RT][RT];
-    uint32_t fa[RT][RF > 0 ? RF : 1][4], seen[RT][RF > 0 ? RF : 1];
-#pragma unroll
-    for (int a = 0; a < RT; ++a) {
-#pragma unroll
-      for (int b = 0; b < RT; ++b) acc[a][b] = 0.0;
-#pragma unroll
-      for (int b = 0; b < RF; ++b) {
-        fa[a][b][0] = fa[a][b][1] = fa[a][b][2] = fa[a][b][3] = 0u;
-        seen[a][b] = 0u;
-      }
-    }
-    for (int k0 = 0; k0 < m; k0 += KP) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < KP * TILE; e += 256) {
-        const int k = e / TILE, i = e % TILE;
-        As[k][i] = k0 + k < m && i0 + i < m ? Nl[(size_t)(k0 + k) * m + i0 + i] : 0.0;
-        const int kk = e % KP, j = e / KP;
-        const double v = k0 + kk < m && j0 + j < m ? T[(size_t)(j0 + j) * m + k0 + kk] : 0.0;
-        Bs[kk][j] = v;
-        Bx[kk][j] = fixed_entry(v);
-      }
-      __syncthreads();
-      if (fix) {
-#pragma unroll 2
-        for (int k = 0; k < KP; ++k) {
-          double a[RT];
-#pragma unroll
-          for (int q = 0; q < RT; ++q) a[q] = As[k][ti + 16 * q];
-#pragma unroll
-          for (int b = 0; b < RT; ++b) {
-            if (b < RF) {
-              const uint64_t x = Bx[k][tj + 16 * b];
-              const uint32_t xl = (uint32_t)x & 0xfffff800u, xh = (uint32_t)(x >> 32);
-              const int sh = etot - (int)((uint32_t)x & 0x7ffu);
-#pragma unroll
-              for (int q = 0; q < RT; ++q) fixed_fma(fa[q][b < RF ? b : 0], seen[q][b < RF ? b : 0], a[q], xl, xh, sh);
-            } else {
-              const double v = Bs[k][tj + 16 * b];
-#pragma unroll
-              for (int q = 0; q < RT; ++q) acc[q][b] = fma(a[q], v, acc[q][b]);
-            }
-          }
-        }
-      } else {
-#pragma unroll 2
-        for (int k = 0; k < KP; ++k) {
-          double a[RT];
-#pragma unroll
-          for (int q = 0; q < RT; ++q) a[q] = As[k][ti + 16 * q];
-#pragma unroll
-          for (int b = 0; b < RT; ++b) {
-            const double v = Bs[k][tj + 16 * b];
-#pragma unroll
-            for (int q = 0; q < RT; ++q) acc[q][b] = fma(a[q], v, acc[q][b]);
-          }
-        }
-      }
-    }
+    const bool fix = dev::fixed_ok(ea) && dev::fixed_ok(eb);
     unsigned e = 0u;
-#pragma unroll
-    for (int b = 0; b < RT; ++b)
-#pragma unroll
-      for (int a = 0; a < RT; ++a) {
-        const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
-        if (i >= m || j >= m) continue;
-        double v = acc[a][b];
-        if (b < RF && fix) {
-          bool bad = false;
-          v = fixed_value(fa[a][b < RF ? b : 0], seen[a][b < RF ? b : 0], etot, bad);
-          if (bad) {
-            v = 0.0;
-            for (int k = 0; k < m; ++k) v = fma(Nl[(size_t)k * m + i], T[(size_t)j * m + k], v);
-          }
-        }
-        W[(size_t)j * m + i] = v;
-        e = max(e, (unsigned)__double2hiint(v) >> 20);
-      }
+    auto run = [&](auto ra, auto rb) {
+      constexpr int RA = decltype(ra)::value, RB = decltype(rb)::value;
+      if constexpr (RA <= RT && RB <= RT)
+        e = fix && RB > 1 ? coupled_tile<TILE, RA, RB, (RB > 1)>(sh, Nl, T, W, etot, i0, j0, m)
+                          : coupled_tile<TILE, RA, RB, false>(sh, Nl, T, W, etot, i0, j0, m);
+    };
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
+    using I4 = std::integral_constant<int, 4>;
+    switch (tile_groups(i0, m) * 8 + tile_groups(j0, m)) {
+      case 9: run(I1(), I1()); break;
+      case 10: run(I1(), I2()); break;
+      case 12: run(I1(), I4()); break;
+      case 17: run(I2(), I1()); break;
+      case 18: run(I2(), I2()); break;
+      case 20: run(I2(), I4()); break;
+      case 33: run(I4(), I1()); break;
+      case 34: run(I4(), I2()); break;
+      default: run(I4(), I4()); break;
+    }
     e = __reduce_max_sync(0xffffffffu, e);
     if ((threadIdx.x & 31) == 0) atomicMax((h == 0 ? ewlo : ewup) + l, (int)e);
+  }
+}
+
+// W for m <= 16: one entry per thread over all blocks (the sweeps of such blocks
+// use no exponents).
+__global__ void __launch_bounds__(256) k_coupled_small(const double* __restrict__ ninv,
+                                                       const double* __restrict__ tlo,
+                                                       const double* __restrict__ tup,
+                                                       double* __restrict__ wlo,
+                                                       double* __restrict__ wup, int64_t L, int m,
+                                                       int ms) {
+  const int mm = m * m;
+  const int64_t total = 2 * L * mm;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = t / mm, l = b >> 1;
+    const int e = (int)(t - b * mm), j = e / m, i = e - j * m;
+    const double* N = ninv + (size_t)l * ms + i;
+    const double* T = ((b & 1) ? tup : tlo) + (size_t)l * ms + j * m;
+    double acc = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < m; ++k) acc = fma(N[k * m], T[k], acc);
+    ((b & 1) ? wup : wlo)[(size_t)l * ms + e] = acc;
   }
 }
 
@@ -655,11 +712,17 @@ cudaError_t launch_factor(double* planes, int* bexp, const Layout& lay, Header* 
                      bexp + kPlaneNINV * L, L, m, lay.ms, num_sms, hdr};
   const cudaError_t e = gj_dispatch(f, s);
   if (e != cudaSuccess || !coupled) return e;
-  const int rt = m <= 16 ? 1 : m <= 32 ? 2 : 4, tiles = (m + 16 * rt - 1) / (16 * rt);
+  if (m <= 16) {
+    const int64_t nb = (2 * L * m * m + 255) / 256;
+    k_coupled_small<<<(int)(nb < 8192 ? nb : 8192), 256, 0, s>>>(
+        planes + kPlaneNINV * pe, planes + kPlaneTLO * pe, planes + kPlaneTUP * pe,
+        planes + kPlaneWLO * pe, planes + kPlaneWUP * pe, L, m, lay.ms);
+    return cudaGetLastError();
+  }
+  const int rt = m <= 32 ? 2 : 4, tiles = (m + 16 * rt - 1) / (16 * rt);
   int64_t nb = L * 2 * tiles * tiles;
-  if (nb > 8ll * num_sms) nb = 8ll * num_sms;
-  if (nb > 2ll * num_sms && m > 32) nb = 2ll * num_sms;
-  auto kernel = rt == 1 ? k_coupled<1> : rt == 2 ? k_coupled<2> : k_coupled<4>;
+  if (nb > 2ll * num_sms) nb = 2ll * num_sms;
+  auto kernel = rt == 2 ? k_coupled<2> : k_coupled<4>;
   kernel<<<(int)nb, 256, 0, s>>>(planes + kPlaneNINV * pe, planes + kPlaneTLO * pe,
                                  planes + kPlaneTUP * pe, planes + kPlaneWLO * pe,
                                  planes + kPlaneWUP * pe, bexp + kPlaneNINV * L,

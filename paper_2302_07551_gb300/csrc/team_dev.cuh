@@ -144,12 +144,13 @@ __device__ __forceinline__ void rows_f64(double (&acc)[RW], const double* __rest
 
 // acc += M v on both pipes where the block's and the vector's exponents allow
 // it, on the FP64 pipe alone otherwise or when a row's sum left the window
-// (decided per warp from the data alone).
+// (decided per warp from the data alone), and for m <= 16: joining the two sums
+// costs more than the few columns save.
 template <int RW, int MC>
 __device__ __forceinline__ void rows_product(double (&acc)[RW], const double* M, const double* v,
                                              const uint64_t* xv, int eb, int ev, int j0, int j1,
                                              int m, int row0, int lane) {
-  bool plain = !fixed_ok(eb) || !fixed_ok(ev);
+  bool plain = m <= 16 || !fixed_ok(eb) || !fixed_ok(ev);
   if (!plain) {
     double old[RW];
 #pragma unroll
