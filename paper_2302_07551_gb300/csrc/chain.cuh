@@ -9,7 +9,8 @@ struct mc_chain {
   char* ws;
   cudaStream_t user;         // caller's stream: every enqueue goes here
   cudaStream_t cap;          // private stream used only to capture graphs
-  int num_sms;
+  int num_sms, dev;
+  int hh_busy;               // a copy into hh may be in flight
   int factored;
   int nb_phase, nw;          // persistent sweep grid (blocks, warps)
   int nb_norm, nb_resid;
