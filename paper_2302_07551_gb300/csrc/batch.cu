@@ -8,6 +8,7 @@
 
 #include "batch.cuh"
 #include "lowprec_dev.cuh"
+#include "lpteam_dev.cuh"
 #include "sweep_dev.cuh"
 #include "wave_dev.cuh"
 
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(256) k_b_zero_d(const BTable* __restrict__ t) 
   for (int64_t i = gw; i < tot; i += nw) {
     const int r = find_req(t->off_lv, 0, t->n, i);
     const BReq* q = &t->r[r];
+    if (q->path != kPathQueue) continue;
     const int64_t l = i - t->off_lv[r];
     for (int k = lane; k < q->m; k += 32) q->d[l * q->m + k] = 0.0f;
   }
@@ -338,6 +340,67 @@ __global__ void __launch_bounds__(256) k_b_sweeps_lp(const BTable* __restrict__ 
     publish_levels(Q->ver, u.l, 2, u.n, base + (int)u.k + 1, lane);
     q = __shfl_sync(kFull, q0, 0);
   }
+}
+
+// Correction sweeps of the team-path requests of one size class: units are single
+// levels in the order (sweep, half-sweep, request, level), claimed by teams of TW
+// warps.  Versions go on from chunk to chunk (the epoch), so the words need no
+// reset.
+template <typename S, int ROWS, int TW, bool COUPLED>
+__global__ void __launch_bounds__(256, 2) k_b_team(const BTable* __restrict__ t, int K, int cls,
+                                                   unsigned long long* claim, BOut* out) {
+  extern __shared__ __align__(16) unsigned char lp_smem[];
+  if ((int)blockIdx.x >= t->team_ctas[cls]) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / TW, w = warp % TW, tt = threadIdx.x - team * TW * 32, bar = 1 + team;
+  auto& sh = reinterpret_cast<LpTeamShared<ROWS, TW>*>(lp_smem)[team];
+  int r0, r1;
+  class_range(t, cls, cls + 1, r0, r1);
+  const int64_t a0 = t->off_t1[r0], b0 = t->off_t2[r0];
+  const int64_t n1 = t->off_t1[r1] - a0, U = n1 + (t->off_t2[r1] - b0);
+  const unsigned long long total = (unsigned long long)K * (unsigned long long)U;
+  const int base = t->epoch;
+  unsigned long long q0 = w == 0 ? claim_unit(claim, lane) : 0ull, q;
+  if (w == 0 && lane == 0) sh.next[1] = q0;
+  if (w == 0) q0 = claim_unit(claim, lane);
+  lp_sync<TW>(bar);
+  q = sh.next[1];
+  int turn = 0;
+  while (q < total) {
+    unsigned long long qn = 0ull;
+    if (w == 0 && lane == 0) sh.next[turn] = q0;
+    const int64_t k = (int64_t)(q / (unsigned long long)U), rr = (int64_t)q - k * U;
+    const bool h2 = rr >= n1;
+    const int64_t* off = h2 ? t->off_t2 : t->off_t1;
+    const int64_t i = h2 ? b0 + (rr - n1) : a0 + rr;
+    const int r = find_req(off, r0, r1, i);
+    const BReq* Q = &t->r[r];
+    const LpLevels v{Q->lA, Q->lB, Q->lC, Q->sc, Q->q, Q->dv, Q->d, Q->L, Q->lp_bs, Q->lp_cbs,
+                     Q->m};
+    const LpUnit u{2 * (i - off[r]) + (h2 ? 1 - Q->p1 : Q->p1), base + (int)(h2 ? k + 1 : k),
+                   base + (int)k + 1, k == 0 && !h2, k == K - 1};
+    LpAhead<S, ROWS, TW, COUPLED> p;
+    p.load(v, u, w, tt, lane);
+    lp_team_unit<S, ROWS, TW, COUPLED>(v, sh, u, p, w, tt, lane, bar, &out[r].status, kWaitNs,
+                                       [&]() {
+                                         qn = sh.next[turn];
+                                         turn ^= 1;
+                                         if (w == 0) q0 = claim_unit(claim, lane);
+                                       });
+    q = qn;
+  }
+}
+
+template <typename S, bool C>
+cudaError_t team_launches(const BTable* t, unsigned long long* claim, BOut* out, int K, int sms,
+                          const cudaStream_t* b) {
+  k_b_team<S, 64, 4, C><<<2 * sms, 256, 2 * sizeof(LpTeamShared<64, 4>), b[0]>>>(t, K, 1,
+                                                                               claim + 1, out);
+  k_b_team<S, 128, 8, C><<<2 * sms, 256, sizeof(LpTeamShared<128, 8>), b[1]>>>(t, K, 2, claim + 2,
+                                                                              out);
+  k_b_team<S, 256, 8, C><<<2 * sms, 256, sizeof(LpTeamShared<256, 8>), b[2]>>>(t, K, 3, claim + 3,
+                                                                              out);
+  return cudaGetLastError();
 }
 
 template <typename K>
@@ -438,6 +501,23 @@ cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out,
     e = coupled ? lp_buckets<float, float, true>(t, t_claim, out, inner, g, s)
                 : lp_buckets<float, float, false>(t, t_claim, out, inner, g, s);
   return e;
+}
+
+int b_lp_path(const Layout& y, int coupled, int num_sms) {
+  if (resident_batch_fits(y, coupled)) return kPathResident;
+  if (y.m > 32 && (y.lp == 1 || y.m % 8 == 0) &&
+      y.L / 2 * (y.m <= 64 ? 4 : 8) <= 16ll * num_sms)   // as launch_sweeps_lp
+    return kPathTeam;
+  return kPathQueue;
+}
+
+cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out, int bf16,
+                      int coupled, int inner, int num_sms, const cudaStream_t* b) {
+  if (bf16)
+    return coupled ? team_launches<unsigned short, true>(t, team_claim, out, inner, num_sms, b)
+                   : team_launches<unsigned short, false>(t, team_claim, out, inner, num_sms, b);
+  return coupled ? team_launches<float, true>(t, team_claim, out, inner, num_sms, b)
+                 : team_launches<float, false>(t, team_claim, out, inner, num_sms, b);
 }
 
 cudaError_t b_lp_finish(const BTable* t, BOut* out, BTune g, cudaStream_t s) {

@@ -53,8 +53,10 @@ struct BReq {
   double* lsum2;        // fused sweeps: [2][L] level sums of the last two sweeps
   int* ver;             // fused sweeps: per-level completion counters
   int64_t L;
+  unsigned long long* dv;   // versioned words of the correction (team path)
   int32_t m, ms, R, p1;  // p1: 0-based parity of the diagonal-only rows
-  int32_t G, pad;        // levels per unit of this request (the table's G scaled by size class)
+  int32_t G, path;       // levels per unit of this request (the table's G scaled by size
+                         // class); kPathQueue, ...
   int64_t lp_bs, lp_cbs;
 };
 
@@ -70,17 +72,38 @@ __host__ __device__ inline int class_group(int G, int m) {
   return g > 16 ? 16 : g;
 }
 
+// How a request's low-precision correction sweeps run, by its own size alone (so
+// that its iterates do not depend on the batch):
+//   kPathQueue: one warp per unit of G levels, all such requests in shared launches
+//     by size class (k_b_sweeps_lp);
+//   kPathTeam: short chains of blocks of more than 32 rows, a team of warps per
+//     level (lpteam_dev.cuh), all such requests of a size class in one launch;
+//   kPathResident: small blocks that fit one cluster's shared memory, one cluster
+//     per request (resident_dev.cuh).
+// The launches of the three paths run side by side; the host deals out CTAs to
+// them with the table.  Eight requests of 131 KB to 17 MB
+// (BF16 coupled, m = 16 to 128): a chunk of 64 sweeps 2.70 -> 0.99 ms with all of them
+// running, 1.32 -> 0.24 ms with the last two small ones.
+enum { kPathQueue = 0, kPathTeam = 1, kPathResident = 2 };
+constexpr int kResidentClusters = 8;   // clusters of 16 in a launch
+
 struct BTable {
   int32_t n;            // active requests, ordered by size class
   int32_t cls_end[kClasses];     // requests [0, cls_end[c]) have size class <= c
   int32_t epoch;        // completion-counter base of this chunk
   int32_t G;            // levels per unit of the fused sweep launches (1, 2 or 4), scaled
                         // per request by class_group
-  int32_t pad;
+  int32_t res_n;        // resident requests, and the clusters that take them
+  int32_t res_clusters;
+  int32_t team_ctas[kClasses];   // CTAs of the team launch of a size class
   unsigned long long claim[kClasses];   // queue counters of one chunk's buckets (0 in t_host)
   int64_t off_h1[kMaxReq + 1];   // prefix counts of half-sweep-1 units (groups of G levels)
   int64_t off_h2[kMaxReq + 1];   // prefix counts of half-sweep-2 units
   int64_t off_lv[kMaxReq + 1];   // prefix counts of all levels
+  unsigned long long team_claim[kClasses];   // queue counters of the team launches
+  int64_t off_t1[kMaxReq + 1];   // prefix counts of the team path's levels by half-sweep
+  int64_t off_t2[kMaxReq + 1];
+  int32_t res[kMaxReq];          // table positions of the resident requests
   BReq r[kMaxReq];
 };
 
@@ -131,11 +154,20 @@ cudaError_t b_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, in
 cudaError_t b_sweeps_finish(const BTable* t, BOut* out, int K, BTune g, cudaStream_t s);
 // Direct residual of every request's iterate (with_q: also q for refinement).
 cudaError_t b_resid(const BTable* t, BOut* out, int with_q, BTune g, cudaStream_t s);
-// Mixed precision: d = 0 (b_lp_zero); `inner` fused correction sweeps
+// Mixed precision: d = 0 (b_lp_zero; queue path only, the others write d once); `inner` fused correction sweeps
 // (b_lp_sweeps); pi <- (pi + d)/e^T(pi + d) with the step error (b_lp_finish).
 cudaError_t b_lp_zero(const BTable* t, BTune g, cudaStream_t s);
 cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, int bf16,
                         int coupled, int inner, BTune g, cudaStream_t s);
+// The team requests' correction sweeps, a launch per size class on b[0..2].
+cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out, int bf16,
+                      int coupled, int inner, int num_sms, const cudaStream_t* b);
+// Path of a request of this layout.
+int b_lp_path(const Layout& lay, int coupled, int num_sms);
+// resident.cu: whether a request fits one cluster; the resident requests' launch.
+bool resident_batch_fits(const Layout& lay, int coupled);
+cudaError_t launch_resident_batch(const BTable* t, int bf16, int coupled, int K, BOut* out,
+                                  cudaStream_t s);
 cudaError_t b_lp_finish(const BTable* t, BOut* out, BTune g, cudaStream_t s);
 
 }  // namespace mc

@@ -5,6 +5,7 @@
 
 #include <mutex>
 
+#include "batch.cuh"
 #include "resident_dev.cuh"
 
 namespace mc {
@@ -16,6 +17,7 @@ using namespace res;
 template <typename V>
 __device__ __forceinline__ void attach(ClusterLink<V>& ln, const ResidentWords&, int* status) {
   ln.status = status;
+  ln.c = (int)cg::this_cluster().num_blocks();
 }
 template <typename V>
 __device__ __forceinline__ void attach(GridLink<V>& ln, const ResidentWords& w, int* status) {
@@ -148,11 +150,66 @@ __global__ void __launch_bounds__(kThreads) k_resident_lp(ResidentLpArgs a) {
   finish(ln);
 }
 
+// CTAs of a cluster of `most` that share L levels, at least two each.
+__host__ __device__ inline int cluster_ctas(int64_t L, int most) {
+  int C = most;
+  while (C > 1 && L < 2 * C) C /= 2;
+  return C;
+}
+
+// The resident requests of a batch, one cluster each in turn; the CTAs of a short
+// chain's cluster that have no levels only take part in its barriers.
+template <typename S, bool COUPLED>
+__global__ void __launch_bounds__(kThreads) k_b_resident(const BTable* __restrict__ t, int K,
+                                                         BOut* out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned long long two[2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int most = (int)cl.num_blocks(), cid = (int)blockIdx.x / most;
+  if (cid >= t->res_clusters) return;
+  for (int i = cid; i < t->res_n; i += t->res_clusters) {
+    const int r = t->res[i];
+    const BReq& Q = t->r[r];
+    ClusterLink<float> ln;
+    ln.status = &out[r].status;
+    ln.c = cluster_ctas(Q.L, most);
+    if ((int)cl.block_rank() < ln.c) {
+      Chain<S, float, float> h{};
+      h.A = reinterpret_cast<const S*>(Q.lA);
+      h.B = reinterpret_cast<const S*>(Q.lB);
+      h.C = Q.lC;
+      h.as = Q.lp_bs;
+      h.cs = Q.lp_cbs;
+      h.sc = Q.sc;
+      h.q = Q.q;
+      h.L = (int)Q.L;
+      h.m = Q.m;
+      h.par0 = Q.p1;
+      sweeps<S, float, float, COUPLED>(h, K, smem, two, ln);
+      const int l0 = ln.s.l0, n = ln.s.n;
+      for (int e = threadIdx.x; e < n * h.m; e += kThreads)
+        Q.d[(int64_t)l0 * h.m + e] = ln.s.x[h.m + e];
+    } else {
+      ln.ready();
+    }
+    cl.sync();   // shared memory and barriers are used again
+    if ((int)cl.block_rank() < ln.c && threadIdx.x == 0) {
+      bar_free(ln.bar[0]);
+      bar_free(ln.bar[1]);
+    }
+  }
+}
+
 constexpr size_t kMaxDyn = 227 * 1024 - 1024;   // opt-in limit less the static arrays
 
 // Kernels by storage type (FP64, FP32, BF16), apply mode and link.
 using Kernel64 = void (*)(ResidentArgs);
 using KernelLp = void (*)(ResidentLpArgs);
+using KernelBatch = void (*)(const BTable*, int, BOut*);
+KernelBatch kernel_batch(int lp, int coupled) {
+  if (lp == 1) return coupled ? k_b_resident<float, true> : k_b_resident<float, false>;
+  return coupled ? k_b_resident<unsigned short, true> : k_b_resident<unsigned short, false>;
+}
 Kernel64 kernel64(int coupled, bool grid) {
   if (grid)
     return coupled ? k_resident<true, GridLink<double>> : k_resident<false, GridLink<double>>;
@@ -235,7 +292,8 @@ Limits limits() {
            opt_in((const void*)kernel64(c, true), false);
       for (int lp = 1; lp <= 2; ++lp)
         ok = ok && opt_in((const void*)kernel_lp(lp, c, false), true) &&
-             opt_in((const void*)kernel_lp(lp, c, true), false);
+             opt_in((const void*)kernel_lp(lp, c, true), false) &&
+             opt_in((const void*)kernel_batch(lp, c), true);
     }
     if (ok) {
       for (int C = 16; C >= 8 && !l.cluster; C /= 2) {
@@ -243,7 +301,8 @@ Limits limits() {
         for (int c = 0; c < 2; ++c) {
           runs = runs && cluster_runs((const void*)kernel64(c, false), C);
           for (int lp = 1; lp <= 2; ++lp)
-            runs = runs && cluster_runs((const void*)kernel_lp(lp, c, false), C);
+            runs = runs && cluster_runs((const void*)kernel_lp(lp, c, false), C) &&
+                   cluster_runs((const void*)kernel_batch(lp, c), C);
         }
         if (runs) l.cluster = C;
       }
@@ -268,8 +327,7 @@ int resident_ctas(const Layout& y, int coupled, int* grid) {
   *grid = 0;
   if (y.L > (1 << 20)) return 0;
   const Limits lim = limits();
-  int C = lim.cluster;
-  while (C > 1 && y.L < 2 * C) C /= 2;
+  const int C = cluster_ctas(y.L, lim.cluster);
   const double entries = (double)y.L * y.m * y.m * (coupled ? 2 : 3);
   const size_t most = y.lp ? 64 * 1024 : kMaxDyn;
   // low precision, m > 32: the team kernel (lpteam_dev.cuh) keeps more warps on a
@@ -300,6 +358,22 @@ cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& y, int cou
   cudaLaunchAttribute at{};
   config(cfg, at, grid != 0, ctas, smem_bytes(y, coupled, ctas), s);
   return cudaLaunchKernelEx(&cfg, kernel_lp(y.lp, coupled, grid != 0), a);
+}
+
+bool resident_batch_fits(const Layout& y, int coupled) {
+  const int C = cluster_ctas(y.L, limits().cluster);
+  return y.lp && C > 0 && y.m <= 32 && y.L <= (1 << 20) && smem_bytes(y, coupled, C) <= kMaxDyn;
+}
+
+cudaError_t launch_resident_batch(const BTable* t, int bf16, int coupled, int K, BOut* out,
+                                  cudaStream_t s) {
+  const int C = limits().cluster;
+  if (C == 0) return cudaSuccess;   // no request has this path
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  config(cfg, at, false, C, kMaxDyn, s);
+  cfg.gridDim = dim3(C * kResidentClusters);
+  return cudaLaunchKernelEx(&cfg, kernel_batch(bf16 ? 2 : 1, coupled), t, K, out);
 }
 
 }  // namespace mc

@@ -207,6 +207,9 @@ __device__ __forceinline__ void push(uint32_t dst, uint32_t bar, float v) {
 __device__ __forceinline__ void bar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void bar_free(uint32_t bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
@@ -269,8 +272,9 @@ struct ClusterLink {
   uint32_t bar[2];                 // own barriers: left, right halo
   uint32_t xl, xr, zl, zr, bl, br; // the neighbours' halo slots and barriers
   int* status;
+  int c;                           // CTAs that take part (the first c of the cluster)
 
-  __device__ __forceinline__ int ctas() const { return (int)cg::this_cluster().num_blocks(); }
+  __device__ __forceinline__ int ctas() const { return c; }
   __device__ __forceinline__ int rank() const { return (int)cg::this_cluster().block_rank(); }
   // n_left: levels of the left neighbour.  bars: two mbarriers.
   __device__ __forceinline__ void open(const Side<V>& side, int n_left, unsigned long long* bars) {

@@ -37,6 +37,7 @@ struct Req {
   double* lsum;
   int64_t sweeps;
   double step_prev;
+  int path;             // kPathQueue / kPathTeam / kPathResident
   bool fresh;           // factor status not yet checked
 };
 
@@ -64,6 +65,8 @@ struct mc_server {
   std::vector<Req*> active;
   std::deque<Done> done;
   cudaStream_t cap;
+  cudaStream_t side[4];             // the short requests' launches run beside the others
+  cudaEvent_t fork[2], join[4];
   cudaGraphExec_t gexec;
   BTune g_tune;          // configuration of the captured graph
   int g_chunk;
@@ -143,6 +146,7 @@ void fill_req(const mc_server* s, const Req* r, BReq* q) {
     q->lC = chain_lpC(c);
     q->sc = chain_lpSc(c);
     q->d = chain_lpD(c);
+    q->dv = (unsigned long long*)c->z;   // FP64 sweeps only write z
     q->q = chain_lpQ(c);
     q->lp_bs = c->lay.lp_bs;
     q->lp_cbs = c->lay.lp_cbs;
@@ -158,6 +162,7 @@ void fill_req(const mc_server* s, const Req* r, BReq* q) {
   q->ms = c->lay.ms;
   q->R = (c->lay.m + 31) / 32;
   q->p1 = s->d.stair == 1 ? 0 : 1;
+  q->path = r->path;
 }
 
 // Retire request i of the active list: copy pi to the host, free its memory.
@@ -194,6 +199,13 @@ int retire(mc_server* s, size_t i, int status, double resid, double step, double
   return rc;
 }
 
+// The words of a team-path request to version 0.
+cudaError_t reset_team_words(mc_server* s, const Req* r) {
+  if (r->path != kPathTeam) return cudaSuccess;
+  return cudaMemsetAsync(r->chain->z, 0, (size_t)r->chain->lay.N * sizeof(unsigned long long),
+                         s->user);
+}
+
 // The next chunk (about to run) uses the current counter base; the one after
 // it starts c higher.  Called before each execution of a chunk (a direct
 // enqueue or a graph launch), while no chunk is in flight.  Before the 32-bit
@@ -203,7 +215,8 @@ int begin_chunk(mc_server* s, int c) {
   if (s->epoch_next > (1 << 30)) {
     for (Req* r : s->active)
       if (cudaMemsetAsync(r->chain->fver, 0, (size_t)r->chain->lay.L * sizeof(int), s->user) !=
-          cudaSuccess)
+              cudaSuccess ||
+          reset_team_words(s, r) != cudaSuccess)
         return MC_ERR_CUDA;
     s->epoch_next = 0;
   }
@@ -223,12 +236,28 @@ int enqueue_chunk(mc_server* s, BTune g, int c, cudaStream_t st, cudaEvent_t* ev
       cudaMemsetAsync(s->out_dev, 0, sizeof(BOut) * kMaxReq, st) != cudaSuccess)
     return MC_ERR_CUDA;
   unsigned long long* claim = &s->t_dev->claim[0];
-  if (lp && b_lp_zero(s->t_dev, g, st) != cudaSuccess) return MC_ERR_CUDA;
   if (ev && cudaEventRecord(ev[0], st) != cudaSuccess) return MC_ERR_CUDA;
   if (lp) {
-    if (b_lp_sweeps(s->t_dev, claim, s->out_dev, s->d.dtype == MC_BF16, coupled, c, g, st) !=
-        cudaSuccess)
+    // The resident launch starts first (its clusters need whole SMs), the team and
+    // queue launches run beside it after the short launch that zeroes d.
+    const int bf16 = s->d.dtype == MC_BF16;
+    if (cudaEventRecord(s->fork[0], st) != cudaSuccess ||
+        cudaStreamWaitEvent(s->side[0], s->fork[0], 0) != cudaSuccess ||
+        launch_resident_batch(s->t_dev, bf16, coupled, c, s->out_dev, s->side[0]) !=
+            cudaSuccess ||
+        b_lp_zero(s->t_dev, g, st) != cudaSuccess ||
+        cudaEventRecord(s->fork[1], st) != cudaSuccess)
       return MC_ERR_CUDA;
+    for (int i = 1; i < 4; ++i)
+      if (cudaStreamWaitEvent(s->side[i], s->fork[1], 0) != cudaSuccess) return MC_ERR_CUDA;
+    if (b_lp_team(s->t_dev, &s->t_dev->team_claim[0], s->out_dev, bf16, coupled, c, s->num_sms,
+                  s->side + 1) != cudaSuccess ||
+        b_lp_sweeps(s->t_dev, claim, s->out_dev, bf16, coupled, c, g, st) != cudaSuccess)
+      return MC_ERR_CUDA;
+    for (int i = 0; i < 4; ++i)
+      if (cudaEventRecord(s->join[i], s->side[i]) != cudaSuccess ||
+          cudaStreamWaitEvent(st, s->join[i], 0) != cudaSuccess)
+        return MC_ERR_CUDA;
   } else {
     if (b_sweeps(s->t_dev, claim, s->out_dev, coupled, c, g, st) != cudaSuccess)
       return MC_ERR_CUDA;
@@ -312,6 +341,27 @@ int check_fresh(mc_server* s) {
   return MC_OK;
 }
 
+// CTAs of the launches that run side by side.  A cluster takes 16 SMs whole; the
+// team launches share the others, two CTAs each, in proportion to their levels
+// (no more than one team per level), so that each gets its part at once instead
+// of the first launch filling the GPU for a chunk's time.  No result depends on it.
+void deal_ctas(const mc_server* s, BTable* t, const int64_t* team_levels) {
+  const bool teams = team_levels[1] + team_levels[2] + team_levels[3] > 0;
+  const int most = teams ? kResidentClusters / 2 : kResidentClusters;
+  t->res_clusters = t->res_n < most ? t->res_n : most;
+  const int64_t free_ctas = 2 * (int64_t)(s->num_sms - 16 * t->res_clusters);
+  int64_t want[kClasses] = {0, 0, 0, 0}, sum = 0;
+  for (int c = 1; c < kClasses; ++c) {
+    want[c] = c == 1 ? (team_levels[c] + 1) / 2 : team_levels[c];   // teams per CTA: 2, 1, 1
+    sum += want[c];
+  }
+  for (int c = 0; c < kClasses; ++c) {
+    int64_t n = want[c];
+    if (sum > free_ctas) n = (n * free_ctas + sum - 1) / sum;
+    t->team_ctas[c] = (int32_t)n;
+  }
+}
+
 // Fill the pinned request table from the active list (small blocks first);
 // returns the table order.
 std::vector<Req*> build_table(mc_server* s) {
@@ -323,7 +373,9 @@ std::vector<Req*> build_table(mc_server* s) {
   t->n = (int32_t)s->active.size();
   for (int c = 0; c < kClasses; ++c) t->cls_end[c] = 0;
   t->G = s->G;
-  t->off_h1[0] = t->off_h2[0] = t->off_lv[0] = 0;
+  t->off_h1[0] = t->off_h2[0] = t->off_lv[0] = t->off_t1[0] = t->off_t2[0] = 0;
+  t->res_n = 0;
+  int64_t team_levels[kClasses] = {0, 0, 0, 0};
   const int p1 = s->d.stair == 1 ? 0 : 1;
   for (int i = 0; i < t->n; ++i) {
     const Req* r = s->active[(size_t)i];
@@ -334,10 +386,16 @@ std::vector<Req*> build_table(mc_server* s) {
     t->r[i].G = (int32_t)G;
     // units: groups of G levels of each half-sweep
     const int64_t P1 = (L - p1 + 1) / 2, P2 = (L - (1 - p1) + 1) / 2;
-    t->off_h1[i + 1] = t->off_h1[i] + (P1 + G - 1) / G;
-    t->off_h2[i + 1] = t->off_h2[i] + (P2 + G - 1) / G;
+    const bool queue = r->path == kPathQueue, team = r->path == kPathTeam;
+    t->off_h1[i + 1] = t->off_h1[i] + (queue ? (P1 + G - 1) / G : 0);
+    t->off_h2[i + 1] = t->off_h2[i] + (queue ? (P2 + G - 1) / G : 0);
+    t->off_t1[i + 1] = t->off_t1[i] + (team ? P1 : 0);
+    t->off_t2[i + 1] = t->off_t2[i] + (team ? P2 : 0);
     t->off_lv[i + 1] = t->off_lv[i] + L;
+    if (team) team_levels[cls(r)] += L;
+    if (r->path == kPathResident) t->res[t->res_n++] = i;
   }
+  deal_ctas(s, t, team_levels);
   return std::vector<Req*>(s->active.begin(), s->active.end());
 }
 
@@ -367,6 +425,19 @@ int process_outputs(mc_server* s, const std::vector<Req*>& order, int c) {
     }
   }
   return nd;
+}
+
+// Pinned memory, streams and events (those that exist).
+void free_host_side(mc_server* s) {
+  if (s->cap) cudaStreamDestroy(s->cap);
+  for (cudaEvent_t f : s->fork)
+    if (f) cudaEventDestroy(f);
+  for (int i = 0; i < 4; ++i) {
+    if (s->side[i]) cudaStreamDestroy(s->side[i]);
+    if (s->join[i]) cudaEventDestroy(s->join[i]);
+  }
+  if (s->t_host) cudaFreeHost(s->t_host);
+  if (s->out_host) cudaFreeHost(s->out_host);
 }
 
 }  // namespace
@@ -401,10 +472,16 @@ int mc_server_create(const mc_server_desc* desc, void* arena, size_t arena_bytes
     delete s;
     return MC_ERR_CUDA;
   }
-  if (cudaHostAlloc((void**)&s->out_host, sizeof(BOut) * kMaxReq, cudaHostAllocDefault) !=
-          cudaSuccess ||
-      cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaFreeHost(s->t_host);
+  bool ok = cudaHostAlloc((void**)&s->out_host, sizeof(BOut) * kMaxReq, cudaHostAllocDefault) ==
+                cudaSuccess &&
+            cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaEventCreateWithFlags(&s->fork[0], cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventCreateWithFlags(&s->fork[1], cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < 4 && ok; ++i)
+    ok = cudaStreamCreateWithFlags(&s->side[i], cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    free_host_side(s);
     delete s;
     return MC_ERR_CUDA;
   }
@@ -479,7 +556,14 @@ int mc_server_submit(mc_server* s, int64_t tag, int64_t L, int32_t m, const doub
   r->lsum = (double*)(s->arena + off + ws);
   r->sweeps = 0;
   r->step_prev = NAN;
+  r->path = y.lp ? b_lp_path(y, s->d.apply == MC_APPLY_COUPLED, s->num_sms) : kPathQueue;
   r->fresh = true;
+  if (reset_team_words(s, r) != cudaSuccess) {
+    mc_destroy(c);
+    release(s, off, bytes);
+    delete r;
+    return MC_ERR_CUDA;
+  }
   s->active.push_back(r);
   return MC_OK;
 }
@@ -646,9 +730,7 @@ void mc_server_destroy(mc_server* s) {
   }
   for (Done& dn : s->done) free(dn.pi);
   if (s->gexec) cudaGraphExecDestroy(s->gexec);
-  if (s->cap) cudaStreamDestroy(s->cap);
-  if (s->t_host) cudaFreeHost(s->t_host);
-  if (s->out_host) cudaFreeHost(s->out_host);
+  free_host_side(s);
   delete s;
 }
 
