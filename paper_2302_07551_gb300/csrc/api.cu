@@ -188,6 +188,27 @@ static ResidentWords resident_words(const mc_chain* c) {
   return w;
 }
 
+// Everything of a resident launch but its vectors, sweeps and outputs.
+static ResidentArgs resident_args(mc_chain* c) {
+  const bool coupled = c->d.apply == MC_APPLY_COUPLED;
+  const size_t pe = c->lay.plane_bytes / sizeof(double);
+  ResidentArgs a{};
+  a.A = c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe;
+  a.B = c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe;
+  a.C = c->planes + kPlaneNINV * pe;
+  a.TLO = c->planes + kPlaneTLO * pe;
+  a.TUP = c->planes + kPlaneTUP * pe;
+  a.part = c->rpart;
+  a.hdr = c->hdr;
+  a.words = resident_words(c);
+  a.L = c->lay.L;
+  a.m = c->lay.m;
+  a.ms = c->lay.ms;
+  a.par0 = c->d.stair == 1 ? 0 : 1;
+  a.chunks = 1;
+  return a;
+}
+
 // n stair sweeps src -> dst (in place allowed) as fused launches of at most
 // kMaxFusedSweeps sweeps, each followed by the normalisation (with the step
 // error after the last).  With resid (block-tridiagonal chains only) the last
@@ -215,25 +236,13 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
     const int64_t K = n - done < kMaxFusedSweeps ? n - done : kMaxFusedSweeps;
     const bool final = done + K == n;
     if (c->res_ctas) {
-      ResidentArgs a{};
-      a.A = c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe;
-      a.B = c->planes + (coupled ? kPlaneWUP : kPlaneTUP) * pe;
-      a.C = c->planes + kPlaneNINV * pe;
-      a.TLO = c->planes + kPlaneTLO * pe;
-      a.TUP = c->planes + kPlaneTUP * pe;
+      ResidentArgs a = resident_args(c);
       a.x_in = in;
       a.x_out = dst;
-      a.hdr = c->hdr;
       a.stats_out = final ? stats_out : nullptr;
-      a.L = L;
       a.K = K;
-      a.m = c->lay.m;
-      a.ms = c->lay.ms;
-      a.par0 = c->d.stair == 1 ? 0 : 1;
       a.with_step = final && step;
       a.with_resid = final && resid;
-      a.part = c->rpart;
-      a.words = resident_words(c);
       CK(launch_resident(a, c->lay, coupled, c->res_ctas, c->res_grid, s));
       if (ev && final) {
         CK(cudaEventRecord(ev[1], s));
@@ -930,10 +939,31 @@ int mc_solve(mc_chain* c, const double* x0, double* pi, double tol, double eps, 
   double d = NAN, d_prev = NAN, r = NAN, kappa = NAN;
   int converged = 0;
   bool direct = mode == kResidDirect;   // r is the direct residual of xa
+  // resident chains run several chunks per launch and stop by themselves; a
+  // launch is kept to about kResidentSweeps sweeps
+  constexpr int64_t kResidentSweeps = 8192;
+  const bool many = c->res_ctas && check_every <= kMaxFusedSweeps;
   while (k < maxit) {
     const int64_t chunk = (maxit - k < check_every) ? (maxit - k) : check_every;
+    int64_t ran = 1;
     direct = mode == kResidDirect;
-    if (chunk == check_every) {
+    if (chunk == check_every && many) {
+      ResidentArgs a = resident_args(c);
+      a.x_in = a.x_out = c->xa;
+      a.K = check_every;
+      a.with_step = 1;
+      a.with_resid = mode == kResidSplit;
+      a.tol = mode == kResidSplit ? tol : 0.0;
+      a.eps = eps;
+      a.chunks = kResidentSweeps / check_every;
+      if (a.chunks > (maxit - k) / check_every) a.chunks = (maxit - k) / check_every;
+      CK(launch_resident(a, c->lay, c->d.apply == MC_APPLY_COUPLED, c->res_ctas, c->res_grid,
+                         c->user));
+      rc = fetch_header(c);
+      if (rc != MC_OK) return rc;
+      ran = c->hh->chunks;
+      if (ran > 1) d_prev = c->hh->prev_step;
+    } else if (chunk == check_every) {
       if (!c->gexec || c->g_chunk != check_every || c->g_resid != mode) {
         rc = capture_chunk(c, check_every, mode);
         if (rc != MC_OK) return rc;
@@ -946,7 +976,7 @@ int mc_solve(mc_chain* c, const double* x0, double* pi, double tol, double eps, 
       rc = fetch_header(c);
       if (rc != MC_OK) return rc;
     }
-    k += chunk;
+    k += ran * chunk;
     st = clear_status(c);
     if (st != 0) return st;
     d = c->hh->stats[1];

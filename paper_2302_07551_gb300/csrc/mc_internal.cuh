@@ -33,6 +33,8 @@ struct Header {
                          // [1] residual, [2] half-sweep 2, [3] low-precision update,
                          // [4] fused scale
   double stats[4];       // [e^T z, step_l1, resid_l1, spare]
+  double prev_step;      // resident solves: step error of the chunk before the last
+  int64_t chunks;        // and the chunks run
 };
 
 // Off-staircase block diagonals |d| >= 2 of a block-banded Q^T (device
@@ -169,6 +171,10 @@ struct ResidentArgs {
   int64_t L, K;
   int m, ms, par0;
   int with_step, with_resid;
+  // a solve: up to `chunks` chunks of K sweeps, each normalised, until the
+  // residual is <= tol (tol > 0) or the step error <= eps (eps > 0)
+  int64_t chunks;
+  double tol, eps;
 };
 struct ResidentLpArgs {
   const void* A;

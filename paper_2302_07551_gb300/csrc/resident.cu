@@ -40,9 +40,12 @@ __device__ __forceinline__ void finish(const GridLink<V>& ln) {
 
 // K FP64 sweeps from x_in, then x_out = z_K / e^T z_K with the step error
 // (with_step) and ||Q^T x_out||_1 from the splitting (with_resid, see
-// fused.cu) into the header and stats_out.
+// fused.cu) into the header and stats_out.  A solve runs several such chunks in
+// one launch, the iterate staying on chip: a launch, a copy and a wait of the
+// host per chunk of 32 sweeps were a third of a small solve (64 levels of 8 to
+// 1e-12: 3.8 -> 3.0 ms).
 template <bool COUPLED, typename Link>
-__global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) k_resident(ResidentArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double sh[2][kThreads / 32 + 1][3];
   __shared__ double rcp[2];
@@ -59,75 +62,91 @@ __global__ void __launch_bounds__(kThreads) k_resident(ResidentArgs a) {
   h.L = (int)a.L;
   h.m = a.m;
   h.par0 = a.par0;
-  sweeps<double, double, double, COUPLED>(h, (int)a.K, smem, two, ln);
   const int L = h.L, m = h.m;
   const int l0 = range_begin(L, C, r), n = range_begin(L, C, r + 1) - l0;
   const Carve k = carve<double, double, double, COUPLED>((L + C - 1) / C, m);
-  const double* x = reinterpret_cast<double*>(smem + k.x);
-  const double* z = reinterpret_cast<double*>(smem + k.z);
-  double v[3] = {0.0, 0.0, 0.0};   // e^T z_K, e^T z_{K-1}, ||Q^T z_K||_1
+  double* x = reinterpret_cast<double*>(smem + k.x);
+  double* z = reinterpret_cast<double*>(smem + k.z);
   // sums by as few warps as keep about 8 entries a lane
   int warps = (n * m + 255) / 256;
   if (warps > kThreads / 32) warps = kThreads / 32;
-  for (int e = threadIdx.x; e < n * m && threadIdx.x < 32 * warps; e += 32 * warps) {
-    v[0] += z[m + e];
-    if (a.K > 1) v[1] += x[m + e];
-  }
-  if (a.with_resid) {
-    // N (x - z) on the diagonal-only rows: T_lo d_{l-1} + T_up d_{l+1}, d = z - x
-    const int t0 = (l0 ^ a.par0) & 1, nh = n > t0 ? (n - t0 + 1) / 2 : 0;
-    const Cover c = cover(m, (n + 1) / 2);
-    double* rs = reinterpret_cast<double*>(smem + k.g);   // |r| per row
-    for_rows<double>(
-        c, m, nh, reinterpret_cast<double*>(smem + k.p),
-        [&](int u, int i, int j0, int S) {
-          const int t = t0 + 2 * u;
-          const int64_t l = l0 + t;
-          const double* A = a.TLO + (size_t)l * a.ms;   // once a launch: from L2
-          const double* B = a.TUP + (size_t)l * a.ms;
-          // d at a halo beyond the chain is 0 - 0 and its block zero
-          double s0 = 0.0;
-#pragma unroll 4
-          for (int j = j0; j < m; j += S) {
-            s0 = fma(A[j * m + i], z[t * m + j] - x[t * m + j], s0);
-            s0 = fma(B[j * m + i], z[(t + 2) * m + j] - x[(t + 2) * m + j], s0);
-          }
-          return s0;
-        },
-        [&](int u, int i, double s) { rs[u * m + i] = fabs(s); });
-    __syncthreads();
-    for (int e = threadIdx.x; e < nh * m && threadIdx.x < 32 * warps; e += 32 * warps)
-      v[2] += rs[e];
-  }
-  all_sum3(v, warps, sh[0], ln, a.part);
-  const double s = v[0], so = a.K > 1 ? v[1] : 1.0, res = v[2];
-  if (threadIdx.x == 0) {   // divisions are many FP64 instructions: one thread
-    rcp[0] = 1.0 / s;
-    rcp[1] = a.K > 1 ? 1.0 / so : 1.0;
-  }
-  __syncthreads();
-  const double inv = rcp[0], pinv = rcp[1];
-  double w[3] = {0.0, 0.0, 0.0};
-  for (int e = threadIdx.x; e < n * m && threadIdx.x < 32 * warps; e += 32 * warps) {
-    const double p = z[m + e] * inv;
-    if (a.with_step) w[0] += fabs(p - x[m + e] * pinv);
-    a.x_out[(int64_t)l0 * m + e] = p;
-  }
-  all_sum3(w, warps, sh[1], ln, a.part + 3 * C);   // after its barrier no CTA reads sh[0] of another
-  if (r == 0 && threadIdx.x == 0) {
-    if (!((s > 0.0) && isfinite(s))) latch(a.hdr, MC_ERR_BREAKDOWN);
-    const double st[3] = {a.K > 1 ? s / so : s, w[0], a.with_resid ? res * inv : nan("")};
-    for (int i = 0; i < 3; ++i) {
-      a.hdr->stats[i] = st[i];
-      if (a.stats_out) a.stats_out[i] = st[i];
+  double step = nan(""), prev = nan("");
+  for (int64_t chunk = 1;; ++chunk) {
+    sweeps<double, double, double, COUPLED>(h, (int)a.K, smem, two, ln, chunk == 1);
+    double v[3] = {0.0, 0.0, 0.0};   // e^T z_K, e^T z_{K-1}, ||Q^T z_K||_1
+    for (int e = threadIdx.x; e < n * m && threadIdx.x < 32 * warps; e += 32 * warps) {
+      v[0] += z[m + e];
+      if (a.K > 1) v[1] += x[m + e];
     }
+    if (a.with_resid) {
+      // N (x - z) on the diagonal-only rows: T_lo d_{l-1} + T_up d_{l+1}, d = z - x
+      const int t0 = (l0 ^ a.par0) & 1, nh = n > t0 ? (n - t0 + 1) / 2 : 0;
+      const Cover c = cover(m, (n + 1) / 2);
+      double* rs = reinterpret_cast<double*>(smem + k.g);   // |r| per row
+      for_rows<double>(
+          c, m, nh, reinterpret_cast<double*>(smem + k.p),
+          [&](int u, int i, int j0, int S) {
+            const int t = t0 + 2 * u;
+            const int64_t l = l0 + t;
+            const double* A = a.TLO + (size_t)l * a.ms;   // once a chunk: from L2
+            const double* B = a.TUP + (size_t)l * a.ms;
+            // d at a halo beyond the chain is 0 - 0 and its block zero
+            double s0 = 0.0;
+#pragma unroll 4
+            for (int j = j0; j < m; j += S) {
+              s0 = fma(A[j * m + i], z[t * m + j] - x[t * m + j], s0);
+              s0 = fma(B[j * m + i], z[(t + 2) * m + j] - x[(t + 2) * m + j], s0);
+            }
+            return s0;
+          },
+          [&](int u, int i, double s) { rs[u * m + i] = fabs(s); });
+      __syncthreads();
+      for (int e = threadIdx.x; e < nh * m && threadIdx.x < 32 * warps; e += 32 * warps)
+        v[2] += rs[e];
+    }
+    all_sum3(v, warps, sh[0], ln, a.part);
+    const double s = v[0], so = a.K > 1 ? v[1] : 1.0, res = v[2];
+    // divisions are many FP64 instructions: one thread each, of different warps
+    if (threadIdx.x == 0) rcp[0] = 1.0 / s;
+    if (threadIdx.x == 32) rcp[1] = a.K > 1 ? 1.0 / so : 1.0;
+    __syncthreads();
+    const double inv = rcp[0], pinv = rcp[1];
+    double w[3] = {0.0, 0.0, 0.0};
+    if (a.with_step) {
+      for (int e = threadIdx.x; e < n * m && threadIdx.x < 32 * warps; e += 32 * warps)
+        w[0] += fabs(z[m + e] * inv - x[m + e] * pinv);
+      all_sum3(w, warps, sh[1], ln, a.part + 3 * C);   // no CTA reads sh[0] of another after it
+      prev = step;
+      step = w[0];
+    }
+    const double resid = a.with_resid ? res * inv : nan("");
+    const bool ok = s > 0.0 && isfinite(s);
+    // the same decision in every CTA
+    if (!ok || chunk >= a.chunks || (a.tol > 0.0 && resid <= a.tol) ||
+        (a.eps > 0.0 && step <= a.eps)) {
+      for (int e = threadIdx.x; e < n * m; e += kThreads)
+        a.x_out[(int64_t)l0 * m + e] = z[m + e] * inv;
+      if (r == 0 && threadIdx.x == 0) {
+        if (!ok) latch(a.hdr, MC_ERR_BREAKDOWN);
+        const double st[3] = {a.K > 1 ? s / so : s, w[0], resid};
+        for (int i = 0; i < 3; ++i) {
+          a.hdr->stats[i] = st[i];
+          if (a.stats_out) a.stats_out[i] = st[i];
+        }
+        a.hdr->prev_step = prev;
+        a.hdr->chunks = chunk;
+      }
+      break;
+    }
+    for (int e = threadIdx.x; e < (n + 2) * m; e += kThreads) x[e] = z[e] * inv;
+    // (the next run's barrier comes before any CTA writes another's halo)
   }
   finish(ln);
 }
 
 // The K correction sweeps of a refinement step from the zero vector.
 template <typename S, bool COUPLED, template <typename> class LinkT>
-__global__ void __launch_bounds__(kThreads) k_resident_lp(ResidentLpArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) k_resident_lp(ResidentLpArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long two[2];
   LinkT<float> ln;
@@ -160,7 +179,7 @@ __host__ __device__ inline int cluster_ctas(int64_t L, int most) {
 // The resident requests of a batch, one cluster each in turn; the CTAs of a short
 // chain's cluster that have no levels only take part in its barriers.
 template <typename S, bool COUPLED>
-__global__ void __launch_bounds__(kThreads) k_b_resident(const BTable* __restrict__ t, int K,
+__global__ void __launch_bounds__(kThreads, 1) k_b_resident(const BTable* __restrict__ t, int K,
                                                          BOut* out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long two[2];

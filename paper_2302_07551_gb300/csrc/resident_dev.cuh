@@ -273,12 +273,14 @@ struct ClusterLink {
   uint32_t xl, xr, zl, zr, bl, br; // the neighbours' halo slots and barriers
   int* status;
   int c;                           // CTAs that take part (the first c of the cluster)
+  int used;                        // phases completed by earlier runs
 
   __device__ __forceinline__ int ctas() const { return c; }
   __device__ __forceinline__ int rank() const { return (int)cg::this_cluster().block_rank(); }
   // n_left: levels of the left neighbour.  bars: two mbarriers.
   __device__ __forceinline__ void open(const Side<V>& side, int n_left, unsigned long long* bars) {
     s = side;
+    used = 0;
     const int r = rank();
     bar[0] = smem_addr(bars);
     bar[1] = smem_addr(bars + 1);
@@ -296,9 +298,20 @@ struct ClusterLink {
       bar_init(bar[0]);
       bar_init(bar[1]);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    arm();
+  }
+  // the barriers expect the first version of a run of K sweeps
+  __device__ __forceinline__ void arm() const {
+    if (threadIdx.x == 0) {
       if (s.left) bar_expect(bar[0], (uint32_t)(s.m * sizeof(V)));
       if (s.right) bar_expect(bar[1], (uint32_t)(s.m * sizeof(V)));
     }
+  }
+  // another run after a finished one
+  __device__ __forceinline__ void again() {
+    used += s.K;
+    arm();
   }
   // every CTA is ready for pushes
   __device__ __forceinline__ void ready() { cg::this_cluster().sync(); }
@@ -306,7 +319,7 @@ struct ClusterLink {
   __device__ __forceinline__ void wait(int side, int kk, int hs) const {
     const int need = kk + hs;
     if (need > 0 && (side == 0 ? s.left : s.right))
-      bar_wait(bar[side], (uint32_t)(need - 1) & 1u, status);
+      bar_wait(bar[side], (uint32_t)(used + need - 1) & 1u, status);
   }
   // value i of boundary level t of sweep kk
   __device__ __forceinline__ void send(int t, int i, V v, int, bool last) const {
@@ -400,6 +413,7 @@ struct GridLink {
     __syncthreads();
     base = (unsigned)*reinterpret_cast<volatile unsigned long long*>(sh);
   }
+  __device__ __forceinline__ void again() { base += (unsigned)s.K; }
   __device__ __forceinline__ void ready() { __syncthreads(); }
   // the halos that half-sweep hs of sweep kk reads, into shared memory
   __device__ __forceinline__ void fill(int kk, int hs) {
@@ -729,10 +743,11 @@ __device__ __forceinline__ void load_plane(T* dst, const T* src, int64_t gs, int
 
 // K sweeps.  On return z (FP64) / x (low precision) holds the CTA's levels of
 // the result and FP64 x the iterate before the last sweep, halos included.
-// sh: two words of shared memory for the link.
+// sh: two words of shared memory for the link.  first = false: another run from
+// the iterate in x (halos included), with the operators as they are.
 template <typename T, typename TC, typename V, bool COUPLED, typename Link>
 __device__ __forceinline__ void sweeps(const Chain<T, TC, V>& h, int K, unsigned char* smem,
-                                       unsigned long long* sh, Link& ln) {
+                                       unsigned long long* sh, Link& ln, bool first = true) {
   const int C = ln.ctas(), r = ln.rank();
   const int L = h.L, m = h.m;
   const int ms = (int)packed<T>(m), mc = (int)packed<TC>(m);
@@ -751,19 +766,23 @@ __device__ __forceinline__ void sweeps(const Chain<T, TC, V>& h, int K, unsigned
   const Cover c = cover(m, (nmax + 1) / 2);   // the same in every CTA
   const int cpl = (m + c.S - 1) / c.S;
   const bool tiny = m <= 16 && ((nmax + 1) / 2) * c.gs <= kThreads && cpl <= 8;
-  ln.open(Side<V>{x, z, l0, n, m, h.par0, K, r > 0, r < C - 1},
-          r > 0 ? l0 - range_begin(L, C, r - 1) : 0, sh);
-  // operators, blocks packed; blocks that lead out of the chain are zero
-  if (!tiny) {
-    load_plane(A, h.A + (size_t)l0 * h.as, h.as, n, m, l0 == 0 ? 0 : -1);
-    load_plane(B, h.B + (size_t)l0 * h.as, h.as, n, m, l0 + n == L ? n - 1 : -1);
-    if (!COUPLED) load_plane(Cp, h.C + (size_t)l0 * h.cs, h.cs, n, m, -1);
-  }
-  for (int e = tid; e < (n + 2) * m; e += kThreads) {
-    const int64_t j = (int64_t)(l0 - 1) * m + e;
-    const V v = h.in && j >= 0 && j < (int64_t)L * m ? h.in[j] : V(0);
-    x[e] = v;
-    if (sizeof(V) == 8) z[e] = V(0);
+  if (first) {
+    ln.open(Side<V>{x, z, l0, n, m, h.par0, K, r > 0, r < C - 1},
+            r > 0 ? l0 - range_begin(L, C, r - 1) : 0, sh);
+    // operators, blocks packed; blocks that lead out of the chain are zero
+    if (!tiny) {
+      load_plane(A, h.A + (size_t)l0 * h.as, h.as, n, m, l0 == 0 ? 0 : -1);
+      load_plane(B, h.B + (size_t)l0 * h.as, h.as, n, m, l0 + n == L ? n - 1 : -1);
+      if (!COUPLED) load_plane(Cp, h.C + (size_t)l0 * h.cs, h.cs, n, m, -1);
+    }
+    for (int e = tid; e < (n + 2) * m; e += kThreads) {
+      const int64_t j = (int64_t)(l0 - 1) * m + e;
+      const V v = h.in && j >= 0 && j < (int64_t)L * m ? h.in[j] : V(0);
+      x[e] = v;
+      if (sizeof(V) == 8) z[e] = V(0);
+    }
+  } else {
+    ln.again();
   }
   float* sc = reinterpret_cast<float*>(smem + k.s);
   if (sizeof(V) == 4 && !tiny) {

@@ -87,3 +87,29 @@ def test_refinement_solutions(L, m, apply, dtype):
     assert np.abs(pi.cpu().numpy() - ref).sum() <= 1e-10
     again, _ = ch.solve(tol=1e-12, check_every=24, maxit=40000)
     assert torch.equal(pi, again)
+
+
+@pytest.mark.parametrize("L,m,apply", [(64, 8, "inverse"), (300, 20, "coupled")])
+def test_solve_is_its_chunks(L, m, apply):
+    """A solve runs its chunks on the device: the iterate, the sweep count, the step error and the
+    contraction are those of the same chunks called one by one (bitwise), whatever stops it."""
+    C, n = 7, 5
+    ch = mc.Chain(*(torch.from_numpy(b).cuda() for b in synth.qbd(L, m, 0.8, seed=2)), apply=apply)
+    x = torch.full((L * m,), 1.0 / (L * m), dtype=torch.float64, device="cuda")
+    xs, steps = [], []
+    for k in range(n):
+        st = torch.zeros(3, dtype=torch.float64, device="cuda")
+        x = ch.sweep(x, nsweeps=C, stats=st)
+        xs.append(x)
+        steps.append(float(st[1]))
+    tail = ch.sweep(x, nsweeps=3)
+    pi, res = ch.solve(tol=1e-30, maxit=n * C + 3, check_every=C, raise_on_maxit=False)
+    assert res["sweeps"] == n * C + 3 and not res["converged"] and torch.equal(pi, tail)
+    pi, res = ch.solve(tol=0.0, eps=steps[2], maxit=n * C, check_every=C)
+    assert res["sweeps"] == 3 * C and res["converged"] and torch.equal(pi, xs[2])
+    assert res["step"] == steps[2]
+    assert abs(res["contraction"] - (steps[2] / steps[1]) ** (1 / C)) <= 1e-12
+    r = ch.residual(xs[3])
+    if r < min(ch.residual(v) for v in xs[:3]):
+        pi, res = ch.solve(tol=r * (1 + 1e-6), maxit=n * C, check_every=C)
+        assert res["sweeps"] == 4 * C and torch.equal(pi, xs[3])
