@@ -434,9 +434,9 @@ __global__ void __launch_bounds__(256) k_fused_scale(const double* lsum, int64_t
     const int64_t p1 = p0 + pc < P ? p0 + pc : P;
     for (int64_t u = p0 + threadIdx.x; u < p1; u += blockDim.x) tr += rsum[u];
   }
-  ta = block_sum(ta, sh);
-  tb = block_sum(tb, sh);
-  tr = block_sum(tr, sh);
+  ta = block_sum0(ta, sh);
+  if (K >= 2) tb = block_sum0(tb, sh);
+  if (rsum) tr = block_sum0(tr, sh);
   if (threadIdx.x == 0) {
     part[3 * blockIdx.x] = ta;
     part[3 * blockIdx.x + 1] = tb;

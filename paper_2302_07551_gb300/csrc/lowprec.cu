@@ -21,6 +21,7 @@
 #include "mc_internal.cuh"
 #include "lowprec_dev.cuh"
 #include "lpteam_dev.cuh"
+#include "sweep_dev.cuh"
 #include "wave_dev.cuh"
 
 namespace mc {
@@ -206,23 +207,20 @@ __global__ void __launch_bounds__(256) k_update(const double* __restrict__ pi,
     out[i] = v;
     t += v;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
-  __syncthreads();
+  t = block_sum0(t, sh);
   if (threadIdx.x == 0) {
-    double b = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += sh[w];
-    bpart[blockIdx.x] = b;
+    bpart[blockIdx.x] = t;
     __threadfence();
     last = (atomicAdd(&hdr->ticket[3], 1u) == gridDim.x - 1);
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
-    __threadfence();
-    double s = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(bpart + b);
-    *s_out = s;
+  if (!last) return;
+  __threadfence();
+  t = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t += __ldcg(bpart + b);
+  t = block_sum0(t, sh);
+  if (threadIdx.x == 0) {
+    *s_out = t;
     hdr->ticket[3] = 0u;
   }
 }

@@ -103,10 +103,8 @@ __global__ void __launch_bounds__(kNormThreads) k_normalise(NormArgs a) {
   if (!ok && blockIdx.x == 0 && threadIdx.x == 0) latch(a.hdr, MC_ERR_BREAKDOWN);
   const double so = a.s_old ? *a.s_old : 1.0;
   // the reciprocals once per block: FP64 division is costly at this FP64 rate
-  if (threadIdx.x == 0) {
-    rcp[0] = 1.0 / s;
-    rcp[1] = 1.0 / so;   // exactly 1 for a normalised x_old
-  }
+  if (threadIdx.x == 0) rcp[0] = 1.0 / s;
+  if (threadIdx.x == 32) rcp[1] = a.s_old ? 1.0 / so : 1.0;   // (another sub-partition's pipe)
   __syncthreads();
   const double inv = rcp[0];
   const double pinv = rcp[1];
@@ -172,7 +170,7 @@ __global__ void __launch_bounds__(kNormThreads) k_normalise(NormArgs a) {
       a.x_new[i] = p;
     }
   }
-  d = block_sum(d, sh);
+  if (a.x_old) d = block_sum0(d, sh);
   if (threadIdx.x == 0) {
     a.dpart[blockIdx.x] = d;
     __threadfence();
@@ -183,8 +181,10 @@ __global__ void __launch_bounds__(kNormThreads) k_normalise(NormArgs a) {
   if (last) {
     __threadfence();
     double e = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) e += __ldcg(a.dpart + i);
-    e = block_sum(e, sh);
+    if (a.x_old) {
+      for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) e += __ldcg(a.dpart + i);
+      e = block_sum0(e, sh);
+    }
     if (threadIdx.x == 0) {
       // e^T z relative to the previous iterate (s itself when that was normalised)
       const double sr = s / so;

@@ -174,6 +174,22 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return t;
 }
 
+// As block_sum, valid on thread 0 only: the second stage by one warp (every warp
+// that adds costs 16 clocks of the SM's FP64 pipe per instruction).
+__device__ __forceinline__ double block_sum0(double v, double* sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  v = warp_sum(v);
+  __syncthreads();
+  if (lane == 0) sh[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    v = lane < nw ? sh[lane] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);   // nw <= 8
+  }
+  return v;
+}
+
 // One level of a half-sweep (Algorithm 2): z_l = (-T_dd)^{-1}(T_lo v_{l-1} +
 // T_up v_{l+1}) (inverse mode: A = T_lo, B = T_up, C = (-T_dd)^{-1}) or
 // z_l = W_lo v_{l-1} + W_up v_{l+1} (coupled: A = W_lo, B = W_up), written to
