@@ -10,6 +10,7 @@
 #include "lowprec_dev.cuh"
 #include "lpteam_dev.cuh"
 #include "sweep_dev.cuh"
+#include "team_dev.cuh"
 #include "wave_dev.cuh"
 
 namespace mc {
@@ -70,18 +71,17 @@ __device__ __forceinline__ BUnit unit_of(const BTable* t, unsigned long long q, 
   return u;
 }
 
-// K FP64 sweeps of every request of one bucket (size classes [c0, c1), rows
-// per lane up to RMAX) in one launch.  Per request: sweep 0 reads x, sweeps
-// 0..K-2 write xb in place, sweep K-1 writes z (so xb keeps the previous
-// sweep for the step error).
-template <bool COUPLED, int RMAX>
-__global__ void __launch_bounds__(256) k_b_sweeps(const BTable* __restrict__ t, int K, int c0,
-                                                  int c1, unsigned long long* claim, BOut* out) {
+// K FP64 sweeps of the queue-path requests (m <= 16, b_path) in one launch.  Per
+// request: sweep 0 reads x, sweeps 0..K-2 write xb in place, sweep K-1 writes z (so
+// xb keeps the previous sweep for the step error).
+template <bool COUPLED>
+__global__ void __launch_bounds__(256) k_b_sweeps(const BTable* __restrict__ t, int K,
+                                                  unsigned long long* claim, BOut* out) {
   extern __shared__ double vsh[];
   const int lane = threadIdx.x & 31;
-  double* slice = vsh + (threadIdx.x >> 5) * 3 * 32 * RMAX;
+  double* slice = vsh + (threadIdx.x >> 5) * 3 * 32;
   int r0, r1;
-  class_range(t, c0, c1, r0, r1);
+  class_range(t, 0, 1, r0, r1);
   const int64_t a0 = t->off_h1[r0], a1 = t->off_h1[r1];
   const int64_t b0 = t->off_h2[r0], b1 = t->off_h2[r1];
   const int64_t n1 = a1 - a0, U = n1 + (b1 - b0);
@@ -103,19 +103,9 @@ __global__ void __launch_bounds__(256) k_b_sweeps(const BTable* __restrict__ t, 
     const bool want = u.k >= K - 2;   // e^T z of the last two sweeps only
     for (int i = 0; i < u.n; ++i) {
       const int64_t l = u.l + 2 * i;
-      double ls;
-      if constexpr (RMAX == 8) {
-        ls = level_sweep2<8, COUPLED, false, true, true>(Q->A, Q->B, Q->C, src, src, dst, l,
-                                                         Q->L, Q->m, Q->ms, slice, lane, 1.0,
-                                                         nullptr, nullptr, nullptr, want);
-      } else {
-        switch (Q->R) {
-          case 1: ls = level_sweep2<1, COUPLED, false, true, true>(Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr, nullptr, nullptr, want); break;
-          case 2: ls = level_sweep2<2, COUPLED, false, true, true>(Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr, nullptr, nullptr, want); break;
-          case 3: ls = level_sweep2<RMAX == 4 ? 3 : 2, COUPLED, false, true, true>(Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr, nullptr, nullptr, want); break;
-          default: ls = level_sweep2<RMAX, COUPLED, false, true, true>(Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr, nullptr, nullptr, want); break;
-        }
-      }
+      const double ls = level_sweep2<1, COUPLED, false, true, true>(
+          Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr,
+          nullptr, nullptr, want);
       if (want && lane == 0) Q->lsum2[(u.k & 1) * Q->L + l] = ls;
     }
     publish_levels(Q->ver, u.l, 2, u.n, base + (int)u.k + 1, lane);
@@ -391,15 +381,118 @@ __global__ void __launch_bounds__(256, 2) k_b_team(const BTable* __restrict__ t,
   }
 }
 
+// FP64 sweeps of the team-path requests of one size class, one row per lane (as
+// k_sweeps).  Bound by the unit's latency where a batch has fewer levels than
+// teams, by HBM and the FP64 pipe elsewhere.  Against one warp per unit of 4 to 16
+// levels on the FP64 pipe alone, a chunk of 64 sweeps: 2000 x 32 + 1500 x 16 +
+// 2500 x 24 coupled 3.20 -> 1.41 ms, 4000 x 64 inverse 8.43 -> 4.46, eight requests
+// of 16 to 128 rows coupled 9.9 -> 4.5, four of 48 to 200 rows 37.8 -> 6.4.
+template <int TW, bool COUPLED>
+__global__ void __launch_bounds__(256, 3) k_b_team64(const BTable* __restrict__ t, int K, int cls,
+                                                     unsigned long long* claim, BOut* out) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  if ((int)blockIdx.x >= t->team_ctas[cls]) return;
+  using Sh = TeamShared<TW, 1>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / TW, w = warp % TW, tt = threadIdx.x - team * TW * 32, bar = 1 + team;
+  const int row0 = 32 * w;
+  Sh& sh = reinterpret_cast<Sh*>(team_smem)[team];
+  int r0, r1;
+  class_range(t, cls, cls + 1, r0, r1);
+  const int64_t a0 = t->off_t1[r0], b0 = t->off_t2[r0];
+  const int64_t n1 = t->off_t1[r1] - a0, U = n1 + (t->off_t2[r1] - b0);
+  const unsigned long long total = (unsigned long long)K * (unsigned long long)U;
+  unsigned long long q0 = w == 0 ? claim_unit(claim, lane) : 0ull, q;
+  if (w == 0 && lane == 0) sh.next[1] = q0;
+  if (w == 0) q0 = claim_unit(claim, lane);
+  team_sync<TW>(bar);
+  q = sh.next[1];
+  int turn = 0, s = 0;
+  while (q < total) {
+    if (w == 0 && lane == 0) sh.next[turn] = q0;
+    const int64_t k = (int64_t)(q / (unsigned long long)U), rr = (int64_t)q - k * U;
+    const bool h2 = rr >= n1;
+    const int64_t* off = h2 ? t->off_t2 : t->off_t1;
+    const int64_t i = h2 ? b0 + (rr - n1) : a0 + rr;
+    const int r = find_req(off, r0, r1, i);
+    const BReq* Q = &t->r[r];
+    const int64_t l = 2 * (i - off[r]) + (h2 ? 1 - Q->p1 : Q->p1), L = Q->L;
+    const int m = Q->m;
+    const size_t at = (size_t)l * Q->ms;
+    const bool has_lo = l > 0, has_up = l < L - 1;
+    double* dst = k == K - 1 ? Q->z : Q->xb;
+    const double* src = h2 ? dst : (k == 0 ? Q->x : Q->xb);
+    const int ea = Q->eA[l], eb = Q->eB[l], ec = COUPLED ? 0 : Q->eC[l];
+    if (h2 || k > 0)
+      wait_neighbours(Q->ver, l, L, (Q->vbase + (int)(h2 ? k + 1 : k)) * TW, &out[r].status, lane,
+                      kWaitNs);
+    const double x0[1] = {has_lo && tt < m ? __ldcg(src + (l - 1) * m + tt) : 0.0};
+    const double x1[1] = {has_up && tt < m ? __ldcg(src + (l + 1) * m + tt) : 0.0};
+    stage_rows<TW, 1>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], x0, tt, 32, w, lane);
+    stage_rows<TW, 1>(sh.slot[s].v[1], sh.slot[s].x[1], sh.emax[s][1], x1, tt, 32, w, lane);
+    team_sync<TW>(bar);
+    const unsigned long long qn = sh.next[turn];
+    turn ^= 1;
+    if (w == 0) q0 = claim_unit(claim, lane);
+    double acc[1] = {0.0};
+    if (has_lo)
+      rows_product<1, 0>(acc, Q->A + at, sh.slot[s].v[0], sh.slot[s].x[0], ea,
+                         team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
+    if (has_up)
+      rows_product<1, 0>(acc, Q->B + at, sh.slot[s].v[1], sh.slot[s].x[1], eb,
+                         team_max<TW>(sh.emax[s][1]), 0, m, m, row0, lane);
+    if constexpr (!COUPLED) {
+      s ^= 1;
+      stage_rows<TW, 1>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], acc, row0 + lane, 32, w,
+                        lane);
+      team_sync<TW>(bar);
+      acc[0] = 0.0;
+      rows_product<1, 0>(acc, Q->C + at, sh.slot[s].v[0], sh.slot[s].x[0], ec,
+                         team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
+    }
+    double ls = 0.0;
+    if (row0 + lane < m) {
+      dst[l * m + row0 + lane] = acc[0];
+      ls = acc[0];
+    }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) red_release(Q->ver + l, 1);
+    if (k >= K - 2) {   // e^T z of the last two sweeps only
+      ls = team_total<TW>(warp_sum(ls), sh.part, w, lane, bar);
+      if (w == 0 && lane == 0) Q->lsum2[(k & 1) * L + l] = ls;
+    }
+    s ^= 1;
+    q = qn;
+  }
+}
+
+template <bool C>
+cudaError_t team64_launches(const BTable* t, unsigned long long* claim, BOut* out, int paths,
+                            int K, int sms, cudaStream_t b0, const cudaStream_t* b) {
+  const int n = 3 * sms;
+  if (paths & path_bit(kPathTeam, 0))
+    k_b_team64<1, C><<<n, 256, 8 * sizeof(TeamShared<1, 1>), b0>>>(t, K, 0, claim, out);
+  if (paths & path_bit(kPathTeam, 1))
+    k_b_team64<2, C><<<n, 256, 4 * sizeof(TeamShared<2, 1>), b[0]>>>(t, K, 1, claim + 1, out);
+  if (paths & path_bit(kPathTeam, 2))
+    k_b_team64<4, C><<<n, 256, 2 * sizeof(TeamShared<4, 1>), b[1]>>>(t, K, 2, claim + 2, out);
+  if (paths & path_bit(kPathTeam, 3))
+    k_b_team64<8, C><<<n, 256, sizeof(TeamShared<8, 1>), b[2]>>>(t, K, 3, claim + 3, out);
+  return cudaGetLastError();
+}
+
 template <typename S, bool C>
-cudaError_t team_launches(const BTable* t, unsigned long long* claim, BOut* out, int K, int sms,
-                          const cudaStream_t* b) {
-  k_b_team<S, 64, 4, C><<<2 * sms, 256, 2 * sizeof(LpTeamShared<64, 4>), b[0]>>>(t, K, 1,
-                                                                               claim + 1, out);
-  k_b_team<S, 128, 8, C><<<2 * sms, 256, sizeof(LpTeamShared<128, 8>), b[1]>>>(t, K, 2, claim + 2,
-                                                                              out);
-  k_b_team<S, 256, 8, C><<<2 * sms, 256, sizeof(LpTeamShared<256, 8>), b[2]>>>(t, K, 3, claim + 3,
-                                                                              out);
+cudaError_t team_launches(const BTable* t, unsigned long long* claim, BOut* out, int paths, int K,
+                          int sms, const cudaStream_t* b) {
+  const int n = 2 * sms;
+  if (paths & path_bit(kPathTeam, 1))
+    k_b_team<S, 64, 4, C><<<n, 256, 2 * sizeof(LpTeamShared<64, 4>), b[0]>>>(t, K, 1, claim + 1,
+                                                                            out);
+  if (paths & path_bit(kPathTeam, 2))
+    k_b_team<S, 128, 8, C><<<n, 256, sizeof(LpTeamShared<128, 8>), b[1]>>>(t, K, 2, claim + 2, out);
+  if (paths & path_bit(kPathTeam, 3))
+    k_b_team<S, 256, 8, C><<<n, 256, sizeof(LpTeamShared<256, 8>), b[2]>>>(t, K, 3, claim + 3, out);
   return cudaGetLastError();
 }
 
@@ -407,29 +500,6 @@ template <typename K>
 cudaError_t allow(K kernel, size_t bytes) {
   if (bytes <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-// Every bucket of a tuning: FP64 kernels sized for R <= 2, 4 or 8 rows per
-// lane by the bucket's largest class.
-template <bool C>
-cudaError_t sweeps_buckets(const BTable* t, unsigned long long* claim, BOut* out, int K,
-                           BTune g, cudaStream_t s) {
-  const BBuckets b = buckets_of(g.split64);
-  for (int i = 0; i < b.n; ++i) {
-    const int rmax = b.c1[i] <= 2 ? 2 : b.c1[i] <= 3 ? 4 : 8;
-    const size_t sm = (size_t)(g.threads / 32) * 3 * 32 * rmax * sizeof(double);
-    cudaError_t e = cudaSuccess;
-    if (rmax == 2) {
-      k_b_sweeps<C, 2><<<g.blocks, g.threads, sm, s>>>(t, K, b.c0[i], b.c1[i], claim + i, out);
-    } else if (rmax == 4) {
-      k_b_sweeps<C, 4><<<g.blocks, g.threads, sm, s>>>(t, K, b.c0[i], b.c1[i], claim + i, out);
-    } else {
-      e = allow(k_b_sweeps<C, 8>, sm);
-      if (e != cudaSuccess) return e;
-      k_b_sweeps<C, 8><<<g.blocks, g.threads, sm, s>>>(t, K, b.c0[i], b.c1[i], claim + i, out);
-    }
-  }
-  return cudaGetLastError();
 }
 
 template <typename TS, typename TL, bool C>
@@ -462,10 +532,14 @@ cudaError_t lp_buckets(const BTable* t, unsigned long long* claim, BOut* out, in
 
 }  // namespace
 
-cudaError_t b_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, int coupled, int K,
+cudaError_t b_sweeps(const BTable* t, unsigned long long* claim, BOut* out, int coupled, int K,
                      BTune g, cudaStream_t s) {
-  return coupled ? sweeps_buckets<true>(t, t_claim, out, K, g, s)
-                 : sweeps_buckets<false>(t, t_claim, out, K, g, s);
+  const size_t sm = (size_t)(g.threads / 32) * 3 * 32 * sizeof(double);
+  if (coupled)
+    k_b_sweeps<true><<<g.blocks, g.threads, sm, s>>>(t, K, claim, out);
+  else
+    k_b_sweeps<false><<<g.blocks, g.threads, sm, s>>>(t, K, claim, out);
+  return cudaGetLastError();
 }
 
 cudaError_t b_sweeps_finish(const BTable* t, BOut* out, int K, BTune g, cudaStream_t s) {
@@ -503,21 +577,34 @@ cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out,
   return e;
 }
 
-int b_lp_path(const Layout& y, int coupled, int num_sms) {
+int b_path(const Layout& y, int coupled, int num_sms) {
   if (resident_batch_fits(y, coupled)) return kPathResident;
-  if (y.m > 32 && (y.lp == 1 || y.m % 8 == 0) &&
+  // FP64, m <= 16: a chain with a level for every warp in flight is bound by the
+  // fence and claim of each unit, which units of 4 levels share (six of 16384 x 16,
+  // coupled, a chunk of 64 sweeps: teams 12.3 ms, queue 11.0); shorter ones by the
+  // unit's latency (1500 x 16 with two of 24 and 32 rows: teams 1.41, queue 3.20).
+  if (y.lp == 0) return y.m <= 16 && y.L / 2 >= 24ll * num_sms ? kPathQueue : kPathTeam;
+  if (y.m <= 32) return kPathQueue;
+  if ((y.lp == 1 || y.m % 8 == 0) &&
       y.L / 2 * (y.m <= 64 ? 4 : 8) <= 16ll * num_sms)   // as launch_sweeps_lp
     return kPathTeam;
   return kPathQueue;
 }
 
-cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out, int bf16,
-                      int coupled, int inner, int num_sms, const cudaStream_t* b) {
+cudaError_t b_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
+                   int coupled, int K, int num_sms, cudaStream_t b0,
+                   const cudaStream_t* b) {
+  return coupled ? team64_launches<true>(t, team_claim, out, paths, K, num_sms, b0, b)
+                 : team64_launches<false>(t, team_claim, out, paths, K, num_sms, b0, b);
+}
+
+cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
+                      int bf16, int coupled, int inner, int num_sms, const cudaStream_t* b) {
   if (bf16)
-    return coupled ? team_launches<unsigned short, true>(t, team_claim, out, inner, num_sms, b)
-                   : team_launches<unsigned short, false>(t, team_claim, out, inner, num_sms, b);
-  return coupled ? team_launches<float, true>(t, team_claim, out, inner, num_sms, b)
-                 : team_launches<float, false>(t, team_claim, out, inner, num_sms, b);
+    return coupled ? team_launches<unsigned short, true>(t, team_claim, out, paths, inner, num_sms, b)
+                   : team_launches<unsigned short, false>(t, team_claim, out, paths, inner, num_sms, b);
+  return coupled ? team_launches<float, true>(t, team_claim, out, paths, inner, num_sms, b)
+                 : team_launches<float, false>(t, team_claim, out, paths, inner, num_sms, b);
 }
 
 cudaError_t b_lp_finish(const BTable* t, BOut* out, BTune g, cudaStream_t s) {

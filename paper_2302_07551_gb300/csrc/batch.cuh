@@ -53,10 +53,14 @@ struct BReq {
   double* lsum2;        // fused sweeps: [2][L] level sums of the last two sweeps
   int* ver;             // fused sweeps: per-level completion counters
   int64_t L;
-  unsigned long long* dv;   // versioned words of the correction (team path)
+  unsigned long long* dv;   // low precision: versioned words of the correction (team path)
+  const int* eA;        // FP64: block_exp of A, B, C (team path)
+  const int* eB;
+  const int* eC;
   int32_t m, ms, R, p1;  // p1: 0-based parity of the diagonal-only rows
   int32_t G, path;       // levels per unit of this request (the table's G scaled by size
                          // class); kPathQueue, ...
+  int32_t vbase, pad2;   // FP64 team path: sweeps that the counters have seen
   int64_t lp_bs, lp_cbs;
 };
 
@@ -72,19 +76,22 @@ __host__ __device__ inline int class_group(int G, int m) {
   return g > 16 ? 16 : g;
 }
 
-// How a request's low-precision correction sweeps run, by its own size alone (so
-// that its iterates do not depend on the batch):
+// How a request's sweeps run, by its own size alone (so that its iterates do not
+// depend on the batch):
 //   kPathQueue: one warp per unit of G levels, all such requests in shared launches
-//     by size class (k_b_sweeps_lp);
-//   kPathTeam: short chains of blocks of more than 32 rows, a team of warps per
-//     level (lpteam_dev.cuh), all such requests of a size class in one launch;
-//   kPathResident: small blocks that fit one cluster's shared memory, one cluster
-//     per request (resident_dev.cuh).
+//     by size class (k_b_sweeps: FP64 blocks of up to 16 rows, long chains; k_b_sweeps_lp);
+//   kPathTeam: a team of warps per level, all such requests of a size class in one
+//     launch: all other FP64 requests (team_dev.cuh), low-precision short chains
+//     of blocks of more than 32 rows (lpteam_dev.cuh);
+//   kPathResident: blocks of up to 32 rows that fit one cluster's shared memory, one
+//     cluster per request (resident_dev.cuh).
 // The launches of the three paths run side by side; the host deals out CTAs to
 // them with the table.  Eight requests of 131 KB to 17 MB
 // (BF16 coupled, m = 16 to 128): a chunk of 64 sweeps 2.70 -> 0.99 ms with all of them
 // running, 1.32 -> 0.24 ms with the last two small ones.
 enum { kPathQueue = 0, kPathTeam = 1, kPathResident = 2 };
+// One bit per path and size class (class 0 but for teams).
+inline int path_bit(int path, int cls) { return 1 << (4 * path + cls); }
 constexpr int kResidentClusters = 8;   // clusters of 16 in a launch
 
 struct BTable {
@@ -149,8 +156,6 @@ inline BBuckets buckets_of(int split64) {
 // between); then (b_sweeps_finish) e^T z, normalisation and the step error of
 // the last sweep.  t_claim: the device table's claim counters.  coupled:
 // server-wide apply mode.
-cudaError_t b_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, int coupled, int K,
-                     BTune g, cudaStream_t s);
 cudaError_t b_sweeps_finish(const BTable* t, BOut* out, int K, BTune g, cudaStream_t s);
 // Direct residual of every request's iterate (with_q: also q for refinement).
 cudaError_t b_resid(const BTable* t, BOut* out, int with_q, BTune g, cudaStream_t s);
@@ -159,14 +164,21 @@ cudaError_t b_resid(const BTable* t, BOut* out, int with_q, BTune g, cudaStream_
 cudaError_t b_lp_zero(const BTable* t, BTune g, cudaStream_t s);
 cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, int bf16,
                         int coupled, int inner, BTune g, cudaStream_t s);
-// The team requests' correction sweeps, a launch per size class on b[0..2].
-cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out, int bf16,
-                      int coupled, int inner, int num_sms, const cudaStream_t* b);
+// The team requests' correction sweeps, a launch per size class on b0, b[0..2].
+// paths: the path_bit of every path and size class of the table.
+cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
+                      int bf16, int coupled, int inner, int num_sms, const cudaStream_t* b);
 // Path of a request of this layout.
-int b_lp_path(const Layout& lay, int coupled, int num_sms);
+int b_path(const Layout& lay, int coupled, int num_sms);
+cudaError_t b_sweeps(const BTable* t, unsigned long long* claim, BOut* out, int coupled, int K,
+                     BTune g, cudaStream_t s);
+// The FP64 team requests' sweeps, a launch per size class on b0, b[0..2].
+cudaError_t b_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
+                   int coupled, int K, int num_sms, cudaStream_t b0, const cudaStream_t* b);
 // resident.cu: whether a request fits one cluster; the resident requests' launch.
 bool resident_batch_fits(const Layout& lay, int coupled);
-cudaError_t launch_resident_batch(const BTable* t, int bf16, int coupled, int K, BOut* out,
+// lp: 0 FP64, 1 FP32, 2 BF16.
+cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int K, BOut* out,
                                   cudaStream_t s);
 cudaError_t b_lp_finish(const BTable* t, BOut* out, BTune g, cudaStream_t s);
 

@@ -46,57 +46,6 @@ namespace {
 
 using namespace dev;
 
-// Largest exponent over the team's warps.
-template <int TW>
-__device__ __forceinline__ int team_max(const int* e) {
-  int v = e[0];
-#pragma unroll
-  for (int i = 1; i < TW; ++i) v = max(v, e[i]);
-  return v;
-}
-
-// Rows first, first + stride, ... of one vector into a staged slot.
-template <int TW, int RW>
-__device__ __forceinline__ void stage_rows(double* v, uint64_t* x, int* emax,
-                                           const double (&y)[RW], int first, int stride, int w,
-                                           int lane) {
-  unsigned e = 0u;
-#pragma unroll
-  for (int i = 0; i < RW; ++i) {
-    v[first + stride * i] = y[i];
-    x[first + stride * i] = fixed_entry(y[i]);
-    e = max(e, (unsigned)__double2hiint(y[i]) >> 20);
-  }
-  e = __reduce_max_sync(kFull, e);
-  if (lane == 0) emax[w] = (int)e;
-}
-
-// Sum of the warps' values in warp order (valid on the team's first warp).
-template <int TW>
-__device__ __forceinline__ double team_total(double t, double* part, int w, int lane, int bar) {
-  if constexpr (TW == 1) return t;
-  if (lane == 0) part[w] = t;
-  team_sync<TW>(bar);
-  double v = part[0];
-#pragma unroll
-  for (int i = 1; i < TW; ++i) v += part[i];
-  return v;
-}
-
-// Shared memory of one team: a ring of two staged products (a warp that writes
-// slot i + 1 has passed the barrier of slot i, so every warp of the team has
-// finished reading slot i - 1), the largest exponents found by each warp, the
-// units to come, and partial level sums.
-// The staged vectors are read in 16-byte pairs, so every team's slots start on a
-// 16-byte boundary.
-template <int TW, int RW>
-struct alignas(16) TeamShared {
-  TeamSlot<32 * RW * TW> slot[2];
-  int emax[2][2][TW];
-  unsigned long long next[2];
-  double part[TW];
-};
-
 // MC: the block size if it equals 32 RW TW, else 0.  BANDED: block-banded
 // chains (Algorithm 2 with off-staircase terms, inverse mode): every row also
 // adds sum_d T_{l,l+d} x_{l+d} over the far diagonals |d| >= 2 from the sweep's

@@ -219,6 +219,55 @@ __global__ void __launch_bounds__(kThreads, 1) k_b_resident(const BTable* __rest
   }
 }
 
+// FP64: also the level sums of the last two sweeps, for the batch's reductions.
+template <bool COUPLED>
+__global__ void __launch_bounds__(kThreads, 1) k_b_resident64(const BTable* __restrict__ t, int K,
+                                                              BOut* out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned long long two[2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int most = (int)cl.num_blocks(), cid = (int)blockIdx.x / most;
+  if (cid >= t->res_clusters) return;
+  for (int i = cid; i < t->res_n; i += t->res_clusters) {
+    const int r = t->res[i];
+    const BReq& Q = t->r[r];
+    ClusterLink<double> ln;
+    ln.status = &out[r].status;
+    ln.c = cluster_ctas(Q.L, most);
+    if ((int)cl.block_rank() < ln.c) {
+      Chain<double, double, double> h{};
+      h.A = Q.A;
+      h.B = Q.B;
+      h.C = Q.C;
+      h.as = h.cs = Q.ms;
+      h.in = Q.x;
+      h.L = (int)Q.L;
+      h.m = Q.m;
+      h.par0 = Q.p1;
+      sweeps<double, double, double, COUPLED>(h, K, smem, two, ln);
+      const int l0 = ln.s.l0, n = ln.s.n, m = h.m;
+      for (int e = threadIdx.x; e < n * m; e += kThreads) {
+        Q.z[(int64_t)l0 * m + e] = ln.s.z[m + e];
+        if (K > 1) Q.xb[(int64_t)l0 * m + e] = ln.s.x[m + e];
+      }
+      for (int q = threadIdx.x; q < 2 * n; q += kThreads) {   // in row order
+        const int lev = q >> 1, prev = q & 1;
+        const double* v = (prev ? ln.s.x : ln.s.z) + (lev + 1) * m;
+        double sum = 0.0;
+        for (int j = 0; j < m; ++j) sum += v[j];
+        if (!prev || K > 1) Q.lsum2[((K - 1 - prev) & 1) * Q.L + l0 + lev] = sum;
+      }
+    } else {
+      ln.ready();
+    }
+    cl.sync();   // shared memory and barriers are used again
+    if ((int)cl.block_rank() < ln.c && threadIdx.x == 0) {
+      bar_free(ln.bar[0]);
+      bar_free(ln.bar[1]);
+    }
+  }
+}
+
 constexpr size_t kMaxDyn = 227 * 1024 - 1024;   // opt-in limit less the static arrays
 
 // Kernels by storage type (FP64, FP32, BF16), apply mode and link.
@@ -226,6 +275,7 @@ using Kernel64 = void (*)(ResidentArgs);
 using KernelLp = void (*)(ResidentLpArgs);
 using KernelBatch = void (*)(const BTable*, int, BOut*);
 KernelBatch kernel_batch(int lp, int coupled) {
+  if (lp == 0) return coupled ? k_b_resident64<true> : k_b_resident64<false>;
   if (lp == 1) return coupled ? k_b_resident<float, true> : k_b_resident<float, false>;
   return coupled ? k_b_resident<unsigned short, true> : k_b_resident<unsigned short, false>;
 }
@@ -308,7 +358,8 @@ Limits limits() {
     bool ok = true;
     for (int c = 0; c < 2; ++c) {
       ok = ok && opt_in((const void*)kernel64(c, false), true) &&
-           opt_in((const void*)kernel64(c, true), false);
+           opt_in((const void*)kernel64(c, true), false) &&
+           opt_in((const void*)kernel_batch(0, c), true);
       for (int lp = 1; lp <= 2; ++lp)
         ok = ok && opt_in((const void*)kernel_lp(lp, c, false), true) &&
              opt_in((const void*)kernel_lp(lp, c, true), false) &&
@@ -318,7 +369,8 @@ Limits limits() {
       for (int C = 16; C >= 8 && !l.cluster; C /= 2) {
         bool runs = true;
         for (int c = 0; c < 2; ++c) {
-          runs = runs && cluster_runs((const void*)kernel64(c, false), C);
+          runs = runs && cluster_runs((const void*)kernel64(c, false), C) &&
+                 cluster_runs((const void*)kernel_batch(0, c), C);
           for (int lp = 1; lp <= 2; ++lp)
             runs = runs && cluster_runs((const void*)kernel_lp(lp, c, false), C) &&
                    cluster_runs((const void*)kernel_batch(lp, c), C);
@@ -381,10 +433,10 @@ cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& y, int cou
 
 bool resident_batch_fits(const Layout& y, int coupled) {
   const int C = cluster_ctas(y.L, limits().cluster);
-  return y.lp && C > 0 && y.m <= 32 && y.L <= (1 << 20) && smem_bytes(y, coupled, C) <= kMaxDyn;
+  return C > 0 && y.m <= 32 && y.L <= (1 << 20) && smem_bytes(y, coupled, C) <= kMaxDyn;
 }
 
-cudaError_t launch_resident_batch(const BTable* t, int bf16, int coupled, int K, BOut* out,
+cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int K, BOut* out,
                                   cudaStream_t s) {
   const int C = limits().cluster;
   if (C == 0) return cudaSuccess;   // no request has this path
@@ -392,7 +444,7 @@ cudaError_t launch_resident_batch(const BTable* t, int bf16, int coupled, int K,
   cudaLaunchAttribute at{};
   config(cfg, at, false, C, kMaxDyn, s);
   cfg.gridDim = dim3(C * kResidentClusters);
-  return cudaLaunchKernelEx(&cfg, kernel_batch(bf16 ? 2 : 1, coupled), t, K, out);
+  return cudaLaunchKernelEx(&cfg, kernel_batch(lp, coupled), t, K, out);
 }
 
 }  // namespace mc

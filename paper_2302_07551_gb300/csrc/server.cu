@@ -38,6 +38,7 @@ struct Req {
   int64_t sweeps;
   double step_prev;
   int path;             // kPathQueue / kPathTeam / kPathResident
+  int64_t vbase;        // sweeps that the completion counters have seen (FP64 teams)
   bool fresh;           // factor status not yet checked
 };
 
@@ -70,6 +71,7 @@ struct mc_server {
   cudaGraphExec_t gexec;
   BTune g_tune;          // configuration of the captured graph
   int g_chunk;
+  int g_paths;           // table_paths of the captured graph
   int G;                 // levels per unit of the table being built
   std::map<uint64_t, BTune> tuned;
   std::map<uint64_t, int> tuned_G;
@@ -140,6 +142,10 @@ void fill_req(const mc_server* s, const Req* r, BReq* q) {
   q->TDD = c->planes + kPlaneTDD * pe;
   q->TUP = c->planes + kPlaneTUP * pe;
   q->NINV = c->planes + kPlaneNINV * pe;
+  q->eA = chain_bexp(c, coupled ? kPlaneWLO : kPlaneTLO);
+  q->eB = chain_bexp(c, coupled ? kPlaneWUP : kPlaneTUP);
+  q->eC = chain_bexp(c, kPlaneNINV);
+  q->vbase = (int32_t)r->vbase;
   if (c->lay.lp) {
     q->lA = chain_lpA(c);
     q->lB = chain_lpB(c);
@@ -201,7 +207,7 @@ int retire(mc_server* s, size_t i, int status, double resid, double step, double
 
 // The words of a team-path request to version 0.
 cudaError_t reset_team_words(mc_server* s, const Req* r) {
-  if (r->path != kPathTeam) return cudaSuccess;
+  if (r->path != kPathTeam || !r->chain->lay.lp) return cudaSuccess;
   return cudaMemsetAsync(r->chain->z, 0, (size_t)r->chain->lay.N * sizeof(unsigned long long),
                          s->user);
 }
@@ -212,17 +218,29 @@ cudaError_t reset_team_words(mc_server* s, const Req* r) {
 // counters could wrap, every active request's counters are zeroed (stream
 // ordered before the chunk) and the base restarts at 0.
 int begin_chunk(mc_server* s, int c) {
-  if (s->epoch_next > (1 << 30)) {
-    for (Req* r : s->active)
+  if (s->epoch_next > (1 << 27)) {   // the teams' counters advance by up to 8 a sweep
+    for (size_t i = 0; i < s->active.size(); ++i) {
+      Req* r = s->active[i];
+      r->vbase = 0;
+      s->t_host->r[i].vbase = 0;   // the table is in the order of the active list
       if (cudaMemsetAsync(r->chain->fver, 0, (size_t)r->chain->lay.L * sizeof(int), s->user) !=
               cudaSuccess ||
           reset_team_words(s, r) != cudaSuccess)
         return MC_ERR_CUDA;
+    }
     s->epoch_next = 0;
   }
   s->t_host->epoch = s->epoch_next;
   s->epoch_next += c;
   return MC_OK;
+}
+
+// The paths and team size classes that the table's requests use.
+int table_paths(const BTable* t) {
+  int p = 0;
+  for (int i = 0; i < t->n; ++i)
+    p |= path_bit(t->r[i].path, t->r[i].path == kPathTeam ? size_class(t->r[i].m) : 0);
+  return p;
 }
 
 // Chunk body on stream st: c fused sweeps (FP64) or one refinement step of c
@@ -237,31 +255,40 @@ int enqueue_chunk(mc_server* s, BTune g, int c, cudaStream_t st, cudaEvent_t* ev
     return MC_ERR_CUDA;
   unsigned long long* claim = &s->t_dev->claim[0];
   if (ev && cudaEventRecord(ev[0], st) != cudaSuccess) return MC_ERR_CUDA;
-  if (lp) {
-    // The resident launch starts first (its clusters need whole SMs), the team and
-    // queue launches run beside it after the short launch that zeroes d.
-    const int bf16 = s->d.dtype == MC_BF16;
-    if (cudaEventRecord(s->fork[0], st) != cudaSuccess ||
-        cudaStreamWaitEvent(s->side[0], s->fork[0], 0) != cudaSuccess ||
-        launch_resident_batch(s->t_dev, bf16, coupled, c, s->out_dev, s->side[0]) !=
-            cudaSuccess ||
-        b_lp_zero(s->t_dev, g, st) != cudaSuccess ||
-        cudaEventRecord(s->fork[1], st) != cudaSuccess)
-      return MC_ERR_CUDA;
+  // The resident launch starts first (its clusters need whole SMs), the team and
+  // queue launches run beside it (low precision: after the short b_lp_zero).  Only
+  // the paths in use are launched.
+  const int kind = s->d.dtype == MC_F64 ? 0 : s->d.dtype == MC_F32 ? 1 : 2;
+  const int paths = table_paths(s->t_host);
+  const bool queue = paths & path_bit(kPathQueue, 0);
+  const bool on[4] = {(paths & path_bit(kPathResident, 0)) != 0,
+                      (paths & path_bit(kPathTeam, 1)) != 0, (paths & path_bit(kPathTeam, 2)) != 0,
+                      (paths & path_bit(kPathTeam, 3)) != 0};
+  if (on[0] &&
+      (cudaEventRecord(s->fork[0], st) != cudaSuccess ||
+       cudaStreamWaitEvent(s->side[0], s->fork[0], 0) != cudaSuccess ||
+       launch_resident_batch(s->t_dev, kind, coupled, c, s->out_dev, s->side[0]) != cudaSuccess))
+    return MC_ERR_CUDA;
+  if (lp && queue && b_lp_zero(s->t_dev, g, st) != cudaSuccess) return MC_ERR_CUDA;
+  if (on[1] || on[2] || on[3]) {
+    if (cudaEventRecord(s->fork[1], st) != cudaSuccess) return MC_ERR_CUDA;
     for (int i = 1; i < 4; ++i)
-      if (cudaStreamWaitEvent(s->side[i], s->fork[1], 0) != cudaSuccess) return MC_ERR_CUDA;
-    if (b_lp_team(s->t_dev, &s->t_dev->team_claim[0], s->out_dev, bf16, coupled, c, s->num_sms,
-                  s->side + 1) != cudaSuccess ||
-        b_lp_sweeps(s->t_dev, claim, s->out_dev, bf16, coupled, c, g, st) != cudaSuccess)
-      return MC_ERR_CUDA;
-    for (int i = 0; i < 4; ++i)
-      if (cudaEventRecord(s->join[i], s->side[i]) != cudaSuccess ||
-          cudaStreamWaitEvent(st, s->join[i], 0) != cudaSuccess)
+      if (on[i] && cudaStreamWaitEvent(s->side[i], s->fork[1], 0) != cudaSuccess)
         return MC_ERR_CUDA;
-  } else {
-    if (b_sweeps(s->t_dev, claim, s->out_dev, coupled, c, g, st) != cudaSuccess)
-      return MC_ERR_CUDA;
   }
+  unsigned long long* team = &s->t_dev->team_claim[0];
+  cudaError_t e =
+      lp ? b_lp_team(s->t_dev, team, s->out_dev, paths, kind == 2, coupled, c, s->num_sms,
+                     s->side + 1)
+         : b_team(s->t_dev, team, s->out_dev, paths, coupled, c, s->num_sms, st, s->side + 1);
+  if (e == cudaSuccess && queue)
+    e = lp ? b_lp_sweeps(s->t_dev, claim, s->out_dev, kind == 2, coupled, c, g, st)
+           : b_sweeps(s->t_dev, claim, s->out_dev, coupled, c, g, st);
+  if (e != cudaSuccess) return MC_ERR_CUDA;
+  for (int i = 0; i < 4; ++i)
+    if (on[i] && (cudaEventRecord(s->join[i], s->side[i]) != cudaSuccess ||
+                  cudaStreamWaitEvent(st, s->join[i], 0) != cudaSuccess))
+      return MC_ERR_CUDA;
   if (ev && cudaEventRecord(ev[1], st) != cudaSuccess) return MC_ERR_CUDA;
   if (lp) {
     if (b_lp_finish(s->t_dev, s->out_dev, g, st) != cudaSuccess) return MC_ERR_CUDA;
@@ -342,17 +369,20 @@ int check_fresh(mc_server* s) {
 }
 
 // CTAs of the launches that run side by side.  A cluster takes 16 SMs whole; the
-// team launches share the others, two CTAs each, in proportion to their levels
+// team launches share the others, two or three CTAs each, in proportion to their levels
 // (no more than one team per level), so that each gets its part at once instead
 // of the first launch filling the GPU for a chunk's time.  No result depends on it.
 void deal_ctas(const mc_server* s, BTable* t, const int64_t* team_levels) {
-  const bool teams = team_levels[1] + team_levels[2] + team_levels[3] > 0;
+  const bool teams = team_levels[0] + team_levels[1] + team_levels[2] + team_levels[3] > 0;
   const int most = teams ? kResidentClusters / 2 : kResidentClusters;
   t->res_clusters = t->res_n < most ? t->res_n : most;
-  const int64_t free_ctas = 2 * (int64_t)(s->num_sms - 16 * t->res_clusters);
+  // CTAs per SM, teams per CTA by class
+  static const int kTeams[2][kClasses] = {{8, 4, 2, 1}, {1, 2, 1, 1}};
+  const int lp = s->d.dtype != MC_F64, per_sm = lp ? 2 : 3;
+  const int64_t free_ctas = (int64_t)per_sm * (s->num_sms - 16 * t->res_clusters);
   int64_t want[kClasses] = {0, 0, 0, 0}, sum = 0;
-  for (int c = 1; c < kClasses; ++c) {
-    want[c] = c == 1 ? (team_levels[c] + 1) / 2 : team_levels[c];   // teams per CTA: 2, 1, 1
+  for (int c = 0; c < kClasses; ++c) {
+    want[c] = (team_levels[c] + kTeams[lp][c] - 1) / kTeams[lp][c];
     sum += want[c];
   }
   for (int c = 0; c < kClasses; ++c) {
@@ -408,6 +438,7 @@ int process_outputs(mc_server* s, const std::vector<Req*>& order, int c) {
     const BOut& o = s->out_host[k];
     Req* r = order[k];
     r->sweeps += c;
+    r->vbase += c;
     const size_t i =
         (size_t)(std::find(s->active.begin(), s->active.end(), r) - s->active.begin());
     const double kap =
@@ -556,7 +587,8 @@ int mc_server_submit(mc_server* s, int64_t tag, int64_t L, int32_t m, const doub
   r->lsum = (double*)(s->arena + off + ws);
   r->sweeps = 0;
   r->step_prev = NAN;
-  r->path = y.lp ? b_lp_path(y, s->d.apply == MC_APPLY_COUPLED, s->num_sms) : kPathQueue;
+  r->path = b_path(y, s->d.apply == MC_APPLY_COUPLED, s->num_sms);
+  r->vbase = 0;
   r->fresh = true;
   if (reset_team_words(s, r) != cudaSuccess) {
     mc_destroy(c);
@@ -650,7 +682,8 @@ int mc_server_step(mc_server* s, int32_t* n_active, int32_t* n_done) {
         s->G = G;
         order = build_table(s);
       }
-      if (!s->gexec || s->g_chunk != c || s->g_tune.blocks != g.blocks ||
+      const int paths = table_paths(s->t_host);
+      if (!s->gexec || s->g_chunk != c || s->g_paths != paths || s->g_tune.blocks != g.blocks ||
           s->g_tune.threads != g.threads || s->g_tune.split64 != g.split64 ||
           s->g_tune.deep != g.deep) {
         if (s->gexec) {
@@ -674,6 +707,7 @@ int mc_server_step(mc_server* s, int32_t* n_active, int32_t* n_done) {
           return MC_ERR_CUDA;
         }
         s->g_chunk = c;
+        s->g_paths = paths;
         s->g_tune = g;
       }
       rc = begin_chunk(s, c);

@@ -41,3 +41,49 @@ def test_every_path_alone_and_together(dtype, apply, stair):
         (_, pa, ra, _), = alone.run_until_idle()
         assert ra["sweeps"] == r["sweeps"] and np.array_equal(pa, pi), (L, m)
     alone.close()
+
+
+# FP64: clusters of 1 to 16 CTAs, below and above one cluster's shared memory (147 and 300 levels of
+# 32), teams of 2, 4 and 8 warps at the edges of their rows, odd sizes
+SIZES64 = [(2, 3), (31, 8), (33, 16), (140, 32), (300, 32), (2, 33), (41, 64), (20, 65), (17, 100), (16, 128), (9, 129), (7, 256)]
+
+
+@pytest.mark.parametrize("apply,stair", [("inverse", 1), ("inverse", 2), ("coupled", 1), ("coupled", 2)])
+@pytest.mark.parametrize("check", [1, 24])
+def test_every_fp64_path_alone_and_together(apply, stair, check):
+    kw = dict(dtype="f64", apply=apply, stair=stair, tol=1e-12, check_every=check)
+    sizes = SIZES64 if check > 1 else SIZES64[::3]
+    srv = mc.Server(2 << 30, autotune=check > 1, **kw)
+    for i, (L, m) in enumerate(sizes):
+        assert srv.submit(i, *blocks(i, L, m))
+    mixed = {t: (pi, r, st) for t, pi, r, st in srv.run_until_idle()}
+    srv.close()
+    alone = mc.Server(1 << 30, autotune=False, **kw)
+    for i, (L, m) in enumerate(sizes):
+        pi, r, st = mixed[i]
+        assert st == 0 and r["residual"] <= 1e-12
+        ref = oracle.Chain(*blocks(i, L, m)).solve(tol=1e-13, maxit=2000, check_every=24)["x"]   # 864 at most; 7 x 256 ends at its floor, 1.6e-13
+        assert np.abs(pi - ref).sum() <= 1e-10
+        alone.submit(i, *blocks(i, L, m))
+        (_, pa, ra, _), = alone.run_until_idle()
+        assert ra["sweeps"] == r["sweeps"] and np.array_equal(pa, pi), (L, m)
+    alone.close()
+
+
+def test_long_chains_of_small_fp64_blocks():
+    """Both sides of the line between teams of one warp and the shared queue (m <= 16, a level a half-sweep for
+    each of 24 warps an SM), against the oracle and bitwise as alone."""
+    n = 2 * 24 * torch.cuda.get_device_properties(0).multi_processor_count
+    kw = dict(dtype="f64", apply="coupled", tol=0.0, check_every=4, autotune=False, maxit=4)
+    sizes = [(n, 3), (n - 2, 4), (n + 1, 16), (n + 3, 17)]
+    srv = mc.Server(4 << 30, **kw)
+    for i, (L, m) in enumerate(sizes):
+        assert srv.submit(i, *blocks(i, L, m))
+    mixed = {t: pi for t, pi, r, st in srv.run_until_idle()}
+    for i, (L, m) in enumerate(sizes):
+        srv.submit(i, *blocks(i, L, m))
+        (_, pa, _, _), = srv.run_until_idle()
+        assert np.array_equal(pa, mixed[i])
+        ref = oracle.Chain(*blocks(i, L, m)).sweeps(np.full(L * m, 1.0 / (L * m)), 4)
+        assert np.abs(pa - ref).sum() <= 1e-12     # 4 sweeps of sums of 3 m terms >= 0: below 1e-14
+    srv.close()
