@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) k_b_sweeps(const BTable* __restrict__ t, 
     const bool want = u.k >= K - 2;   // e^T z of the last two sweeps only
     for (int i = 0; i < u.n; ++i) {
       const int64_t l = u.l + 2 * i;
-      const double ls = level_sweep2<1, COUPLED, false, true, true>(
+      const double ls = level_sweep2<1, COUPLED, true, true>(
           Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr,
           nullptr, nullptr, want);
       if (want && lane == 0) Q->lsum2[(u.k & 1) * Q->L + l] = ls;

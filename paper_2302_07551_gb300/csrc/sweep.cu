@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256, Tune<R>::MINB) k_phase(PhaseArgs a) {
   double wsum = 0.0;
   for (int64_t u = gw; u < a.P; u += nw) {
     const int64_t l = a.stride * u + a.parity;
-    wsum += level_sweep2<R, COUPLED, false, false>(a.A, a.B, a.C, a.src, a.src, a.dst, l, a.L,
+    wsum += level_sweep2<R, COUPLED, false>(a.A, a.B, a.C, a.src, a.src, a.dst, l, a.L,
                                                     a.m, a.ms, slice, lane, 1.0, a.far, a.xfar,
                                                     a.xfar);
   }
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kNormThreads) k_normalise(NormArgs a) {
 // Direct residual ||Q^T x||_1 from the stored FP64 blocks (Eq. (1)).  With
 // WITH_Q the level's residual r_l also yields q_l = (-T_dd)^{-1} r_l, stored
 // in FP32 for the correction sweeps of iterative refinement.
-template <int R, bool WITH_Q, bool PAIRED>
+template <int R, bool WITH_Q>
 __global__ void __launch_bounds__(256, Tune<R>::MINB) k_residual(ResidArgs a) {
   extern __shared__ double vsh[];
   __shared__ double sh[32];
@@ -217,8 +217,8 @@ __global__ void __launch_bounds__(256, Tune<R>::MINB) k_residual(ResidArgs a) {
   const int gw = sched_warp(a.L, nw);
   double wsum = 0.0;
   for (int64_t l = gw; l < a.L; l += nw)
-    wsum += level_resid<R, PAIRED>(a.TLO, a.TDD, a.TUP, a.NINV, a.x, WITH_Q ? a.q : nullptr, l,
-                                   a.L, a.m, a.ms, slice, lane, a.far);
+    wsum += level_resid<R>(a.TLO, a.TDD, a.TUP, a.NINV, a.x, WITH_Q ? a.q : nullptr, l, a.L,
+                           a.m, a.ms, slice, lane, a.far);
   if (lane == 0) {
     a.rpart[gw] = wsum;
     __threadfence();
@@ -463,9 +463,9 @@ cudaError_t launch_residual(const ResidArgs& a, int nb, int sms, cudaStream_t s)
   switch (r) {
     case 1:
       if (a.q)
-        k_residual<1, true, false><<<nb, 256, vec_smem<1>(), s>>>(a);
+        k_residual<1, true><<<nb, 256, vec_smem<1>(), s>>>(a);
       else
-        k_residual<1, false, false><<<nb, 256, vec_smem<1>(), s>>>(a);
+        k_residual<1, false><<<nb, 256, vec_smem<1>(), s>>>(a);
       return cudaGetLastError();
     case 2: return resid_m<2>(a, sms, s);
     case 3:

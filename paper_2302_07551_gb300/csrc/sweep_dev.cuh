@@ -102,24 +102,6 @@ __device__ __forceinline__ void gemv_acc_part(double (&acc)[R][Tune<R>::NA],
   }
 }
 
-// Products with the off-diagonal Q^T blocks of a paired block-pentadiagonal
-// chain (m = 32 R, R even): T_lo is zero in rows m/2.. of columns ..m/2,
-// T_up in rows ..m/2 of columns m/2..; only the nonzero quadrants are read.
-template <int R>
-__device__ __forceinline__ void gemv_lo_paired(double (&acc)[R][Tune<R>::NA],
-                                               const double* __restrict__ M, const double* v,
-                                               int m, int lane) {
-  gemv_acc_part<R, 0, R / 2>(acc, M, v, 0, m / 2, m, lane);
-  gemv_acc_part<R, 0, R>(acc, M, v, m / 2, m, m, lane);
-}
-template <int R>
-__device__ __forceinline__ void gemv_up_paired(double (&acc)[R][Tune<R>::NA],
-                                               const double* __restrict__ M, const double* v,
-                                               int m, int lane) {
-  gemv_acc_part<R, 0, R>(acc, M, v, 0, m / 2, m, lane);
-  gemv_acc_part<R, R / 2, R>(acc, M, v, m / 2, m, m, lane);
-}
-
 // v = p * scale (scale = 1 / e^T z of the previous sweep when the previous
 // sweep was not normalised in memory; 1 otherwise: fl(z * (1/s)) is exactly
 // the value the normalisation would have stored).
@@ -219,7 +201,7 @@ __device__ __forceinline__ void far_terms(double (&acc)[R][Tune<R>::NA], const F
 // share of an FP64-bound kernel, and a fused launch only needs the sums of its
 // last two sweeps.
 // CG: neighbour vectors written by other SMs during this kernel (L2 reads).
-template <int R, bool COUPLED, bool PAIRED = false, bool WARP_TOTAL = true, bool CG = false,
+template <int R, bool COUPLED, bool WARP_TOTAL = true, bool CG = false,
           int UM = 1>
 __device__ __forceinline__ double level_sweep2(const double* A, const double* B, const double* C,
                                                const double* src, const double* src_up,
@@ -239,13 +221,8 @@ __device__ __forceinline__ double level_sweep2(const double* A, const double* B,
   __syncwarp();
   double acc[R][NA];
   zero_acc<R>(acc);
-  if constexpr (PAIRED) {
-    if (has_lo) gemv_lo_paired<R>(acc, A + (size_t)l * ms, v_lo, m, lane);
-    if (has_up) gemv_up_paired<R>(acc, B + (size_t)l * ms, v_up, m, lane);
-  } else {
-    if (has_lo) gemv_acc<R, UM>(acc, A + (size_t)l * ms, v_lo, m, lane);
-    if (has_up) gemv_acc<R, UM>(acc, B + (size_t)l * ms, v_up, m, lane);
-  }
+  if (has_lo) gemv_acc<R, UM>(acc, A + (size_t)l * ms, v_lo, m, lane);
+  if (has_up) gemv_acc<R, UM>(acc, B + (size_t)l * ms, v_up, m, lane);
   if (far) far_terms<R, CG>(acc, far, xfar_lo, xfar_up, l, L, m, ms, v_lo, lane);
   if (!COUPLED) {
 #pragma unroll
@@ -280,7 +257,7 @@ __device__ __forceinline__ double level_sweep2(const double* A, const double* B,
 // One level of the direct residual r_l = (Q^T x)_l = T_lo x_{l-1} + T_dd x_l +
 // T_up x_{l+1} (Eq. (1)); returns ||r_l||_1 on every lane.  With q != NULL
 // also stores q_l = (-T_dd)^{-1} r_l in FP32.
-template <int R, bool PAIRED = false>
+template <int R>
 __device__ __forceinline__ double level_resid(const double* TLO, const double* TDD,
                                               const double* TUP, const double* NINV,
                                               const double* x, float* q, int64_t l, int64_t L,
@@ -297,17 +274,11 @@ __device__ __forceinline__ double level_resid(const double* TLO, const double* T
   double acc[R][NA];
   zero_acc<R>(acc);
   if (l > 0) {
-    if constexpr (PAIRED)
-      gemv_lo_paired<R>(acc, TLO + (size_t)l * ms, v_lo, m, lane);
-    else
-      gemv_acc<R>(acc, TLO + (size_t)l * ms, v_lo, m, lane);
+    gemv_acc<R>(acc, TLO + (size_t)l * ms, v_lo, m, lane);
   }
   gemv_acc<R>(acc, TDD + (size_t)l * ms, v_dd, m, lane);
   if (l < L - 1) {
-    if constexpr (PAIRED)
-      gemv_up_paired<R>(acc, TUP + (size_t)l * ms, v_up, m, lane);
-    else
-      gemv_acc<R>(acc, TUP + (size_t)l * ms, v_up, m, lane);
+    gemv_acc<R>(acc, TUP + (size_t)l * ms, v_up, m, lane);
   }
   if (far) far_terms<R>(acc, far, x, x, l, L, m, ms, v_lo, lane);
   double ls = 0.0;
