@@ -196,7 +196,8 @@ int mc_factor(mc_chain* chain);
  * Gauss-Seidel on block-tridiagonal chains run the nsweeps sweeps as one
  * persistent launch per 1024 sweeps, with no normalisation between the sweeps
  * of a launch (the scale of the iterate does not change the next one, Eq. (2)
- * up to rounding); x_out is normalised and stats refer to the last sweep as
+ * up to rounding); chains that fit on chip run the whole call, normalisation
+ * included, in one launch, which mc_set_tuning does not affect; x_out is normalised and stats refer to the last sweep as
  * above.  Block Jacobi (and banded block Gauss-Seidel) run one launch per
  * sweep.  Results are bitwise reproducible for equal calls and independent of
  * the launch configuration (mc_set_tuning); a run split into several calls
@@ -332,8 +333,9 @@ int mc_residual_noalloc(const double* dn, const double* loc, const double* up, i
  * (mc_server_request_bytes each) and at most max_active are running.  Each
  * mc_server_step runs check_every sweeps (dtype MC_F64) or one refinement
  * step of check_every correction sweeps (MC_F32 / MC_BF16) for ALL active
- * requests in shared fused persistent launches (one per block-size bucket
- * for all sweeps of the step), then every request's FP64 residual; requests with residual <= tol
+ * requests in fused persistent launches side by side (one cluster per small
+ * request, teams of warps by block size, a shared queue; which one follows
+ * from the request's own size), then every request's FP64 residual; requests with residual <= tol
  * (or a latched error, or maxit sweeps) are retired, their pi copied to host
  * memory and their arena memory freed.  Requests submitted between steps
  * join the next chunk.  A request's iterates are bitwise independent of the
