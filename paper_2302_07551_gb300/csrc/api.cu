@@ -179,13 +179,26 @@ int* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); 
 
 // Versioned words of a resident cooperative launch.  FP64: two words a value in
 // z and xb (such chains use neither otherwise); low precision: one, both rows in
-// z (xb holds the refinement update).
+// z (xb holds the refinement update; FP64 sweeps of such a chain write z, and
+// reset the words behind them).
 static ResidentWords resident_words(const mc_chain* c) {
   ResidentWords w{};
   w.first = (unsigned long long*)c->z;
   w.last = c->lay.lp ? w.first + (size_t)c->res_ctas * c->lay.m : (unsigned long long*)c->xb;
   w.state = (char*)c->hdr + kGridStateOffset;
   return w;
+}
+
+// Words of a resident cooperative launch to version 0.
+static cudaError_t reset_words(mc_chain* c, cudaStream_t s) {
+  if (!c->res_ctas || !c->res_grid) return cudaSuccess;
+  const size_t row = (size_t)c->res_ctas * c->lay.m * sizeof(unsigned long long);
+  const ResidentWords w = resident_words(c);
+  const size_t bytes = c->lay.lp ? row : 2 * row;
+  cudaError_t e = cudaMemsetAsync(w.state, 0, 16, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.first, 0, bytes, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.last, 0, bytes, s);
+  return e;
 }
 
 // Everything of a resident launch but its vectors, sweeps and outputs.
@@ -214,7 +227,9 @@ static ResidentArgs resident_args(mc_chain* c) {
 // error after the last).  With resid (block-tridiagonal chains only) the last
 // launch also forms ||Q^T dst||_1 from the splitting into stats[2].  ev
 // (optional, 4 events): before the first launch, after the last fused kernel,
-// after its scale reduction, after the last normalisation.
+// after its scale reduction, after the last normalisation.  Low-precision
+// chains stay on chip in their own layout only: their FP64 sweeps run through
+// global memory.
 static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int64_t n,
                                 double* stats_out, cudaStream_t s, cudaEvent_t* ev,
                                 bool resid, bool step) {
@@ -235,7 +250,7 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
   for (int64_t done = 0; done < n;) {
     const int64_t K = n - done < kMaxFusedSweeps ? n - done : kMaxFusedSweeps;
     const bool final = done + K == n;
-    if (c->res_ctas) {
+    if (c->res_ctas && !c->lay.lp) {
       ResidentArgs a = resident_args(c);
       a.x_in = in;
       a.x_out = dst;
@@ -311,6 +326,7 @@ static int enqueue_sweeps_fused(mc_chain* c, const double* src, double* dst, int
     in = dst;
     done += K;
   }
+  if (c->lay.lp) CK(reset_words(c, s));   // z held them
   if (ev) CK(cudaEventRecord(ev[3], s));
   return MC_OK;
 }
@@ -425,25 +441,13 @@ const float* mc::chain_lpSc(mc_chain* c) { return lpSc(c); }
 float* mc::chain_lpQ(mc_chain* c) { return lpQ(c); }
 float* mc::chain_lpD(mc_chain* c) { return lpD(c); }
 
-// Words of a resident cooperative launch to version 0.
-static cudaError_t reset_words(mc_chain* c) {
-  if (!c->res_ctas || !c->res_grid) return cudaSuccess;
-  const size_t row = (size_t)c->res_ctas * c->lay.m * sizeof(unsigned long long);
-  const ResidentWords w = resident_words(c);
-  const size_t bytes = c->lay.lp ? row : 2 * row;
-  cudaError_t e = cudaMemsetAsync(w.state, 0, 16, c->user);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.first, 0, bytes, c->user);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.last, 0, bytes, c->user);
-  return e;
-}
-
 // Clear the status latched in the fetched header and return it (a wait that
 // gave up leaves a resident launch's counters anywhere: they start again).
 static int clear_status(mc_chain* c) {
   const int st = c->hh->status;
   if (st != 0) {
     CK(cudaMemsetAsync(&c->hdr->status, 0, sizeof(int32_t), c->user));
-    if (st == MC_ERR_TIMEOUT) CK(reset_words(c));
+    if (st == MC_ERR_TIMEOUT) CK(reset_words(c, c->user));
     CK(cudaStreamSynchronize(c->user));
   }
   return st;
@@ -577,7 +581,7 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   if (cudaMemsetAsync(c->ws + lay.off_hdr, 0, 4096, c->user) != cudaSuccess ||
       cudaMemsetAsync(c->ws + lay.off_bexp, 0, (size_t)(7 + lay.nfar) * lay.L * sizeof(int),
                       c->user) != cudaSuccess ||
-      reset_words(c) != cudaSuccess)
+      reset_words(c, c->user) != cudaSuccess)
     rc = MC_ERR_CUDA;
   if (rc != MC_OK) {
     mc_destroy(c);

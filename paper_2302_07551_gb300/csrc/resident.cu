@@ -417,6 +417,7 @@ int resident_ctas(const Layout& y, int coupled, int* grid) {
 
 cudaError_t launch_resident(const ResidentArgs& a, const Layout& y, int coupled, int ctas,
                             int grid, cudaStream_t s) {
+  if (y.lp != 0) return cudaErrorInvalidValue;   // ctas and smem_bytes follow the storage type
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   config(cfg, at, grid != 0, ctas, smem_bytes(y, coupled, ctas), s);
@@ -425,6 +426,7 @@ cudaError_t launch_resident(const ResidentArgs& a, const Layout& y, int coupled,
 
 cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& y, int coupled, int ctas,
                                int grid, cudaStream_t s) {
+  if (y.lp == 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   config(cfg, at, grid != 0, ctas, smem_bytes(y, coupled, ctas), s);

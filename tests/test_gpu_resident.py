@@ -113,3 +113,28 @@ def test_solve_is_its_chunks(L, m, apply):
     if r < min(ch.residual(v) for v in xs[:3]):
         pi, res = ch.solve(tol=r * (1 + 1e-6), maxit=n * C, check_every=C)
         assert res["sweeps"] == 4 * C and torch.equal(pi, xs[3])
+
+
+# both links, the low-precision teams, and chains that never stay on chip
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("apply,stair", [("inverse", 1), ("coupled", 2)])
+@pytest.mark.parametrize("L,m", [(2, 4), (64, 8), (305, 32), (600, 24), (2048, 24), (400, 64), (900, 96)])
+def test_fp64_sweeps_of_low_precision_chains(L, m, apply, stair, dtype):
+    """sweep and sweep_host of a low-precision chain run on its FP64 blocks: the FP64 chain's iterates (the
+    suite's 1e-12 relative L1), and they leave the chain's refinement as it was (bitwise)."""
+    blocks = [torch.from_numpy(b).cuda() for b in synth.qbd(L, m, 0.5, seed=L + m)]
+    ch, ref = mc.Chain(*blocks, apply=apply, stair=stair, dtype=dtype), mc.Chain(*blocks, apply=apply, stair=stair)
+    before, _ = ch.solve(tol=1e-12, check_every=24, maxit=40000)
+    x = torch.rand(L * m, dtype=torch.float64, device="cuda") + 0.05
+    x /= x.sum()
+    xh, yh = x.cpu().pin_memory(), torch.empty(L * m, dtype=torch.float64).pin_memory()
+    for K in (1, 2, 33):
+        st, rs = (torch.zeros(3, dtype=torch.float64, device="cuda") for _ in range(2))
+        y, r = ch.sweep(x, nsweeps=K, stats=st), ref.sweep(x, nsweeps=K, stats=rs)
+        assert float((y - r).abs().sum()) <= 1e-12
+        assert torch.allclose(st[:2], rs[:2], rtol=1e-11, atol=1e-14)
+        sh = ch.sweep_host(xh, yh, K)
+        assert torch.equal(yh, y.cpu()) and sh == st.tolist()
+        after, _ = ch.solve(tol=1e-12, check_every=24, maxit=40000)
+        assert torch.equal(before, after)
+    ch.sync()
