@@ -78,8 +78,72 @@ __global__ void __launch_bounds__(256) k_layout(const double* dn, const double* 
 // pivot) and the sum of its updates, added where it is used: m updates rounded
 // at the size of the dominant diagonal would be most of the inverse's error
 // (m = 256: 6.9e-16 against 0.9e-16 relative, 3.3e-16 for blocked LU and solves).
-// Bound: the FP64 pipe (89 % busy at m = 64; a tenth of its instructions are the
-// pivot's).  8192 blocks of 64: 7.7 -> 4.65 ms (3.4 at the pipe's rate).
+// Whether a pivot vanishes is decided by plain LU: a block one of whose pivots
+// cancels to below 2^-45 of its diagonal entry, or is no number, is given up here
+// and formed again by plain_block, with true divisions (a / -a is -1, a * (1 / -a)
+// need not be) and the diagonal in one part, so that two phases whose rates balance
+// still meet their zero pivot and nothing else is refused.  8192 blocks of 64 take
+// the same time with the check.
+// Bound: the FP64 pipe (a tenth of its instructions are the pivot's).  8192 blocks
+// of 64: 7.7 -> 4.65 ms (3.4 at the pipe's rate).
+__device__ __forceinline__ bool cancels(double piv, double diag) {
+  return (((unsigned)__double2hiint(piv) >> 20) & 0x7ffu) + 45u <
+         (((unsigned)__double2hiint(diag) >> 20) & 0x7ffu);
+}
+
+// LU of one block without pivoting and (-T)^{-1} by substitution, in place in
+// global memory, by a CTA: rare, so that only the call costs the kernels above
+// registers.  The pivot test of the set-up.
+__device__ __noinline__ void plain_block(const double* T, double* lu, double* ninv, int* eninv,
+                                         int m, Header* hdr) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int e = tid; e < m * m; e += nt) {
+    lu[e] = T[e];
+    ninv[e] = e % m == e / m ? -1.0 : 0.0;
+  }
+  __syncthreads();
+  for (int k = 0; k < m; ++k) {
+    const double piv = lu[k * m + k];
+    if (!(piv != 0.0) || !isfinite(piv)) {
+      if (tid == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
+      return;
+    }
+    const int n = m - k - 1;
+    for (int i = k + 1 + tid; i < m; i += nt) lu[k * m + i] = lu[k * m + i] / piv;
+    __syncthreads();
+    for (int e = tid; e < n * n; e += nt) {
+      const int i = k + 1 + e % n, j = k + 1 + e / n;
+      lu[j * m + i] = fma(-lu[k * m + i], lu[j * m + k], lu[j * m + i]);
+    }
+    __syncthreads();
+  }
+  for (int k = 0; k < m; ++k) {   // L^{-1}
+    const int n = m - k - 1;
+    for (int e = tid; e < n * m; e += nt) {
+      const int i = k + 1 + e % n, c = e / n;
+      ninv[c * m + i] = fma(-lu[k * m + i], ninv[c * m + k], ninv[c * m + i]);
+    }
+    __syncthreads();
+  }
+  for (int k = m - 1; k >= 0; --k) {   // U^{-1}
+    for (int c = tid; c < m; c += nt) ninv[c * m + k] = ninv[c * m + k] / lu[k * m + k];
+    __syncthreads();
+    for (int e = tid; e < k * m; e += nt) {
+      const int i = e % k, c = e / k;
+      ninv[c * m + i] = fma(-lu[k * m + i], ninv[c * m + k], ninv[c * m + i]);
+    }
+    __syncthreads();
+  }
+  unsigned big = 0u;
+  for (int e = tid; e < m * m; e += nt) {
+    const double v = ninv[e] + 0.0;   // no -0
+    ninv[e] = v;
+    big = max(big, (unsigned)__double2hiint(v) >> 20);
+  }
+  big = __reduce_max_sync(0xffffffffu, big);
+  if ((tid & 31) == 0) atomicMax(eninv, (int)big);
+}
+
 template <int G, int R>
 __device__ __forceinline__ void gj_update(double (&A)[R][R], const double* row, const double* cs,
                                           int ti, int tj, int kb, bool own_row, bool own_col) {
@@ -175,7 +239,7 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
         const double* cl = col + (k & 1) * MP;
         if (G != 16 || (threadIdx.x >> 5) == (k & 7)) {
           const double piv = base[k] + rw[k];
-          if (!(piv != 0.0) || !isfinite(piv)) s_bad[grp] = 1;
+          if (!(piv != 0.0) || !isfinite(piv) || cancels(piv, base[k])) s_bad[grp] = 1;
           const double p = 1.0 / piv;
           for (int i = G == 16 ? (int)(threadIdx.x & 31) : t; i < m; i += G == 16 ? 32 : G * G) {
             const double c = cl[i] * p;
@@ -204,9 +268,7 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
         sync();
       }
     }
-    if (bad) {
-      if (live && t == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
-    } else if (live) {
+    if (live && !bad) {
       unsigned e = 0u;
 #pragma unroll
       for (int a = 0; a < R; ++a)
@@ -227,7 +289,14 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
         for (int i = ti; i < m; i += G)
           lu[(size_t)l * ms + (size_t)j * m + i] = LU[j * (m + 1) + i];
     }
-    sync();   // the buffers are rewritten for the next block
+    if (__syncthreads_or(live && bad)) {   // (also: the buffers are rewritten for the next block)
+      for (int g = 0; g < N; ++g)
+        if (s_bad[g] != 0 && l0 + g < L) {
+          const size_t o = (size_t)(l0 + g) * ms;
+          plain_block(tdd + o, lu + o, ninv + o, eninv + l0 + g, m, hdr);
+        }
+      __syncthreads();   // s_bad is cleared for the next block
+    }
   }
 }
 
@@ -296,9 +365,11 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
             for (int a = 0; a < R; ++a) {
               col[f * H + ti + 16 * a] = A[a][b];
               col_peer[f * H + ti + 16 * a] = A[a][b];
-              if (a == q && cr == (s >> 4) && ti == (s & 15))
+              if (a == q && cr == (s >> 4) && ti == (s & 15)) {
+                const double d = base[ti + 16 * a], v = d + A[a][b];
                 for (int p = 0; p < 4; ++p)
-                  cl.map_shared_rank(piv, p)[f] = base[ti + 16 * a] + A[a][b];
+                  cl.map_shared_rank(piv, p)[f] = cancels(v, d) ? 0.0 : v;
+              }
             }
           }
       }
@@ -342,7 +413,8 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
       }
     }
     if (bad) {
-      if (rank == 0 && threadIdx.x == 0) latch(hdr, MC_ERR_SINGULAR_BLOCK);
+      const size_t o = (size_t)l * ms;
+      if (rank == 0) plain_block(tdd + o, lu + o, ninv + o, eninv + l, m, hdr);
     } else {
       unsigned e = 0u;
 #pragma unroll
