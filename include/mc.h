@@ -464,7 +464,9 @@ int mc_tune(mc_chain* chain, const double* x, int64_t nsweeps, mc_tuning* best,
 /* Wait for the handle's stream and return (and clear) the device status. */
 int mc_sync(mc_chain* chain);
 
-/* Release the handle (host memory only; the workspace stays the caller's). */
+/* Release the handle (host memory only; the workspace stays the caller's).
+ * Does not wait: work that mc_sweep or mc_export left on the stream still uses
+ * the workspace until the stream has reached its end. */
 void mc_destroy(mc_chain* chain);
 
 /* Static description of a status code. */

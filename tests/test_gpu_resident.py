@@ -138,3 +138,21 @@ def test_fp64_sweeps_of_low_precision_chains(L, m, apply, stair, dtype):
         after, _ = ch.solve(tol=1e-12, check_every=24, maxit=40000)
         assert torch.equal(before, after)
     ch.sync()
+
+
+@pytest.mark.parametrize("L,m", [(64, 8), (6000, 64)])
+def test_close_waits_for_the_chains_stream(L, m):
+    """Sweeps may still run on a side stream when a chain is closed: its workspace, which belongs to the
+    stream current at construction, is given back only after them."""
+    blocks = [torch.from_numpy(b).cuda() for b in synth.qbd(L, m, 0.8, seed=1)]
+    x = torch.full((L * m,), 1.0 / (L * m), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    ch = mc.Chain(*blocks, stream=st)
+    ref = ch.sweep(x, nsweeps=64)
+    for _ in range(20):
+        ref = ch.sweep(x, ref, nsweeps=1024)     # some milliseconds at least
+    ws = ch._ws                                  # not handed out here, whatever close() does
+    ch.close()
+    assert st.query()
+    del ws
