@@ -175,14 +175,10 @@ class Chain:
         nat.check(self._lib.mc_sync(self._h), "mc_sync")
 
     def close(self):
-        """Release the handle.  Waits for the chain's stream: sweeps and exports that are still running use the
-        workspace, which the allocator gives out again in the order of the stream current at construction.  While
-        a graph is being captured it only ties the workspace to the chain's stream."""
+        """Release the handle.  Does not wait: sweeps and exports that still run on the chain's stream keep the
+        workspace until they are done, whatever stream was current at construction."""
         if getattr(self, "_h", None):
-            if torch.cuda.is_current_stream_capturing():
-                self._ws.record_stream(self.stream)
-            else:
-                self.stream.synchronize()
+            self._ws.record_stream(self.stream)
             self._lib.mc_destroy(self._h)
             self._h = None
 

@@ -141,18 +141,25 @@ def test_fp64_sweeps_of_low_precision_chains(L, m, apply, stair, dtype):
 
 
 @pytest.mark.parametrize("L,m", [(64, 8), (6000, 64)])
-def test_close_waits_for_the_chains_stream(L, m):
-    """Sweeps may still run on a side stream when a chain is closed: its workspace, which belongs to the
-    stream current at construction, is given back only after them."""
+def test_close_keeps_the_workspace_until_the_stream_is_done(L, m):
+    """Sweeps may still run on a side stream when a chain is closed: the allocator does not give its workspace,
+    which belongs to the stream current at construction, to anyone before they end."""
     blocks = [torch.from_numpy(b).cuda() for b in synth.qbd(L, m, 0.8, seed=1)]
     x = torch.full((L * m,), 1.0 / (L * m), dtype=torch.float64, device="cuda")
     torch.cuda.synchronize()
     st = torch.cuda.Stream()
     ch = mc.Chain(*blocks, stream=st)
     ref = ch.sweep(x, nsweeps=64)
-    for _ in range(20):
-        ref = ch.sweep(x, ref, nsweeps=1024)     # some milliseconds at least
-    ws = ch._ws                                  # not handed out here, whatever close() does
+    torch.cuda.synchronize()
+    y = torch.empty_like(ref)
+    for _ in range(40):
+        ch.sweep(x, y, nsweeps=1024)             # tens of milliseconds
+    ch.sweep(x, y, nsweeps=64)
+    at, size = ch._ws.data_ptr(), ch._ws.numel()
     ch.close()
-    assert st.query()
-    del ws
+    del ch
+    other = torch.empty(size, dtype=torch.uint8, device="cuda")     # never written
+    busy = not st.query()
+    assert busy and other.data_ptr() != at
+    st.synchronize()
+    assert torch.equal(y, ref)
