@@ -57,7 +57,8 @@ class Chain:
         self._ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
         base = self._ws.data_ptr()
         self._ws_ptr = (base + 255) // 256 * 256
-        self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+        self._ws_stream = torch.cuda.current_stream(self.device)
+        self.stream = stream if stream is not None else self._ws_stream
         h = ctypes.c_void_p()
         if diags is not None:
             arr = (ctypes.c_void_p * (lower + upper + 1))(
@@ -178,7 +179,8 @@ class Chain:
         """Release the handle.  Does not wait: sweeps and exports that still run on the chain's stream keep the
         workspace until they are done, whatever stream was current at construction."""
         if getattr(self, "_h", None):
-            self._ws.record_stream(self.stream)
+            if self.stream != self._ws_stream:
+                self._ws.record_stream(self.stream)
             self._lib.mc_destroy(self._h)
             self._h = None
 
