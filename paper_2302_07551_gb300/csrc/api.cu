@@ -65,7 +65,7 @@ Layout make_layout(const mc_desc& d) {
   y.off_fver = o;
   o += round_up(sizeof(unsigned long long) + (size_t)d.L * sizeof(int), 256);
   y.off_bexp = o;
-  o += round_up((size_t)(7 + y.nfar) * (size_t)d.L * sizeof(int), 256);   // either apply mode
+  o += round_up((size_t)(7 + y.nfar) * (size_t)d.L * sizeof(int2), 256);   // either apply mode
   y.lp = d.dtype == MC_F32 ? 1 : d.dtype == MC_BF16 ? 2 : 0;
   if (y.lp) {
     const size_t es = y.lp == 1 ? 4 : 2;
@@ -172,10 +172,10 @@ static bool fused_ok(const mc_chain* c) {
 static bool split_resid_ok(const mc_chain* c) { return c->d.stair <= 2 && c->lay.nfar == 0; }
 
 // block_exp of a plane's blocks (written by the factorisation).
-static int* plane_exp(const mc_chain* c, int plane) {
-  return (int*)(c->ws + c->lay.off_bexp) + (size_t)plane * (size_t)c->lay.L;
+static int2* plane_exp(const mc_chain* c, int plane) {
+  return (int2*)(c->ws + c->lay.off_bexp) + (size_t)plane * (size_t)c->lay.L;
 }
-int* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); }
+int2* mc::chain_bexp(const mc_chain* c, int plane) { return plane_exp(c, plane); }
 
 // Versioned words of a resident cooperative launch.  FP64: two words a value in
 // z and xb (such chains use neither otherwise); low precision: one, both rows in
@@ -579,7 +579,7 @@ int mc::chain_init(const mc_desc* desc, void* workspace, size_t ws_bytes, cudaSt
   memset(c->hh, 0, sizeof(Header));
   int rc = MC_OK;
   if (cudaMemsetAsync(c->ws + lay.off_hdr, 0, 4096, c->user) != cudaSuccess ||
-      cudaMemsetAsync(c->ws + lay.off_bexp, 0, (size_t)(7 + lay.nfar) * lay.L * sizeof(int),
+      cudaMemsetAsync(c->ws + lay.off_bexp, 0, (size_t)(7 + lay.nfar) * lay.L * sizeof(int2),
                       c->user) != cudaSuccess ||
       reset_words(c, c->user) != cudaSuccess)
     rc = MC_ERR_CUDA;
@@ -681,6 +681,9 @@ int mc::chain_factor_async(mc_chain* c) {
   const size_t pe = c->lay.plane_bytes / sizeof(double);
   const bool coupled = c->d.apply == MC_APPLY_COUPLED;
   CK(launch_factor(c->planes, plane_exp(c, 0), c->lay, c->hdr, coupled, c->num_sms, c->user));
+  // the sweeps of blocks of up to 16 rows, on chip or in low precision do not ask for it
+  if (c->lay.m > 16 && !c->lay.lp && !c->res_ctas)
+    CK(launch_weak_rows(c->planes, plane_exp(c, 0), c->lay, coupled, c->user));
   if (c->lay.lp) {
     const int bf16 = c->lay.lp == 2;
     CK(launch_lp_convert(c->planes + (coupled ? kPlaneWLO : kPlaneTLO) * pe, c->ws + c->lay.off_lpA,

@@ -422,14 +422,14 @@ __global__ void __launch_bounds__(256, 3) k_b_team64(const BTable* __restrict__ 
     const bool has_lo = l > 0, has_up = l < L - 1;
     double* dst = k == K - 1 ? Q->z : Q->xb;
     const double* src = h2 ? dst : (k == 0 ? Q->x : Q->xb);
-    const int ea = Q->eA[l], eb = Q->eB[l], ec = COUPLED ? 0 : Q->eC[l];
+    const int2 ea = Q->eA[l], eb = Q->eB[l], ec = COUPLED ? make_int2(0, 0) : Q->eC[l];
     if (h2 || k > 0)
       wait_neighbours(Q->ver, l, L, (Q->vbase + (int)(h2 ? k + 1 : k)) * TW, &out[r].status, lane,
                       kWaitNs);
     const double x0[1] = {has_lo && tt < m ? __ldcg(src + (l - 1) * m + tt) : 0.0};
     const double x1[1] = {has_up && tt < m ? __ldcg(src + (l + 1) * m + tt) : 0.0};
-    stage_rows<TW, 1>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], x0, tt, 32, w, lane);
-    stage_rows<TW, 1>(sh.slot[s].v[1], sh.slot[s].x[1], sh.emax[s][1], x1, tt, 32, w, lane);
+    stage_rows<1>(sh.slot[s].v[0], sh.slot[s].x[0], sh.exps[s][0], x0, m, tt, 32, w, lane);
+    stage_rows<1>(sh.slot[s].v[1], sh.slot[s].x[1], sh.exps[s][1], x1, m, tt, 32, w, lane);
     team_sync<TW>(bar);
     const unsigned long long qn = sh.next[turn];
     turn ^= 1;
@@ -437,18 +437,18 @@ __global__ void __launch_bounds__(256, 3) k_b_team64(const BTable* __restrict__ 
     double acc[1] = {0.0};
     if (has_lo)
       rows_product<1, 0>(acc, Q->A + at, sh.slot[s].v[0], sh.slot[s].x[0], ea,
-                         team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
+                         team_exp<TW>(sh.exps[s][0]), 0, m, m, row0, lane);
     if (has_up)
       rows_product<1, 0>(acc, Q->B + at, sh.slot[s].v[1], sh.slot[s].x[1], eb,
-                         team_max<TW>(sh.emax[s][1]), 0, m, m, row0, lane);
+                         team_exp<TW>(sh.exps[s][1]), 0, m, m, row0, lane);
     if constexpr (!COUPLED) {
       s ^= 1;
-      stage_rows<TW, 1>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], acc, row0 + lane, 32, w,
-                        lane);
+      stage_rows<1>(sh.slot[s].v[0], sh.slot[s].x[0], sh.exps[s][0], acc, m, row0 + lane, 32, w,
+                    lane);
       team_sync<TW>(bar);
       acc[0] = 0.0;
       rows_product<1, 0>(acc, Q->C + at, sh.slot[s].v[0], sh.slot[s].x[0], ec,
-                         team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
+                         team_exp<TW>(sh.exps[s][0]), 0, m, m, row0, lane);
     }
     double ls = 0.0;
     if (row0 + lane < m) {

@@ -54,9 +54,9 @@ struct BReq {
   int* ver;             // fused sweeps: per-level completion counters
   int64_t L;
   unsigned long long* dv;   // low precision: versioned words of the correction (team path)
-  const int* eA;        // FP64: block_exp of A, B, C (team path)
-  const int* eB;
-  const int* eC;
+  const int2* eA;       // FP64: block_exp of A, B, C (team path)
+  const int2* eB;
+  const int2* eC;
   int32_t m, ms, R, p1;  // p1: 0-based parity of the diagonal-only rows
   int32_t G, path;       // levels per unit of this request (the table's G scaled by size
                          // class); kPathQueue, ...

@@ -38,7 +38,7 @@ int chain_factor_async(mc_chain* c);
 // Enqueue the direct residual of x (and q = (-T_dd)^{-1} r when q != NULL).
 int chain_residual_async(mc_chain* c, const double* x, cudaStream_t s, float* q);
 // block_exp per level of one plane (mc_internal.cuh).
-int* chain_bexp(const mc_chain* c, int plane);
+int2* chain_bexp(const mc_chain* c, int plane);
 const void* chain_lpA(mc_chain* c);
 const void* chain_lpB(mc_chain* c);
 const float* chain_lpC(mc_chain* c);

@@ -12,13 +12,30 @@ namespace mc {
 
 namespace {
 
+// Exponents of a lane's entries of a block, joined over the lanes of `mask` and into
+// its block_exp (the rows' part comes later, k_weak_rows).
+struct Exps {
+  unsigned most = 0u, low = 0u;
+  __device__ __forceinline__ void take(double v) {
+    most = max(most, dev::exp_field(v));
+    low = max(low, dev::exp_low(v));
+  }
+  __device__ __forceinline__ void join(int2* to, bool first, unsigned mask = 0xffffffffu) {
+    most = __reduce_max_sync(mask, most);
+    low = __reduce_max_sync(mask, low);
+    if (first) {
+      atomicMax(&to->x, (int)most);
+      atomicMax(&to->y, (int)low);
+    }
+  }
+};
+
 // Copy of one block (or of a 2048-entry chunk of it) by a warp, zero where the
-// block is missing and beyond m * m; returns the largest exponent field of its
-// entries on every lane (block_exp).
+// block is missing and beyond m * m.
 constexpr int kChunk = 2048;
-__device__ __forceinline__ unsigned copy_chunk(const double* src, double* dst, int e0, int mm,
-                                               int ms, int lane) {
-  unsigned big = 0u;
+__device__ __forceinline__ Exps copy_chunk(const double* src, double* dst, int e0, int mm, int ms,
+                                           int lane) {
+  Exps x;
   const int e1 = min(e0 + kChunk, ms);
   for (int e = e0 + lane; e < e1; e += 8 * 32) {
     double v[8];
@@ -27,10 +44,10 @@ __device__ __forceinline__ unsigned copy_chunk(const double* src, double* dst, i
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       if (e + 32 * q < e1) dst[e + 32 * q] = v[q];
-      big = max(big, (unsigned)__double2hiint(v[q]) >> 20);
+      x.take(v[q]);
     }
   }
-  return __reduce_max_sync(0xffffffffu, big);
+  return x;
 }
 
 // Planes TLO, TUP, TDD from the generator blocks (Sect. 2 block partition of
@@ -41,7 +58,7 @@ __device__ __forceinline__ unsigned copy_chunk(const double* src, double* dst, i
 // copy, without another pass.
 __global__ void __launch_bounds__(256) k_layout(const double* dn, const double* loc,
                                                 const double* up, double* tlo, double* tup,
-                                                double* tdd, int* elo, int* eup, int64_t L, int m,
+                                                double* tdd, int2* elo, int2* eup, int64_t L, int m,
                                                 int ms) {
   const int64_t mm = (int64_t)m * m;
   const int chunks = (ms + kChunk - 1) / kChunk, lane = threadIdx.x & 31;
@@ -53,8 +70,8 @@ __global__ void __launch_bounds__(256) k_layout(const double* dn, const double* 
                         : p == 1 ? (l < L - 1 ? dn + (l + 1) * mm : nullptr)
                                  : loc + l * mm;
     double* dst = (p == 0 ? tlo : p == 1 ? tup : tdd) + (size_t)l * ms;
-    const unsigned e = copy_chunk(src, dst, e0, (int)mm, ms, lane);
-    if (p < 2 && lane == 0) atomicMax((p == 0 ? elo : eup) + l, (int)e);
+    Exps x = copy_chunk(src, dst, e0, (int)mm, ms, lane);
+    if (p < 2) x.join((p == 0 ? elo : eup) + l, lane == 0);
   }
 }
 
@@ -94,7 +111,7 @@ __device__ __forceinline__ bool cancels(double piv, double diag) {
 // LU of one block without pivoting and (-T)^{-1} by substitution, in place in
 // global memory, by a CTA: rare, so that only the call costs the kernels above
 // registers.  The pivot test of the set-up.
-__device__ __noinline__ void plain_block(const double* T, double* lu, double* ninv, int* eninv,
+__device__ __noinline__ void plain_block(const double* T, double* lu, double* ninv, int2* eninv,
                                          int m, Header* hdr) {
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int e = tid; e < m * m; e += nt) {
@@ -134,14 +151,13 @@ __device__ __noinline__ void plain_block(const double* T, double* lu, double* ni
     }
     __syncthreads();
   }
-  unsigned big = 0u;
+  Exps x;
   for (int e = tid; e < m * m; e += nt) {
     const double v = ninv[e] + 0.0;   // no -0
     ninv[e] = v;
-    big = max(big, (unsigned)__double2hiint(v) >> 20);
+    x.take(v);
   }
-  big = __reduce_max_sync(0xffffffffu, big);
-  if ((tid & 31) == 0) atomicMax(eninv, (int)big);
+  x.join(eninv, (tid & 31) == 0);
 }
 
 template <int G, int R>
@@ -186,7 +202,7 @@ struct GjBlock {
 
 template <int G, int R>
 __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __restrict__ tdd,
-                                                             double* lu, double* ninv, int* eninv,
+                                                             double* lu, double* ninv, int2* eninv,
                                                              int64_t L, int m, int ms, int per,
                                                              Header* hdr) {
   extern __shared__ double sm[];
@@ -269,7 +285,7 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
       }
     }
     if (live && !bad) {
-      unsigned e = 0u;
+      Exps x;
 #pragma unroll
       for (int a = 0; a < R; ++a)
 #pragma unroll
@@ -279,12 +295,11 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
             // 0 - x: no -0, whose sign bit would read as negative
             const double v = (i == j ? -base[i] : 0.0) - A[a][b];
             ninv[(size_t)l * ms + (size_t)j * m + i] = v;
-            e = max(e, (unsigned)__double2hiint(v) >> 20);
+            x.take(v);
           }
         }
-      const unsigned mask = G == 16 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
-      e = __reduce_max_sync(mask, e);
-      if ((threadIdx.x & (G == 16 ? 31 : 15)) == 0) atomicMax(eninv + l, (int)e);
+      x.join(eninv + l, (threadIdx.x & (G == 16 ? 31 : 15)) == 0,
+             G == 16 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16));
       for (int j = tj; j < m; j += G)
         for (int i = ti; i < m; i += G)
           lu[(size_t)l * ms + (size_t)j * m + i] = LU[j * (m + 1) + i];
@@ -313,7 +328,7 @@ struct GjBig {
 
 template <int R>
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
-    k_gj_cluster(const double* __restrict__ tdd, double* lu, double* ninv, int* eninv, int64_t L,
+    k_gj_cluster(const double* __restrict__ tdd, double* lu, double* ninv, int2* eninv, int64_t L,
                  int m, int ms, Header* hdr) {
   extern __shared__ double sm[];
   constexpr int H = GjBig<R>::H;
@@ -416,7 +431,7 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
       const size_t o = (size_t)l * ms;
       if (rank == 0) plain_block(tdd + o, lu + o, ninv + o, eninv + l, m, hdr);
     } else {
-      unsigned e = 0u;
+      Exps x;
 #pragma unroll
       for (int a = 0; a < R; ++a)
 #pragma unroll
@@ -426,11 +441,10 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256, 1)
             const double v = (i == j ? -base[ti + 16 * a] : 0.0) - A[a][b];
             ninv[(size_t)l * ms + (size_t)j * m + i] = v;
             lu[(size_t)l * ms + (size_t)j * m + i] = LU[(tj + 16 * b) * (H + 1) + ti + 16 * a];
-            e = max(e, (unsigned)__double2hiint(v) >> 20);
+            x.take(v);
           }
         }
-      e = __reduce_max_sync(0xffffffffu, e);
-      if ((threadIdx.x & 31) == 0) atomicMax(eninv + l, (int)e);
+      x.join(eninv + l, (threadIdx.x & 31) == 0);
     }
     cl.sync();   // the buffers are rewritten for the next block
   }
@@ -456,7 +470,7 @@ struct CoupledShared {
 
 // One tile: rows i0 + ti + 16 a (a < RA), columns j0 + tj + 16 b (b < RB) of W.
 template <int TILE, int RA, int RB, bool FIX>
-__device__ __forceinline__ unsigned coupled_tile(CoupledShared<TILE>& sh, const double* Nl,
+__device__ __forceinline__ Exps coupled_tile(CoupledShared<TILE>& sh, const double* Nl,
                                                  const double* T, double* W, int etot, int i0,
                                                  int j0, int m) {
   using namespace dev;
@@ -500,7 +514,7 @@ __device__ __forceinline__ unsigned coupled_tile(CoupledShared<TILE>& sh, const 
           const int s = etot - (int)((uint32_t)x & 0x7ffu);
 #pragma unroll
           for (int q = 0; q < RA; ++q)
-            fixed_fma(fa[q][b < RF ? b : 0], seen[q][b < RF ? b : 0], a[q], xl, xh, s);
+            fixed_fma(fa[q][b < RF ? b : 0], a[q], xl, xh, s, &seen[q][b < RF ? b : 0]);
         } else {
           const double v = sh.B[k][tj + 16 * b];
 #pragma unroll
@@ -509,7 +523,7 @@ __device__ __forceinline__ unsigned coupled_tile(CoupledShared<TILE>& sh, const 
       }
     }
   }
-  unsigned e = 0u;
+  Exps e;
 #pragma unroll
   for (int b = 0; b < RB; ++b)
 #pragma unroll
@@ -519,14 +533,14 @@ __device__ __forceinline__ unsigned coupled_tile(CoupledShared<TILE>& sh, const 
       double v = acc[a][b];
       if (b < RF) {
         bool bad = false;
-        v = fixed_value(fa[a][b < RF ? b : 0], seen[a][b < RF ? b : 0], etot, bad);
-        if (bad) {
+        v = fixed_value(fa[a][b < RF ? b : 0], etot, bad);
+        if (bad && seen[a][b < RF ? b : 0] != 0u) {
           v = 0.0;
           for (int k = 0; k < m; ++k) v = fma(Nl[(size_t)k * m + i], T[(size_t)j * m + k], v);
         }
       }
       W[(size_t)j * m + i] = v;
-      e = max(e, (unsigned)__double2hiint(v) >> 20);
+      e.take(v);
     }
   return e;
 }
@@ -542,9 +556,9 @@ __global__ void __launch_bounds__(256, 2) k_coupled(const double* __restrict__ n
                                                     const double* __restrict__ tlo,
                                                     const double* __restrict__ tup,
                                                     double* __restrict__ wlo,
-                                                    double* __restrict__ wup, const int* en,
-                                                    const int* elo, const int* eup, int* ewlo,
-                                                    int* ewup, int64_t L, int m, int ms,
+                                                    double* __restrict__ wup, const int2* en,
+                                                    const int2* elo, const int2* eup, int2* ewlo,
+                                                    int2* ewup, int64_t L, int m, int ms,
                                                     int tiles) {
   constexpr int TILE = 16 * RT;
   __shared__ CoupledShared<TILE> sh;
@@ -558,9 +572,9 @@ __global__ void __launch_bounds__(256, 2) k_coupled(const double* __restrict__ n
     const double* Nl = ninv + (size_t)l * ms;
     const double* T = (h == 0 ? tlo : tup) + (size_t)l * ms;
     double* W = (h == 0 ? wlo : wup) + (size_t)l * ms;
-    const int ea = en[l], eb = (h == 0 ? elo : eup)[l], etot = ea + eb;
+    const int ea = en[l].x, eb = (h == 0 ? elo : eup)[l].x, etot = ea + eb;
     const bool fix = dev::fixed_ok(ea) && dev::fixed_ok(eb);
-    unsigned e = 0u;
+    Exps e;
     auto run = [&](auto ra, auto rb) {
       constexpr int RA = decltype(ra)::value, RB = decltype(rb)::value;
       if constexpr (RA <= RT && RB <= RT)
@@ -581,8 +595,7 @@ __global__ void __launch_bounds__(256, 2) k_coupled(const double* __restrict__ n
       case 34: run(I4(), I2()); break;
       default: run(I4(), I4()); break;
     }
-    e = __reduce_max_sync(0xffffffffu, e);
-    if ((threadIdx.x & 31) == 0) atomicMax((h == 0 ? ewlo : ewup) + l, (int)e);
+    e.join((h == 0 ? ewlo : ewup) + l, (threadIdx.x & 31) == 0);
   }
 }
 
@@ -628,35 +641,70 @@ __global__ void k_check_paired(const double* __restrict__ tlo, const double* __r
 }
 
 __global__ void __launch_bounds__(256) k_layout_diag(const double* diag, int d, double* plane,
-                                                     int* bexp, int64_t L, int m, int ms) {
+                                                     int2* bexp, int64_t L, int m, int ms) {
   const int64_t mm = (int64_t)m * m;
   const int chunks = (ms + kChunk - 1) / kChunk, lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < L * chunks;
        t += nw) {
     const int64_t l = t / chunks, k = l + d;
-    const unsigned e = copy_chunk(k >= 0 && k < L ? diag + k * mm : nullptr,
-                                  plane + (size_t)l * ms, (int)(t - l * chunks) * kChunk, (int)mm,
-                                  ms, lane);
-    if (lane == 0) atomicMax(bexp + l, (int)e);
+    Exps x = copy_chunk(k >= 0 && k < L ? diag + k * mm : nullptr, plane + (size_t)l * ms,
+                        (int)(t - l * chunks) * kChunk, (int)mm, ms, lane);
+    x.join(bexp + l, lane == 0);
   }
 }
 
-// block_exp of TLO and TUP where the blocks did not come through k_layout.
+// block_exp (but for the rows) of TLO and TUP where the blocks did not come through k_layout.
 __global__ void __launch_bounds__(256) k_block_exp(const double* __restrict__ tlo,
-                                                   const double* __restrict__ tup, int* elo,
-                                                   int* eup, int64_t L, int m, int ms) {
+                                                   const double* __restrict__ tup, int2* elo,
+                                                   int2* eup, int64_t L, int m, int ms) {
   const int chunks = (ms + kChunk - 1) / kChunk, lane = threadIdx.x & 31;
   const int64_t total = 2 * L * chunks, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total; t += nw) {
     const int64_t b = t / chunks, l = b >> 1;
     const int e0 = (int)(t - b * chunks) * kChunk, e1 = min(e0 + kChunk, m * m);
     const double* p = ((b & 1) ? tup : tlo) + (size_t)l * ms;
-    unsigned e = 0u;
-    for (int i = e0 + lane; i < e1; i += 32)
-      e = max(e, (unsigned)__double2hiint(__ldcs(p + i)) >> 20);
-    e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0) atomicMax(((b & 1) ? eup : elo) + l, (int)e);
+    Exps x;
+    for (int i = e0 + lane; i < e1; i += 32) x.take(__ldcs(p + i));
+    x.join(((b & 1) ? eup : elo) + l, lane == 0);
+  }
+}
+
+// The rows' part of block_exp: the smallest over the rows (that are not zero) of a
+// row's largest entry.  Local blocks whose phases form a long line have inverses
+// whose entries span hundreds of bits with every row's largest at the same size.
+// Blocks that span up to 2^16 are left at their smallest entry, which loses little
+// there, and are not read again; a warp per other block.
+struct WeakRows {
+  int n;
+  const double* plane[3 + kMaxFar];
+  int2* exps[3 + kMaxFar];
+};
+__global__ void __launch_bounds__(256) k_weak_rows(WeakRows p, int64_t L, int m, int ms) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < p.n * L; t += nw) {
+    const int64_t l = t % L;
+    const int k = (int)(t / L);
+    int2* to = p.exps[k] + l;
+    const int2 e = *to;
+    if (e.x >= 2047 || e.x + e.y <= 4096 + 16) continue;   // (no entries: 0 + 0)
+    const double* M = p.plane[k] + (size_t)l * ms;
+    unsigned weak = 0u;
+    for (int r0 = 0; r0 < m; r0 += 32) {
+      const int row = r0 + lane;
+      unsigned most = 0u;
+      bool any = false;
+      if (row < m)
+        for (int j = 0; j < m; ++j) {
+          const double v = M[(size_t)j * m + row];
+          any = any || !dev::is_zero(v);
+          most = max(most, dev::exp_field(v));
+        }
+      if (any) weak = max(weak, 4096u - most);
+    }
+    weak = __reduce_max_sync(0xffffffffu, weak);
+    if (lane == 0) to->y = (int)(weak << 16) | (e.y & 0xffff);
   }
 }
 
@@ -667,7 +715,23 @@ int copy_blocks(int64_t warps) {
 
 }  // namespace
 
-cudaError_t launch_block_exp(const double* planes, int* bexp, const Layout& y, cudaStream_t s) {
+cudaError_t launch_weak_rows(const double* planes, int2* bexp, const Layout& y, int coupled,
+                             cudaStream_t s) {
+  const size_t pe = y.plane_bytes / sizeof(double);
+  WeakRows p{};
+  auto add = [&](int k) {
+    p.plane[p.n] = planes + (size_t)k * pe;
+    p.exps[p.n++] = bexp + (size_t)k * y.L;
+  };
+  add(coupled ? kPlaneWLO : kPlaneTLO);
+  add(coupled ? kPlaneWUP : kPlaneTUP);
+  if (!coupled) add(kPlaneNINV);
+  for (int j = 0; j < y.nfar; ++j) add(y.far_base + j);
+  k_weak_rows<<<copy_blocks(p.n * y.L), 256, 0, s>>>(p, y.L, y.m, y.ms);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_block_exp(const double* planes, int2* bexp, const Layout& y, cudaStream_t s) {
   const size_t pe = y.plane_bytes / sizeof(double);
   const int chunks = (y.ms + kChunk - 1) / kChunk;
   k_block_exp<<<copy_blocks(2 * y.L * chunks), 256, 0, s>>>(
@@ -676,7 +740,7 @@ cudaError_t launch_block_exp(const double* planes, int* bexp, const Layout& y, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_layout_diag(const double* diag, int d, double* plane, int* bexp,
+cudaError_t launch_layout_diag(const double* diag, int d, double* plane, int2* bexp,
                                const Layout& lay, cudaStream_t s) {
   const int chunks = (lay.ms + kChunk - 1) / kChunk;
   k_layout_diag<<<copy_blocks(lay.L * chunks), 256, 0, s>>>(diag, d, plane, bexp, lay.L, lay.m,
@@ -691,7 +755,7 @@ cudaError_t launch_check_paired(const double* tlo, const double* tup, const Layo
 }
 
 cudaError_t launch_layout(const double* dn, const double* loc, const double* up, double* planes,
-                          int* bexp, const Layout& lay, cudaStream_t s) {
+                          int2* bexp, const Layout& lay, cudaStream_t s) {
   const size_t pe = lay.plane_bytes / sizeof(double);
   const int chunks = (lay.ms + kChunk - 1) / kChunk;
   k_layout<<<copy_blocks(3 * lay.L * chunks), 256, 0, s>>>(
@@ -705,7 +769,7 @@ namespace {
 struct FactorArgs {
   const double* tdd;
   double *lu, *ninv;
-  int* eninv;
+  int2* eninv;
   int64_t L;
   int m, ms, sms;
   Header* hdr;
@@ -775,7 +839,7 @@ cudaError_t gj_dispatch(const FactorArgs& f, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_factor(double* planes, int* bexp, const Layout& lay, Header* hdr, int coupled,
+cudaError_t launch_factor(double* planes, int2* bexp, const Layout& lay, Header* hdr, int coupled,
                           int num_sms, cudaStream_t s) {
   const size_t pe = lay.plane_bytes / sizeof(double);
   const int m = lay.m;

@@ -109,8 +109,9 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
     const double* src = resid ? a.Z : h2 ? dst : y;
     const int need = (int)(h2 ? k + 1 : k);
     // the blocks' exponents: loaded while this team waits
-    const int ea = resid ? 0 : a.eA[l], eb = resid ? 0 : a.eB[l];
-    const int ec = COUPLED || resid ? 0 : a.eC[l];
+    const int2 none = make_int2(0, 0);
+    const int2 ea = resid ? none : a.eA[l], eb = resid ? none : a.eB[l];
+    const int2 ec = COUPLED || resid ? none : a.eC[l];
     if constexpr (BANDED) {
       if (need > 0)
         wait_band(a.ver, l, a.L, a.bw, (int)k * TW, need * TW, &a.hdr->status, lane, a.wait_ns);
@@ -119,7 +120,6 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
     }
     // stage both neighbours: thread tt of the team loads rows tt, tt + 32 TW
     {
-      unsigned e0 = 0u, e1 = 0u;
       double x0[RW], x1[RW];
 #pragma unroll
       for (int i = 0; i < RW; ++i) {
@@ -135,22 +135,8 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
           if (has_up && row < m) x1[i] -= __ldcg(a.prev + (l + 1) * m + row);
         }
       }
-#pragma unroll
-      for (int i = 0; i < RW; ++i) {
-        const int row = tt + 32 * TW * i;
-        sh.slot[s].v[0][row] = x0[i];
-        sh.slot[s].v[1][row] = x1[i];
-        sh.slot[s].x[0][row] = fixed_entry(x0[i]);
-        sh.slot[s].x[1][row] = fixed_entry(x1[i]);
-        e0 = max(e0, (unsigned)__double2hiint(x0[i]) >> 20);
-        e1 = max(e1, (unsigned)__double2hiint(x1[i]) >> 20);
-      }
-      e0 = __reduce_max_sync(kFull, e0);
-      e1 = __reduce_max_sync(kFull, e1);
-      if (lane == 0) {
-        sh.emax[s][0][w] = (int)e0;
-        sh.emax[s][1][w] = (int)e1;
-      }
+      stage_rows<RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.exps[s][0], x0, m, tt, 32 * TW, w, lane);
+      stage_rows<RW>(sh.slot[s].v[1], sh.slot[s].x[1], sh.exps[s][1], x1, m, tt, 32 * TW, w, lane);
     }
     team_sync<TW>(bar);
     if constexpr (TW > 1) {
@@ -178,40 +164,40 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
     }
     if (has_lo)
       rows_product<RW, MC>(acc, a.A + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], ea,
-                           team_max<TW>(sh.emax[s][0]), lo0, m, m, row0, lane);
+                           team_exp<TW>(sh.exps[s][0]), lo0, m, m, row0, lane);
     if (has_up)
       rows_product<RW, MC>(acc, a.B + (size_t)l * a.ms, sh.slot[s].v[1], sh.slot[s].x[1], eb,
-                           team_max<TW>(sh.emax[s][1]), 0, up1, m, row0, lane);
+                           team_exp<TW>(sh.exps[s][1]), 0, up1, m, row0, lane);
     if constexpr (BANDED) {
       const int n = a.far->n;
       for (int j = 0; j < n; ++j) {
         const int64_t kk = l + a.far->off[j];
         if (kk < 0 || kk >= a.L) continue;
         s ^= 1;
-        const int ef = a.far->bexp[j][l];
+        const int2 ef = a.far->bexp[j][l];
         double x0[RW];
 #pragma unroll
         for (int i = 0; i < RW; ++i) {
           const int row = tt + 32 * TW * i;
           x0[i] = row < m ? __ldcg(y + kk * m + row) : 0.0;
         }
-        stage_rows<TW, RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], x0, tt, 32 * TW, w,
-                           lane);
+        stage_rows<RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.exps[s][0], x0, m, tt, 32 * TW, w,
+                       lane);
         team_sync<TW>(bar);
         rows_product<RW, MC>(acc, a.far->plane[j] + (size_t)l * a.ms, sh.slot[s].v[0],
-                             sh.slot[s].x[0], ef, team_max<TW>(sh.emax[s][0]), 0,
+                             sh.slot[s].x[0], ef, team_exp<TW>(sh.exps[s][0]), 0,
                              m, m, row0, lane);
       }
     }
     if constexpr (!COUPLED) {
       s ^= 1;
-      stage_rows<TW, RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.emax[s][0], acc, row0 + lane, 32, w,
-                         lane);
+      stage_rows<RW>(sh.slot[s].v[0], sh.slot[s].x[0], sh.exps[s][0], acc, m, row0 + lane, 32, w,
+                     lane);
       team_sync<TW>(bar);
 #pragma unroll
       for (int i = 0; i < RW; ++i) acc[i] = 0.0;
       rows_product<RW, MC>(acc, a.C + (size_t)l * a.ms, sh.slot[s].v[0], sh.slot[s].x[0], ec,
-                           team_max<TW>(sh.emax[s][0]), 0, m, m, row0, lane);
+                           team_exp<TW>(sh.exps[s][0]), 0, m, m, row0, lane);
     }
     double t = 0.0;
 #pragma unroll

@@ -44,7 +44,7 @@ struct FarDesc {
   int32_t n;
   int32_t off[kMaxFar];           // d: the Q^T block (l, l + d)
   const double* plane[kMaxFar];   // L blocks, column-major, stride ms
-  const int* bexp[kMaxFar];       // per block: largest exponent (block_exp)
+  const int2* bexp[kMaxFar];      // per block: block_exp
 };
 constexpr size_t kFarDescOffset = 512;   // byte offset inside the 4 KB header
 
@@ -65,7 +65,7 @@ struct Layout {
   // per-level residual sums, the scales, queue counter + per-level completion
   // counters
   size_t off_fsum, off_fver;
-  size_t off_bexp;       // per plane and level: largest exponent of the block (block_exp)
+  size_t off_bexp;       // per plane and level: exponents of the block (block_exp, int2)
   // low-precision storage (dtype MC_F32 / MC_BF16)
   int lp;                // 0: none, 1: FP32, 2: BF16
   int64_t lp_bs;         // elements per stored block of the A/B planes
@@ -75,9 +75,11 @@ struct Layout {
 
 Layout make_layout(const mc_desc& d);
 
-// block_exp of a block: the largest exponent field of its entries, sign bit
-// included (fixed_ok in fixed_dev.cuh decides what it allows); per plane and
-// level, zero before set-up.
+// block_exp of a block: .x the largest exponent field of its entries, sign bit
+// included; .y 4096 - the smallest one of a nonzero entry in the low half and
+// 4096 - the smallest over the rows of a row's largest one in the upper half (0: as
+// the low half).  What they allow: fixed_safe in fixed_dev.cuh.  Per plane and level,
+// zero before set-up.
 
 // Arguments of one half-sweep (Algorithm 2, step 1+2 or step 3).
 struct PhaseArgs {
@@ -110,9 +112,9 @@ struct FusedArgs {
   const double* A;       // TLO / WLO plane
   const double* B;       // TUP / WUP plane
   const double* C;       // NINV plane (inverse mode)
-  const int* eA;         // block_exp of A, B, C per level
-  const int* eB;
-  const int* eC;
+  const int2* eA;        // block_exp of A, B, C per level
+  const int2* eB;
+  const int2* eC;
   const double* x_in;    // z_0 (read by the first half-sweep only)
   double* W;             // z_1 .. z_{K-1}, in place
   double* Z;             // z_K
@@ -221,15 +223,18 @@ struct ResidArgs {
 // Launchers (return cudaGetLastError()).
 // bexp: block_exp of all planes (L per plane).
 cudaError_t launch_layout(const double* dn, const double* loc, const double* up, double* planes,
-                          int* bexp, const Layout& lay, cudaStream_t s);
+                          int2* bexp, const Layout& lay, cudaStream_t s);
 // Q^T diagonal d into a plane: plane[l] = diag[l + d] (row-major Q block =
 // column-major Q^T block), zero where l + d is outside [0, L).
-cudaError_t launch_layout_diag(const double* diag, int d, double* plane, int* bexp,
+cudaError_t launch_layout_diag(const double* diag, int d, double* plane, int2* bexp,
                                const Layout& lay, cudaStream_t s);
-cudaError_t launch_factor(double* planes, int* bexp, const Layout& lay, Header* hdr, int coupled,
+cudaError_t launch_factor(double* planes, int2* bexp, const Layout& lay, Header* hdr, int coupled,
                           int num_sms, cudaStream_t s);
 // block_exp of TLO and TUP (blocks that did not come through launch_layout).
-cudaError_t launch_block_exp(const double* planes, int* bexp, const Layout& lay, cudaStream_t s);
+cudaError_t launch_block_exp(const double* planes, int2* bexp, const Layout& lay, cudaStream_t s);
+// The rows' part of block_exp of the sweeps' planes (after launch_factor).
+cudaError_t launch_weak_rows(const double* planes, int2* bexp, const Layout& lay, int coupled,
+                             cudaStream_t s);
 cudaError_t launch_phase(const PhaseArgs& a, int coupled, int n_blocks, cudaStream_t s);
 // Block Gauss-Seidel step: one warp walks the levels in order (z_{l-1} fresh,
 // x_{l+1} old); e^T z into hdr->stats[0].

@@ -12,8 +12,8 @@
 // The multiply-adds are shared between the FP64 pipe and the integer pipes
 // (fixed_dev.cuh), which moves the bound from the FP64 pipe (98 % busy, 74 % of
 // the HBM copy rate) to HBM.  64 sweeps with residual units: L = 32768, m = 64
-// 41.8 -> 29.4 ms (4.98 -> 7.1 TB/s streamed, FP64 pipe 87 %, ALU 40 %); 32
-// coupled sweeps, L = 5001, m = 100, 7.32 -> 5.63 ms; 16 sweeps of 4096 paired
+// 41.8 -> 29.5 ms (4.98 -> 7.1 TB/s streamed); 32 coupled sweeps, L = 5001,
+// m = 100, 7.32 -> 5.47 ms; 16 sweeps of 4096 paired
 // levels of 256, 19.2 -> 12.7 ms (one warp per level with 8 rows a lane: 21.2);
 // block Hessenberg, L = 4096, 64 sweeps, 11.9 -> 8.0 ms (with four of eight
 // entries on the integer pipes 8.3, L = 32768 unchanged).
@@ -64,19 +64,16 @@ __device__ __forceinline__ void team_sync(int bar) {
 
 // acc[r] += sum over columns [j0b, j1) of M(row0 + lane + 32 r, j) v_j.  MC:
 // the block size when it fills the team's rows (no bounds checks), else 0.
-// b0 = etot = largest exponent of the block + of the vector.
+// etot = largest exponent of the block + of the vector.
 template <int RW, int MC>
 __device__ __forceinline__ void rows_mix(double (&acc)[RW], const double* __restrict__ M,
                                          const double* v, const uint64_t* xv, int etot, int j0b,
-                                         int j1, int m_, int row0, int lane, bool& bad) {
+                                         int j1, int m_, int row0, int lane) {
   constexpr int U = TeamTune<RW>::U, T = U * RW, N8 = MC ? 3 : 4;
   const int m = MC ? MC : m_;
-  uint32_t fa[RW][4], seen[RW];
+  uint32_t fa[RW][4];
 #pragma unroll
-  for (int r = 0; r < RW; ++r) {
-    fa[r][0] = fa[r][1] = fa[r][2] = fa[r][3] = 0u;
-    seen[r] = 0u;
-  }
+  for (int r = 0; r < RW; ++r) fa[r][0] = fa[r][1] = fa[r][2] = fa[r][3] = 0u;
   const double* p = M + (size_t)j0b * m + row0 + lane;
 #pragma unroll 1
   for (int j0 = j0b; j0 < j1; j0 += U, p += (size_t)U * m) {
@@ -101,15 +98,17 @@ __device__ __forceinline__ void rows_mix(double (&acc)[RW], const double* __rest
 #pragma unroll
         for (int r = 0; r < RW; ++r) {
           if (fixed_slot((q + h) * RW + r, T, N8))
-            fixed_fma(fa[r], seen[r], t[q + h][r], xl, xh, b);
+            fixed_fma(fa[r], t[q + h][r], xl, xh, b);
           else
             acc[r] = fma(t[q + h][r], vj, acc[r]);
         }
       }
     }
   }
+  // truncations of up to m terms: below 2^-57 of the row's whole sum (fixed_safe)
+  bool bad = false;
 #pragma unroll
-  for (int r = 0; r < RW; ++r) acc[r] += fixed_value(fa[r], seen[r], etot, bad);
+  for (int r = 0; r < RW; ++r) acc[r] += fixed_value(fa[r], etot, bad);
 }
 
 // As rows_mix on the FP64 pipe alone.
@@ -142,53 +141,47 @@ __device__ __forceinline__ void rows_f64(double (&acc)[RW], const double* __rest
   }
 }
 
-// acc += M v on both pipes where the block's and the vector's exponents allow
-// it, on the FP64 pipe alone otherwise or when a row's sum left the window
-// (decided per warp from the data alone), and for m <= 16: joining the two sums
-// costs more than the few columns save.
+// acc += M v on both pipes where the exponents of block and vector allow it, else
+// and for m <= 16 on the FP64 pipe alone: joining the two sums costs more than the
+// few columns save.
 template <int RW, int MC>
 __device__ __forceinline__ void rows_product(double (&acc)[RW], const double* M, const double* v,
-                                             const uint64_t* xv, int eb, int ev, int j0, int j1,
+                                             const uint64_t* xv, int2 eb, int ev, int j0, int j1,
                                              int m, int row0, int lane) {
-  bool plain = m <= 16 || !fixed_ok(eb) || !fixed_ok(ev);
-  if (!plain) {
-    double old[RW];
-#pragma unroll
-    for (int r = 0; r < RW; ++r) old[r] = acc[r];
-    bool bad = false;
-    rows_mix<RW, MC>(acc, M, v, xv, eb + ev, j0, j1, m, row0, lane, bad);
-    plain = __any_sync(kFull, bad);
-    if (plain) {
-#pragma unroll
-      for (int r = 0; r < RW; ++r) acc[r] = old[r];
-    }
-  }
-  if (plain) rows_f64<RW, MC>(acc, M, v, j0, j1, m, row0, lane);
+  if (m > 16 && fixed_safe(eb, ev))
+    rows_mix<RW, MC>(acc, M, v, xv, eb.x + (ev & 0xfff), j0, j1, m, row0, lane);
+  else
+    rows_f64<RW, MC>(acc, M, v, j0, j1, m, row0, lane);
 }
 
-// Largest exponent over the team's warps.
+// Exponents over the team's warps.
 template <int TW>
-__device__ __forceinline__ int team_max(const int* e) {
+__device__ __forceinline__ int team_exp(const int* e) {
   int v = e[0];
 #pragma unroll
-  for (int i = 1; i < TW; ++i) v = max(v, e[i]);
+  for (int i = 1; i < TW; ++i) v = exp_join(v, e[i]);
   return v;
 }
 
-// Rows first, first + stride, ... of one vector into a staged slot.
-template <int TW, int RW>
-__device__ __forceinline__ void stage_rows(double* v, uint64_t* x, int* emax,
-                                           const double (&y)[RW], int first, int stride, int w,
-                                           int lane) {
-  unsigned e = 0u;
+// Rows first, first + stride, ... of one vector of m rows into a staged slot.
+template <int RW>
+__device__ __forceinline__ void stage_rows(double* v, uint64_t* x, int* exps,
+                                           const double (&y)[RW], int m, int first, int stride,
+                                           int w, int lane) {
+  unsigned most = 0u, low = 0u;
+  bool zero = false;
 #pragma unroll
   for (int i = 0; i < RW; ++i) {
     v[first + stride * i] = y[i];
     x[first + stride * i] = fixed_entry(y[i]);
-    e = max(e, (unsigned)__double2hiint(y[i]) >> 20);
+    most = max(most, exp_field(y[i]));
+    low = max(low, exp_low(y[i]));
+    zero = zero || (first + stride * i < m && is_zero(y[i]));
   }
-  e = __reduce_max_sync(kFull, e);
-  if (lane == 0) emax[w] = (int)e;
+  most = __reduce_max_sync(kFull, most);
+  low = __reduce_max_sync(kFull, low);
+  zero = __any_sync(kFull, zero);
+  if (lane == 0) exps[w] = exp_pack(most, low, zero);
 }
 
 // Sum of the warps' values in warp order (valid on the team's first warp).
@@ -205,14 +198,14 @@ __device__ __forceinline__ double team_total(double t, double* part, int w, int 
 
 // Shared memory of one team: a ring of two staged products (a warp that writes
 // slot i + 1 has passed the barrier of slot i, so every warp of the team has
-// finished reading slot i - 1), the largest exponents found by each warp, the
+// finished reading slot i - 1), the exponents found by each warp, the
 // units to come, and partial level sums.
 // The staged vectors are read in 16-byte pairs, so every team's slots start on a
 // 16-byte boundary.
 template <int TW, int RW>
 struct alignas(16) TeamShared {
   TeamSlot<32 * RW * TW> slot[2];
-  int emax[2][2][TW];
+  int exps[2][2][TW];
   unsigned long long next[2];
   double part[TW];
 };

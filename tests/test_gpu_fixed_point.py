@@ -114,3 +114,161 @@ def test_not_a_number_propagates(m):
     with pytest.raises(mc.McError):
         ch.sync()
     assert torch.isnan(y).any()
+
+
+# ---- chains through global memory, in every team form ----------------------------------------
+
+def rates(L, m, seed, ratio=0.8, line=False):
+    """Generator blocks on the GPU: random rates, or (line) phases that only exchange with their neighbours, weakly
+    upwards, and levels that keep the phase."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    r = lambda: (torch.rand(L, m, m, generator=g, device="cuda", dtype=torch.float64) * 0.9 + 0.1)  # noqa: E731
+    up, dn, loc = r(), r(), r()
+    if line:
+        i = torch.arange(m, device="cuda")
+        near = (i[:, None] - i[None, :]).abs()
+        up, dn = up * (near == 0), dn * (near == 0)
+        loc = loc * (near == 1) * torch.where(i[None, :] > i[:, None], 0.1, 1.0)
+    return dn / ratio, loc, up
+
+
+def close_rows(dn, loc, up):
+    up[-1] = 0.0
+    dn[0] = 0.0
+    loc.diagonal(dim1=1, dim2=2).zero_()
+    loc.diagonal(dim1=1, dim2=2).sub_(dn.sum(2) + loc.sum(2) + up.sum(2))
+    return dn, loc, up
+
+
+def check_levels(ch, x, coupled, levels, stair=1):
+    """check() on some levels of a long chain: the sweep's own e^T z scales them, and the result sums to 1."""
+    L, m = ch.L, ch.m
+    st = torch.zeros(3, dtype=torch.float64, device="cuda")
+    got = ch.sweep(torch.from_numpy(x).cuda(), nsweeps=1, stats=st).cpu().numpy().reshape(L, m)
+    ch.sync()
+    s = float(st[0])
+    assert abs(got.sum() - 1.0) <= (L * m / 64 + 32) * U * np.abs(got).sum()
+    x = x.reshape(L, m).astype(np.longdouble)
+
+    def level(l, y, f):
+        names = ("wlo", "wup") if coupled else ("tlo", "tup", "ninv")
+        ops = [f(ch.export(n, l, 1).cpu().numpy()[0].T.astype(np.longdouble)) for n in names]
+        g = sum((op @ y(l + d) for op, d in zip(ops, (-1, 1)) if 0 <= l + d < L), np.zeros(m, np.longdouble))
+        return g if coupled else ops[2] @ g
+
+    for l in levels:
+        for f in (lambda a: a, np.abs):
+            first = lambda k: f(x[k])  # noqa: E731
+            z = level(l, first if l % 2 == stair - 1 else lambda k: level(k, first, f), f)
+            if f is np.abs:
+                mag = z
+            else:
+                ref = z
+        tol = (6 * m + ch.N / 64 + 32) * U * (mag / abs(s) + 2 * np.abs(ref / s))
+        err = np.abs(got[l] - ref / s)
+        assert np.all(err <= tol + 5e-324), (l, float((err / (tol + 1e-320)).max()))
+
+
+# teams of one to eight warps with one or two rows a lane, with and without bounds checks: shorter and
+# longer than half as many levels again as a half-sweep has teams
+TEAMS = [(4000, 24), (2200, 32), (2200, 33), (600, 64), (40, 100), (30, 128), (24, 150), (20, 192), (16, 224), (16, 256),
+         (11000, 40), (11000, 64), (5500, 72), (5500, 128), (3700, 136), (3700, 192), (2750, 200), (2750, 256)]
+
+
+def sample(L, n=10, seed=1):
+    return sorted({0, 1, L - 2, L - 1, *(int(v) for v in np.random.default_rng(seed).integers(0, L, n))})
+
+
+@pytest.mark.parametrize("apply,stair", [("inverse", 1), ("coupled", 2)])
+@pytest.mark.parametrize("L,m", TEAMS)
+def test_every_team(L, m, apply, stair):
+    ch = mc.Chain(*close_rows(*rates(L, m, m)), apply=apply, stair=stair)
+    x = start(L, m)
+    assert ch.profile(torch.from_numpy(x).cuda())[1]["launches"] == 3     # sweeps, scale, normalisation
+    check_levels(ch, x, apply == "coupled", sample(L), stair)
+
+
+KINDS = ["negative", "weak_rows", "zero_rows", "small_block", "wide_vector", "wide_both", "small_level", "zeros", "line", "line_zeros"]
+
+
+@pytest.mark.parametrize("apply", ["inverse", "coupled"])
+@pytest.mark.parametrize("L,m", [(4000, 24), (2200, 32), (2200, 33), (600, 64), (40, 100), (11000, 64), (5500, 100)])
+@pytest.mark.parametrize("kind", KINDS)
+def test_outside_the_window_in_every_form(kind, L, m, apply):
+    dn, loc, up = rates(L, m, 7, line=kind.startswith("line"))
+    x = start(L, m).reshape(L, m)
+    k = L // 2
+    if kind == "weak_rows":           # rows of Q^T below the block's largest entry by more than the window
+        up[:, :, : m // 3] *= 2.0 ** -75
+    elif kind == "zero_rows":
+        dn[:, :, : m // 3] = 0.0
+        up[:, :, : m // 3] = 0.0
+    elif kind == "small_block":
+        up[k] *= 1e-270
+    elif kind == "wide_vector":       # rows keep a large entry, but it may meet a small one
+        x[:, ::3] *= 2.0 ** -60
+    elif kind == "wide_both":         # block and vector together beyond the window, neither alone
+        dn[:, :, : m // 3] *= 2.0 ** -30
+        up[:, :, : m // 3] *= 2.0 ** -30
+        x[:, 1::2] *= 2.0 ** -30
+    elif kind == "small_level":
+        x[k:] *= 1e-290
+    elif kind in ("zeros", "line_zeros"):
+        x[:, m // 2:] = 0.0
+        x[k] = 0.0
+    elif kind == "line":
+        x *= 0.1 ** np.arange(m)
+    close_rows(dn, loc, up)
+    if kind == "negative":
+        up[k, 2, 4] = -0.25
+    ch = mc.Chain(dn, loc, up, apply=apply)
+    x = np.ascontiguousarray(x.reshape(-1) / x.sum())
+    assert ch.profile(torch.from_numpy(x).cuda())[1]["launches"] == 3
+    check_levels(ch, x, apply == "coupled", sorted({*sample(L, 4), k - 1, k, k + 1}))
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("L,m", [(4000, 24), (600, 64), (40, 100), (11000, 64)])
+def test_non_finite_entries_propagate(L, m, value):
+    ch = mc.Chain(*close_rows(*rates(L, m, 3)))
+    x = start(L, m)
+    x[m + 3] = value         # level 1: read by the first half-sweep
+    y = ch.sweep(torch.from_numpy(x).cuda(), nsweeps=1)
+    with pytest.raises(mc.McError):
+        ch.sync()
+    assert not torch.isfinite(y).all()
+
+
+@pytest.mark.parametrize("kind", ["weak_rows", "line", "transient"])
+@pytest.mark.parametrize("apply", ["inverse", "coupled"])
+def test_banded_and_served_chains_outside_the_window(kind, apply):
+    """192 sweeps by the server's teams against a chain of its own and, inverse, the far terms of a banded chain against
+    the same chain with its near blocks only (the further ones vanish beside them): 6 m roundings a sweep."""
+    L, m, K, n = 600, 40, 64, 3
+    dn, loc, up = rates(L, m, 9, line=kind == "line")
+    if kind == "weak_rows":
+        up[:, :, : m // 3] *= 2.0 ** -75
+    elif kind == "transient":         # the second half of the phases is left and never entered
+        for t in (dn, loc, up):
+            t[:, : m // 2, m // 2:] = 0.0
+    dn, loc, up = close_rows(dn, loc, up)
+
+    def sweeps(ch):
+        x = torch.full((L * m,), 1.0 / (L * m), dtype=torch.float64, device="cuda")
+        for _ in range(n):
+            x = ch.sweep(x, nsweeps=K)
+        ch.sync()
+        return x.cpu().numpy()
+
+    pi = sweeps(mc.Chain(dn, loc, up, apply=apply))
+    srv = mc.Server(1 << 30, dtype="f64", apply=apply, check_every=K, tol=0.0, maxit=n * K, autotune=False)
+    assert srv.submit(0, *(t.cpu().numpy() for t in (dn, loc, up)))
+    (_, ps, _, _), = srv.run_until_idle()
+    assert np.abs(ps - pi).sum() <= n * K * 6 * m * U
+    srv.close()
+    if apply == "inverse":
+        far = torch.zeros_like(dn)
+        far[:L - 2] = 2.0 ** -80 * dn[:L - 2]          # its rows lie far below those of the near blocks
+        pb = sweeps(mc.Chain.banded({-1: dn, 0: loc, 1: up, 2: far}))
+        assert np.abs(pb - pi).sum() <= n * K * 6 * m * U
