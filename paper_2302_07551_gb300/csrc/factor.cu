@@ -533,8 +533,8 @@ __device__ __forceinline__ Exps coupled_tile(CoupledShared<TILE>& sh, const doub
       double v = acc[a][b];
       if (b < RF) {
         bool bad = false;
-        v = fixed_value(fa[a][b < RF ? b : 0], etot, bad);
-        if (bad && seen[a][b < RF ? b : 0] != 0u) {
+        v = fixed_value(fa[a][b < RF ? b : 0], seen[a][b < RF ? b : 0], etot, bad);
+        if (bad) {
           v = 0.0;
           for (int k = 0; k < m; ++k) v = fma(Nl[(size_t)k * m + i], T[(size_t)j * m + k], v);
         }

@@ -106,9 +106,8 @@ __device__ __forceinline__ void rows_mix(double (&acc)[RW], const double* __rest
     }
   }
   // truncations of up to m terms: below 2^-57 of the row's whole sum (fixed_safe)
-  bool bad = false;
 #pragma unroll
-  for (int r = 0; r < RW; ++r) acc[r] += fixed_value(fa[r], etot, bad);
+  for (int r = 0; r < RW; ++r) acc[r] += fixed_part(fa[r], etot);
 }
 
 // As rows_mix on the FP64 pipe alone.
