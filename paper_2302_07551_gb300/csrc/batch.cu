@@ -9,6 +9,7 @@
 #include "batch.cuh"
 #include "lowprec_dev.cuh"
 #include "lpteam_dev.cuh"
+#include "resident_dev.cuh"
 #include "sweep_dev.cuh"
 #include "team_dev.cuh"
 #include "wave_dev.cuh"
@@ -71,11 +72,109 @@ __device__ __forceinline__ BUnit unit_of(const BTable* t, unsigned long long q, 
   return u;
 }
 
-// K FP64 sweeps of the queue-path requests (m <= 16, b_path) in one launch.  Per
+// One level (m <= 32, lane = row) with every sum in the order of the resident kernels:
+// S column groups, column j in group j % S, the terms of A and B in turn; the groups'
+// sums added by a tree (rows shared by lanes) or in order (by warps); the level's sum
+// row by row.
+template <int S, bool TREE, bool COUPLED>
+__device__ __forceinline__ double level_grouped(const BReq* Q, const double* src, double* dst,
+                                                int64_t l, double* slice, int lane,
+                                                bool want_sum) {
+  static_assert(S == 1 || S == 2 || S == 4, "");
+  constexpr int U = 8;
+  const int m = Q->m;
+  const bool has_lo = l > 0, has_up = l < Q->L - 1, in = lane < m;
+  double *lo = slice, *up = slice + 32, *g = slice + 64;
+  lo[lane] = has_lo && in ? __ldcg(src + (l - 1) * m + lane) : 0.0;
+  up[lane] = has_up && in ? __ldcg(src + (l + 1) * m + lane) : 0.0;
+  __syncwarp();
+  auto total = [](const double (&p)[S]) {
+    if constexpr (S == 1)
+      return p[0];
+    else if constexpr (S == 2)
+      return p[0] + p[1];
+    else if constexpr (TREE)
+      return (p[0] + p[1]) + (p[2] + p[3]);
+    else
+      return ((p[0] + p[1]) + p[2]) + p[3];
+  };
+  double p[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) p[s] = 0.0;
+  const double* A = Q->A + (size_t)l * Q->ms + lane;
+  const double* B = Q->B + (size_t)l * Q->ms + lane;
+  for (int j0 = 0; j0 < m; j0 += U) {
+    double a[U], b[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const bool ok = in && j0 + q < m;
+      a[q] = ok && has_lo ? ld_stream(A + (size_t)(j0 + q) * m) : 0.0;
+      b[q] = ok && has_up ? ld_stream(B + (size_t)(j0 + q) * m) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      p[q % S] = fma(a[q], lo[j0 + q], p[q % S]);
+      p[q % S] = fma(b[q], up[j0 + q], p[q % S]);
+    }
+  }
+  double v = total(p);
+  if constexpr (!COUPLED) {
+    g[lane] = v;
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < S; ++s) p[s] = 0.0;
+    const double* C = Q->C + (size_t)l * Q->ms + lane;
+    for (int j0 = 0; j0 < m; j0 += 2 * U) {
+      double c[2 * U];
+#pragma unroll
+      for (int q = 0; q < 2 * U; ++q)
+        c[q] = in && j0 + q < m ? ld_stream(C + (size_t)(j0 + q) * m) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 2 * U; ++q) p[q % S] = fma(c[q], g[j0 + q], p[q % S]);
+    }
+    v = total(p);
+  }
+  if (in) dst[l * m + lane] = v;
+  double sum = 0.0;
+  if (want_sum) {
+    __syncwarp();   // lo has been read
+    lo[lane] = v;
+    __syncwarp();
+    if (lane == 0)
+      for (int j = 0; j < m; ++j) sum += lo[j];
+  }
+  __syncwarp();   // the slice is rewritten for the next level
+  return sum;
+}
+
+// Column groups of level l of a request in the resident order.
+__device__ __forceinline__ int level_groups(const BReq* Q, int64_t l) {
+  if (Q->res_s) return Q->res_s;
+  const int C = Q->res_c, L = (int)Q->L, base = L / C, rem = L % C, long_end = (base + 1) * rem;
+  const int r = l < long_end ? (int)l / (base + 1) : rem + ((int)l - long_end) / base;
+  const int l0 = res::range_begin(L, C, r), n = res::range_begin(L, C, r + 1) - l0;
+  const int t0 = (l0 ^ (int)l) & 1;   // the CTA's first level of this half-sweep
+  return res::flat_split((n - t0 + 1) / 2 * Q->m);
+}
+
+template <bool COUPLED>
+__device__ __forceinline__ double level_resident(const BReq* Q, const double* src, double* dst,
+                                                 int64_t l, double* slice, int lane,
+                                                 bool want_sum) {
+  switch (level_groups(Q, l)) {
+    case 1: return level_grouped<1, false, COUPLED>(Q, src, dst, l, slice, lane, want_sum);
+    case 2: return level_grouped<2, false, COUPLED>(Q, src, dst, l, slice, lane, want_sum);
+    default:
+      return Q->res_s ? level_grouped<4, true, COUPLED>(Q, src, dst, l, slice, lane, want_sum)
+                      : level_grouped<4, false, COUPLED>(Q, src, dst, l, slice, lane, want_sum);
+  }
+}
+
+// K FP64 sweeps of the queue-path requests (b_path: m <= 16; build_table: m <= 32) in one launch.  Per
 // request: sweep 0 reads x, sweeps 0..K-2 write xb in place, sweep K-1 writes z (so
 // xb keeps the previous sweep for the step error).
 template <bool COUPLED>
-__global__ void __launch_bounds__(256) k_b_sweeps(const BTable* __restrict__ t, int K,
+__global__ void __launch_bounds__(256, 4) k_b_sweeps(const BTable* __restrict__ t, int K,
                                                   unsigned long long* claim, BOut* out) {
   extern __shared__ double vsh[];
   const int lane = threadIdx.x & 31;
@@ -103,9 +202,11 @@ __global__ void __launch_bounds__(256) k_b_sweeps(const BTable* __restrict__ t, 
     const bool want = u.k >= K - 2;   // e^T z of the last two sweeps only
     for (int i = 0; i < u.n; ++i) {
       const int64_t l = u.l + 2 * i;
-      const double ls = level_sweep2<1, COUPLED, true, true>(
-          Q->A, Q->B, Q->C, src, src, dst, l, Q->L, Q->m, Q->ms, slice, lane, 1.0, nullptr,
-          nullptr, nullptr, want);
+      const double ls =
+          Q->res_c ? level_resident<COUPLED>(Q, src, dst, l, slice, lane, want)
+                   : level_sweep2<1, COUPLED, true, true>(Q->A, Q->B, Q->C, src, src, dst, l, Q->L,
+                                                          Q->m, Q->ms, slice, lane, 1.0, nullptr,
+                                                          nullptr, nullptr, want);
       if (want && lane == 0) Q->lsum2[(u.k & 1) * Q->L + l] = ls;
     }
     publish_levels(Q->ver, u.l, 2, u.n, base + (int)u.k + 1, lane);
@@ -578,7 +679,7 @@ cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out,
 }
 
 int b_path(const Layout& y, int coupled, int num_sms) {
-  if (resident_batch_fits(y, coupled)) return kPathResident;
+  if (resident_batch_group(y, coupled) >= 0) return kPathResident;
   // FP64, m <= 16: a chain with a level for every warp in flight is bound by the
   // fence and claim of each unit, which units of 4 levels share (six of 16384 x 16,
   // coupled, a chunk of 64 sweeps: teams 12.3 ms, queue 11.0); shorter ones by the

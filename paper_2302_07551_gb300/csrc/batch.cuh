@@ -60,7 +60,9 @@ struct BReq {
   int32_t m, ms, R, p1;  // p1: 0-based parity of the diagonal-only rows
   int32_t G, path;       // levels per unit of this request (the table's G scaled by size
                          // class); kPathQueue, ...
-  int32_t vbase, pad2;   // FP64 team path: sweeps that the counters have seen
+  int32_t vbase;         // FP64 team path: sweeps that the counters have seen
+  int16_t res_c, res_s;  // FP64 queue: CTAs of the cluster whose order of sums applies (0:
+                         // columns in order) and its column groups (0: by the level)
   int64_t lp_bs, lp_cbs;
 };
 
@@ -76,8 +78,8 @@ __host__ __device__ inline int class_group(int G, int m) {
   return g > 16 ? 16 : g;
 }
 
-// How a request's sweeps run, by its own size alone (so that its iterates do not
-// depend on the batch):
+// How a request's sweeps run.  Its arithmetic follows from its own size alone (so that
+// its iterates do not depend on the batch):
 //   kPathQueue: one warp per unit of G levels, all such requests in shared launches
 //     by size class (k_b_sweeps: FP64 blocks of up to 16 rows, long chains; k_b_sweeps_lp);
 //   kPathTeam: a team of warps per level, all such requests of a size class in one
@@ -85,14 +87,33 @@ __host__ __device__ inline int class_group(int G, int m) {
 //     of blocks of more than 32 rows (lpteam_dev.cuh);
 //   kPathResident: blocks of up to 32 rows that fit one cluster's shared memory, one
 //     cluster per request (resident_dev.cuh).
+// FP64 requests of the resident path run on the queue, with the sums in the resident
+// order (res_order), while so many are active that the clusters would take longer.
 // The launches of the three paths run side by side; the host deals out CTAs to
 // them with the table.  Eight requests of 131 KB to 17 MB
 // (BF16 coupled, m = 16 to 128): a chunk of 64 sweeps 2.70 -> 0.99 ms with all of them
 // running, 1.32 -> 0.24 ms with the last two small ones.
 enum { kPathQueue = 0, kPathTeam = 1, kPathResident = 2 };
-// One bit per path and size class (class 0 but for teams).
-inline int path_bit(int path, int cls) { return 1 << (4 * path + cls); }
-constexpr int kResidentClusters = 8;   // clusters of 16 in a launch
+// One bit per path and size class (queue: 0) or resident group.
+inline int path_bit(int path, int cls) { return 1 << (5 * path + cls); }
+
+// Resident requests by group, a launch each.  A cluster alone leaves most of its SMs'
+// time to latency, so a batch of many small low-precision requests needs several
+// clusters on the same SMs: a group is a number of CTAs that share an SM, given by
+// their shared memory and by the registers of the kernel (blocks of up to 16 rows hold
+// their operators in registers, wider ones, `wide`, do not).  A chunk of 64 sweeps,
+// one CTA an SM -> shared (the queue): 250 of 128 x 16, BF16 coupled, 2.97 -> 1.61 ms
+// (2.15); 200 of 90 x 24, FP32 inverse, 7.3 -> 1.76 (2.81); 100 of 400 x 20, BF16
+// coupled, 3.18 -> 1.12 (3.97).  What fits an SM only once is as before: below the
+// queue's rate where 60 or more of FP32 or inverse mode with m > 16 run at once (100
+// of 200 x 28, FP32 inverse: 4.1, queue 2.7), far above it where few do (one of
+// 300 x 32: 0.20, queue 1.27).
+constexpr int kResGroups = 5;
+constexpr int kResidentSlots = 8;      // sets of 16 SMs given to clusters
+__host__ __device__ constexpr int group_share(int group) {
+  return group == 0 ? 2 : group == 2 ? 4 : group == 3 ? 2 : 1;
+}
+__host__ __device__ constexpr bool group_wide(int group) { return group >= 2; }
 
 struct BTable {
   int32_t n;            // active requests, ordered by size class
@@ -100,17 +121,19 @@ struct BTable {
   int32_t epoch;        // completion-counter base of this chunk
   int32_t G;            // levels per unit of the fused sweep launches (1, 2 or 4), scaled
                         // per request by class_group
-  int32_t res_n;        // resident requests, and the clusters that take them
-  int32_t res_clusters;
+  int32_t res_end[kResGroups];        // resident requests of the groups up to this one
+  int32_t res_clusters[kResGroups];   // and the clusters that take a group's
   int32_t team_ctas[kClasses];   // CTAs of the team launch of a size class
-  unsigned long long claim[kClasses];   // queue counters of one chunk's buckets (0 in t_host)
-  int64_t off_h1[kMaxReq + 1];   // prefix counts of half-sweep-1 units (groups of G levels)
+  // (the counters on lines of their own: next to the offsets that every unit reads a
+  // chunk of three chains of 6000 levels took 1.48 ms instead of 1.42)
+  alignas(128) unsigned long long claim[kClasses];   // queue counters of one chunk's buckets (0 in t_host)
+  alignas(128) int64_t off_h1[kMaxReq + 1];   // prefix counts of half-sweep-1 units (groups of G levels)
   int64_t off_h2[kMaxReq + 1];   // prefix counts of half-sweep-2 units
   int64_t off_lv[kMaxReq + 1];   // prefix counts of all levels
-  unsigned long long team_claim[kClasses];   // queue counters of the team launches
-  int64_t off_t1[kMaxReq + 1];   // prefix counts of the team path's levels by half-sweep
+  alignas(128) unsigned long long team_claim[kClasses];   // queue counters of the team launches
+  alignas(128) int64_t off_t1[kMaxReq + 1];   // prefix counts of the team path's levels by half-sweep
   int64_t off_t2[kMaxReq + 1];
-  int32_t res[kMaxReq];          // table positions of the resident requests
+  int32_t res[kMaxReq];          // table positions of the resident requests, by group
   BReq r[kMaxReq];
 };
 
@@ -175,11 +198,12 @@ cudaError_t b_sweeps(const BTable* t, unsigned long long* claim, BOut* out, int 
 // The FP64 team requests' sweeps, a launch per size class on b0, b[0..2].
 cudaError_t b_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
                    int coupled, int K, int num_sms, cudaStream_t b0, const cudaStream_t* b);
-// resident.cu: whether a request fits one cluster; the resident requests' launch.
-bool resident_batch_fits(const Layout& lay, int coupled);
-// lp: 0 FP64, 1 FP32, 2 BF16.
-cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int K, BOut* out,
+// resident.cu: the group of a request that fits one cluster, else -1; the launch of
+// a group's requests (lp: 0 FP64, 1 FP32, 2 BF16); res_c and res_s of an FP64 request.
+int resident_batch_group(const Layout& lay, int coupled);
+cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int group, int K, BOut* out,
                                   cudaStream_t s);
+void resident_order(const Layout& lay, int16_t* c, int16_t* s);
 cudaError_t b_lp_finish(const BTable* t, BOut* out, BTune g, cudaStream_t s);
 
 }  // namespace mc

@@ -176,22 +176,37 @@ __host__ __device__ inline int cluster_ctas(int64_t L, int most) {
   return C;
 }
 
-// The resident requests of a batch, one cluster each in turn; the CTAs of a short
-// chain's cluster that have no levels only take part in its barriers.
-template <typename S, bool COUPLED>
-__global__ void __launch_bounds__(kThreads, 1) k_b_resident(const BTable* __restrict__ t, int K,
-                                                         BOut* out) {
+// Dynamic shared memory of this launch: a request whose share does not fit it (none
+// does not: its group follows from its size) is reported and left out.
+__device__ __forceinline__ size_t dyn_smem() {
+  unsigned v;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(v));
+  return v;
+}
+
+// The resident requests of a group of a batch, one cluster each in turn; the CTAs of
+// a short chain's cluster that have no levels only take part in its barriers.
+// GROUP: the first group of this kernel.
+template <typename S, bool COUPLED, int GROUP>
+__global__ void __launch_bounds__(kThreads, group_share(GROUP))
+    k_b_resident(const BTable* __restrict__ t, int group, int K, BOut* out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long two[2];
   cg::cluster_group cl = cg::this_cluster();
   const int most = (int)cl.num_blocks(), cid = (int)blockIdx.x / most;
-  if (cid >= t->res_clusters) return;
-  for (int i = cid; i < t->res_n; i += t->res_clusters) {
+  const int clusters = t->res_clusters[group];
+  if (cid >= clusters) return;
+  const int i1 = t->res_end[group];
+  for (int i = (group > 0 ? t->res_end[group - 1] : 0) + cid; i < i1; i += clusters) {
     const int r = t->res[i];
     const BReq& Q = t->r[r];
     ClusterLink<float> ln;
     ln.status = &out[r].status;
     ln.c = cluster_ctas(Q.L, most);
+    if (carve<S, float, float, COUPLED>((int)((Q.L + ln.c - 1) / ln.c), Q.m).total > dyn_smem()) {
+      atomicCAS(ln.status, 0, (int)MC_ERR_CUDA);
+      continue;   // the whole cluster
+    }
     if ((int)cl.block_rank() < ln.c) {
       Chain<S, float, float> h{};
       h.A = reinterpret_cast<const S*>(Q.lA);
@@ -204,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_b_resident(const BTable* __rest
       h.L = (int)Q.L;
       h.m = Q.m;
       h.par0 = Q.p1;
-      sweeps<S, float, float, COUPLED>(h, K, smem, two, ln);
+      sweeps<S, float, float, COUPLED, group_wide(GROUP)>(h, K, smem, two, ln);
       const int l0 = ln.s.l0, n = ln.s.n;
       for (int e = threadIdx.x; e < n * h.m; e += kThreads)
         Q.d[(int64_t)l0 * h.m + e] = ln.s.x[h.m + e];
@@ -221,19 +236,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_b_resident(const BTable* __rest
 
 // FP64: also the level sums of the last two sweeps, for the batch's reductions.
 template <bool COUPLED>
-__global__ void __launch_bounds__(kThreads, 1) k_b_resident64(const BTable* __restrict__ t, int K,
-                                                              BOut* out) {
+__global__ void __launch_bounds__(kThreads, 1)
+    k_b_resident64(const BTable* __restrict__ t, int group, int K, BOut* out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long two[2];
   cg::cluster_group cl = cg::this_cluster();
   const int most = (int)cl.num_blocks(), cid = (int)blockIdx.x / most;
-  if (cid >= t->res_clusters) return;
-  for (int i = cid; i < t->res_n; i += t->res_clusters) {
+  const int clusters = t->res_clusters[group];
+  if (cid >= clusters) return;
+  const int i1 = t->res_end[group];
+  for (int i = (group > 0 ? t->res_end[group - 1] : 0) + cid; i < i1; i += clusters) {
     const int r = t->res[i];
     const BReq& Q = t->r[r];
     ClusterLink<double> ln;
     ln.status = &out[r].status;
     ln.c = cluster_ctas(Q.L, most);
+    if (carve<double, double, double, COUPLED>((int)((Q.L + ln.c - 1) / ln.c), Q.m).total > dyn_smem()) {
+      atomicCAS(ln.status, 0, (int)MC_ERR_CUDA);
+      continue;   // the whole cluster
+    }
     if ((int)cl.block_rank() < ln.c) {
       Chain<double, double, double> h{};
       h.A = Q.A;
@@ -273,11 +294,24 @@ constexpr size_t kMaxDyn = 227 * 1024 - 1024;   // opt-in limit less the static 
 // Kernels by storage type (FP64, FP32, BF16), apply mode and link.
 using Kernel64 = void (*)(ResidentArgs);
 using KernelLp = void (*)(ResidentLpArgs);
-using KernelBatch = void (*)(const BTable*, int, BOut*);
-KernelBatch kernel_batch(int lp, int coupled) {
+using KernelBatch = void (*)(const BTable*, int, int, BOut*);
+template <int GROUP>
+KernelBatch kernel_batch_lp(int lp, int coupled) {
+  if (lp == 1) return coupled ? k_b_resident<float, true, GROUP> : k_b_resident<float, false, GROUP>;
+  return coupled ? k_b_resident<unsigned short, true, GROUP>
+                 : k_b_resident<unsigned short, false, GROUP>;
+}
+KernelBatch kernel_batch(int lp, int coupled, int group) {
   if (lp == 0) return coupled ? k_b_resident64<true> : k_b_resident64<false>;
-  if (lp == 1) return coupled ? k_b_resident<float, true> : k_b_resident<float, false>;
-  return coupled ? k_b_resident<unsigned short, true> : k_b_resident<unsigned short, false>;
+  return group < 2    ? kernel_batch_lp<0>(lp, coupled)
+         : group == 2 ? kernel_batch_lp<2>(lp, coupled)
+                      : kernel_batch_lp<3>(lp, coupled);
+}
+// Dynamic shared memory of a group's CTAs: an SM's 228 KB by the CTAs that share it,
+// less 1 KB each and the static arrays.
+size_t group_smem(int group) {
+  const int n = group_share(group);
+  return n == 1 ? kMaxDyn : (size_t)(228 / n - 2) * 1024;
 }
 Kernel64 kernel64(int coupled, bool grid) {
   if (grid)
@@ -359,21 +393,25 @@ Limits limits() {
     for (int c = 0; c < 2; ++c) {
       ok = ok && opt_in((const void*)kernel64(c, false), true) &&
            opt_in((const void*)kernel64(c, true), false) &&
-           opt_in((const void*)kernel_batch(0, c), true);
+           opt_in((const void*)kernel_batch(0, c, 1), true);
       for (int lp = 1; lp <= 2; ++lp)
         ok = ok && opt_in((const void*)kernel_lp(lp, c, false), true) &&
              opt_in((const void*)kernel_lp(lp, c, true), false) &&
-             opt_in((const void*)kernel_batch(lp, c), true);
+             opt_in((const void*)kernel_batch(lp, c, 0), true) &&
+             opt_in((const void*)kernel_batch(lp, c, 2), true) &&
+             opt_in((const void*)kernel_batch(lp, c, 3), true);
     }
     if (ok) {
       for (int C = 16; C >= 8 && !l.cluster; C /= 2) {
         bool runs = true;
         for (int c = 0; c < 2; ++c) {
           runs = runs && cluster_runs((const void*)kernel64(c, false), C) &&
-                 cluster_runs((const void*)kernel_batch(0, c), C);
+                 cluster_runs((const void*)kernel_batch(0, c, 1), C);
           for (int lp = 1; lp <= 2; ++lp)
             runs = runs && cluster_runs((const void*)kernel_lp(lp, c, false), C) &&
-                   cluster_runs((const void*)kernel_batch(lp, c), C);
+                   cluster_runs((const void*)kernel_batch(lp, c, 0), C) &&
+                   cluster_runs((const void*)kernel_batch(lp, c, 2), C) &&
+                   cluster_runs((const void*)kernel_batch(lp, c, 3), C);
         }
         if (runs) l.cluster = C;
       }
@@ -433,20 +471,33 @@ cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& y, int cou
   return cudaLaunchKernelEx(&cfg, kernel_lp(y.lp, coupled, grid != 0), a);
 }
 
-bool resident_batch_fits(const Layout& y, int coupled) {
+int resident_batch_group(const Layout& y, int coupled) {
   const int C = cluster_ctas(y.L, limits().cluster);
-  return C > 0 && y.m <= 32 && y.L <= (1 << 20) && smem_bytes(y, coupled, C) <= kMaxDyn;
+  if (C == 0 || y.m > 32 || y.L > (1 << 20)) return -1;
+  const size_t need = smem_bytes(y, coupled, C);
+  if (need > kMaxDyn) return -1;
+  if (y.lp == 0) return 1;
+  int g = y.m > 16 ? 2 : 0;
+  while (need > group_smem(g)) ++g;
+  return g;
 }
 
-cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int K, BOut* out,
+void resident_order(const Layout& y, int16_t* c, int16_t* s) {
+  *c = (int16_t)cluster_ctas(y.L, limits().cluster);
+  const int n_half = (int)(((y.L + *c - 1) / *c + 1) / 2);
+  const Cover v = cover(y.m, n_half);
+  *s = (int16_t)(v.S > 1 ? v.S : is_tiny(y.m, n_half, v) ? 1 : 0);
+}
+
+cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int group, int K, BOut* out,
                                   cudaStream_t s) {
   const int C = limits().cluster;
   if (C == 0) return cudaSuccess;   // no request has this path
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
-  config(cfg, at, false, C, kMaxDyn, s);
-  cfg.gridDim = dim3(C * kResidentClusters);
-  return cudaLaunchKernelEx(&cfg, kernel_batch(lp, coupled), t, K, out);
+  config(cfg, at, false, C, group_smem(group), s);
+  cfg.gridDim = dim3(C * kResidentSlots * group_share(group));
+  return cudaLaunchKernelEx(&cfg, kernel_batch(lp, coupled, group), t, group, K, out);
 }
 
 }  // namespace mc

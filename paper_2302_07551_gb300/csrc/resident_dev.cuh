@@ -92,13 +92,26 @@ __host__ __device__ inline int range_begin(int L, int C, int r) {
 struct Cover {
   int mp, S, gs;   // S = 1: flattened rows; else gs = mp S lanes per level
 };
-__device__ __forceinline__ Cover cover(int m, int n_half) {
+__host__ __device__ inline Cover cover(int m, int n_half) {
   Cover c{1, 1, 1};
   if (m > 16) return c;
   while (c.mp < m) c.mp *= 2;
   while (c.mp * c.S < 32 && c.S < m && n_half * c.mp * c.S * 2 <= kThreads) c.S *= 2;
   c.gs = c.mp * c.S;
   return c;
+}
+
+// Whether the operators fit the threads' registers (sweeps_tiny).
+__host__ __device__ inline bool is_tiny(int m, int n_half, const Cover& c) {
+  return m <= 16 && n_half * c.gs <= kThreads && (m + c.S - 1) / c.S <= 8;
+}
+
+// Column groups of flattened rows of a half-sweep (for_rows): with fewer than 32 rows
+// per sub-partition (each has its own FP64 pipe) the columns are split over warps as
+// well, and the parts of a row added in order.
+__host__ __device__ inline int flat_split(int rows) {
+  const int chunks = (rows + 31) / 32;
+  return chunks * 2 <= 4 ? 4 / chunks : 1;
 }
 
 // sum_j A(i, j) p_j + B(i, j) q_j over this thread's columns, in one chain: a
@@ -131,11 +144,8 @@ template <typename V, typename F, typename G>
 __device__ __forceinline__ void for_rows(const Cover& c, int m, int n_half, V* part, F value,
                                          G store) {
   if (c.S == 1) {
-    // flattened rows; with fewer than 32 per sub-partition (each has its own
-    // FP64 pipe) the columns are split over warps as well
-    constexpr int W = 4;
     const int rows = n_half * m, chunks = (rows + 31) / 32;
-    const int S = chunks * 2 <= W ? W / chunks : 1;
+    const int S = flat_split(rows);
     if (S == 1) {
       for (int t = threadIdx.x; t < rows; t += kThreads) {
         const int u = t / m, i = t - u * m;
@@ -744,8 +754,8 @@ __device__ __forceinline__ void load_plane(T* dst, const T* src, int64_t gs, int
 // K sweeps.  On return z (FP64) / x (low precision) holds the CTA's levels of
 // the result and FP64 x the iterate before the last sweep, halos included.
 // sh: two words of shared memory for the link.  first = false: another run from
-// the iterate in x (halos included), with the operators as they are.
-template <typename T, typename TC, typename V, bool COUPLED, typename Link>
+// the iterate in x (halos included), with the operators as they are.  WIDE: m > 16.
+template <typename T, typename TC, typename V, bool COUPLED, bool WIDE = false, typename Link>
 __device__ __forceinline__ void sweeps(const Chain<T, TC, V>& h, int K, unsigned char* smem,
                                        unsigned long long* sh, Link& ln, bool first = true) {
   const int C = ln.ctas(), r = ln.rank();
@@ -765,7 +775,7 @@ __device__ __forceinline__ void sweeps(const Chain<T, TC, V>& h, int K, unsigned
   const int tid = threadIdx.x;
   const Cover c = cover(m, (nmax + 1) / 2);   // the same in every CTA
   const int cpl = (m + c.S - 1) / c.S;
-  const bool tiny = m <= 16 && ((nmax + 1) / 2) * c.gs <= kThreads && cpl <= 8;
+  const bool tiny = !WIDE && is_tiny(m, (nmax + 1) / 2, c);
   if (first) {
     ln.open(Side<V>{x, z, l0, n, m, h.par0, K, r > 0, r < C - 1},
             r > 0 ? l0 - range_begin(L, C, r - 1) : 0, sh);
@@ -790,7 +800,7 @@ __device__ __forceinline__ void sweeps(const Chain<T, TC, V>& h, int K, unsigned
     for (int e = tid; e < 2 * n; e += kThreads) sc[e] = h.sc[2 * l0 + e];
   }
   ln.ready();
-  if (tiny) {
+  if (!WIDE && tiny) {
     if (cpl <= 1)
       sweeps_tiny<T, TC, V, COUPLED, 1>(h, K, c, ln);
     else if (cpl <= 2)

@@ -38,9 +38,12 @@ struct Req {
   int64_t sweeps;
   double step_prev;
   int path;             // kPathQueue / kPathTeam / kPathResident
+  int group;            // of the resident path
   int64_t vbase;        // sweeps that the completion counters have seen (FP64 teams)
   bool fresh;           // factor status not yet checked
 };
+
+constexpr int kSides = kResGroups + kClasses - 1;
 
 struct Done {
   int64_t tag;
@@ -66,8 +69,8 @@ struct mc_server {
   std::vector<Req*> active;
   std::deque<Done> done;
   cudaStream_t cap;
-  cudaStream_t side[4];             // the short requests' launches run beside the others
-  cudaEvent_t fork[2], join[4];
+  cudaStream_t side[kSides];        // resident groups and team classes run beside the others
+  cudaEvent_t fork[2], join[kSides];
   cudaGraphExec_t gexec;
   BTune g_tune;          // configuration of the captured graph
   int g_chunk;
@@ -235,11 +238,14 @@ int begin_chunk(mc_server* s, int c) {
   return MC_OK;
 }
 
-// The paths and team size classes that the table's requests use.
+// The paths, team size classes and resident groups that the table's requests use.
 int table_paths(const BTable* t) {
   int p = 0;
   for (int i = 0; i < t->n; ++i)
-    p |= path_bit(t->r[i].path, t->r[i].path == kPathTeam ? size_class(t->r[i].m) : 0);
+    if (t->r[i].path != kPathResident)
+      p |= path_bit(t->r[i].path, t->r[i].path == kPathTeam ? size_class(t->r[i].m) : 0);
+  for (int g = 0; g < kResGroups; ++g)
+    if (t->res_end[g] > (g ? t->res_end[g - 1] : 0)) p |= path_bit(kPathResident, g);
   return p;
 }
 
@@ -261,31 +267,36 @@ int enqueue_chunk(mc_server* s, BTune g, int c, cudaStream_t st, cudaEvent_t* ev
   const int kind = s->d.dtype == MC_F64 ? 0 : s->d.dtype == MC_F32 ? 1 : 2;
   const int paths = table_paths(s->t_host);
   const bool queue = paths & path_bit(kPathQueue, 0);
-  const bool on[4] = {(paths & path_bit(kPathResident, 0)) != 0,
-                      (paths & path_bit(kPathTeam, 1)) != 0, (paths & path_bit(kPathTeam, 2)) != 0,
-                      (paths & path_bit(kPathTeam, 3)) != 0};
-  if (on[0] &&
-      (cudaEventRecord(s->fork[0], st) != cudaSuccess ||
-       cudaStreamWaitEvent(s->side[0], s->fork[0], 0) != cudaSuccess ||
-       launch_resident_batch(s->t_dev, kind, coupled, c, s->out_dev, s->side[0]) != cudaSuccess))
-    return MC_ERR_CUDA;
+  bool on[kSides];
+  for (int i = 0; i < kSides; ++i)
+    on[i] = (paths & (i < kResGroups ? path_bit(kPathResident, i)
+                                     : path_bit(kPathTeam, i - kResGroups + 1))) != 0;
+  auto fork = [&](cudaEvent_t e, int i0, int i1) {
+    bool any = false;
+    for (int i = i0; i < i1; ++i) any = any || on[i];
+    if (any && cudaEventRecord(e, st) != cudaSuccess) return false;
+    for (int i = i0; i < i1; ++i)
+      if (on[i] && cudaStreamWaitEvent(s->side[i], e, 0) != cudaSuccess) return false;
+    return true;
+  };
+  if (!fork(s->fork[0], 0, kResGroups)) return MC_ERR_CUDA;
+  for (int i = kResGroups - 1; i >= 0; --i)   // the larger ones first
+    if (on[i] && launch_resident_batch(s->t_dev, kind, coupled, i, c, s->out_dev, s->side[i]) !=
+                     cudaSuccess)
+      return MC_ERR_CUDA;
   if (lp && queue && b_lp_zero(s->t_dev, g, st) != cudaSuccess) return MC_ERR_CUDA;
-  if (on[1] || on[2] || on[3]) {
-    if (cudaEventRecord(s->fork[1], st) != cudaSuccess) return MC_ERR_CUDA;
-    for (int i = 1; i < 4; ++i)
-      if (on[i] && cudaStreamWaitEvent(s->side[i], s->fork[1], 0) != cudaSuccess)
-        return MC_ERR_CUDA;
-  }
+  if (!fork(s->fork[1], kResGroups, kSides)) return MC_ERR_CUDA;
   unsigned long long* team = &s->t_dev->team_claim[0];
   cudaError_t e =
       lp ? b_lp_team(s->t_dev, team, s->out_dev, paths, kind == 2, coupled, c, s->num_sms,
-                     s->side + 1)
-         : b_team(s->t_dev, team, s->out_dev, paths, coupled, c, s->num_sms, st, s->side + 1);
+                     s->side + kResGroups)
+         : b_team(s->t_dev, team, s->out_dev, paths, coupled, c, s->num_sms, st,
+                  s->side + kResGroups);
   if (e == cudaSuccess && queue)
     e = lp ? b_lp_sweeps(s->t_dev, claim, s->out_dev, kind == 2, coupled, c, g, st)
            : b_sweeps(s->t_dev, claim, s->out_dev, coupled, c, g, st);
   if (e != cudaSuccess) return MC_ERR_CUDA;
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < kSides; ++i)
     if (on[i] && (cudaEventRecord(s->join[i], s->side[i]) != cudaSuccess ||
                   cudaStreamWaitEvent(st, s->join[i], 0) != cudaSuccess))
       return MC_ERR_CUDA;
@@ -368,18 +379,33 @@ int check_fresh(mc_server* s) {
   return MC_OK;
 }
 
-// CTAs of the launches that run side by side.  A cluster takes 16 SMs whole; the
-// team launches share the others, two or three CTAs each, in proportion to their levels
-// (no more than one team per level), so that each gets its part at once instead
-// of the first launch filling the GPU for a chunk's time.  No result depends on it.
+// CTAs of the launches that run side by side.  Clusters take 16 SMs whole, a slot that
+// group_share clusters of a group share; the slots go one by one to the group with the
+// most requests in turn.  The team launches share the other SMs, two or three CTAs each,
+// in proportion to their levels (no more than one team per level), so that each gets
+// its part at once instead of the first launch filling the GPU for a chunk's time.  No
+// result depends on it.
 void deal_ctas(const mc_server* s, BTable* t, const int64_t* team_levels) {
   const bool teams = team_levels[0] + team_levels[1] + team_levels[2] + team_levels[3] > 0;
-  const int most = teams ? kResidentClusters / 2 : kResidentClusters;
-  t->res_clusters = t->res_n < most ? t->res_n : most;
+  const int lp = s->d.dtype != MC_F64, per_sm = lp ? 2 : 3;
+  int n[kResGroups], slots[kResGroups] = {}, used = 0;
+  for (int g = 0; g < kResGroups; ++g) n[g] = t->res_end[g] - (g ? t->res_end[g - 1] : 0);
+  for (int left = teams ? kResidentSlots / 2 : kResidentSlots; left > 0; --left) {
+    int best = -1;
+    double turns = 1.0;   // requests per cluster: no group needs more clusters than requests
+    for (int g = 0; g < kResGroups; ++g) {
+      const double r = n[g] == 0 ? 0.0 : slots[g] ? (double)n[g] / (slots[g] * group_share(g)) : 1e9;
+      if (r > turns) best = g, turns = r;
+    }
+    if (best < 0) break;
+    ++slots[best];
+    ++used;
+  }
+  for (int g = 0; g < kResGroups; ++g)
+    t->res_clusters[g] = n[g] < slots[g] * group_share(g) ? n[g] : slots[g] * group_share(g);
   // CTAs per SM, teams per CTA by class
   static const int kTeams[2][kClasses] = {{8, 4, 2, 1}, {1, 2, 1, 1}};
-  const int lp = s->d.dtype != MC_F64, per_sm = lp ? 2 : 3;
-  const int64_t free_ctas = (int64_t)per_sm * (s->num_sms - 16 * t->res_clusters);
+  const int64_t free_ctas = (int64_t)per_sm * (s->num_sms - 16 * used);
   int64_t want[kClasses] = {0, 0, 0, 0}, sum = 0;
   for (int c = 0; c < kClasses; ++c) {
     want[c] = (team_levels[c] + kTeams[lp][c] - 1) / kTeams[lp][c];
@@ -390,6 +416,22 @@ void deal_ctas(const mc_server* s, BTable* t, const int64_t* team_levels) {
     if (sum > free_ctas) n = (n * free_ctas + sum - 1) / sum;
     t->team_ctas[c] = (int32_t)n;
   }
+}
+
+// Whether so many FP64 requests of the resident path are active that the queue takes
+// less time than the clusters, eight at a time.  By block size, requests at which the
+// two took the same time for a chunk of 64 sweeps (inverse, coupled): 64 x 8 104, 105;
+// 128 x 16 50, 60; 300 x 12 57; 140 x 32 25, 26; 90 x 24 23, 23; 200 x 8 none.  With
+// all of them there: 250 of 128 x 16 11.0 -> 5.7 ms, 200 of 140 x 32 31.4 -> 9.6.
+bool residents_overflow(const mc_server* s) {
+  if (s->d.dtype != MC_F64) return false;
+  double load = 0.0;
+  for (const Req* r : s->active)
+    if (r->path == kPathResident) {
+      const int64_t m = r->chain->lay.m;
+      load += m > 16 ? 1.0 / 24 : m > 8 ? 1.0 / 52 : r->chain->lay.N < 1200 ? 1.0 / 100 : 0.0;
+    }
+  return load > 1.0;
 }
 
 // Fill the pinned request table from the active list (small blocks first);
@@ -404,7 +446,7 @@ std::vector<Req*> build_table(mc_server* s) {
   for (int c = 0; c < kClasses; ++c) t->cls_end[c] = 0;
   t->G = s->G;
   t->off_h1[0] = t->off_h2[0] = t->off_lv[0] = t->off_t1[0] = t->off_t2[0] = 0;
-  t->res_n = 0;
+  const bool overflow = residents_overflow(s);
   int64_t team_levels[kClasses] = {0, 0, 0, 0};
   const int p1 = s->d.stair == 1 ? 0 : 1;
   for (int i = 0; i < t->n; ++i) {
@@ -412,18 +454,27 @@ std::vector<Req*> build_table(mc_server* s) {
     const int64_t L = r->chain->lay.L;
     for (int c = cls(r); c < kClasses; ++c) t->cls_end[c] = i + 1;
     fill_req(s, r, &t->r[i]);
+    if (overflow && r->path == kPathResident) {
+      t->r[i].path = kPathQueue;
+      resident_order(r->chain->lay, &t->r[i].res_c, &t->r[i].res_s);
+    }
+    const int path = t->r[i].path;
     const int64_t G = class_group(s->G, r->chain->lay.m);
     t->r[i].G = (int32_t)G;
     // units: groups of G levels of each half-sweep
     const int64_t P1 = (L - p1 + 1) / 2, P2 = (L - (1 - p1) + 1) / 2;
-    const bool queue = r->path == kPathQueue, team = r->path == kPathTeam;
+    const bool queue = path == kPathQueue, team = path == kPathTeam;
     t->off_h1[i + 1] = t->off_h1[i] + (queue ? (P1 + G - 1) / G : 0);
     t->off_h2[i + 1] = t->off_h2[i] + (queue ? (P2 + G - 1) / G : 0);
     t->off_t1[i + 1] = t->off_t1[i] + (team ? P1 : 0);
     t->off_t2[i + 1] = t->off_t2[i] + (team ? P2 : 0);
     t->off_lv[i + 1] = t->off_lv[i] + L;
     if (team) team_levels[cls(r)] += L;
-    if (r->path == kPathResident) t->res[t->res_n++] = i;
+  }
+  for (int g = 0, n = 0; g < kResGroups; ++g) {
+    for (int i = 0; i < t->n; ++i)
+      if (t->r[i].path == kPathResident && s->active[(size_t)i]->group == g) t->res[n++] = i;
+    t->res_end[g] = n;
   }
   deal_ctas(s, t, team_levels);
   return std::vector<Req*>(s->active.begin(), s->active.end());
@@ -463,7 +514,7 @@ void free_host_side(mc_server* s) {
   if (s->cap) cudaStreamDestroy(s->cap);
   for (cudaEvent_t f : s->fork)
     if (f) cudaEventDestroy(f);
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < kSides; ++i) {
     if (s->side[i]) cudaStreamDestroy(s->side[i]);
     if (s->join[i]) cudaEventDestroy(s->join[i]);
   }
@@ -508,7 +559,7 @@ int mc_server_create(const mc_server_desc* desc, void* arena, size_t arena_bytes
             cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) == cudaSuccess &&
             cudaEventCreateWithFlags(&s->fork[0], cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&s->fork[1], cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 4 && ok; ++i)
+  for (int i = 0; i < kSides && ok; ++i)
     ok = cudaStreamCreateWithFlags(&s->side[i], cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
@@ -588,6 +639,7 @@ int mc_server_submit(mc_server* s, int64_t tag, int64_t L, int32_t m, const doub
   r->sweeps = 0;
   r->step_prev = NAN;
   r->path = b_path(y, s->d.apply == MC_APPLY_COUPLED, s->num_sms);
+  r->group = resident_batch_group(y, s->d.apply == MC_APPLY_COUPLED);
   r->vbase = 0;
   r->fresh = true;
   if (reset_team_words(s, r) != cudaSuccess) {

@@ -87,3 +87,44 @@ def test_long_chains_of_small_fp64_blocks():
         ref = oracle.Chain(*blocks(i, L, m)).sweeps(np.full(L * m, 1.0 / (L * m)), 4)
         assert np.abs(pa - ref).sum() <= 1e-12     # 4 sweeps of sums of 3 m terms >= 0: below 1e-14
     srv.close()
+
+
+def copies(sizes, n, **kw):
+    """Every size n times in one server, and once in a server of its own: statuses and results."""
+    srv = mc.Server(4 << 30, autotune=False, max_active=1000, **kw)
+    for c in range(n):
+        for i, (L, m) in enumerate(sizes):
+            assert srv.submit(c * len(sizes) + i, *blocks(i, L, m))
+    mixed = {t: (pi, r["sweeps"]) for t, pi, r, st in srv.run_until_idle()}
+    assert len(mixed) == n * len(sizes)
+    srv.close()
+    alone = mc.Server(1 << 30, autotune=False, **kw)
+    for i, (L, m) in enumerate(sizes):
+        alone.submit(i, *blocks(i, L, m))
+        (_, pa, ra, _), = alone.run_until_idle()
+        for c in range(n):
+            pi, sweeps = mixed[c * len(sizes) + i]
+            assert sweeps == ra["sweeps"] and np.array_equal(pa, pi), (L, m, c)
+    alone.close()
+
+
+# every way the resident kernels split a row's columns (by lanes, by warps, not at all), clusters of 1 to
+# 16 CTAs with equal and unequal shares; four of each are more than clusters are given, and fewer again
+# once the first have converged
+SMALL64 = [(2, 3), (3, 1), (5, 2), (8, 4), (31, 8), (33, 16), (60, 32), (140, 32), (90, 24), (64, 5), (200, 8), (100, 13),
+           (35, 20), (17, 31), (500, 3), (16, 17), (70, 11), (33, 2), (400, 10), (250, 16)]
+
+
+@pytest.mark.parametrize("apply,stair", [("inverse", 1), ("coupled", 2)])
+@pytest.mark.parametrize("check,stop", [(24, dict(tol=1e-12)), (1, dict(tol=0.0, maxit=5)), (2, dict(tol=0.0, maxit=6))])
+def test_many_small_fp64_requests_are_as_alone(apply, stair, check, stop):
+    """Below and above the line between clusters and the shared queue the iterates are the same bits."""
+    copies(SMALL64, 4, dtype="f64", apply=apply, stair=stair, check_every=check, **stop)
+
+
+# shared memory of a CTA for four, two and one to an SM, blocks of up to 16 rows and wider
+@pytest.mark.parametrize("apply", ["inverse", "coupled"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_many_small_low_precision_requests_are_as_alone(dtype, apply):
+    copies([(128, 16), (33, 4), (1500, 8), (2600, 8), (64, 32), (40, 24), (100, 28), (140, 32), (200, 32), (300, 32), (450, 32)], 4,
+           dtype=dtype, apply=apply, check_every=24, tol=1e-11)
