@@ -680,11 +680,7 @@ cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out,
 
 int b_path(const Layout& y, int coupled, int num_sms) {
   if (resident_batch_group(y, coupled) >= 0) return kPathResident;
-  // FP64, m <= 16: a chain with a level for every warp in flight is bound by the
-  // fence and claim of each unit, which units of 4 levels share (six of 16384 x 16,
-  // coupled, a chunk of 64 sweeps: teams 12.3 ms, queue 11.0); shorter ones by the
-  // unit's latency (1500 x 16 with two of 24 and 32 rows: teams 1.41, queue 3.20).
-  if (y.lp == 0) return y.m <= 16 && y.L / 2 >= 24ll * num_sms ? kPathQueue : kPathTeam;
+  if (y.lp == 0) return kPathTeam;   // (m <= 16: or the queue, by the batch)
   if (y.m <= 32) return kPathQueue;
   if ((y.lp == 1 || y.m % 8 == 0) &&
       y.L / 2 * (y.m <= 64 ? 4 : 8) <= 16ll * num_sms)   // as launch_sweeps_lp

@@ -81,14 +81,16 @@ __host__ __device__ inline int class_group(int G, int m) {
 // How a request's sweeps run.  Its arithmetic follows from its own size alone (so that
 // its iterates do not depend on the batch):
 //   kPathQueue: one warp per unit of G levels, all such requests in shared launches
-//     by size class (k_b_sweeps: FP64 blocks of up to 16 rows, long chains; k_b_sweeps_lp);
+//     by size class (k_b_sweeps, k_b_sweeps_lp);
 //   kPathTeam: a team of warps per level, all such requests of a size class in one
-//     launch: all other FP64 requests (team_dev.cuh), low-precision short chains
-//     of blocks of more than 32 rows (lpteam_dev.cuh);
+//     launch: FP64 requests (team_dev.cuh), low-precision short chains of blocks of
+//     more than 32 rows (lpteam_dev.cuh);
 //   kPathResident: blocks of up to 32 rows that fit one cluster's shared memory, one
 //     cluster per request (resident_dev.cuh).
 // FP64 requests of the resident path run on the queue, with the sums in the resident
-// order (res_order), while so many are active that the clusters would take longer.
+// order (res_c), while so many are active that the clusters would take longer, and
+// FP64 blocks of up to 16 rows of the team path, which adds as the queue does, while
+// their levels fill the GPU several times over (build_table).
 // The launches of the three paths run side by side; the host deals out CTAs to
 // them with the table.  Eight requests of 131 KB to 17 MB
 // (BF16 coupled, m = 16 to 128): a chunk of 64 sweeps 2.70 -> 0.99 ms with all of them

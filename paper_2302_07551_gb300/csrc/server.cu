@@ -39,7 +39,7 @@ struct Req {
   double step_prev;
   int path;             // kPathQueue / kPathTeam / kPathResident
   int group;            // of the resident path
-  int64_t vbase;        // sweeps that the completion counters have seen (FP64 teams)
+  int64_t vbase;        // value of the completion counters per warp of a level's team (FP64)
   bool fresh;           // factor status not yet checked
 };
 
@@ -434,6 +434,19 @@ bool residents_overflow(const mc_server* s) {
   return load > 1.0;
 }
 
+// Whether the FP64 requests of up to 16 rows on the team path run on the queue, whose
+// units of several levels share a fence and a claim: from about 26000 levels together.
+// A chunk of 64 sweeps by teams and by the queue, inverse: 10 of 1500 x 16 2.64, 3.19 ms,
+// 6 of 3000 x 13 3.14, 3.47, 10 5.19, 5.04, 4 of 7000 x 10 4.82, 4.71, 40 of 1500 x 16
+// 10.5, 9.94; coupled: 10 of 1500 x 16 1.94, 2.32, 40 7.87, 6.77.  The sums are the same.
+bool small_teams_overflow(const mc_server* s) {
+  int64_t levels = 0;
+  for (const Req* r : s->active)
+    if (r->path == kPathTeam && r->chain->lay.lp == 0 && r->chain->lay.m <= 16)
+      levels += r->chain->lay.L;
+  return levels >= 170ll * s->num_sms;
+}
+
 // Fill the pinned request table from the active list (small blocks first);
 // returns the table order.
 std::vector<Req*> build_table(mc_server* s) {
@@ -446,7 +459,7 @@ std::vector<Req*> build_table(mc_server* s) {
   for (int c = 0; c < kClasses; ++c) t->cls_end[c] = 0;
   t->G = s->G;
   t->off_h1[0] = t->off_h2[0] = t->off_lv[0] = t->off_t1[0] = t->off_t2[0] = 0;
-  const bool overflow = residents_overflow(s);
+  const bool overflow = residents_overflow(s), small_queue = small_teams_overflow(s);
   int64_t team_levels[kClasses] = {0, 0, 0, 0};
   const int p1 = s->d.stair == 1 ? 0 : 1;
   for (int i = 0; i < t->n; ++i) {
@@ -458,6 +471,7 @@ std::vector<Req*> build_table(mc_server* s) {
       t->r[i].path = kPathQueue;
       resident_order(r->chain->lay, &t->r[i].res_c, &t->r[i].res_s);
     }
+    if (small_queue && r->path == kPathTeam && r->chain->lay.m <= 16) t->r[i].path = kPathQueue;
     const int path = t->r[i].path;
     const int64_t G = class_group(s->G, r->chain->lay.m);
     t->r[i].G = (int32_t)G;
@@ -489,7 +503,8 @@ int process_outputs(mc_server* s, const std::vector<Req*>& order, int c) {
     const BOut& o = s->out_host[k];
     Req* r = order[k];
     r->sweeps += c;
-    r->vbase += c;
+    // (the queue writes the epoch's counts, teams count on from their own)
+    r->vbase = s->t_host->r[k].path == kPathQueue ? s->t_host->epoch + c : r->vbase + c;
     const size_t i =
         (size_t)(std::find(s->active.begin(), s->active.end(), r) - s->active.begin());
     const double kap =

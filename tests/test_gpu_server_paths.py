@@ -128,3 +128,28 @@ def test_many_small_fp64_requests_are_as_alone(apply, stair, check, stop):
 def test_many_small_low_precision_requests_are_as_alone(dtype, apply):
     copies([(128, 16), (33, 4), (1500, 8), (2600, 8), (64, 32), (40, 24), (100, 28), (140, 32), (200, 32), (300, 32), (450, 32)], 4,
            dtype=dtype, apply=apply, check_every=24, tol=1e-11)
+
+
+@pytest.mark.parametrize("apply,check", [("inverse", 24), ("coupled", 24), ("coupled", 1)])
+def test_small_blocks_move_between_teams_and_queue(apply, check):
+    """Long FP64 chains of up to 16 rows run by teams while few are active and on the queue while many are; a
+    request that goes from one to the other and back has the bits of one that never did."""
+    kw = dict(dtype="f64", apply=apply, check_every=check, tol=0.0, maxit=5 * check, autotune=False)
+    waves = {0: [(2000, 16), (9000, 5), (4000, 9)], 2: [(2500, 12)] * 6 + [(3001, 10)], 3: [(2000, 16), (4001, 9)]}
+    srv, got, want, tag = mc.Server(4 << 30, **kw), {}, [], 0
+    for step in range(8):
+        for size in waves.get(step, []):
+            assert srv.submit(tag, *blocks(tag, *size))
+            want.append(size)
+            tag += 1
+        srv.step()
+        while (r := srv.fetch()) is not None:
+            got[r[0]] = r[1]
+    srv.close()
+    assert len(got) == len(want)
+    alone = mc.Server(1 << 30, **kw)
+    for i, size in enumerate(want):
+        alone.submit(i, *blocks(i, *size))
+        (_, pa, _, _), = alone.run_until_idle()
+        assert np.array_equal(pa, got[i]), (i, size)
+    alone.close()
