@@ -243,10 +243,10 @@ __global__ void __launch_bounds__(256, Tune<R>::MINB) k_residual(ResidArgs a) {
 }
 
 // k_residual for blocks of more than 32 rows: a team of TW warps per level, one
-// row per lane (team_dev.cuh).  One warp per level with up to 8 rows a lane kept
-// few loads in flight and left most of the GPU idle on short chains (512 levels
+// row per lane (team_dev.cuh).  One warp per level with up to 8 rows a lane keeps
+// few loads in flight and leaves most of the GPU idle on short chains (512 levels
 // of 256 with q: the refinement's outer step 563 -> 320 us, of which the FP64
-// pipe needs 213).
+// pipe needs 213).  launch_residual says where one warp is the better.
 template <int TW>
 struct ResidShared {
   double v[3][32 * TW];
@@ -449,8 +449,36 @@ cudaError_t launch_normalise(const NormArgs& a, int n_blocks, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <int R>
+cudaError_t resid_warp(const ResidArgs& a, int nb, cudaStream_t s) {
+  static_assert(vec_smem<R>() <= 40 * 1024, "no opt-in");
+  if (a.q)
+    k_residual<R, true><<<nb, 256, vec_smem<R>(), s>>>(a);
+  else
+    k_residual<R, false><<<nb, 256, vec_smem<R>(), s>>>(a);
+  return cudaGetLastError();
+}
+
+// Teams where a chain is short or its teams' rows (32 TW, TW even) are in use: long
+// chains, us, team and one warp per level: 8000 x 40 161, 146; 8000 x 48 163, 172 (aligned
+// columns); 8000 x 56 211, 187; 8000 x 72 455, 335; 8000 x 96 535, 433; 3600 x 100 298, 270;
+// 8000 x 104 605, 605; 8000 x 112 617, 652; 8000 x 128 694, 733; 2600 x 136 407, 447;
+// 8000 x 136 1162, 953; 3600 x 200 999, 1140; 3600 x 256 1213, 1628; short: 300 x 40 40, 49;
+// 300 x 72 48, 72; 300 x 136 76, 197.
 cudaError_t launch_residual(const ResidArgs& a, int nb, int sms, cudaStream_t s) {
   const int r = (a.m + 31) / 32;
+  const bool warp = r == 2   ? a.m % 16 != 0
+                    : r == 3 ? true
+                    : r == 4 ? a.m % 8 != 0
+                             : r == 5 && a.L >= 30ll * sms;
+  if (!a.paired && warp && a.L >= 6ll * sms) {
+    switch (r) {
+      case 2: return resid_warp<2>(a, nb, s);
+      case 3: return resid_warp<3>(a, nb, s);
+      case 4: return resid_warp<4>(a, nb, s);
+      default: return resid_warp<5>(a, nb, s);
+    }
+  }
   if (a.paired) {
     switch (r) {
       case 2: return resid_m<2, true>(a, sms, s);
@@ -461,12 +489,7 @@ cudaError_t launch_residual(const ResidArgs& a, int nb, int sms, cudaStream_t s)
     }
   }
   switch (r) {
-    case 1:
-      if (a.q)
-        k_residual<1, true><<<nb, 256, vec_smem<1>(), s>>>(a);
-      else
-        k_residual<1, false><<<nb, 256, vec_smem<1>(), s>>>(a);
-      return cudaGetLastError();
+    case 1: return resid_warp<1>(a, nb, s);
     case 2: return resid_m<2>(a, sms, s);
     case 3:
     case 4: return resid_m<4>(a, sms, s);
