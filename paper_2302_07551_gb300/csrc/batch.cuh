@@ -200,8 +200,9 @@ cudaError_t b_sweeps(const BTable* t, unsigned long long* claim, BOut* out, int 
 // The FP64 team requests' sweeps, a launch per size class on b0, b[0..2].
 cudaError_t b_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
                    int coupled, int K, int num_sms, cudaStream_t b0, const cudaStream_t* b);
-// resident.cu: the group of a request that fits one cluster, else -1; the launch of
+// resident.cu: CTAs of a cluster (0: none can run); the group of a request that fits one cluster, else -1; the launch of
 // a group's requests (lp: 0 FP64, 1 FP32, 2 BF16); res_c and res_s of an FP64 request.
+int resident_cluster();
 int resident_batch_group(const Layout& lay, int coupled);
 cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int group, int K, BOut* out,
                                   cudaStream_t s);

@@ -471,6 +471,8 @@ cudaError_t launch_resident_lp(const ResidentLpArgs& a, const Layout& y, int cou
   return cudaLaunchKernelEx(&cfg, kernel_lp(y.lp, coupled, grid != 0), a);
 }
 
+int resident_cluster() { return limits().cluster; }
+
 int resident_batch_group(const Layout& y, int coupled) {
   const int C = cluster_ctas(y.L, limits().cluster);
   if (C == 0 || y.m > 32 || y.L > (1 << 20)) return -1;

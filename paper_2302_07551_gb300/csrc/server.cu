@@ -21,6 +21,7 @@
 
 #include "batch.cuh"
 #include "chain.cuh"
+#include "deal.h"
 
 using namespace mc;
 
@@ -379,43 +380,19 @@ int check_fresh(mc_server* s) {
   return MC_OK;
 }
 
-// CTAs of the launches that run side by side.  Clusters take 16 SMs whole, a slot that
-// group_share clusters of a group share; the slots go one by one to the group with the
-// most requests in turn.  The team launches share the other SMs, two or three CTAs each,
-// in proportion to their levels (no more than one team per level), so that each gets
-// its part at once instead of the first launch filling the GPU for a chunk's time.  No
-// result depends on it.
+// CTAs of the launches that run side by side (deal.h).
 void deal_ctas(const mc_server* s, BTable* t, const int64_t* team_levels) {
-  const bool teams = team_levels[0] + team_levels[1] + team_levels[2] + team_levels[3] > 0;
-  const int lp = s->d.dtype != MC_F64, per_sm = lp ? 2 : 3;
-  int n[kResGroups], slots[kResGroups] = {}, used = 0;
-  for (int g = 0; g < kResGroups; ++g) n[g] = t->res_end[g] - (g ? t->res_end[g - 1] : 0);
-  for (int left = teams ? kResidentSlots / 2 : kResidentSlots; left > 0; --left) {
-    int best = -1;
-    double turns = 1.0;   // requests per cluster: no group needs more clusters than requests
-    for (int g = 0; g < kResGroups; ++g) {
-      const double r = n[g] == 0 ? 0.0 : slots[g] ? (double)n[g] / (slots[g] * group_share(g)) : 1e9;
-      if (r > turns) best = g, turns = r;
-    }
-    if (best < 0) break;
-    ++slots[best];
-    ++used;
+  static const int kTeams[2][kClasses] = {{8, 4, 2, 1}, {1, 2, 1, 1}};   // per CTA, by class
+  const int lp = s->d.dtype != MC_F64;
+  int n[kResGroups], share[kResGroups];
+  for (int g = 0; g < kResGroups; ++g) {
+    n[g] = t->res_end[g] - (g ? t->res_end[g - 1] : 0);
+    share[g] = group_share(g);
   }
-  for (int g = 0; g < kResGroups; ++g)
-    t->res_clusters[g] = n[g] < slots[g] * group_share(g) ? n[g] : slots[g] * group_share(g);
-  // CTAs per SM, teams per CTA by class
-  static const int kTeams[2][kClasses] = {{8, 4, 2, 1}, {1, 2, 1, 1}};
-  const int64_t free_ctas = (int64_t)per_sm * (s->num_sms - 16 * used);
-  int64_t want[kClasses] = {0, 0, 0, 0}, sum = 0;
-  for (int c = 0; c < kClasses; ++c) {
-    want[c] = (team_levels[c] + kTeams[lp][c] - 1) / kTeams[lp][c];
-    sum += want[c];
-  }
-  for (int c = 0; c < kClasses; ++c) {
-    int64_t n = want[c];
-    if (sum > free_ctas) n = (n * free_ctas + sum - 1) / sum;
-    t->team_ctas[c] = (int32_t)n;
-  }
+  const int cluster = resident_cluster();
+  deal(DealIn{kResGroups, kClasses, n, share, team_levels, kTeams[lp], lp ? 2 : 3, s->num_sms,
+              cluster > 0 ? cluster : 16, kResidentSlots},
+       t->res_clusters, t->team_ctas);
 }
 
 // Whether so many FP64 requests of the resident path are active that the queue takes

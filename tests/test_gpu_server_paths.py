@@ -153,3 +153,10 @@ def test_small_blocks_move_between_teams_and_queue(apply, check):
         (_, pa, _, _), = alone.run_until_idle()
         assert np.array_equal(pa, got[i]), (i, size)
     alone.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_every_group_beside_teams(dtype):
+    """All resident groups, teams of all size classes and the queue in one batch: each gets its part."""
+    copies([(128, 16), (2600, 8), (64, 32), (100, 28), (200, 32), (450, 32), (40, 40), (21, 72), (12, 136), (1300, 64)], 2,
+           dtype=dtype, apply="inverse", check_every=24, tol=1e-11)
