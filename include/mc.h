@@ -409,7 +409,8 @@ int mc_server_grid(const mc_server* server, int32_t* blocks, int32_t* threads,
  */
 typedef struct {
   uint64_t signature;       /* bit c set: requests of size class c present (m <= 32, 64,
-                               128, 256); bits 8..: ceil(log2(total levels)) / 2      */
+                               128, 256); bit 4: requests on the shared queue; bits
+                               8..: ceil(log2(total levels)) / 2                      */
   int32_t blocks_per_sm;    /* resident 256-thread blocks per SM of the fused launches  */
   int32_t levels_per_unit;  /* adjacent same-parity levels per claimed unit (1, 2, 4)
                                for m > 64; x2 for m <= 64, x4 for m <= 32 (at most 16) */

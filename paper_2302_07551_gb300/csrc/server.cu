@@ -336,8 +336,8 @@ double chunk_sweep_bytes(const mc_server* s, int c) {
   return b;
 }
 
-// Autotuner: for each batch signature (size classes present, size class of
-// the total level count) time one live chunk per candidate configuration
+// Autotuner: for each batch signature (size classes present, whether any
+// request is on the queue, size class of the total level count) time one live chunk per candidate configuration
 // (real work, counted as such: results do not depend on the configuration)
 // and keep the fastest.  Coordinate search: the persistent grid (1, 2, 3, 4,
 // 6, 8 resident 256-thread blocks per SM) with one level per unit, then 2
@@ -351,6 +351,9 @@ uint64_t signature(const mc_server* s) {
   uint64_t sig = (uint64_t)(lg / 2) << 8;
   for (int c = 0; c < kClasses; ++c)
     if (t->cls_end[c] > (c ? t->cls_end[c - 1] : 0)) sig |= 1ull << c;
+  // the sweeps of teams and clusters do not depend on the tuned configuration: what
+  // was found without a queue says nothing about one
+  if (table_paths(t) & path_bit(kPathQueue, 0)) sig |= 1ull << kClasses;
   return sig;
 }
 

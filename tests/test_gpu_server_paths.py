@@ -160,3 +160,19 @@ def test_every_group_beside_teams(dtype):
     """All resident groups, teams of all size classes and the queue in one batch: each gets its part."""
     copies([(128, 16), (2600, 8), (64, 32), (100, 28), (200, 32), (450, 32), (40, 40), (21, 72), (12, 136), (1300, 64)], 2,
            dtype=dtype, apply="inverse", check_every=24, tol=1e-11)
+
+
+def test_a_queue_has_a_signature_of_its_own():
+    """Batches of the same size classes and level count, one by teams alone, one with the queue: what the autotuner
+    kept for the first does not decide for the second."""
+    srv = mc.Server(4 << 30, dtype="f32", apply="coupled", check_every=8, tol=0.0, maxit=160, max_active=1000)
+    sigs = []
+    for L, m, n in [(300, 64, 8), (2400, 64, 1)]:       # 2400 levels: more than teams for all of a half-sweep
+        before = len(srv.trials())
+        for i in range(n):
+            assert srv.submit(i, *blocks(i, L, m))
+        srv.run_until_idle()
+        sigs.append({t["signature"] for t in srv.trials()[before:]})
+    srv.close()
+    assert sigs[0] and sigs[1] and not sigs[0] & sigs[1]
+    assert all(s & 16 for s in sigs[1]) and not any(s & 16 for s in sigs[0])
