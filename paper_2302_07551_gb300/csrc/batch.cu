@@ -205,8 +205,8 @@ __global__ void __launch_bounds__(256, 4) k_b_sweeps(const BTable* __restrict__ 
       const double ls =
           Q->res_c ? level_resident<COUPLED>(Q, src, dst, l, slice, lane, want)
                    : level_sweep2<1, COUPLED, true, true>(Q->A, Q->B, Q->C, src, src, dst, l, Q->L,
-                                                          Q->m, Q->ms, slice, lane, 1.0, nullptr,
-                                                          nullptr, nullptr, want);
+                                                          Q->m, Q->ms, slice, lane, nullptr, nullptr,
+                                                          nullptr, want);
       if (want && lane == 0) Q->lsum2[(u.k & 1) * Q->L + l] = ls;
     }
     publish_levels(Q->ver, u.l, 2, u.n, base + (int)u.k + 1, lane);
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(256, 2) k_b_team(const BTable* __restrict__ t,
   unsigned long long q0 = w == 0 ? claim_unit(claim, lane) : 0ull, q;
   if (w == 0 && lane == 0) sh.next[1] = q0;
   if (w == 0) q0 = claim_unit(claim, lane);
-  lp_sync<TW>(bar);
+  team_sync<TW>(bar);
   q = sh.next[1];
   int turn = 0;
   while (q < total) {

@@ -251,13 +251,8 @@ __global__ void __launch_bounds__(TeamBlock<TW>::T, TeamBlock<TW>::B) k_sweeps(F
 constexpr int kBgsWarps = 4;
 
 __device__ __forceinline__ double bgs_parts(const double* part, int W, int i) {
-  if constexpr (kBgsWarps == 8)
-    return ((part[i] + part[W + i]) + (part[2 * W + i] + part[3 * W + i])) +
-           ((part[4 * W + i] + part[5 * W + i]) + (part[6 * W + i] + part[7 * W + i]));
-  else if constexpr (kBgsWarps == 4)
-    return (part[i] + part[W + i]) + (part[2 * W + i] + part[3 * W + i]);
-  else
-    return part[i] + part[W + i];
+  static_assert(kBgsWarps == 4, "");
+  return (part[i] + part[W + i]) + (part[2 * W + i] + part[3 * W + i]);
 }
 
 template <int R, bool COUPLED>
@@ -298,22 +293,22 @@ __global__ void __launch_bounds__(32 * kBgsWarps, 16 / kBgsWarps) k_bgs_cta(Fuse
       v_up[i] = has_up ? __ldcg(up + (l + 1) * m + i) : 0.0;
     }
     __syncthreads();
-    double acc[R][Tune<R>::NA];
+    double acc[R];
     zero_acc<R>(acc);
     if (j0 < j1) {
-      if (has_lo) gemv_acc_part<R, 0, R>(acc, a.A + (size_t)l * a.ms, v_lo, j0, j1, m, lane);
-      if (has_up) gemv_acc_part<R, 0, R>(acc, a.B + (size_t)l * a.ms, v_up, j0, j1, m, lane);
+      if (has_lo) gemv_acc<R>(acc, a.A + (size_t)l * a.ms, v_lo, j0, j1, m, lane);
+      if (has_up) gemv_acc<R>(acc, a.B + (size_t)l * a.ms, v_up, j0, j1, m, lane);
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) part[w * W + lane + 32 * r] = fold<R>(acc[r]);
+    for (int r = 0; r < R; ++r) part[w * W + lane + 32 * r] = acc[r];
     __syncthreads();
     if (!COUPLED) {
       for (int i = threadIdx.x; i < m; i += nt) v_g[i] = bgs_parts(part, W, i);
       __syncthreads();
       zero_acc<R>(acc);
-      if (j0 < j1) gemv_acc_part<R, 0, R>(acc, a.C + (size_t)l * a.ms, v_g, j0, j1, m, lane);
+      if (j0 < j1) gemv_acc<R>(acc, a.C + (size_t)l * a.ms, v_g, j0, j1, m, lane);
 #pragma unroll
-      for (int r = 0; r < R; ++r) part[w * W + lane + 32 * r] = fold<R>(acc[r]);
+      for (int r = 0; r < R; ++r) part[w * W + lane + 32 * r] = acc[r];
       __syncthreads();
     }
     double ls = 0.0;

@@ -123,15 +123,12 @@ __global__ void __launch_bounds__(256, 2) k_lp_team(LpLevels a, int64_t K, int p
   auto& sh = reinterpret_cast<LpTeamShared<ROWS, TW>*>(lp_smem)[team];
   const int64_t P0 = (a.L - parity + 1) / 2;
   const unsigned long long total = (unsigned long long)K * (unsigned long long)a.L;
+  static_assert(TW > 1, "the next unit travels through shared memory");
   unsigned long long q0 = w == 0 ? claim_unit(claim, lane) : 0ull, q;
-  if constexpr (TW == 1) {
-    q = __shfl_sync(0xffffffffu, q0, 0);
-  } else {
-    if (w == 0 && lane == 0) sh.next[1] = q0;
-    if (w == 0) q0 = claim_unit(claim, lane);
-    lp_sync<TW>(bar);
-    q = sh.next[1];
-  }
+  if (w == 0 && lane == 0) sh.next[1] = q0;
+  if (w == 0) q0 = claim_unit(claim, lane);
+  team_sync<TW>(bar);
+  q = sh.next[1];
   auto unit = [&](unsigned long long i) {
     const int64_t k = (int64_t)(i / (unsigned long long)a.L);
     const int64_t r = (int64_t)i - k * a.L;
@@ -142,22 +139,17 @@ __global__ void __launch_bounds__(256, 2) k_lp_team(LpLevels a, int64_t K, int p
   int turn = 0;
   while (q < total) {
     unsigned long long qn = 0ull;
-    if constexpr (TW == 1)
-      q0 = claim_unit(claim, lane);
-    else if (w == 0 && lane == 0)
-      sh.next[turn] = q0;
+    if (w == 0 && lane == 0) sh.next[turn] = q0;
     const LpUnit u = unit(q);
     LpAhead<S, ROWS, TW, COUPLED> p;
     p.load(a, u, w, tt, lane);
     lp_team_unit<S, ROWS, TW, COUPLED>(a, sh, u, p, w, tt, lane, bar, &hdr->status, wait_ns,
                                        [&]() {
-                                         if constexpr (TW > 1) {
-                                           qn = sh.next[turn];
-                                           turn ^= 1;
-                                           if (w == 0) q0 = claim_unit(claim, lane);
-                                         }
+                                         qn = sh.next[turn];
+                                         turn ^= 1;
+                                         if (w == 0) q0 = claim_unit(claim, lane);
                                        });
-    q = TW == 1 ? __shfl_sync(0xffffffffu, q0, 0) : qn;
+    q = qn;
   }
 }
 

@@ -122,17 +122,6 @@ __device__ __forceinline__ void wide_store(
   }
 }
 
-__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_word(unsigned long long* p, float v, int version) {
-  const unsigned long long w =
-      ((unsigned long long)(unsigned)version << 32) | __float_as_uint(v);
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
-
 // The words at p and q (either may be NULL: zero) once they carry `version`
 // (bounded: after wait_ns, or once a timeout is latched, MC_ERR_TIMEOUT is
 // latched and the last values are taken).
@@ -168,14 +157,6 @@ struct alignas(16) LpTeamShared {
   unsigned long long next[2];
 };
 
-template <int TW>
-__device__ __forceinline__ void lp_sync(int bar) {
-  if constexpr (TW == 1)
-    __syncwarp();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(TW * 32) : "memory");
-}
-
 // Operators and vectors of a chain (or one request of a batch).
 struct LpLevels {
   const void* A;
@@ -193,7 +174,6 @@ struct LpLevels {
 // every lane layout start on a whole load; at most ROWS / TW (>= 16) columns.
 template <int TW>
 __device__ __forceinline__ int lp_col(int m, int w) {
-  if (TW == 1) return w ? m : 0;
   const int cw = ((m + TW - 1) / TW + 15) / 16 * 16, j = w * cw;
   return j < m ? j : m;
 }
@@ -252,7 +232,7 @@ __device__ __forceinline__ void lp_team_unit(const LpLevels& a, LpTeamShared<ROW
       sh.v[1][i] = v.y * p.s_up;
     }
   }
-  lp_sync<TW>(bar);
+  team_sync<TW>(bar);
   hand();
   const float q = p.q;
   if (!u.zero) {
@@ -272,7 +252,7 @@ __device__ __forceinline__ void lp_team_unit(const LpLevels& a, LpTeamShared<ROW
     }
     wide_store<S, ROWS>(acc, sh.part[w], lane);
   }
-  lp_sync<TW>(bar);
+  team_sync<TW>(bar);
   auto total = [&](int row) {
     float t = sh.part[0][row];
 #pragma unroll
@@ -282,7 +262,7 @@ __device__ __forceinline__ void lp_team_unit(const LpLevels& a, LpTeamShared<ROW
   if constexpr (!COUPLED) {
     if (!u.zero) {
       for (int i = tt; i < ROWS + 64; i += 32 * TW) sh.g[i] = i < m ? total(i) : 0.0f;
-      lp_sync<TW>(bar);
+      team_sync<TW>(bar);
       using P = WideLane<float, ROWS>;
       float acc[P::RG][P::E];
 #pragma unroll
@@ -292,15 +272,14 @@ __device__ __forceinline__ void lp_team_unit(const LpLevels& a, LpTeamShared<ROW
       if (j0 < j1)
         wide_product<float, ROWS, CW>(acc, p.c, a.C + l * a.cbs, sh.g, j0, j1, m, lane);
       wide_store<float, ROWS>(acc, sh.part[w], lane);
-      lp_sync<TW>(bar);
+      team_sync<TW>(bar);
     }
   }
   if (tt < m) {
     const float v = (u.zero ? 0.0f : total(tt)) + q;
-    st_word(a.dv + l * m + tt, v, u.out);
+    st_word(a.dv + l * m + tt, __float_as_uint(v), (unsigned)u.out);
     if (u.last) a.d[l * m + tt] = v;
   }
-  if constexpr (TW == 1) __syncwarp();   // part is rewritten for the next level
 }
 
 }  // namespace dev

@@ -353,17 +353,9 @@ struct ClusterLink {
   }
 };
 
-// Words {32 bits of the value, version} in global memory; a double takes two.
-__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_word(unsigned long long* p, unsigned bits, unsigned version) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p),
-               "l"(((unsigned long long)version << 32) | bits)
-               : "memory");
-}
+// Words (wave_dev.cuh) of a vector in global memory; a double takes two.
+using dev::ld_word;
+using dev::st_word;
 __device__ __forceinline__ void put(unsigned long long* p, int i, float v, unsigned version) {
   st_word(p + i, __float_as_uint(v), version);
 }

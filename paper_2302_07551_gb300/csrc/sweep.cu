@@ -18,9 +18,7 @@
 // m % 32 == 0.  The level's input vectors sit in a per-warp slice of shared
 // memory and v_j, v_{j+1} reach all lanes with one broadcast 16-byte load;
 // the intermediate g of the inverse mode goes through the same slice, so the
-// second product needs no block barrier.  Each row keeps NA independent
-// accumulators (columns interleaved) so that consecutive DFMAs do not wait
-// on each other.  Warps stream levels with a static stride; each warp writes
+// second product needs no block barrier.  Warps stream levels with a static stride; each warp writes
 // one partial of e^T z and the last block of half-sweep 2 sums them in a
 // fixed order (bitwise deterministic).
 #include <math.h>
@@ -51,8 +49,7 @@ __global__ void __launch_bounds__(256, Tune<R>::MINB) k_phase(PhaseArgs a) {
   for (int64_t u = gw; u < a.P; u += nw) {
     const int64_t l = a.stride * u + a.parity;
     wsum += level_sweep2<R, COUPLED, false>(a.A, a.B, a.C, a.src, a.src, a.dst, l, a.L,
-                                                    a.m, a.ms, slice, lane, 1.0, a.far, a.xfar,
-                                                    a.xfar);
+                                                    a.m, a.ms, slice, lane, a.far, a.xfar, a.xfar);
   }
   wsum = warp_sum(wsum);   // the lanes' partials over all of this warp's levels
   if (lane == 0) {
@@ -88,7 +85,7 @@ __global__ void __launch_bounds__(32) k_bgs(PhaseArgs a) {
   double s = 0.0;
   for (int64_t l = 0; l < a.L; ++l) {
     s += level_sweep2<R, COUPLED>(a.A, a.B, a.C, a.dst, a.src_up, a.dst, l, a.L, a.m, a.ms, slice,
-                                  lane, 1.0, a.far, a.dst, a.src_up);
+                                  lane, a.far, a.dst, a.src_up);
     __syncwarp();   // z_l (global, written by all lanes) is read by all lanes next
   }
   if (lane == 0) a.hdr->stats[0] = s;

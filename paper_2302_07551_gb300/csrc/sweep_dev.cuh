@@ -35,20 +35,17 @@ __device__ __forceinline__ int sched_warp(int64_t P, int nw) {
 template <int R>
 struct Tune {
   static constexpr int U = R <= 1 ? 16 : R <= 2 ? 8 : R <= 4 ? 4 : 2;  // columns per batch
-  static constexpr int NA = 1;                                         // accumulators per row
   static constexpr int MINB = R <= 4 ? 3 : 2;                          // blocks per SM
 };
 
-// acc[r][c] += M(row_r, j) * v[j] for the m columns j of a column-major block
-// M; column j feeds accumulator j % NA.  v: per-warp shared slice, zero
-// beyond m (so the pair load at an odd m reads a zero).  UM multiplies the
-// columns per batch (more loads in flight for kernels with few warps).
-template <int R, int UM = 1>
-__device__ __forceinline__ void gemv_acc(double (&acc)[R][Tune<R>::NA],
-                                         const double* __restrict__ M, const double* v, int m,
-                                         int lane) {
-  constexpr int U = Tune<R>::U * UM, NA = Tune<R>::NA;
-  for (int j0 = 0; j0 < m; j0 += U) {
+// acc[r] += sum over columns [j0b, j1) of M(row_r, j) * v[j] of a column-major block M.
+// v: shared, zero beyond m and readable to the end of the last batch (so the pair load
+// at an odd end reads a zero, or meets a zero block entry).
+template <int R>
+__device__ __forceinline__ void gemv_acc(double (&acc)[R], const double* __restrict__ M,
+                                         const double* v, int j0b, int j1, int m, int lane) {
+  constexpr int U = Tune<R>::U;
+  for (int j0 = j0b; j0 < j1; j0 += U) {
     double t[U][R];
 #pragma unroll
     for (int q = 0; q < U; ++q) {
@@ -56,7 +53,7 @@ __device__ __forceinline__ void gemv_acc(double (&acc)[R][Tune<R>::NA],
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int row = lane + 32 * r;
-        t[q][r] = (j < m && row < m) ? ld_stream(M + (size_t)j * m + row) : 0.0;
+        t[q][r] = (j < j1 && row < m) ? ld_stream(M + (size_t)j * m + row) : 0.0;
       }
     }
 #pragma unroll
@@ -64,84 +61,29 @@ __device__ __forceinline__ void gemv_acc(double (&acc)[R][Tune<R>::NA],
       const double2 vv = *reinterpret_cast<const double2*>(v + j0 + q);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        acc[r][q % NA] = fma(t[q][r], vv.x, acc[r][q % NA]);
-        acc[r][(q + 1) % NA] = fma(t[q + 1][r], vv.y, acc[r][(q + 1) % NA]);
+        acc[r] = fma(t[q][r], vv.x, acc[r]);
+        acc[r] = fma(t[q + 1][r], vv.y, acc[r]);
       }
     }
   }
 }
 
-// As gemv_acc, restricted to columns [j0, j1) and row groups r in [R0, R1)
-// (rows lane + 32 r): the structurally nonzero part of a block.
-template <int R, int R0, int R1>
-__device__ __forceinline__ void gemv_acc_part(double (&acc)[R][Tune<R>::NA],
-                                              const double* __restrict__ M, const double* v,
-                                              int j0b, int j1, int m, int lane) {
-  // batch size follows the rows actually read (about 16 loads in flight)
-  constexpr int U = Tune<R1 - R0>::U, NA = Tune<R>::NA;
-  for (int j0 = j0b; j0 < j1; j0 += U) {
-    double t[U][R1 - R0];
-#pragma unroll
-    for (int q = 0; q < U; ++q) {
-      const int j = j0 + q;
-#pragma unroll
-      for (int r = R0; r < R1; ++r) {
-        const int row = lane + 32 * r;
-        t[q][r - R0] = (j < j1 && row < m) ? ld_stream(M + (size_t)j * m + row) : 0.0;
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < U; q += 2) {
-      const double2 vv = *reinterpret_cast<const double2*>(v + j0 + q);
-#pragma unroll
-      for (int r = R0; r < R1; ++r) {
-        acc[r][q % NA] = fma(t[q][r - R0], vv.x, acc[r][q % NA]);
-        acc[r][(q + 1) % NA] = fma(t[q + 1][r - R0], vv.y, acc[r][(q + 1) % NA]);
-      }
-    }
-  }
-}
-
-// v = p * scale (scale = 1 / e^T z of the previous sweep when the previous
-// sweep was not normalised in memory; 1 otherwise: fl(z * (1/s)) is exactly
-// the value the normalisation would have stored).
 // CG: p was written by other SMs during this kernel, so it is read from L2
 // (ld.global.cg), never from a possibly stale L1 line.
 template <int R, bool CG = false>
 __device__ __forceinline__ void stage_vec(double* v, const double* __restrict__ p, int m,
-                                          int lane, double scale = 1.0) {
-  if (scale != 1.0) {
+                                          int lane) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int row = lane + 32 * r;
-      v[row] = row < m ? (CG ? __ldcg(p + row) : p[row]) * scale : 0.0;
-    }
-  } else {
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int row = lane + 32 * r;
-      v[row] = row < m ? (CG ? __ldcg(p + row) : p[row]) : 0.0;
-    }
+  for (int r = 0; r < R; ++r) {
+    const int row = lane + 32 * r;
+    v[row] = row < m ? (CG ? __ldcg(p + row) : p[row]) : 0.0;
   }
 }
 
 template <int R>
-__device__ __forceinline__ void zero_acc(double (&acc)[R][Tune<R>::NA]) {
+__device__ __forceinline__ void zero_acc(double (&acc)[R]) {
 #pragma unroll
-  for (int r = 0; r < R; ++r)
-#pragma unroll
-    for (int c = 0; c < Tune<R>::NA; ++c) acc[r][c] = 0.0;
-}
-
-template <int R>
-__device__ __forceinline__ double fold(const double (&a)[Tune<R>::NA]) {
-  if constexpr (Tune<R>::NA == 1) {
-    return a[0];
-  } else if constexpr (Tune<R>::NA == 4) {
-    return (a[0] + a[1]) + (a[2] + a[3]);
-  } else {
-    return a[0] + a[1];
-  }
+  for (int r = 0; r < R; ++r) acc[r] = 0.0;
 }
 
 // Deterministic block-wide sum (fixed shuffle tree, fixed warp order).
@@ -180,7 +122,7 @@ __device__ __forceinline__ double block_sum0(double v, double* sh) {
 // Off-staircase terms of a block-banded Q^T: acc += sum_j T_{l,l+d_j} v_{l+d_j}
 // with v = xlo for d_j < 0 and xup for d_j > 0 (staged through slice).
 template <int R, bool CG = false>
-__device__ __forceinline__ void far_terms(double (&acc)[R][Tune<R>::NA], const FarDesc* far,
+__device__ __forceinline__ void far_terms(double (&acc)[R], const FarDesc* far,
                                           const double* xlo, const double* xup, int64_t l,
                                           int64_t L, int m, int ms, double* slice, int lane) {
   const int n = far->n;
@@ -190,7 +132,7 @@ __device__ __forceinline__ void far_terms(double (&acc)[R][Tune<R>::NA], const F
     __syncwarp();
     stage_vec<R, CG>(slice, (far->off[j] < 0 ? xlo : xup) + k * m, m, lane);
     __syncwarp();
-    gemv_acc<R>(acc, far->plane[j] + (size_t)l * ms, slice, m, lane);
+    gemv_acc<R>(acc, far->plane[j] + (size_t)l * ms, slice, 0, m, m, lane);
   }
   __syncwarp();
 }
@@ -201,45 +143,43 @@ __device__ __forceinline__ void far_terms(double (&acc)[R][Tune<R>::NA], const F
 // share of an FP64-bound kernel, and a fused launch only needs the sums of its
 // last two sweeps.
 // CG: neighbour vectors written by other SMs during this kernel (L2 reads).
-template <int R, bool COUPLED, bool WARP_TOTAL = true, bool CG = false,
-          int UM = 1>
+template <int R, bool COUPLED, bool WARP_TOTAL = true, bool CG = false>
 __device__ __forceinline__ double level_sweep2(const double* A, const double* B, const double* C,
                                                const double* src, const double* src_up,
                                                double* dst, int64_t l, int64_t L, int m, int ms,
-                                               double* slice, int lane, double scale = 1.0,
+                                               double* slice, int lane,
                                                const FarDesc* far = nullptr,
                                                const double* xfar_lo = nullptr,
                                                const double* xfar_up = nullptr,
                                                bool want_sum = true) {
-  constexpr int NA = Tune<R>::NA, W = 32 * R;
+  constexpr int W = 32 * R;
   double* v_lo = slice;
   double* v_up = slice + W;
   double* v_g = slice + 2 * W;
   const bool has_lo = l > 0, has_up = l < L - 1;
-  if (has_lo) stage_vec<R, CG>(v_lo, src + (l - 1) * m, m, lane, scale);
-  if (has_up) stage_vec<R, CG>(v_up, src_up + (l + 1) * m, m, lane, scale);
+  if (has_lo) stage_vec<R, CG>(v_lo, src + (l - 1) * m, m, lane);
+  if (has_up) stage_vec<R, CG>(v_up, src_up + (l + 1) * m, m, lane);
   __syncwarp();
-  double acc[R][NA];
+  double acc[R];
   zero_acc<R>(acc);
-  if (has_lo) gemv_acc<R, UM>(acc, A + (size_t)l * ms, v_lo, m, lane);
-  if (has_up) gemv_acc<R, UM>(acc, B + (size_t)l * ms, v_up, m, lane);
+  if (has_lo) gemv_acc<R>(acc, A + (size_t)l * ms, v_lo, 0, m, m, lane);
+  if (has_up) gemv_acc<R>(acc, B + (size_t)l * ms, v_up, 0, m, m, lane);
   if (far) far_terms<R, CG>(acc, far, xfar_lo, xfar_up, l, L, m, ms, v_lo, lane);
   if (!COUPLED) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) v_g[lane + 32 * r] = fold<R>(acc[r]);
+    for (int r = 0; r < R; ++r) v_g[lane + 32 * r] = acc[r];
     __syncwarp();
     zero_acc<R>(acc);
-    gemv_acc<R, UM>(acc, C + (size_t)l * ms, v_g, m, lane);
+    gemv_acc<R>(acc, C + (size_t)l * ms, v_g, 0, m, m, lane);
   }
   double ls = 0.0;
   if (want_sum) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int row = lane + 32 * r;
-      const double zr = fold<R>(acc[r]);
       if (row < m) {
-        dst[l * m + row] = zr;
-        ls += zr;
+        dst[l * m + row] = acc[r];
+        ls += acc[r];
       }
     }
     if (WARP_TOTAL) ls = warp_sum(ls);
@@ -247,7 +187,7 @@ __device__ __forceinline__ double level_sweep2(const double* A, const double* B,
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int row = lane + 32 * r;
-      if (row < m) dst[l * m + row] = fold<R>(acc[r]);
+      if (row < m) dst[l * m + row] = acc[r];
     }
   }
   __syncwarp();   // the slice is rewritten for the next level
@@ -263,7 +203,7 @@ __device__ __forceinline__ double level_resid(const double* TLO, const double* T
                                               const double* x, float* q, int64_t l, int64_t L,
                                               int m, int ms, double* slice, int lane,
                                               const FarDesc* far = nullptr) {
-  constexpr int NA = Tune<R>::NA, W = 32 * R;
+  constexpr int W = 32 * R;
   double* v_lo = slice;
   double* v_dd = slice + W;
   double* v_up = slice + 2 * W;
@@ -271,31 +211,31 @@ __device__ __forceinline__ double level_resid(const double* TLO, const double* T
   stage_vec<R>(v_dd, x + l * m, m, lane);
   if (l < L - 1) stage_vec<R>(v_up, x + (l + 1) * m, m, lane);
   __syncwarp();
-  double acc[R][NA];
+  double acc[R];
   zero_acc<R>(acc);
   if (l > 0) {
-    gemv_acc<R>(acc, TLO + (size_t)l * ms, v_lo, m, lane);
+    gemv_acc<R>(acc, TLO + (size_t)l * ms, v_lo, 0, m, m, lane);
   }
-  gemv_acc<R>(acc, TDD + (size_t)l * ms, v_dd, m, lane);
+  gemv_acc<R>(acc, TDD + (size_t)l * ms, v_dd, 0, m, m, lane);
   if (l < L - 1) {
-    gemv_acc<R>(acc, TUP + (size_t)l * ms, v_up, m, lane);
+    gemv_acc<R>(acc, TUP + (size_t)l * ms, v_up, 0, m, m, lane);
   }
   if (far) far_terms<R>(acc, far, x, x, l, L, m, ms, v_lo, lane);
   double ls = 0.0;
 #pragma unroll
-  for (int r = 0; r < R; ++r) ls += fabs(fold<R>(acc[r]));
+  for (int r = 0; r < R; ++r) ls += fabs(acc[r]);
   const double total = warp_sum(ls);
   if (q) {
     __syncwarp();
 #pragma unroll
-    for (int r = 0; r < R; ++r) v_lo[lane + 32 * r] = fold<R>(acc[r]);
+    for (int r = 0; r < R; ++r) v_lo[lane + 32 * r] = acc[r];
     __syncwarp();
     zero_acc<R>(acc);
-    gemv_acc<R>(acc, NINV + (size_t)l * ms, v_lo, m, lane);
+    gemv_acc<R>(acc, NINV + (size_t)l * ms, v_lo, 0, m, m, lane);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int row = lane + 32 * r;
-      if (row < m) q[l * m + row] = (float)fold<R>(acc[r]);
+      if (row < m) q[l * m + row] = (float)acc[r];
     }
   }
   __syncwarp();

@@ -54,14 +54,6 @@ struct TeamSlot {
   uint64_t x[2][W];
 };
 
-template <int TW>
-__device__ __forceinline__ void team_sync(int bar) {
-  if constexpr (TW == 1)
-    __syncwarp();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(TW * 32) : "memory");
-}
-
 // acc[r] += sum over columns [j0b, j1) of M(row0 + lane + 32 r, j) v_j.  MC:
 // the block size when it fills the team's rows (no bounds checks), else 0.
 // etot = largest exponent of the block + of the vector.
