@@ -393,9 +393,11 @@ def run_mine(args):
     # q) and per refinement step the fused correction sweeps, the update, the
     # normalisation and the residual with q
     n_chunks = -(-args.steps // check)
-    n_kernels = 3 * n_chunks if args.dtype == "f64" else 2 + 4 * n_chunks
+    # FP64 chains that stay on chip: one launch a chunk, which reads the blocks once
+    on_chip = args.dtype == "f64" and fused and prof["launches"] == n_launch
+    n_kernels = (1 if on_chip else 3) * n_chunks if args.dtype == "f64" else 2 + 4 * n_chunks
     kern_ms = prof["sweeps_ms"] / n_launch
-    kern_bytes = bytes_level * L * sweeps_per_launch + tail_bytes
+    kern_bytes = (sweep_bytes if on_chip else bytes_level * L * sweeps_per_launch) + tail_bytes
     kern_flops = flops_level * L * sweeps_per_launch + tail_flops
     kern_ms_per_sweep = {"sweeps": prof["sweeps_ms"] / prof_steps,
                          "scale": prof["scale_ms"] / prof_steps,
@@ -418,7 +420,7 @@ def run_mine(args):
         del oc
         oracle_threads_restore()
     if args.dtype == "f64":
-        kname = ("k_sweeps_banded" if banded else "k_sweeps") if fused else "k_phase"
+        kname = "k_resident" if on_chip else "k_sweeps" if fused else "k_phase"
         key = f"{name}:{args.apply}"
     else:
         kname = "k_sweeps_lp"
@@ -435,14 +437,15 @@ def run_mine(args):
                        if fused else w["bytes_per_launch"])
     if args.dtype == "f64":
         # the products are shared between the FP64 pipe and the integer pipes, so the
-        # fused sweeps are bound by HBM; block Jacobi runs on the FP64 pipe alone
+        # fused sweeps are bound by HBM; block Jacobi and chains on chip run on the FP64
+        # pipe alone
         kn = f"{kname} (fused: {sweeps_per_launch} sweeps + residual units per launch)"
         hbm = {"achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
                "frac": achieved_gbs / hbm_peak, "peak_source": hbm_src}
         fp64 = {"achieved": achieved_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": achieved_tf / FP64_PEAK_TFLOPS,
                 "peak_source": "FP64 pipe alone, derived: 152 SMs x 2 FP64 lanes/clk x 2 flop x 2.07 GHz; the fma-loop probe (--measure-fp64-peak) measures 1.2558 TFLOP/s = 1.996 lanes/clk/SM"}
-        if fused:
+        if fused and not on_chip:
             roof = {"bound": "hbm", **hbm, "traffic": traffic, "kernel": kn, "fp64_pipe": fp64}
         else:
             roof = {"bound": "alu", **fp64, "traffic": traffic, "kernel": kn, "hbm": hbm}

@@ -68,8 +68,8 @@ typedef enum { MC_F64 = 0, MC_F32 = 1, MC_BF16 = 2 } mc_dtype;
 
 /*
  * How the diagonal-block solves Q_{i,i}^{-1} of Algorithm 2 (steps 2 and 3)
- * are applied.  Both are computed from the LU factors of mc_factor and give
- * the same iterates up to rounding.
+ * are applied.  Both come from the inverse that mc_factor forms and give the
+ * same iterates up to rounding.
  *   MC_APPLY_INVERSE: store (-Q_{i,i})^{-1} (entrywise >= 0, Q^T being a
  *     singular M-matrix up to sign) and apply it as a dense product after
  *     the neighbour products: 3 m^2 FP64 multiply-adds and 24 m^2 bytes per
@@ -162,12 +162,13 @@ int mc_create_banded(const mc_desc* desc, const double* const* diags, void* work
                      size_t ws_bytes, void* cuda_stream, mc_chain** out);
 
 /*
- * Factor the diagonal blocks Q_{i,i} (as blocks of Q^T) by batched LU without
- * pivoting (the blocks of a generator's transpose are strictly diagonally
- * dominant by columns, so no row exchange is ever needed) and form the
- * operators that apply Q_{i,i}^{-1} in Algorithm 2 steps 2 and 3 (see
- * mc_apply).  Syncs once.  Errors: MC_ERR_SINGULAR_BLOCK if a pivot is zero
- * or not finite (the handle stays unfactored), MC_ERR_CUDA.
+ * Factor the diagonal blocks Q_{i,i} (as blocks of Q^T): LU without pivoting
+ * (the blocks of a generator's transpose are strictly diagonally dominant by
+ * columns, so no row exchange is ever needed) and the inverse, in one
+ * Gauss-Jordan elimination per block, then the operators that apply
+ * Q_{i,i}^{-1} in Algorithm 2 steps 2 and 3 (see mc_apply).  Syncs once.
+ * Errors: MC_ERR_SINGULAR_BLOCK if a pivot is zero or not finite, as decided
+ * by plain LU (the handle stays unfactored), MC_ERR_CUDA.
  */
 int mc_factor(mc_chain* chain);
 
@@ -196,9 +197,9 @@ int mc_factor(mc_chain* chain);
  * Gauss-Seidel on block-tridiagonal chains run the nsweeps sweeps as one
  * persistent launch per 1024 sweeps, with no normalisation between the sweeps
  * of a launch (the scale of the iterate does not change the next one, Eq. (2)
- * up to rounding); chains that fit on chip run the whole call, normalisation
- * included, in one launch, which mc_set_tuning does not affect; x_out is normalised and stats refer to the last sweep as
- * above.  Block Jacobi (and banded block Gauss-Seidel) run one launch per
+ * up to rounding); FP64 chains that fit on chip run the whole call,
+ * normalisation included, in one launch, which mc_set_tuning does not affect;
+ * x_out is normalised and stats refer to the last sweep as above.  Block Jacobi (and banded block Gauss-Seidel) run one launch per
  * sweep.  Results are bitwise reproducible for equal calls and independent of
  * the launch configuration (mc_set_tuning); a run split into several calls
  * agrees up to rounding.
@@ -273,9 +274,10 @@ int mc_profile(mc_chain* chain, const double* x_in, double* x_out, int64_t nswee
  *   eps: stop when the step error of Sect. 3 is <= eps (evaluated every
  *     check_every sweeps); eps <= 0 disables.
  *   maxit: sweep limit (>= 1).  check_every >= 1: sweeps per check; the
- *     sweeps between checks run as one CUDA graph.
+ *     sweeps between checks run as one CUDA graph.  FP64 chains that fit on
+ *     chip make their checks on the device, up to 8192 sweeps a launch.
  *   res: receives the result (may be NULL).
- * Syncs once per check.  Errors: MC_ERR_ARG (bad sizes, x0 with a negative
+ * Syncs once per check, or launch of several checks.  Errors: MC_ERR_ARG (bad sizes, x0 with a negative
  * entry or zero sum), MC_ERR_NOT_FACTORED, MC_ERR_BREAKDOWN,
  * MC_ERR_NO_CONVERGENCE (maxit reached with tol or eps enabled; pi and res
  * still hold the last iterate), MC_ERR_CUDA.
@@ -334,9 +336,10 @@ int mc_residual_noalloc(const double* dn, const double* loc, const double* up, i
  * mc_server_step runs check_every sweeps (dtype MC_F64) or one refinement
  * step of check_every correction sweeps (MC_F32 / MC_BF16) for ALL active
  * requests in fused persistent launches side by side (one cluster per small
- * request, teams of warps by block size, a shared queue; which one follows
- * from the request's own size), then every request's FP64 residual; requests with residual <= tol
- * (or a latched error, or maxit sweeps) are retired, their pi copied to host
+ * request, teams of warps by block size, a shared queue; the request's own
+ * size decides which, and for some FP64 requests the batch, where two of them
+ * form the same sums), then every request's FP64 residual; requests with
+ * residual <= tol (or a latched error, or maxit sweeps) are retired, their pi copied to host
  * memory and their arena memory freed.  Requests submitted between steps
  * join the next chunk.  A request's iterates are bitwise independent of the
  * other requests in the batch and of every launch configuration.  With

@@ -378,10 +378,7 @@ static float* lpSc(mc_chain* c) { return (float*)(c->ws + c->lay.off_sc); }
 static float* lpQ(mc_chain* c) { return (float*)(c->ws + c->lay.off_q); }
 static float* lpD(mc_chain* c) { return (float*)(c->ws + c->lay.off_d); }
 
-// One correction sweep d <- M^{-1}(N d - r) in low precision (two launches).
-// One outer step on the iterate xa: `inner` correction sweeps from d = 0 (q
-// must hold (-T_dd)^{-1} r for the current xa), pi <- (pi + d)/e^T(pi + d)
-// with the step error, then r and q of the new iterate.
+// K correction sweeps d <- M^{-1}(N d - r) in low precision, one launch.
 static int enqueue_lp_sweeps_fused(mc_chain* c, int64_t K, cudaStream_t s) {
   if (c->res_ctas) {
     ResidentLpArgs a{};
@@ -411,6 +408,9 @@ static int enqueue_lp_sweeps_fused(mc_chain* c, int64_t K, cudaStream_t s) {
   return MC_OK;
 }
 
+// One outer step on the iterate xa: `inner` correction sweeps from d = 0 (q
+// must hold (-T_dd)^{-1} r for the current xa), pi <- (pi + d)/e^T(pi + d)
+// with the step error, then r and q of the new iterate.
 static int enqueue_refine_step(mc_chain* c, int inner, cudaStream_t s) {
   if (!c->res_ctas) CK(cudaMemsetAsync(lpD(c), 0, (size_t)c->lay.N * sizeof(float), s));
   const int rc = enqueue_lp_sweeps_fused(c, inner, s);

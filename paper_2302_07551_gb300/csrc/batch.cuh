@@ -1,24 +1,24 @@
 // Batched (multi-request) sweep: descriptors shared by batch.cu and server.cu.
 //
-// All active requests of the solve server advance together: one fused
-// persistent launch per block-size bucket covers every level of every
-// request for all sweeps of a chunk (details below).  The request
-// table lives in device memory and is rewritten by the host between chunks,
-// so one captured CUDA graph serves any active set.  Requests are ordered by
-// size class (m <= 32, m <= 64, m <= 128, m <= 256: rows per lane R <= 1, 2,
-// 4, 8); a bucket is a run of classes launched as one kernel sized for its
-// largest block, so that register use follows the bucket.  Where the bucket
-// edges lie is a tuning choice (BTune::split64).
+// All active requests of the solve server advance together: fused persistent
+// launches side by side cover every level of every request for all sweeps of
+// a chunk, by path (below).  The request table lives in device memory and is
+// rewritten by the host between chunks, so one captured CUDA graph serves any
+// active set that uses the same launches.  Requests are ordered by size class
+// (m <= 32, m <= 64, m <= 128, m <= 256).  On the low-precision queue a bucket
+// is a run of classes launched as one kernel sized for its largest block, so
+// that register use follows the bucket; where the bucket edges lie is a tuning
+// choice (BTune::split64).
 //
 // Every reduction is per level first (one partial per level), then per
 // request in level order: a request's iterates do not depend on which other
 // requests share the launch, nor on any choice of the autotuner (grid,
 // levels per unit, bucket edges, load depth).
 //
-// The sweeps of a chunk run fused (as the single-chain fused sweeps): one
-// persistent launch per bucket for all sweeps of the chunk, units claimed in
-// order, each waiting for its neighbour levels through the request's
-// completion counters.  A unit covers G adjacent levels of one half-sweep of
+// The sweeps of a chunk run fused (as the single-chain fused sweeps): all of
+// them in one persistent launch, units claimed in order, each waiting for its
+// neighbour levels through the request's completion counters.  On the queue a
+// unit covers G adjacent levels of one half-sweep of
 // one request (levels l0, l0 + 2, ..., l0 + 2 (G - 1); G per request, from
 // the table's G and the request's size class): one claim, one wait for the
 // G + 1 neighbour levels, one completion fence.  Counters grow across
@@ -151,13 +151,13 @@ struct BOut {
 // request table (its unit prefix counts depend on G).
 struct BTune {
   int blocks, threads;  // persistent grid of the fused launches
-  int split64;          // 1: m <= 64 in a launch of its own (kernel for R <= 2);
-                        // 0: m <= 128 in one launch (kernel for R <= 4)
+  int split64;          // low precision: 1: m <= 64 in a launch of its own,
+                        // 0: m <= 128 in one launch
   int deep;             // low-precision blocks of m <= 64: 16 (1) or 8 (0) loads in flight
 };
 
-// The buckets (runs of size classes launched as one kernel) of a tuning:
-// FP64 and low precision alike, [c0[i], c1[i]) for i < n.
+// The buckets (runs of size classes launched as one kernel) of a tuning of the
+// low-precision queue, [c0[i], c1[i]) for i < n.
 struct BBuckets {
   int n;
   int c0[kClasses], c1[kClasses];
@@ -177,15 +177,14 @@ inline BBuckets buckets_of(int split64) {
   return b;
 }
 
-// K FP64 sweeps of every request (fused launches, no normalisation in
-// between); then (b_sweeps_finish) e^T z, normalisation and the step error of
-// the last sweep.  t_claim: the device table's claim counters.  coupled:
-// server-wide apply mode.
+// After K FP64 sweeps of every request: e^T z, normalisation and the step error
+// of the last sweep.
 cudaError_t b_sweeps_finish(const BTable* t, BOut* out, int K, BTune g, cudaStream_t s);
 // Direct residual of every request's iterate (with_q: also q for refinement).
 cudaError_t b_resid(const BTable* t, BOut* out, int with_q, BTune g, cudaStream_t s);
 // Mixed precision: d = 0 (b_lp_zero; queue path only, the others write d once); `inner` fused correction sweeps
-// (b_lp_sweeps); pi <- (pi + d)/e^T(pi + d) with the step error (b_lp_finish).
+// (b_lp_sweeps; t_claim: the device table's claim counters; coupled: server-wide
+// apply mode); pi <- (pi + d)/e^T(pi + d) with the step error (b_lp_finish).
 cudaError_t b_lp_zero(const BTable* t, BTune g, cudaStream_t s);
 cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, int bf16,
                         int coupled, int inner, BTune g, cudaStream_t s);
@@ -195,6 +194,7 @@ cudaError_t b_lp_team(const BTable* t, unsigned long long* team_claim, BOut* out
                       int bf16, int coupled, int inner, int num_sms, const cudaStream_t* b);
 // Path of a request of this layout.
 int b_path(const Layout& lay, int coupled, int num_sms);
+// The FP64 queue's sweeps.
 cudaError_t b_sweeps(const BTable* t, unsigned long long* claim, BOut* out, int coupled, int K,
                      BTune g, cudaStream_t s);
 // The FP64 team requests' sweeps, a launch per size class on b0, b[0..2].

@@ -3,11 +3,11 @@
 // Requests (independent chains of any L and m <= 256) are admitted into a
 // caller-owned device arena as long as their workspace fits; each step runs
 // one chunk of check_every sweeps for ALL active requests with the batched
-// kernels of batch.cu (one fused persistent launch per block-size bucket for
-// all sweeps of the chunk), then reads every request's residual and retires the converged
+// kernels of batch.cu and resident.cu (fused persistent launches side by side,
+// by path: batch.cuh), then reads every request's residual and retires the converged
 // ones.  New requests join at the next chunk, so their work overlaps with the
 // requests already running.  A chunk is one CUDA graph, captured once per
-// (grid, chunk length) and replayed: the kernels read the request table from
+// (grid, chunk length, launches in use) and replayed: the kernels read the request table from
 // device memory, which the graph itself refreshes from pinned host memory.
 #include <math.h>
 #include <stdlib.h>
@@ -635,6 +635,15 @@ int mc_server_submit(mc_server* s, int64_t tag, int64_t L, int32_t m, const doub
   r->step_prev = NAN;
   r->path = b_path(y, s->d.apply == MC_APPLY_COUPLED, s->num_sms);
   r->group = resident_batch_group(y, s->d.apply == MC_APPLY_COUPLED);
+  // a chain that would stay on chip by itself has no row exponents yet; teams use them
+  if (c->res_ctas && y.lp == 0 && m > 16 && r->path == kPathTeam &&
+      launch_weak_rows(P, chain_bexp(c, 0), y, s->d.apply == MC_APPLY_COUPLED, s->user) !=
+          cudaSuccess) {
+    mc_destroy(c);
+    release(s, off, bytes);
+    delete r;
+    return MC_ERR_CUDA;
+  }
   r->vbase = 0;
   r->fresh = true;
   if (reset_team_words(s, r) != cudaSuccess) {
