@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(256) k_b_resid(const BTable* __restrict__ t, i
     if (LARGE) {
       ls = level_resid<8>(q->TLO, q->TDD, q->TUP, q->NINV, q->x, qv, l, q->L, q->m, q->ms, slice, lane);
     } else {
-      switch (q->R) {
+      switch ((q->m + 31) / 32) {
         case 1: ls = level_resid<1>(q->TLO, q->TDD, q->TUP, q->NINV, q->x, qv, l, q->L, q->m, q->ms, slice, lane); break;
         case 2: ls = level_resid<2>(q->TLO, q->TDD, q->TUP, q->NINV, q->x, qv, l, q->L, q->m, q->ms, slice, lane); break;
         case 3: ls = level_resid<3>(q->TLO, q->TDD, q->TUP, q->NINV, q->x, qv, l, q->L, q->m, q->ms, slice, lane); break;

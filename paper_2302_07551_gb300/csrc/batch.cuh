@@ -57,7 +57,8 @@ struct BReq {
   const int2* eA;       // FP64: block_exp of A, B, C (team path)
   const int2* eB;
   const int2* eC;
-  int32_t m, ms, R, p1;  // p1: 0-based parity of the diagonal-only rows
+  int32_t m, ms, smem, p1;  // smem: shared memory of a CTA of the resident path; p1: 0-based
+                            // parity of the diagonal-only rows
   int32_t G, path;       // levels per unit of this request (the table's G scaled by size
                          // class); kPathQueue, ...
   int32_t vbase;         // FP64 team path: sweeps that the counters have seen
@@ -115,7 +116,7 @@ constexpr int kResidentSlots = 8;      // sets of 16 SMs given to clusters
 __host__ __device__ constexpr int group_share(int group) {
   return group == 0 ? 2 : group == 2 ? 4 : group == 3 ? 2 : 1;
 }
-__host__ __device__ constexpr bool group_wide(int group) { return group >= 2; }
+__host__ __device__ constexpr bool group_wide(int group) { return group == 2 || group == 3; }
 
 struct BTable {
   int32_t n;            // active requests, ordered by size class
@@ -204,6 +205,7 @@ cudaError_t b_team(const BTable* t, unsigned long long* team_claim, BOut* out, i
 // a group's requests (lp: 0 FP64, 1 FP32, 2 BF16); res_c and res_s of an FP64 request.
 int resident_cluster();
 int resident_batch_group(const Layout& lay, int coupled);
+int resident_batch_smem(const Layout& lay, int coupled);
 cudaError_t launch_resident_batch(const BTable* t, int lp, int coupled, int group, int K, BOut* out,
                                   cudaStream_t s);
 void resident_order(const Layout& lay, int16_t* c, int16_t* s);

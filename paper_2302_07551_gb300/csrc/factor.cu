@@ -107,6 +107,9 @@ __device__ __forceinline__ bool cancels(double piv, double diag) {
   return (((unsigned)__double2hiint(piv) >> 20) & 0x7ffu) + 45u <
          (((unsigned)__double2hiint(diag) >> 20) & 0x7ffu);
 }
+__device__ __forceinline__ bool no_pivot(double piv, double diag) {
+  return !(piv != 0.0) || !isfinite(piv) || cancels(piv, diag);
+}
 
 // LU of one block without pivoting and (-T)^{-1} by substitution, in place in
 // global memory, by a CTA: rare, so that only the call costs the kernels above
@@ -255,7 +258,6 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
         const double* cl = col + (k & 1) * MP;
         if (G != 16 || (threadIdx.x >> 5) == (k & 7)) {
           const double piv = base[k] + rw[k];
-          if (!(piv != 0.0) || !isfinite(piv) || cancels(piv, base[k])) s_bad[grp] = 1;
           const double p = 1.0 / piv;
           for (int i = G == 16 ? (int)(threadIdx.x & 31) : t; i < m; i += G == 16 ? 32 : G * G) {
             const double c = cl[i] * p;
@@ -263,6 +265,9 @@ __global__ void __launch_bounds__(256, GjBlock<G, R>::B) k_gj(const double* __re
             if (i > k) LU[k * (m + 1) + i] = c;
             if (i >= k) LU[i * (m + 1) + k] = i == k ? piv : rw[i];
           }
+          if (G != 16 && no_pivot(piv, base[k])) s_bad[grp] = 1;
+        } else if (threadIdx.x == 32 * ((k + 1) & 7)) {   // another warp, not on the critical path
+          if (no_pivot(base[k] + rw[k], base[k])) s_bad[grp] = 1;
         }
         sync();
         bad = s_bad[grp] != 0;

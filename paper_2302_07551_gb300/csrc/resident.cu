@@ -178,7 +178,7 @@ __host__ __device__ inline int cluster_ctas(int64_t L, int most) {
 
 // Dynamic shared memory of this launch: a request whose share does not fit it (none
 // does not: its group follows from its size) is reported and left out.
-__device__ __forceinline__ size_t dyn_smem() {
+__device__ __forceinline__ unsigned dyn_smem() {
   unsigned v;
   asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(v));
   return v;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, group_share(GROUP))
     ClusterLink<float> ln;
     ln.status = &out[r].status;
     ln.c = cluster_ctas(Q.L, most);
-    if (carve<S, float, float, COUPLED>((int)((Q.L + ln.c - 1) / ln.c), Q.m).total > dyn_smem()) {
+    if (Q.smem > (int)dyn_smem()) {
       atomicCAS(ln.status, 0, (int)MC_ERR_CUDA);
       continue;   // the whole cluster
     }
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     ClusterLink<double> ln;
     ln.status = &out[r].status;
     ln.c = cluster_ctas(Q.L, most);
-    if (carve<double, double, double, COUPLED>((int)((Q.L + ln.c - 1) / ln.c), Q.m).total > dyn_smem()) {
+    if (Q.smem > (int)dyn_smem()) {
       atomicCAS(ln.status, 0, (int)MC_ERR_CUDA);
       continue;   // the whole cluster
     }
@@ -305,7 +305,8 @@ KernelBatch kernel_batch(int lp, int coupled, int group) {
   if (lp == 0) return coupled ? k_b_resident64<true> : k_b_resident64<false>;
   return group < 2    ? kernel_batch_lp<0>(lp, coupled)
          : group == 2 ? kernel_batch_lp<2>(lp, coupled)
-                      : kernel_batch_lp<3>(lp, coupled);
+         : group == 3 ? kernel_batch_lp<3>(lp, coupled)
+                      : kernel_batch_lp<4>(lp, coupled);
 }
 // Dynamic shared memory of a group's CTAs: an SM's 228 KB by the CTAs that share it,
 // less 1 KB each and the static arrays.
@@ -399,7 +400,8 @@ Limits limits() {
              opt_in((const void*)kernel_lp(lp, c, true), false) &&
              opt_in((const void*)kernel_batch(lp, c, 0), true) &&
              opt_in((const void*)kernel_batch(lp, c, 2), true) &&
-             opt_in((const void*)kernel_batch(lp, c, 3), true);
+             opt_in((const void*)kernel_batch(lp, c, 3), true) &&
+             opt_in((const void*)kernel_batch(lp, c, 4), true);
     }
     if (ok) {
       for (int C = 16; C >= 8 && !l.cluster; C /= 2) {
@@ -411,7 +413,8 @@ Limits limits() {
             runs = runs && cluster_runs((const void*)kernel_lp(lp, c, false), C) &&
                    cluster_runs((const void*)kernel_batch(lp, c, 0), C) &&
                    cluster_runs((const void*)kernel_batch(lp, c, 2), C) &&
-                   cluster_runs((const void*)kernel_batch(lp, c, 3), C);
+                   cluster_runs((const void*)kernel_batch(lp, c, 3), C) &&
+                   cluster_runs((const void*)kernel_batch(lp, c, 4), C);
         }
         if (runs) l.cluster = C;
       }
@@ -482,6 +485,10 @@ int resident_batch_group(const Layout& y, int coupled) {
   int g = y.m > 16 ? 2 : 0;
   while (need > group_smem(g)) ++g;
   return g;
+}
+
+int resident_batch_smem(const Layout& y, int coupled) {
+  return (int)smem_bytes(y, coupled, cluster_ctas(y.L, limits().cluster));
 }
 
 void resident_order(const Layout& y, int16_t* c, int16_t* s) {

@@ -767,7 +767,7 @@ __device__ __forceinline__ void sweeps(const Chain<T, TC, V>& h, int K, unsigned
   const int tid = threadIdx.x;
   const Cover c = cover(m, (nmax + 1) / 2);   // the same in every CTA
   const int cpl = (m + c.S - 1) / c.S;
-  const bool tiny = !WIDE && is_tiny(m, (nmax + 1) / 2, c);
+  const bool tiny = !WIDE && m <= 16 && ((nmax + 1) / 2) * c.gs <= kThreads && cpl <= 8;   // is_tiny
   if (first) {
     ln.open(Side<V>{x, z, l0, n, m, h.par0, K, r > 0, r < C - 1},
             r > 0 ? l0 - range_begin(L, C, r - 1) : 0, sh);

@@ -170,7 +170,7 @@ void fill_req(const mc_server* s, const Req* r, BReq* q) {
   q->L = c->lay.L;
   q->m = c->lay.m;
   q->ms = c->lay.ms;
-  q->R = (c->lay.m + 31) / 32;
+  if (r->path == kPathResident) q->smem = resident_batch_smem(c->lay, coupled);
   q->p1 = s->d.stair == 1 ? 0 : 1;
   q->path = r->path;
 }
@@ -440,6 +440,15 @@ std::vector<Req*> build_table(mc_server* s) {
   t->G = s->G;
   t->off_h1[0] = t->off_h2[0] = t->off_lv[0] = t->off_t1[0] = t->off_t2[0] = 0;
   const bool overflow = residents_overflow(s), small_queue = small_teams_overflow(s);
+  // a few of the wide ones that could share an SM do not, or less, in the kernel with more
+  // registers (two of 168 x 32, BF16: 0.152 -> 0.144 ms a chunk; eight of 140 x 32 two to an
+  // SM 0.157, one 0.234, four 0.177)
+  int wide = 0;
+  for (const Req* r : s->active) wide += r->path == kPathResident && (r->group == 2 || r->group == 3);
+  auto group_now = [wide](int g) {
+    if (g != 2 && g != 3) return g;
+    return wide <= kResidentSlots / 2 ? 4 : wide <= kResidentSlots ? 3 : g;
+  };
   int64_t team_levels[kClasses] = {0, 0, 0, 0};
   const int p1 = s->d.stair == 1 ? 0 : 1;
   for (int i = 0; i < t->n; ++i) {
@@ -466,8 +475,10 @@ std::vector<Req*> build_table(mc_server* s) {
     if (team) team_levels[cls(r)] += L;
   }
   for (int g = 0, n = 0; g < kResGroups; ++g) {
-    for (int i = 0; i < t->n; ++i)
-      if (t->r[i].path == kPathResident && s->active[(size_t)i]->group == g) t->res[n++] = i;
+    for (int i = 0; i < t->n; ++i) {
+      if (t->r[i].path == kPathResident && group_now(s->active[(size_t)i]->group) == g)
+        t->res[n++] = i;
+    }
     t->res_end[g] = n;
   }
   deal_ctas(s, t, team_levels);
@@ -502,6 +513,13 @@ int process_outputs(mc_server* s, const std::vector<Req*>& order, int c) {
     }
   }
   return nd;
+}
+
+// The stream and the event of a side launch, made with its first request.
+bool open_side(mc_server* s, int i) {
+  return (s->side[i] || cudaStreamCreateWithFlags(&s->side[i], cudaStreamNonBlocking) == cudaSuccess) &&
+         (s->join[i] ||
+          cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming) == cudaSuccess);
 }
 
 // Pinned memory, streams and events (those that exist).
@@ -554,9 +572,6 @@ int mc_server_create(const mc_server_desc* desc, void* arena, size_t arena_bytes
             cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) == cudaSuccess &&
             cudaEventCreateWithFlags(&s->fork[0], cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&s->fork[1], cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < kSides && ok; ++i)
-    ok = cudaStreamCreateWithFlags(&s->side[i], cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
     free_host_side(s);
     delete s;
@@ -635,10 +650,16 @@ int mc_server_submit(mc_server* s, int64_t tag, int64_t L, int32_t m, const doub
   r->step_prev = NAN;
   r->path = b_path(y, s->d.apply == MC_APPLY_COUPLED, s->num_sms);
   r->group = resident_batch_group(y, s->d.apply == MC_APPLY_COUPLED);
+  const int side = r->path == kPathResident ? r->group
+                   : r->path == kPathTeam   ? kResGroups - 1 + size_class(m)
+                                            : -1;
+  bool ok = side < (r->path == kPathTeam ? kResGroups : 0) || open_side(s, side);
+  if (side == 2 || side == 3) ok = ok && open_side(s, 3) && open_side(s, 4);   // build_table
   // a chain that would stay on chip by itself has no row exponents yet; teams use them
-  if (c->res_ctas && y.lp == 0 && m > 16 && r->path == kPathTeam &&
-      launch_weak_rows(P, chain_bexp(c, 0), y, s->d.apply == MC_APPLY_COUPLED, s->user) !=
-          cudaSuccess) {
+  if (ok && c->res_ctas && y.lp == 0 && m > 16 && r->path == kPathTeam)
+    ok = launch_weak_rows(P, chain_bexp(c, 0), y, s->d.apply == MC_APPLY_COUPLED, s->user) ==
+         cudaSuccess;
+  if (!ok) {
     mc_destroy(c);
     release(s, off, bytes);
     delete r;
