@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(256) k_layout(const double* dn, const double* 
 // A diagonal entry is kept in two parts, its value at the start (or the inverse
 // pivot) and the sum of its updates, added where it is used: m updates rounded
 // at the size of the dominant diagonal would be most of the inverse's error
-// (m = 256: 6.9e-16 against 0.9e-16 relative, 3.3e-16 for blocked LU and solves).
+// (relative error over 8192 blocks of 64: LU and solves 4.3e-16, this 2.0e-16).
 // Whether a pivot vanishes is decided by plain LU: a block one of whose pivots
 // cancels to below 2^-45 of its diagonal entry, or is no number, is given up here
 // and formed again by plain_block, with true divisions (a / -a is -1, a * (1 / -a)
