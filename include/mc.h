@@ -199,8 +199,8 @@ int mc_factor(mc_chain* chain);
  * of a launch (the scale of the iterate does not change the next one, Eq. (2)
  * up to rounding); FP64 chains that fit on chip run the whole call,
  * normalisation included, in one launch, which mc_set_tuning does not affect;
- * x_out is normalised and stats refer to the last sweep as above.  Block Jacobi (and banded block Gauss-Seidel) run one launch per
- * sweep.  Results are bitwise reproducible for equal calls and independent of
+ * x_out is normalised and stats refer to the last sweep as above.  Block
+ * Jacobi (and banded block Gauss-Seidel) run one launch per sweep.  Results are bitwise reproducible for equal calls and independent of
  * the launch configuration (mc_set_tuning); a run split into several calls
  * agrees up to rounding.
  * Async.  Errors: MC_ERR_ARG, MC_ERR_NOT_FACTORED, MC_ERR_CUDA; a breakdown

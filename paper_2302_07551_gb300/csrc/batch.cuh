@@ -183,8 +183,8 @@ inline BBuckets buckets_of(int split64) {
 cudaError_t b_sweeps_finish(const BTable* t, BOut* out, int K, BTune g, cudaStream_t s);
 // Direct residual of every request's iterate (with_q: also q for refinement).
 cudaError_t b_resid(const BTable* t, BOut* out, int with_q, BTune g, cudaStream_t s);
-// Mixed precision: d = 0 (b_lp_zero; queue path only, the others write d once); `inner` fused correction sweeps
-// (b_lp_sweeps; t_claim: the device table's claim counters; coupled: server-wide
+// Mixed precision: d = 0 (b_lp_zero; queue path only, the others write d once);
+// `inner` fused correction sweeps (b_lp_sweeps; t_claim: the device table's claim counters; coupled: server-wide
 // apply mode); pi <- (pi + d)/e^T(pi + d) with the step error (b_lp_finish).
 cudaError_t b_lp_zero(const BTable* t, BTune g, cudaStream_t s);
 cudaError_t b_lp_sweeps(const BTable* t, unsigned long long* t_claim, BOut* out, int bf16,
@@ -201,8 +201,9 @@ cudaError_t b_sweeps(const BTable* t, unsigned long long* claim, BOut* out, int 
 // The FP64 team requests' sweeps, a launch per size class on b0, b[0..2].
 cudaError_t b_team(const BTable* t, unsigned long long* team_claim, BOut* out, int paths,
                    int coupled, int K, int num_sms, cudaStream_t b0, const cudaStream_t* b);
-// resident.cu: CTAs of a cluster (0: none can run); the group of a request that fits one cluster, else -1; the launch of
-// a group's requests (lp: 0 FP64, 1 FP32, 2 BF16); res_c and res_s of an FP64 request.
+// resident.cu: CTAs of a cluster (0: none can run); the group of a request that fits
+// one cluster, else -1, and a CTA's shared memory; res_c and res_s of an FP64 request;
+// the launch of a group's requests (lp: 0 FP64, 1 FP32, 2 BF16).
 int resident_cluster();
 int resident_batch_group(const Layout& lay, int coupled);
 int resident_batch_smem(const Layout& lay, int coupled);

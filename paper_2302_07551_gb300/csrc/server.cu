@@ -337,9 +337,9 @@ double chunk_sweep_bytes(const mc_server* s, int c) {
 }
 
 // Autotuner: for each batch signature (size classes present, whether any
-// request is on the queue, size class of the total level count) time one live chunk per candidate configuration
-// (real work, counted as such: results do not depend on the configuration)
-// and keep the fastest.  Coordinate search: the persistent grid (1, 2, 3, 4,
+// request is on the queue, size class of the total level count) time one live
+// chunk per candidate configuration (real work, counted as such: results do not
+// depend on the configuration) and keep the fastest.  Coordinate search: the persistent grid (1, 2, 3, 4,
 // 6, 8 resident 256-thread blocks per SM) with one level per unit, then 2
 // and 4 levels per unit, then the other bucket edge, then (low precision
 // with m <= 64 present) the other load depth.
